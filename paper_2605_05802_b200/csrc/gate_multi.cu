@@ -10,10 +10,10 @@
 //   prep     one CTA per (group, pattern rollout): hashes the pattern's symbols
 //            in shared memory, then translates every text paired with it into a
 //            "loc" stream: for text column c the position of the column's symbol in
-//            the pattern (0x7FFF: absent; bit 15 set: several occurrences, walk
-//            the pattern's chain).  A block's match word is then just
-//            1 << (loc - first_row_of_block), no table lookup.  Also bins the pairs
-//            by (team shape, text length).
+//            the pattern (0x7FFF: absent).  A block's match word is then just
+//            1 << (loc - first_row_of_block), no table lookup.  A symbol with several
+//            occurrences gets a row of match words instead, and the stream names the row.
+//            Also bins the pairs by (team shape, text length).
 //   order    counting sort of the pairs by bin: longest warp tasks first, one team
 //            shape and similar text lengths per bin; warp-task table.
 //   dp       persistent warps pull tasks.  A task is a warp of 32/T teams; a team of
@@ -57,8 +57,11 @@ constexpr int kNumClasses = 32;     // team shapes (T lanes x R blocks), see cla
 constexpr int kLenBuckets = 32;     // buckets of estimated task duration
 constexpr int kNumBins = kNumClasses * kLenBuckets;
 constexpr uint32_t kLocNone = 0x7FFFu;    // bit 15 clear, far above any row: shifts to 0
-constexpr uint32_t kLocMulti = 0x8000u;
+constexpr uint32_t kLocRow = 0x8000u;     // | index of the symbol's mask row
+constexpr uint32_t kLocChain = 0xC000u;   // | first position of the symbol's occurrence chain
 constexpr uint32_t kChainEnd = 0xFFFFu;
+constexpr int kRepeatedFlag = 0x10000;    // a text's stream holds row or chain entries
+constexpr int kPosPerThread = SR_MAX_K / kPrepThreads;
 constexpr int kDpWarpsPerCta = 4;
 constexpr uint32_t kBinMask = 0x3FFu;
 constexpr int32_t kCappedFlag = 0x40000000;   // decide mode: the pair's distance exceeds its cap
@@ -88,8 +91,10 @@ struct Ctl {               // int32 control block in the workspace
 };
 
 struct MultiWs {
-    size_t off_dist, off_desc, off_loc, off_next, off_order, off_ctl, off_flag, total;
+    size_t off_dist, off_desc, off_loc, off_next, off_order, off_ctl, off_flag, off_rows, total;
     int pitch;             // uint16 elements per loc / chain row
+    int row_words;         // 32-bit words of a mask row: one per 32 pattern positions
+    int row_cap;           // mask rows a pattern may have
     int min_tlog;          // small batches: teams of at least 2^min_tlog lanes
 };
 
@@ -106,6 +111,13 @@ MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K) {
     w.off_order = off; off = align_up(off + (size_t)n_groups * P * 4, 256);
     w.off_next = off;  off = align_up(off + (size_t)n_groups * N * w.pitch * 2, 256);
     w.off_loc = off;   off = align_up(off + (size_t)n_groups * P * w.pitch * 2, 256);
+    // Mask rows for an eighth of the positions: symbols with at least eight occurrences always
+    // fit, and 1/rank token frequencies put no more than about K / 10 symbols above one.  A team's
+    // lanes cover up to seven words more than the pattern has: slack after the last row.
+    w.row_words = (K + 31) >> 5;
+    w.row_cap = (K + 7) >> 3;
+    w.off_rows = off;
+    off = align_up(off + (size_t)n_groups * N * w.row_cap * w.row_words * 4 + 256, 256);
     w.total = off;
     return w;
 }
@@ -217,19 +229,15 @@ __device__ __forceinline__ unsigned long long make_slot(int32_t sym, uint32_t po
     return ((unsigned long long)(uint32_t)sym << 32) | pos_plus_1;
 }
 
-// Position (or chain head) of `sym` in the pattern hashed in shared memory, given the
-// content `v` of its home slot `h` (read by the caller, so that the first probes of the
-// four look-ups of a quad are in flight together).
+// Stream entry of `sym` (its position, mask row or chain in the pattern hashed in shared
+// memory), given the content `v` of its home slot `h` (read by the caller, so that the first
+// probes of the four look-ups of a quad are in flight together).
 __device__ __forceinline__ uint32_t pattern_lookup(int32_t sym, uint32_t h, unsigned long long v,
-                                                   const unsigned long long* s_slot,
-                                                   const uint32_t* s_next, int hslots) {
+                                                   const unsigned long long* s_slot, int hslots) {
     for (int probe = 0; probe < hslots; ++probe) {     // an empty slot always exists
         const uint32_t o = (uint32_t)v;
         if (o == 0u) break;
-        if ((int32_t)(v >> 32) == sym) {
-            const uint32_t first = o - 1u;
-            return s_next[first] == kChainEnd ? first : (kLocMulti | first);
-        }
+        if ((int32_t)(v >> 32) == sym) return o - 1u;
         h = (h + 1u) & (uint32_t)(hslots - 1);
         v = s_slot[h];
     }
@@ -245,9 +253,10 @@ __global__ void __launch_bounds__(kPrepThreads, 6)
 multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int32_t* dist_out, int g_base) {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned long long* s_slot = reinterpret_cast<unsigned long long*>(smem);    // [hslots_max]
-    uint32_t* s_next = reinterpret_cast<uint32_t*>(s_slot + hslots_max);         // [pitch]
+    uint32_t* s_info = reinterpret_cast<uint32_t*>(s_slot + hslots_max);         // [pitch]
     __shared__ int s_txt[SR_MAX_N], s_len[SR_MAX_N], s_qstart[SR_MAX_N + 1], s_absent[SR_MAX_N];
     __shared__ int s_cp[SR_MAX_N], s_differ[SR_MAX_N];
+    __shared__ int s_repeats[4];     // symbols with >= 2, 3, 4 occurrences; mask rows handed out
     // (At K = 1024 the 36 KB of dynamic plus these 656 bytes of static shared memory sit just
     // under the size at which six CTAs share an SM: 512 bytes more were measured to cost one
     // CTA per SM and a fifth of the kernel's speed.  Smaller tables with more CTAs per SM are
@@ -269,7 +278,8 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
     while (hslots < 4 * m) hslots <<= 1;
     const int hshift = __clz(hslots) + 1;             // 32 - log2(hslots)
     for (int q = tid; 4 * q < m; q += kPrepThreads)
-        reinterpret_cast<uint4*>(s_next)[q] = make_uint4(kChainEnd, kChainEnd, kChainEnd, kChainEnd);
+        reinterpret_cast<uint4*>(s_info)[q] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < 4) s_repeats[tid] = 0;
     for (int h = tid; h < hslots; h += kPrepThreads) s_slot[h] = 0ull;
     // The texts this pattern is paired with, one warp per text.  The warp also measures the
     // common prefix of pattern and text (128 positions per trip, stopping at the first
@@ -324,18 +334,23 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
         int quads = 0;
         for (int t = 0; t < ntxt; ++t) {
             const int lo = min(m, s_len[t]);
-            // the removed prefix is a multiple of four symbols (the match stream is read in
-            // 8-byte quads); if one prefix is the start of the other nothing is left to do
-            const int strip = s_cp[t] >= lo ? -1 : (s_cp[t] & ~3);
-            s_cp[t] = strip;
+            // if one prefix is the start of the other nothing is left to do
+            if (s_cp[t] >= lo) s_cp[t] = -1;
             s_qstart[t] = quads;
-            quads += strip < 0 ? 0 : (s_len[t] - strip + 3) >> 2;
+            quads += s_cp[t] < 0 ? 0 : (s_len[t] - (s_cp[t] & ~31) + 3) >> 2;
         }
         s_qstart[ntxt] = quads;
     }
-    // every position claims the slot of its symbol, or links itself behind the
-    // position that claimed it (the claimant heads the symbol's occurrence chain)
-    for (int p = tid; p < m; p += kPrepThreads) {
+    // Every position claims the slot of its symbol or counts itself as a further occurrence
+    // with the position that did (s_info[claimant]).
+    uint32_t my_slot[kPosPerThread], my_first[kPosPerThread];
+    bool repeated = false;
+#pragma unroll
+    for (int k = 0; k < kPosPerThread; ++k) {
+        const int p = tid + k * kPrepThreads;
+        my_slot[k] = 0u;
+        my_first[k] = (uint32_t)p;
+        if (p >= m) continue;
         const int32_t sym = __ldg(pat + p);
         uint32_t h = ((uint32_t)sym * 0x9E3779B1u) >> hshift;
         const unsigned long long mine = make_slot(sym, (uint32_t)p + 1u);
@@ -344,15 +359,61 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
             if ((uint32_t)v == 0u) v = atomicCAS(&s_slot[h], 0ull, mine);
             if ((uint32_t)v == 0u) break;
             if ((int32_t)(v >> 32) == sym) {
-                s_next[p] = atomicExch(&s_next[(uint32_t)v - 1u], (uint32_t)p);
+                my_first[k] = (uint32_t)v - 1u;
+                atomicAdd(&s_info[my_first[k]], 1u);
+                repeated = true;
                 break;
             }
             h = (h + 1u) & (uint32_t)(hslots - 1);
         }
+        my_slot[k] = h;
     }
-    __syncthreads();
-    uint16_t* g_next = reinterpret_cast<uint16_t*>(ws + W.off_next) + ((size_t)g * N + i) * W.pitch;
-    for (int p = tid; p < m; p += kPrepThreads) g_next[p] = (uint16_t)s_next[p];
+    if (__syncthreads_or(repeated)) {
+        // Symbols with several occurrences.  In written language a few tokens make up much of
+        // every rollout (a third of the columns of such a text meet a symbol that occurs more
+        // than once, the most common one dozens of times), so these get a row of match words,
+        // one per 32 positions, which the recurrence reads in place of its one-hot word.  The
+        // pool has room for every symbol with at least eight occurrences; what does not fit
+        // (the rarest of the repeated ones) is left as a chain of at most seven positions.
+#pragma unroll
+        for (int k = 0; k < kPosPerThread; ++k) {
+            const int p = tid + k * kPrepThreads;
+            if (p >= m || my_first[k] != (uint32_t)p) continue;
+            const uint32_t more = s_info[p];
+            for (uint32_t c = 0; c < 3u && c < more; ++c) atomicAdd(&s_repeats[c], 1);
+        }
+        __syncthreads();
+        const uint32_t need = s_repeats[0] <= W.row_cap ? 1u : (s_repeats[1] <= W.row_cap ? 2u : (s_repeats[2] <= W.row_cap ? 3u : 7u));
+#pragma unroll
+        for (int k = 0; k < kPosPerThread; ++k) {
+            const int p = tid + k * kPrepThreads;
+            if (p >= m || my_first[k] != (uint32_t)p) continue;
+            const uint32_t more = s_info[p];
+            if (more == 0u) continue;
+            const uint32_t code = more >= need ? kLocRow | (uint32_t)atomicAdd(&s_repeats[3], 1) : kLocChain | (uint32_t)p;
+            s_info[p] = more >= need ? code : kChainEnd;
+            s_slot[my_slot[k]] = make_slot(__ldg(pat + p), code + 1u);
+        }
+        __syncthreads();
+        uint32_t* rows = reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * N + i) * W.row_cap * W.row_words;
+        for (int e = tid; e < s_repeats[3] * W.row_words; e += kPrepThreads) rows[e] = 0u;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kPosPerThread; ++k) {
+            const int p = tid + k * kPrepThreads;
+            if (p >= m) continue;
+            const uint32_t f = my_first[k], info = s_info[f];
+            if ((info & kLocChain) == kLocRow)         // not a chain's end (all bits set) nor a count or position
+                atomicOr(&rows[(info & 0x3FFFu) * W.row_words + (p >> 5)], 1u << (p & 31));
+            else if (f != (uint32_t)p)
+                s_info[p] = atomicExch(&s_info[f], (uint32_t)p);
+        }
+        if (s_repeats[0] > s_repeats[3]) {             // some chains: leave them for the recurrence
+            __syncthreads();
+            uint16_t* g_next = reinterpret_cast<uint16_t*>(ws + W.off_next) + ((size_t)g * N + i) * W.pitch;
+            for (int p = tid; p < m; p += kPrepThreads) g_next[p] = (uint16_t)s_info[p];
+        }
+    }
 
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     uint16_t* locs = reinterpret_cast<uint16_t*>(ws + W.off_loc);
@@ -363,7 +424,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
     for (int item = tid; item < total_quads; item += kPrepThreads) {
         int t = 0;
         while (item >= s_qstart[t + 1]) ++t;
-        const int q = (s_cp[t] >> 2) + item - s_qstart[t];      // quad index within the text
+        const int q = ((s_cp[t] & ~31) >> 2) + item - s_qstart[t];      // quad index within the text
         const int j = s_txt[t];
         const int lo = min(i, j), hi = max(i, j);
         const size_t idx = (size_t)g * P + pair_index(lo, hi, N);
@@ -371,19 +432,22 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
         const uint32_t h0 = ((uint32_t)sym.x * 0x9E3779B1u) >> hshift, h1 = ((uint32_t)sym.y * 0x9E3779B1u) >> hshift;
         const uint32_t h2 = ((uint32_t)sym.z * 0x9E3779B1u) >> hshift, h3 = ((uint32_t)sym.w * 0x9E3779B1u) >> hshift;
         const unsigned long long v0 = s_slot[h0], v1 = s_slot[h1], v2 = s_slot[h2], v3 = s_slot[h3];
-        const uint32_t l0 = pattern_lookup(sym.x, h0, v0, s_slot, s_next, hslots);
-        const uint32_t l1 = pattern_lookup(sym.y, h1, v1, s_slot, s_next, hslots);
-        const uint32_t l2 = pattern_lookup(sym.z, h2, v2, s_slot, s_next, hslots);
-        const uint32_t l3 = pattern_lookup(sym.w, h3, v3, s_slot, s_next, hslots);
+        const uint32_t l0 = pattern_lookup(sym.x, h0, v0, s_slot, hslots);
+        const uint32_t l1 = pattern_lookup(sym.y, h1, v1, s_slot, hslots);
+        const uint32_t l2 = pattern_lookup(sym.z, h2, v2, s_slot, hslots);
+        const uint32_t l3 = pattern_lookup(sym.w, h3, v3, s_slot, hslots);
         reinterpret_cast<uint2*>(locs + idx * W.pitch)[q] = make_uint2(l0 | (l1 << 16), l2 | (l3 << 16));
+        // columns past the text's end hold whatever the row holds: harmless to count as repeated
+        if (((l0 | l1 | l2 | l3) & kLocRow) && !(s_absent[t] & kRepeatedFlag)) atomicOr(&s_absent[t], kRepeatedFlag);
         if (kBounds) {
-            // positions below both lengths whose symbol is not the pattern's symbol at the same
-            // place (a symbol with several occurrences may be counted although it matches: the
-            // count only has to be an upper bound of the mismatches)
+            // positions below both lengths whose symbol is not the pattern's symbol at the same place
             const int both = min(m, s_len[t]) - 4 * q;       // columns of this quad below both lengths
-            const uint32_t c0 = 4u * (uint32_t)q;
-            const int differ = (both > 0 && l0 != c0) + (both > 1 && l1 != c0 + 1u) +
-                               (both > 2 && l2 != c0 + 2u) + (both > 3 && l3 != c0 + 3u);
+            int differ = 0;
+            if (both > 0) {
+                const int4 own = __ldg(reinterpret_cast<const int4*>(pat) + q);
+                differ = (sym.x != own.x) + (both > 1 && sym.y != own.y) + (both > 2 && sym.z != own.z) +
+                         (both > 3 && sym.w != own.w);
+            }
             if (differ) atomicAdd(&s_differ[t], differ);
             const int left = s_len[t] - 4 * q;           // columns of this quad that exist
             const int absent = (l0 == kLocNone) + (left > 1 && l1 == kLocNone) +
@@ -391,9 +455,12 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
             if (absent) atomicAdd(&s_absent[t], absent);
         }
     }
-    if (kBounds) __syncthreads();
+    __syncthreads();
     if (tid < ntxt) {                                 // descriptors, bins, trivial pairs
-        const int j = s_txt[tid], n = s_len[tid], strip = s_cp[tid];
+        const int j = s_txt[tid], n = s_len[tid];
+        // the removed prefix is a multiple of four symbols (the match stream is read in 8-byte
+        // quads), and of 32 where the stream refers to mask rows (whose words start there)
+        const int strip = s_cp[tid] < 0 ? -1 : (s_cp[tid] & (s_absent[tid] & kRepeatedFlag ? ~31 : ~3));
         const int lo = min(i, j), hi = max(i, j);
         const size_t idx = (size_t)g * P + pair_index(lo, hi, N);
         if (strip < 0) {                              // one prefix starts the other (or is empty)
@@ -405,7 +472,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
             // the decide mode bands its pairs: 0xFFFF stands for "no bound")
             const int upper = kBounds ? s_differ[tid] + abs(m - n) : 0xFFFF;
             const int bin = shape_and_bin(m - strip, n - strip, upper, W.min_tlog);
-            const int lower = kBounds ? max(abs(m - n), s_absent[tid]) : 0;
+            const int lower = kBounds ? max(abs(m - n), s_absent[tid] & (kRepeatedFlag - 1)) : 0;
             descs[idx] = PairDesc{(uint32_t)m | ((uint32_t)n << 16), (uint32_t)(g * N + i),
                                   (uint32_t)bin | ((uint32_t)strip << kStripShift) | kNeedsDp,
                                   (uint32_t)lower | ((uint32_t)upper << 16)};
@@ -488,28 +555,50 @@ __device__ __forceinline__ uint32_t shl_clamp(uint32_t v, uint32_t s) {
     return r;
 }
 
-// One bit-vector column step over the R blocks a lane owns.  `loc` is the column's
-// entry of the match stream, (inP, inM) the pre-shift horizontal delta words of the
+// Match words of a quad of text columns for the R blocks a lane owns.  A position becomes a
+// one-hot word; an entry that names a mask row is read from it (`rows` points at the lane's
+// first word of the pattern's first row); a chain is walked.  Runs one quad ahead of the
+// recurrence, so that the loads of the rows are in flight while the previous quad is worked on.
+template <int R>
+__device__ __forceinline__ void match_words(uint2 q, uint32_t rowbase, int m, const uint32_t* __restrict__ rows,
+                                            int row_words, const uint16_t* __restrict__ nxt,
+                                            uint32_t (&Eq)[4][R]) {
+    const uint32_t loc[4] = {q.x & 0xFFFFu, q.x >> 16, q.y & 0xFFFFu, q.y >> 16};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const uint32_t d0 = loc[u] - rowbase;
+#pragma unroll
+        for (int r = 0; r < R; ++r) Eq[u][r] = shl_clamp(1u, d0 - 32u * r);
+    }
+    if ((q.x | q.y) & (kLocRow | (kLocRow << 16))) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (!(loc[u] & kLocRow)) continue;
+            if ((loc[u] & kLocChain) == kLocRow) {
+                const uint32_t* row = rows + (loc[u] & 0x3FFFu) * (uint32_t)row_words;
+#pragma unroll
+                for (int r = 0; r < R; ++r) Eq[u][r] = __ldg(row + r);
+            } else {
+                uint32_t p = loc[u] & 0x3FFFu;
+                for (int hop = 0; hop < SR_MAX_K && p < (uint32_t)m; ++hop) {   // chain ends at 0xFFFF
+                    const uint32_t dd = p - rowbase;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) Eq[u][r] |= shl_clamp(1u, dd - 32u * r);
+                    p = __ldg(nxt + p);
+                }
+            }
+        }
+    }
+}
+
+// One bit-vector column step over the R blocks a lane owns.  `Eq` are the column's match
+// words, (inP, inM) the pre-shift horizontal delta words of the
 // block above (only their top bits matter); returns this lane's last block's words in
 // (inP, inM).
 template <int R>
-__device__ __forceinline__ void column_step(uint32_t loc, uint32_t rowbase, int m,
-                                            const uint16_t* __restrict__ nxt,
+__device__ __forceinline__ void column_step(const uint32_t (&Eq)[R],
                                             uint32_t (&Pv)[R], uint32_t (&Mv)[R],
                                             uint32_t& inP, uint32_t& inM, uint32_t two) {
-    const uint32_t d0 = loc - rowbase;
-    uint32_t Eq[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) Eq[r] = shl_clamp(1u, d0 - 32u * r);
-    if (loc & kLocMulti) {          // several occurrences in the pattern: walk the chain
-        uint32_t p = loc & 0x7FFFu;
-        for (int hop = 0; hop < SR_MAX_K && p < (uint32_t)m; ++hop) {   // chain ends at 0xFFFF
-            const uint32_t dd = p - rowbase;
-#pragma unroll
-            for (int r = 0; r < R; ++r) Eq[r] |= shl_clamp(1u, dd - 32u * r);
-            p = __ldg(nxt + p);
-        }
-    }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const uint32_t pv = Pv[r], mv = Mv[r];
@@ -543,8 +632,8 @@ __device__ __forceinline__ void column_step(uint32_t loc, uint32_t rowbase, int 
 template <int R>
 __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDesc* descs,
                                         const int32_t* order, const uint16_t* locs,
-                                        const uint16_t* nexts, int pitch, int32_t* dist_out,
-                                        uint32_t two) {
+                                        const uint16_t* nexts, const uint32_t* masks, MultiWs W,
+                                        int32_t* dist_out, uint32_t two) {
     const int lane = threadIdx.x & 31;
     const int T = 1 << tlog;
     const int lt = lane & (T - 1);
@@ -553,6 +642,7 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
     int idx = 0, m_all = 0, m = 0, n = 0, strip = 0;
     const uint2* loc4 = reinterpret_cast<const uint2*>(locs);
     const uint16_t* nxt = nexts;
+    const uint32_t* rows = masks;
     if (valid) {
         idx = order[pos];
         const PairDesc d = descs[idx];
@@ -561,8 +651,9 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
         m = m_all - strip;
         n = (int)(d.mn >> 16) - strip;
         // rows are 16-byte aligned and strip is a multiple of 4 entries: 8-byte loads
-        loc4 = reinterpret_cast<const uint2*>(locs + (size_t)idx * pitch + strip);
-        nxt = nexts + (size_t)d.pat_row * pitch;
+        loc4 = reinterpret_cast<const uint2*>(locs + (size_t)idx * W.pitch + strip);
+        nxt = nexts + (size_t)d.pat_row * W.pitch;
+        rows = masks + (size_t)d.pat_row * (W.row_cap * W.row_words) + (strip >> 5) + lt * R;
     }
     const uint32_t rowbase = (uint32_t)(lt * R * 32);
     const uint32_t rowabs = rowbase + (uint32_t)strip;          // first pattern position of this lane
@@ -576,13 +667,16 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
     for (int r = 0; r < R; ++r) { Pv[r] = 0xFFFFFFFFu; Mv[r] = 0u; }
     uint32_t outP[4] = {0u, 0u, 0u, 0u}, outM[4] = {0u, 0u, 0u, 0u};
     const uint2 none = make_uint2(kLocNone | (kLocNone << 16), kLocNone | (kLocNone << 16));
-    uint2 q_next = (valid && top) ? __ldg(loc4) : none;
+    uint2 q_next = valid ? (top ? __ldg(loc4) : none) : none;
+    uint32_t Eq[4][R];
+    match_words<R>(q_next, rowabs, m_all, rows, W.row_words, nxt, Eq);
+    q_next = (valid && 1 - lt >= 0 && 1 - lt < nq) ? __ldg(loc4 + 1 - lt) : none;
 
     for (int j = 0; j < iters; ++j) {
         const int qi = j - lt;
         const bool active = valid && qi >= 0 && qi < nq;
-        const uint2 q = q_next;
-        q_next = (valid && qi + 1 >= 0 && qi + 1 < nq) ? __ldg(loc4 + qi + 1) : none;
+        const uint2 q = q_next;                         // the quad after this one
+        q_next = (valid && qi + 2 >= 0 && qi + 2 < nq) ? __ldg(loc4 + qi + 2) : none;
         // delta words leaving the lane above for this quad (it worked on it last iteration)
         uint32_t inP[4], inM[4];
 #pragma unroll
@@ -593,13 +687,14 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
         }
         if (active) {
             const int left = n - 4 * qi;               // columns of this quad that exist (>= 1)
-            column_step<R>(q.x & 0xFFFFu, rowabs, m_all, nxt, Pv, Mv, inP[0], inM[0], two);
-            if (left > 1) column_step<R>(q.x >> 16, rowabs, m_all, nxt, Pv, Mv, inP[1], inM[1], two);
-            if (left > 2) column_step<R>(q.y & 0xFFFFu, rowabs, m_all, nxt, Pv, Mv, inP[2], inM[2], two);
-            if (left > 3) column_step<R>(q.y >> 16, rowabs, m_all, nxt, Pv, Mv, inP[3], inM[3], two);
+            column_step<R>(Eq[0], Pv, Mv, inP[0], inM[0], two);
+            if (left > 1) column_step<R>(Eq[1], Pv, Mv, inP[1], inM[1], two);
+            if (left > 2) column_step<R>(Eq[2], Pv, Mv, inP[2], inM[2], two);
+            if (left > 3) column_step<R>(Eq[3], Pv, Mv, inP[3], inM[3], two);
 #pragma unroll
             for (int u = 0; u < 4; ++u) { outP[u] = inP[u]; outM[u] = inM[u]; }
         }
+        match_words<R>(q, rowabs, m_all, rows, W.row_words, nxt, Eq);
     }
     // D[m][n] = n + (sum of the vertical deltas of the last column over rows 1..m)
     int part = 0;
@@ -628,8 +723,8 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
 template <int R>
 __device__ __noinline__ void dp_task_band(int tlog, int pos, bool valid, const PairDesc* descs,
                                              const int32_t* order, const uint16_t* locs,
-                                             const uint16_t* nexts, int pitch, int32_t* dist_out,
-                                             uint32_t two) {
+                                             const uint16_t* nexts, const uint32_t* masks, MultiWs W,
+                                             int32_t* dist_out, uint32_t two) {
     const int lane = threadIdx.x & 31;
     const int T = 1 << tlog;
     const int lt = lane & (T - 1);
@@ -637,6 +732,7 @@ __device__ __noinline__ void dp_task_band(int tlog, int pos, bool valid, const P
     int idx = 0, m_all = 0, m = 0, n = 0, strip = 0, ub = 0;
     const uint2* loc4 = reinterpret_cast<const uint2*>(locs);
     const uint16_t* nxt = nexts;
+    const uint32_t* rows = masks;
     if (valid) {
         idx = order[pos];
         const PairDesc d = descs[idx];
@@ -645,8 +741,9 @@ __device__ __noinline__ void dp_task_band(int tlog, int pos, bool valid, const P
         m = m_all - strip;
         n = (int)(d.mn >> 16) - strip;
         ub = (int)(d.lower >> 16);
-        loc4 = reinterpret_cast<const uint2*>(locs + (size_t)idx * pitch + strip);
-        nxt = nexts + (size_t)d.pat_row * pitch;
+        loc4 = reinterpret_cast<const uint2*>(locs + (size_t)idx * W.pitch + strip);
+        nxt = nexts + (size_t)d.pat_row * W.pitch;
+        rows = masks + (size_t)d.pat_row * (W.row_cap * W.row_words) + (strip >> 5);
     }
     int dlo, dhi;
     band_of(m, n, ub, dlo, dhi);
@@ -714,21 +811,23 @@ __device__ __noinline__ void dp_task_band(int tlog, int pos, bool valid, const P
             before = base + (int)up - (int)down;
             const uint32_t rowabs = (uint32_t)(strip + 32 * R * g);
             const int left = n - 4 * qi;               // columns of this quad that exist (>= 1)
-            column_step<R>(q.x & 0xFFFFu, rowabs, m_all, nxt, Pv, Mv, inP[0], inM[0], two);
+            uint32_t Eq[4][R];
+            match_words<R>(q, rowabs, m_all, rows + R * g, W.row_words, nxt, Eq);
+            column_step<R>(Eq[0], Pv, Mv, inP[0], inM[0], two);
             up = __umulhi(inP[0], two) + up;           // top bit of the word: the delta leaving the stripe
             down = __umulhi(inM[0], two) + down;
             if (left > 1) {
-                column_step<R>(q.x >> 16, rowabs, m_all, nxt, Pv, Mv, inP[1], inM[1], two);
+                column_step<R>(Eq[1], Pv, Mv, inP[1], inM[1], two);
                 up = __umulhi(inP[1], two) + up;
                 down = __umulhi(inM[1], two) + down;
             }
             if (left > 2) {
-                column_step<R>(q.y & 0xFFFFu, rowabs, m_all, nxt, Pv, Mv, inP[2], inM[2], two);
+                column_step<R>(Eq[2], Pv, Mv, inP[2], inM[2], two);
                 up = __umulhi(inP[2], two) + up;
                 down = __umulhi(inM[2], two) + down;
             }
             if (left > 3) {
-                column_step<R>(q.y >> 16, rowabs, m_all, nxt, Pv, Mv, inP[3], inM[3], two);
+                column_step<R>(Eq[3], Pv, Mv, inP[3], inM[3], two);
                 up = __umulhi(inP[3], two) + up;
                 down = __umulhi(inM[3], two) + down;
             }
@@ -764,6 +863,7 @@ multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
     const int32_t* order = reinterpret_cast<const int32_t*>(ws + W.off_order);
     const uint16_t* locs = reinterpret_cast<const uint16_t*>(ws + W.off_loc);
     const uint16_t* nexts = reinterpret_cast<const uint16_t*>(ws + W.off_next);
+    const uint32_t* masks = reinterpret_cast<const uint32_t*>(ws + W.off_rows);
     const int lane = threadIdx.x & 31;
     const int total = ctl->total_tasks;
     int32_t* counter = kBand ? &ctl->task_counter_band : &ctl->task_counter;
@@ -785,19 +885,19 @@ multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
         const bool valid = pos < ctl->start[k] + ctl->fill[k];     // fill = pairs in the bin
         if (kBand) {
             switch (R) {
-                case 1: dp_task_band<1>(tlog, pos, valid, descs, order, locs, nexts, W.pitch, dist_out, two); break;
-                case 2: dp_task_band<2>(tlog, pos, valid, descs, order, locs, nexts, W.pitch, dist_out, two); break;
-                case 3: dp_task_band<3>(tlog, pos, valid, descs, order, locs, nexts, W.pitch, dist_out, two); break;
-                default: dp_task_band<4>(tlog, pos, valid, descs, order, locs, nexts, W.pitch, dist_out, two); break;
+                case 1: dp_task_band<1>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+                case 2: dp_task_band<2>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+                case 3: dp_task_band<3>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+                default: dp_task_band<4>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
             }
         } else {
             switch (R) {
-                case 1: dp_task<1>(tlog, pos, valid, descs, order, locs, nexts, W.pitch, dist_out, two); break;
-                case 2: dp_task<2>(tlog, pos, valid, descs, order, locs, nexts, W.pitch, dist_out, two); break;
-                case 3: dp_task<3>(tlog, pos, valid, descs, order, locs, nexts, W.pitch, dist_out, two); break;
-                case 4: dp_task<4>(tlog, pos, valid, descs, order, locs, nexts, W.pitch, dist_out, two); break;
-                case 5: dp_task<5>(tlog, pos, valid, descs, order, locs, nexts, W.pitch, dist_out, two); break;
-                default: dp_task<6>(tlog, pos, valid, descs, order, locs, nexts, W.pitch, dist_out, two); break;
+                case 1: dp_task<1>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+                case 2: dp_task<2>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+                case 3: dp_task<3>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+                case 4: dp_task<4>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+                case 5: dp_task<5>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+                default: dp_task<6>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
             }
         }
     }

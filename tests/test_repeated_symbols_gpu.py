@@ -1,0 +1,26 @@
+"""Multi-word gate on prefixes whose symbols occur several times: mask rows, the occurrence
+count from which a symbol gets one, the chains of the others, and common prefixes of such pairs."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import assert_gate_matches, gate_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("K", [33, 64, 500, 1024])
+@pytest.mark.parametrize("times", [2, 3, 4, 7, 8, 60])
+def test_symbols_with_a_given_number_of_occurrences(K, times):
+    rng = np.random.default_rng(1000 * K + times)
+    G, N, stride = 6, 5, (K + 3) // 4 * 4
+    pool = np.arange(stride) // times                       # every symbol `times` times ...
+    seqs = np.stack([[rng.permutation(pool) for _ in range(N)] for _ in range(G)]).astype(np.int32)
+    seqs[1] += rng.integers(0, 40000, size=(N, stride)) * (rng.random((N, stride)) < 0.5)   # ... or some of them once
+    seqs[2:5, :, : K // 2] = seqs[2:5, :1, : K // 2]        # common prefixes
+    seqs[4, :, 31] += np.arange(N)                          # ... that end around a word boundary
+    seqs[5] = seqs[5, :1]
+    lens = rng.integers(K // 3, K + 1, size=(G, N)).astype(np.int32)
+    lens[0] = K
+    want = oracle.gate(seqs, lens, K, 0.4, threads=8)
+    assert_gate_matches(gate_gpu(seqs, lens, K, 0.4), want, f"K={K}, {times} occurrences")
