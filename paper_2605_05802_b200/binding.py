@@ -1,6 +1,8 @@
-"""Thin ctypes binding of the sr_gate C ABI (include/sr_gate.h, include/sr_probe.h).
+"""Thin binding of the sr_gate C ABI (include/sr_gate.h, include/sr_probe.h).
 
-Argument marshalling only: every step of the path runs in the CUDA library.
+Argument marshalling only: every step of the path runs in the CUDA library.  The calls
+a program makes per batch or per step go through a compiled extension
+(csrc/torch_binding.cpp), the host-only and measurement entry points through ctypes.
 PyTorch tensors are used as device (or pinned host) memory and for streams.  There
 is no CPU fallback: if the shared library is missing or fails to load, every call
 raises.
@@ -15,6 +17,7 @@ import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libsr_gate.so")
+NATIVE_PATH = os.path.join(HERE, "_native.so")
 
 SR_OK = 0
 SR_ERR_NULL, SR_ERR_BAD_N, SR_ERR_BAD_K, SR_ERR_ALIGN = -1, -2, -3, -4
@@ -89,8 +92,25 @@ def load() -> ctypes.CDLL:
     return _lib
 
 
-def _check(rc: int) -> None:
-    if rc != SR_OK:
+_native_module = None
+
+
+def _native():
+    """The compiled half of this module (csrc/torch_binding.cpp): argument checks and the calls."""
+    global _native_module
+    if _native_module is None:
+        load()
+        try:
+            from . import _native as module
+        except ImportError as e:
+            raise SrError(SR_ERR_CUDA, f"{NATIVE_PATH} is missing or does not load ({e}): build it with "
+                                       "`python -m paper_2605_05802_b200.build`; there is no fallback path")
+        _native_module = module
+    return _native_module
+
+
+def _check(rc: Optional[int]) -> None:
+    if rc:
         lib = load()
         msg = lib.sr_strerror(rc).decode()
         if rc == SR_ERR_CUDA:
@@ -140,13 +160,8 @@ def sr_gate(seqs: torch.Tensor, lens: Optional[torch.Tensor], K: int, threshold:
             stop: torch.Tensor = None, status: Optional[torch.Tensor] = None,
             workspace: Optional[torch.Tensor] = None, stream=None) -> None:
     """seqs int32 [G, N, stride] on the device; outputs are preallocated tensors."""
-    G, N, stride = seqs.shape
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load().sr_gate(_ptr(seqs, torch.int32), _ptr(lens, torch.int32, need=G * N, name="lens"), G, N, stride, K,
-                          float(threshold), norm_mode, _ptr(pair_dist, torch.int32, need=G * (N * (N - 1) // 2), name="pair_dist"),
-                          _ptr(pair_sum, torch.int32, need=G, name="pair_sum"), _ptr(mean, torch.float64, need=G, name="mean"),
-                          _ptr(stop, torch.uint8, need=G, name="stop"), _ptr(status, torch.int32, need=1, name="status"), _ptr(workspace),
-                          ws_bytes, _stream(stream)))
+    _check(_native().sr_gate(seqs, lens, K, threshold, norm_mode, pair_dist, pair_sum, mean, stop, status,
+                             workspace, stream))
 
 
 def sr_gate_noalloc_limit_bytes() -> int:
@@ -161,12 +176,8 @@ def sr_gate_noalloc(seqs: torch.Tensor, lens: Optional[torch.Tensor], K: int, th
     scratch is a fixed array inside the library; problems whose scratch need exceeds
     sr_gate_noalloc_limit_bytes() are refused with SR_ERR_SCRATCH_LIMIT.  Calls that
     may overlap on the device must be serialised by the caller."""
-    G, N, stride = seqs.shape
-    _check(load().sr_gate_noalloc(_ptr(seqs, torch.int32), _ptr(lens, torch.int32, need=G * N, name="lens"), G, N, stride, K,
-                                  float(threshold), norm_mode, _ptr(pair_dist, torch.int32, need=G * (N * (N - 1) // 2), name="pair_dist"),
-                                  _ptr(pair_sum, torch.int32, need=G, name="pair_sum"), _ptr(mean, torch.float64, need=G, name="mean"),
-                                  _ptr(stop, torch.uint8, need=G, name="stop"), _ptr(status, torch.int32, need=1, name="status"),
-                                  _stream(stream)))
+    _check(_native().sr_gate_noalloc(seqs, lens, K, threshold, norm_mode, pair_dist, pair_sum, mean, stop,
+                                     status, stream))
 
 
 def sr_gate_decide(seqs: torch.Tensor, lens: Optional[torch.Tensor], K: int, threshold: float,
@@ -174,13 +185,8 @@ def sr_gate_decide(seqs: torch.Tensor, lens: Optional[torch.Tensor], K: int, thr
                    stop=None, exact=None, status=None, workspace=None, stream=None) -> None:
     """Same stop mask as sr_gate; groups that a lower bound of d_K already dismisses are
     not computed (exact[g] = 0 marks them, their other outputs are lower bounds)."""
-    G, N, stride = seqs.shape
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load().sr_gate_decide(_ptr(seqs, torch.int32), _ptr(lens, torch.int32, need=G * N, name="lens"), G, N, stride, K,
-                                 float(threshold), norm_mode, _ptr(pair_dist, torch.int32, need=G * (N * (N - 1) // 2), name="pair_dist"),
-                                 _ptr(pair_sum, torch.int32, need=G, name="pair_sum"), _ptr(mean, torch.float64, need=G, name="mean"),
-                                 _ptr(stop, torch.uint8, need=G, name="stop"), _ptr(exact, torch.uint8, need=G, name="exact"),
-                                 _ptr(status, torch.int32, need=1, name="status"), _ptr(workspace), ws_bytes, _stream(stream)))
+    _check(_native().sr_gate_decide(seqs, lens, K, threshold, norm_mode, pair_dist, pair_sum, mean, stop,
+                                    exact, status, workspace, stream))
 
 
 def sr_gate_stages(seqs, lens, K, threshold, norm_mode=SR_NORM_MAXLEN, *, pair_dist=None, pair_sum=None,
@@ -210,13 +216,8 @@ def sr_gate_host(seqs: torch.Tensor, lens: Optional[torch.Tensor], K: int, thres
     for t in (seqs, lens, pair_dist, pair_sum, mean, stop, status):
         if t is not None and t.is_cuda:
             raise ValueError("sr_gate_host takes host tensors")
-    G, N, stride = seqs.shape
-    _check(load().sr_gate_host(_ptr(seqs, torch.int32, host=True, name="seqs"), _ptr(lens, torch.int32, need=G * N, host=True, name="lens"), G, N, stride, K,
-                               float(threshold), norm_mode, _ptr(pair_dist, torch.int32, need=G * (N * (N - 1) // 2), host=True, name="pair_dist"),
-                               _ptr(pair_sum, torch.int32, need=G, host=True, name="pair_sum"), _ptr(mean, torch.float64, need=G, host=True, name="mean"),
-                               _ptr(stop, torch.uint8, need=G, host=True, name="stop"), _ptr(status, torch.int32, need=1, host=True, name="status"), _ptr(arena),
-                               arena.numel() * arena.element_size(), _stream(stream),
-                               None if copy_stream is None else copy_stream.cuda_stream))
+    _check(_native().sr_gate_host(seqs, lens, K, threshold, norm_mode, pair_dist, pair_sum, mean, stop, status,
+                                  arena, stream, copy_stream))
 
 
 def sr_gate_host_packed_arena_bytes(n_groups: int, N: int, stride: int, K: int) -> int:
@@ -232,17 +233,8 @@ def sr_gate_host_packed(symbols: torch.Tensor, row_start: torch.Tensor, N: int, 
     for t in (symbols, row_start, pair_dist, pair_sum, mean, stop, status):
         if t is not None and t.is_cuda:
             raise ValueError("sr_gate_host_packed takes host tensors")
-    rows = row_start.numel() - 1
-    if rows < 0 or rows % N:
-        raise ValueError("row_start needs n_groups * N + 1 entries")
-    G = rows // N
-    _check(load().sr_gate_host_packed(_ptr(symbols, torch.int32, host=True, name="symbols"), _ptr(row_start, torch.int64, host=True, name="row_start"),
-                                      rows // N, N, stride, K, float(threshold), norm_mode,
-                                      _ptr(pair_dist, torch.int32, need=G * (N * (N - 1) // 2), host=True, name="pair_dist"), _ptr(pair_sum, torch.int32, need=G, host=True, name="pair_sum"),
-                                      _ptr(mean, torch.float64, need=G, host=True, name="mean"), _ptr(stop, torch.uint8, need=G, host=True, name="stop"),
-                                      _ptr(status, torch.int32, need=1, host=True, name="status"), _ptr(arena),
-                                      arena.numel() * arena.element_size(), _stream(stream),
-                                      None if copy_stream is None else copy_stream.cuda_stream))
+    _check(_native().sr_gate_host_packed(symbols, row_start, N, stride, K, threshold, norm_mode, pair_dist,
+                                         pair_sum, mean, stop, status, arena, stream, copy_stream))
 
 
 def sr_incr_state_bytes(n_groups: int, N: int, max_steps: int) -> int:
@@ -250,48 +242,33 @@ def sr_incr_state_bytes(n_groups: int, N: int, max_steps: int) -> int:
 
 
 def sr_incr_init(state: torch.Tensor, n_groups: int, N: int, max_steps: int, stream=None) -> None:
-    _check(load().sr_incr_init(_ptr(state), state.numel() * state.element_size(), n_groups, N,
-                               max_steps, _stream(stream)))
+    _check(_native().sr_incr_init(state, n_groups, N, max_steps, stream))
 
 
 def sr_gate_step_incremental(state: torch.Tensor, new_actions: torch.Tensor, threshold: float,
                              norm_mode: int = SR_NORM_MAXLEN, *, pair_dist=None, pair_sum=None,
                              mean=None, stop=None, status=None, stream=None) -> None:
-    G, N = new_actions.shape
-    _check(load().sr_gate_step_incremental(
-        _ptr(state), state.numel() * state.element_size(), _ptr(new_actions, torch.int32, name="new_actions"), G, N,
-        float(threshold), norm_mode, _ptr(pair_dist, torch.int32, need=G * (N * (N - 1) // 2), name="pair_dist"), _ptr(pair_sum, torch.int32, need=G, name="pair_sum"),
-        _ptr(mean, torch.float64, need=G, name="mean"), _ptr(stop, torch.uint8, need=G, name="stop"), _ptr(status, torch.int32, need=1, name="status"),
-        _stream(stream)))
+    _check(_native().sr_gate_step_incremental(state, new_actions, threshold, norm_mode, pair_dist, pair_sum,
+                                              mean, stop, status, stream))
 
 
 def sr_gate_or_rule(mean: torch.Tensor, lens: Optional[torch.Tensor], done: Optional[torch.Tensor],
                     N: int, K: int, threshold: float, tau_high: float, *, tau: Optional[torch.Tensor] = None,
                     stop: torch.Tensor = None, stream=None) -> None:
-    G = mean.shape[0]
-    _check(load().sr_gate_or_rule(_ptr(mean, torch.float64), _ptr(lens, torch.int32, need=G * N, name="lens"),
-                                  _ptr(done, torch.uint8, need=G * N, name="done"), mean.shape[0], N, K, float(threshold),
-                                  float(tau_high), _ptr(tau, torch.float64, need=G, name="tau"), _ptr(stop, torch.uint8, need=G, name="stop"),
-                                  _stream(stream)))
+    _check(_native().sr_gate_or_rule(mean, lens, done, N, K, threshold, tau_high, tau, stop, stream))
 
 
 def sr_group_signals(seqs: torch.Tensor, lens: Optional[torch.Tensor], K: int, *,
                      unique_prefix_ratio=None, unique_action_ratio=None, action_entropy=None,
                      bigram_jaccard_mean=None, stream=None) -> None:
-    G, N, stride = seqs.shape
-    _check(load().sr_group_signals(_ptr(seqs, torch.int32), _ptr(lens, torch.int32, need=G * N, name="lens"), G, N, stride, K,
-                                   _ptr(unique_prefix_ratio, torch.float64, need=G, name="unique_prefix_ratio"),
-                                   _ptr(unique_action_ratio, torch.float64, need=G, name="unique_action_ratio"),
-                                   _ptr(action_entropy, torch.float64, need=G, name="action_entropy"),
-                                   _ptr(bigram_jaccard_mean, torch.float64, need=G, name="bigram_jaccard_mean"), _stream(stream)))
+    _check(_native().sr_group_signals(seqs, lens, K, unique_prefix_ratio, unique_action_ratio, action_entropy,
+                                      bigram_jaccard_mean, stream))
 
 
 def sr_batch_stats(adv: torch.Tensor, stop: Optional[torch.Tensor], *, counts: torch.Tensor,
                    sumsq: torch.Tensor, stream=None) -> None:
     """counts: int64 [3] device tensor, sumsq: float64 [2] device tensor (see sr_gate.h)."""
-    G, N = adv.shape
-    _check(load().sr_batch_stats(_ptr(adv, torch.float32), _ptr(stop, torch.uint8, need=G, name="stop"), G, N,
-                                 _ptr(counts, torch.int64, need=3, name="counts"), _ptr(sumsq, torch.float64, need=2, name="sumsq"), _stream(stream)))
+    _check(_native().sr_batch_stats(adv, stop, counts, sumsq, stream))
 
 
 def sr_kept_groups_workspace_bytes(n_groups: int) -> int:
@@ -303,12 +280,7 @@ def sr_kept_groups(stop: Optional[torch.Tensor], zero_var: Optional[torch.Tensor
                    stream=None) -> None:
     """index int32 [n_groups], count int32 [1] (device): ascending indices of the groups
     with stop == 0 (and zero_var == 0 when given)."""
-    if n_groups is None:
-        n_groups = (stop if stop is not None else zero_var if zero_var is not None else index).shape[0]
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load().sr_kept_groups(_ptr(stop, torch.uint8, need=n_groups, name="stop"), _ptr(zero_var, torch.uint8, need=n_groups, name="zero_var"), n_groups,
-                                 _ptr(index, torch.int32, need=n_groups, name="index"), _ptr(count, torch.int32, need=1, name="count"), _ptr(workspace),
-                                 ws_bytes, _stream(stream)))
+    _check(_native().sr_kept_groups(stop, zero_var, index, count, workspace, n_groups, stream))
 
 
 def sr_savings_fraction(cut: int, n_groups: int, T_max: int, K: int) -> float:
@@ -321,10 +293,7 @@ def sr_dilution_gain(before: float, after: float) -> float:
 
 def sr_grpo_advantage(rewards: torch.Tensor, drop_mask: Optional[torch.Tensor], eps: float, *,
                       adv: torch.Tensor, zero_var: Optional[torch.Tensor] = None, stream=None) -> None:
-    G, N = rewards.shape
-    _check(load().sr_grpo_advantage(_ptr(rewards, torch.float32), _ptr(drop_mask, torch.uint8, need=G, name="drop_mask"), G, N,
-                                    float(eps), _ptr(adv, torch.float32, need=G * N, name="adv"), _ptr(zero_var, torch.uint8, need=G, name="zero_var"),
-                                    _stream(stream)))
+    _check(_native().sr_grpo_advantage(rewards, drop_mask, eps, adv, zero_var, stream))
 
 
 def sr_probe_int32(variant: int, iters: int, blocks: int, threads: int, sink: torch.Tensor,
