@@ -14,6 +14,7 @@ __global__ void __launch_bounds__(256)
 advantage_kernel(const float* __restrict__ rewards, const uint8_t* __restrict__ drop_mask,
                  int n_groups, int n_rt, float eps, float* __restrict__ adv,
                  uint8_t* __restrict__ zero_var) {
+    grid_begin();
     const int N = NT > 0 ? NT : n_rt;
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= n_groups) return;
@@ -81,12 +82,11 @@ int launch_advantage(const float* rewards, const uint8_t* drop_mask, int32_t n_g
     // the vector path needs 16-byte aligned rows
     const bool aligned = ((reinterpret_cast<uintptr_t>(rewards) | reinterpret_cast<uintptr_t>(adv)) & 15) == 0;
     if (N == 8 && aligned)
-        advantage_kernel<8><<<blocks, threads, 0, s>>>(rewards, drop_mask, n_groups, N, eps, adv, zero_var);
+        SR_LAUNCH("advantage_kernel", advantage_kernel<8>, blocks, threads, 0, s, rewards, drop_mask, n_groups, N, eps, adv, zero_var);
     else if (N == 16 && aligned)
-        advantage_kernel<16><<<blocks, threads, 0, s>>>(rewards, drop_mask, n_groups, N, eps, adv, zero_var);
+        SR_LAUNCH("advantage_kernel", advantage_kernel<16>, blocks, threads, 0, s, rewards, drop_mask, n_groups, N, eps, adv, zero_var);
     else
-        advantage_kernel<0><<<blocks, threads, 0, s>>>(rewards, drop_mask, n_groups, N, eps, adv, zero_var);
-    SR_LAUNCH_CHECK("advantage_kernel");
+        SR_LAUNCH("advantage_kernel", advantage_kernel<0>, blocks, threads, 0, s, rewards, drop_mask, n_groups, N, eps, adv, zero_var);
     return SR_OK;
 }
 

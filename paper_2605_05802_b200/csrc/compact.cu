@@ -57,6 +57,7 @@ template <bool kVec>
 __global__ void __launch_bounds__(kTileThreads)
 kept_count_kernel(const uint8_t* __restrict__ stop, const uint8_t* __restrict__ zero_var,
                   int n_groups, int32_t* __restrict__ tile_count) {
+    grid_begin();
     __shared__ int s_warp[kTileThreads / 32];
     const int base = (blockIdx.x * kTileThreads + threadIdx.x) * kPerThread;
     int c = base < n_groups ? __popc(kept_bits<kVec>(stop, zero_var, base, n_groups)) : 0;
@@ -74,6 +75,7 @@ kept_count_kernel(const uint8_t* __restrict__ stop, const uint8_t* __restrict__ 
 // a batch of 4 M groups has about a thousand tiles.
 __global__ void __launch_bounds__(1024)
 kept_offsets_kernel(int32_t* __restrict__ tile_count, int n_tiles, int32_t* __restrict__ count) {
+    grid_begin();
     __shared__ int s_warp[32];
     __shared__ int s_carry;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -115,6 +117,7 @@ __global__ void __launch_bounds__(kTileThreads)
 kept_scatter_kernel(const uint8_t* __restrict__ stop, const uint8_t* __restrict__ zero_var,
                     int n_groups, const int32_t* __restrict__ tile_offset,
                     int32_t* __restrict__ index) {
+    grid_begin();
     __shared__ int s_warp[kTileThreads / 32];
     __shared__ int32_t s_idx[kTile];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -162,14 +165,11 @@ int launch_kept_groups(const uint8_t* stop, const uint8_t* zero_var, int32_t n_g
     int32_t* tiles = static_cast<int32_t*>(ws);
     const int n_tiles = (n_groups + kTile - 1) / kTile;
     const bool vec = ((reinterpret_cast<uintptr_t>(stop) | reinterpret_cast<uintptr_t>(zero_var)) & 15) == 0;
-    if (vec) kept_count_kernel<true><<<n_tiles, kTileThreads, 0, s>>>(stop, zero_var, n_groups, tiles);
-    else kept_count_kernel<false><<<n_tiles, kTileThreads, 0, s>>>(stop, zero_var, n_groups, tiles);
-    SR_LAUNCH_CHECK("kept_count_kernel");
-    kept_offsets_kernel<<<1, 1024, 0, s>>>(tiles, n_tiles, count);
-    SR_LAUNCH_CHECK("kept_offsets_kernel");
-    if (vec) kept_scatter_kernel<true><<<n_tiles, kTileThreads, 0, s>>>(stop, zero_var, n_groups, tiles, index);
-    else kept_scatter_kernel<false><<<n_tiles, kTileThreads, 0, s>>>(stop, zero_var, n_groups, tiles, index);
-    SR_LAUNCH_CHECK("kept_scatter_kernel");
+    if (vec) SR_LAUNCH("kept_count_kernel", kept_count_kernel<true>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles);
+    else SR_LAUNCH("kept_count_kernel", kept_count_kernel<false>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles);
+    SR_LAUNCH("kept_offsets_kernel", kept_offsets_kernel, 1, 1024, 0, s, tiles, n_tiles, count);
+    if (vec) SR_LAUNCH("kept_scatter_kernel", kept_scatter_kernel<true>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles, index);
+    else SR_LAUNCH("kept_scatter_kernel", kept_scatter_kernel<false>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles, index);
     return SR_OK;
 }
 

@@ -251,6 +251,7 @@ __device__ __forceinline__ uint32_t pattern_lookup(int32_t sym, uint32_t h, unsi
 template <bool kBounds>
 __global__ void __launch_bounds__(kPrepThreads, 6)
 multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int32_t* dist_out, int g_base) {
+    grid_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned long long* s_slot = reinterpret_cast<unsigned long long*>(smem);    // [hslots_max]
     uint32_t* s_info = reinterpret_cast<uint32_t*>(s_slot + hslots_max);         // [pitch]
@@ -517,6 +518,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* s_part /* [32] *
 // also leaves the tables the dp kernel reads.  `fill` is zeroed by the caller's memset.
 __global__ void __launch_bounds__(kNumBins)
 multi_order_kernel(const PairDesc* descs, int32_t* order, Ctl* ctl, int n_pairs) {
+    grid_begin();
     __shared__ int s_part[32];
     __shared__ int32_t s_start[kNumBins];
     const int t = threadIdx.x;
@@ -857,6 +859,7 @@ __device__ __noinline__ void dp_task_band(int tlog, int pos, bool valid, const P
 template <bool kBoth>
 __global__ void __launch_bounds__(kDpWarpsPerCta * 32)
 multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
+    grid_begin();
     const bool kBand = kBoth && (blockIdx.x & 1);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
     const PairDesc* descs = reinterpret_cast<const PairDesc*>(ws + W.off_desc);
@@ -917,6 +920,7 @@ multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
 // exceeds its cap is reported as "more than the cap", which is all Eq. 2 needs to know.
 __global__ void __launch_bounds__(128)
 multi_bound_kernel(GateArgs a, PairDesc* descs, Ctl* ctl, uint8_t* flag, uint8_t* exact, int min_tlog) {
+    grid_begin();
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= a.n_groups) return;
     const int N = a.N, P = pairs_of(N);
@@ -966,6 +970,7 @@ constexpr int kFinishThreads = 256;
 
 __global__ void __launch_bounds__(kFinishThreads)
 multi_finish_kernel(GateArgs a, int32_t* dist, const uint8_t* flag, uint8_t* exact, int gpb) {
+    grid_begin();
     __shared__ double s_term[kFinishThreads];
     __shared__ int32_t s_dist[kFinishThreads];
     const int N = a.N, P = pairs_of(N);
@@ -1087,21 +1092,15 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
             if (rc != SR_OK) return rc;
         }
         if (decide)
-            multi_prep_kernel<true><<<(g1 - g0) * a.N, kPrepThreads, prep_smem, s>>>(a, ws, W, hslots, dist, g0);
+            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<true>, (g1 - g0) * a.N, kPrepThreads, prep_smem, s, a, ws, W, hslots, dist, g0);
         else
-            multi_prep_kernel<false><<<(g1 - g0) * a.N, kPrepThreads, prep_smem, s>>>(a, ws, W, hslots, dist, g0);
-        SR_LAUNCH_CHECK("multi_prep_kernel");
+            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<false>, (g1 - g0) * a.N, kPrepThreads, prep_smem, s, a, ws, W, hslots, dist, g0);
     }
     if (decide) {
-        multi_bound_kernel<<<(a.n_groups + 127) / 128, 128, 0, s>>>(
-            a, reinterpret_cast<PairDesc*>(ws + W.off_desc), ctl, flag, exact, W.min_tlog);
-        SR_LAUNCH_CHECK("multi_bound_kernel");
+        SR_LAUNCH("multi_bound_kernel", multi_bound_kernel, (a.n_groups + 127) / 128, 128, 0, s,  a, reinterpret_cast<PairDesc*>(ws + W.off_desc), ctl, flag, exact, W.min_tlog);
     }
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[1], s));
-    multi_order_kernel<<<(n_pairs + kNumBins - 1) / kNumBins, kNumBins, 0, s>>>(
-        reinterpret_cast<const PairDesc*>(ws + W.off_desc),
-        reinterpret_cast<int32_t*>(ws + W.off_order), ctl, n_pairs);
-    SR_LAUNCH_CHECK("multi_order_kernel");
+    SR_LAUNCH("multi_order_kernel", multi_order_kernel, (n_pairs + kNumBins - 1) / kNumBins, kNumBins, 0, s,  reinterpret_cast<const PairDesc*>(ws + W.off_desc), reinterpret_cast<int32_t*>(ws + W.off_order), ctl, n_pairs);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[2], s));
     // persistent grid: a multiple of the SM count; warps pull tasks until none is left
     long long want = (n_pairs_ll + kDpWarpsPerCta - 1) / kDpWarpsPerCta;
@@ -1111,13 +1110,14 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     long long cap = (long long)sms * 3;
     int blocks = (int)(want < cap ? want : cap);
     if (blocks < 1) blocks = 1;
-    if (decide) multi_dp_kernel<true><<<2 * blocks, kDpWarpsPerCta * 32, 0, s>>>(ws, W, dist, 2u);
-    else multi_dp_kernel<false><<<blocks, kDpWarpsPerCta * 32, 0, s>>>(ws, W, dist, 2u);
-    SR_LAUNCH_CHECK("multi_dp_kernel");
+    // (an ordinary launch: CTAs made resident while the tail of prep still fills some SMs would
+    // crowd onto the others, 478 us instead of 434 for the token-level batch of 1024 groups)
+    const int rc = decide ? launch_as(false, "multi_dp_kernel", multi_dp_kernel<true>, 2 * blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u)
+                          : launch_as(false, "multi_dp_kernel", multi_dp_kernel<false>, blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u);
+    if (rc != SR_OK) return rc;
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[3], s));
     const int fin_gpb = P <= kFinishThreads ? kFinishThreads / P : 1;
-    multi_finish_kernel<<<(a.n_groups + fin_gpb - 1) / fin_gpb, kFinishThreads, 0, s>>>(a, dist, flag, exact, fin_gpb);
-    SR_LAUNCH_CHECK("multi_finish_kernel");
+    SR_LAUNCH("multi_finish_kernel", multi_finish_kernel, (a.n_groups + fin_gpb - 1) / fin_gpb, kFinishThreads, 0, s, a, dist, flag, exact, fin_gpb);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[4], s));
     return SR_OK;
 }

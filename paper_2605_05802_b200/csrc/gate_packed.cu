@@ -16,6 +16,7 @@ constexpr int kUnpackThreads = 256;
 __global__ void __launch_bounds__(kUnpackThreads)
 unpack_rows_kernel(const int32_t* __restrict__ packed, const long long* __restrict__ start,
                    int rows, int stride, int32_t* __restrict__ seqs, int32_t* __restrict__ lens) {
+    grid_begin();
     const int row = blockIdx.x * (kUnpackThreads / 32) + (threadIdx.x >> 5);
     if (row >= rows) return;
     const int lane = threadIdx.x & 31;
@@ -43,9 +44,7 @@ struct FeedCtx {
 int unpack_rows(const FeedCtx& f, int g0, int g1, cudaStream_t s) {
     const size_t row0 = (size_t)g0 * f.N;
     const int rows = (g1 - g0) * f.N;
-    unpack_rows_kernel<<<(rows + kUnpackThreads / 32 - 1) / (kUnpackThreads / 32), kUnpackThreads, 0, s>>>(
-        f.d_packed, f.d_start + row0, rows, f.stride, f.d_seqs + row0 * f.stride, f.d_lens + row0);
-    SR_LAUNCH_CHECK("unpack_rows_kernel");
+    SR_LAUNCH("unpack_rows_kernel", unpack_rows_kernel, (rows + kUnpackThreads / 32 - 1) / (kUnpackThreads / 32), kUnpackThreads, 0, s,  f.d_packed, f.d_start + row0, rows, f.stride, f.d_seqs + row0 * f.stride, f.d_lens + row0);
     return SR_OK;
 }
 

@@ -56,6 +56,7 @@ __device__ __forceinline__ void group_sync(bool warp_level) {
 template <bool kWarp>
 __global__ void __launch_bounds__(kWarp ? 256 : 512)
 gate_single_kernel(GateArgs a, SingleLayout L) {
+    grid_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     const int N = a.N, K = a.K, P = pairs_of(N);
     const int t = kWarp ? (threadIdx.x & 31) : threadIdx.x;               // thread within the group
@@ -210,6 +211,7 @@ gate_single_kernel(GateArgs a, SingleLayout L) {
 template <int KR>      // pattern rows / text columns held in registers: K <= KR, KR % 4 == 0
 __global__ void __launch_bounds__(512)
 gate_direct_kernel(GateArgs a, int groups_per_cta, uint32_t one) {
+    grid_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     const int N = a.N, K = a.K, P = pairs_of(N);
     double* s_term = reinterpret_cast<double*>(smem);                               // [groups_per_cta * P]
@@ -277,8 +279,7 @@ int launch_gate_direct(const GateArgs& a, cudaStream_t s) {
     const int gpc = threads / P;
     const int smem = gpc * P * 12;
     const int blocks = (a.n_groups + gpc - 1) / gpc;
-    gate_direct_kernel<KR><<<blocks, threads, smem, s>>>(a, gpc, 1u);
-    SR_LAUNCH_CHECK("gate_direct_kernel");
+    SR_LAUNCH("gate_direct_kernel", gate_direct_kernel<KR>, blocks, threads, smem, s, a, gpc, 1u);
     return SR_OK;
 }
 
@@ -343,9 +344,8 @@ int launch_gate_single(const GateArgs& a, cudaStream_t s) {
             if (dev >= 0 && dev < 64) granted[warp][dev] = smem;
         }
     }
-    if (warp) gate_single_kernel<true><<<blocks, threads, smem, s>>>(a, L);
-    else gate_single_kernel<false><<<blocks, threads, smem, s>>>(a, L);
-    SR_LAUNCH_CHECK("gate_single_kernel");
+    if (warp) SR_LAUNCH("gate_single_kernel", gate_single_kernel<true>, blocks, threads, smem, s, a, L);
+    else SR_LAUNCH("gate_single_kernel", gate_single_kernel<false>, blocks, threads, smem, s, a, L);
     return SR_OK;
 }
 

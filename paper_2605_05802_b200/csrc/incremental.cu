@@ -52,6 +52,7 @@ IncrLayout incr_layout(int32_t n_groups, int32_t N) {
 
 __global__ void incr_init_kernel(unsigned char* state, IncrLayout L, int n_groups, int N,
                                  int max_steps) {
+    grid_begin();
     const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t nthr = (size_t)gridDim.x * blockDim.x;
     uint32_t* hdr = reinterpret_cast<uint32_t*>(state);
@@ -153,6 +154,7 @@ __device__ __forceinline__ void match_masks(const int4* quads, int N, int ri, in
 template <int kN>
 __global__ void __launch_bounds__(512, 3)
 incr_step_kernel(IncrArgs a) {
+    grid_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     const int N = kN ? kN : a.N, P = pairs_of(N);
     const int tid = threadIdx.x;
@@ -291,8 +293,7 @@ int launch_incr_init(void* state, size_t bytes, int32_t n_groups, int32_t N, int
     int blocks = (int)((work + 255) / 256);
     if (blocks < 1) blocks = 1;
     if (blocks > 4096) blocks = 4096;
-    incr_init_kernel<<<blocks, 256, 0, s>>>(static_cast<unsigned char*>(state), L, n_groups, N, max_steps);
-    SR_LAUNCH_CHECK("incr_init_kernel");
+    SR_LAUNCH("incr_init_kernel", incr_init_kernel, blocks, 256, 0, s, static_cast<unsigned char*>(state), L, n_groups, N, max_steps);
     return SR_OK;
 }
 
@@ -326,9 +327,8 @@ int launch_incr_step(void* state, size_t bytes, const int32_t* new_actions, int3
     if (threads < gpb * N) threads = (gpb * N + 31) & ~31;
     if (threads < 64) threads = 64;
     const int blocks = (n_groups + gpb - 1) / gpb;
-    if (N == 8) incr_step_kernel<8><<<blocks, threads, off, s>>>(a);
-    else incr_step_kernel<0><<<blocks, threads, off, s>>>(a);
-    SR_LAUNCH_CHECK("incr_step_kernel");
+    if (N == 8) SR_LAUNCH("incr_step_kernel", incr_step_kernel<8>, blocks, threads, off, s, a);
+    else SR_LAUNCH("incr_step_kernel", incr_step_kernel<0>, blocks, threads, off, s, a);
     return SR_OK;
 }
 

@@ -12,6 +12,7 @@ __global__ void __launch_bounds__(256)
 or_rule_kernel(const double* __restrict__ mean, const int32_t* __restrict__ lens,
                const uint8_t* __restrict__ done, int n_groups, int N, int K, double threshold,
                double tau_high, bool vec4, double* __restrict__ tau, uint8_t* __restrict__ stop) {
+    grid_begin();
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= n_groups) return;
     const double dk = mean[g];
@@ -54,6 +55,7 @@ __global__ void __launch_bounds__(512)
 group_signals_kernel(const int32_t* __restrict__ seqs, const int32_t* __restrict__ lens, int N,
                      int stride, int K, int slots, int slot_shift, double ln_n, SignalLayout L,
                      double* upr, double* uar, double* ent, double* jac) {
+    grid_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     double* s_term = reinterpret_cast<double*>(smem + L.off_term);          // [P]
     double* s_plogp = reinterpret_cast<double*>(smem + L.off_plogp);        // [N]
@@ -192,6 +194,7 @@ group_signals_kernel(const int32_t* __restrict__ seqs, const int32_t* __restrict
 __global__ void __launch_bounds__(256)
 batch_stats_kernel(const float* __restrict__ adv, const uint8_t* __restrict__ stop, int N,
                    int n_groups, bool vec4, unsigned long long* counts, double* sumsq) {
+    grid_begin();
     double ss_all = 0.0, ss_kept = 0.0;
     unsigned z_all = 0, z_kept = 0, kept_groups = 0;
     const int stride = gridDim.x * blockDim.x;
@@ -316,9 +319,7 @@ int launch_group_signals(const int32_t* seqs, const int32_t* lens, int32_t n_gro
     L.off_slot = take(N * 32 * 2);
     L.words = kBgWords;
     L.total = off;
-    group_signals_kernel<<<n_groups, threads, L.total, s>>>(seqs, lens, N, stride, K, slots, slot_shift,
-                                                            log((double)N), L, upr, uar, ent, jac);
-    SR_LAUNCH_CHECK("group_signals_kernel");
+    SR_LAUNCH("group_signals_kernel", group_signals_kernel, n_groups, threads, L.total, s, seqs, lens, N, stride, K, slots, slot_shift, log((double)N), L, upr, uar, ent, jac);
     return SR_OK;
 }
 
@@ -334,9 +335,7 @@ int launch_batch_stats(const float* adv, const uint8_t* stop, int32_t n_groups, 
     const int want = (n_groups + 255) / 256;
     const int cap = sms * 16;
     const int blocks = want < cap ? want : cap;
-    batch_stats_kernel<<<blocks, 256, 0, s>>>(adv, stop, N, n_groups, vec4,
-                                              reinterpret_cast<unsigned long long*>(counts), sumsq);
-    SR_LAUNCH_CHECK("batch_stats_kernel");
+    SR_LAUNCH("batch_stats_kernel", batch_stats_kernel, blocks, 256, 0, s, adv, stop, N, n_groups, vec4, reinterpret_cast<unsigned long long*>(counts), sumsq);
     return SR_OK;
 }
 
@@ -345,9 +344,7 @@ int launch_or_rule(const double* mean, const int32_t* lens, const uint8_t* done,
                    uint8_t* stop, cudaStream_t s) {
     if (n_groups == 0) return SR_OK;
     const bool vec4 = done == nullptr && (N % 4 == 0) && (reinterpret_cast<uintptr_t>(lens) & 15) == 0;
-    or_rule_kernel<<<(n_groups + 255) / 256, 256, 0, s>>>(mean, lens, done, n_groups, N, K, threshold,
-                                                          tau_high, vec4, tau, stop);
-    SR_LAUNCH_CHECK("or_rule_kernel");
+    SR_LAUNCH("or_rule_kernel", or_rule_kernel, (n_groups + 255) / 256, 256, 0, s, mean, lens, done, n_groups, N, K, threshold, tau_high, vec4, tau, stop);
     return SR_OK;
 }
 

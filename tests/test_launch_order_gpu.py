@@ -1,0 +1,62 @@
+"""Calls that follow one another on a stream without synchronisation, each reading what the one
+before it wrote: kernels start early (programmatic stream serialisation) but must not read early."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2605_05802_b200 as sr
+from paper_2605_05802_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("n_groups,K", [(16, 10), (3000, 30), (40, 300)])
+def test_back_to_back_calls_see_each_other(n_groups, K, captured):
+    dev = torch.device("cuda:0")
+    make = (lambda s: W.token_gate(seed=s, n_groups=n_groups, min_len=40, max_len=K)) if K > 32 else \
+        (lambda s: W.agent_gate(seed=s, n_groups=n_groups, K=K))
+    batches = [make(s) for s in range(4)]
+    threshold = 0.4
+    host = [(torch.from_numpy(w.seqs).to(dev), torch.from_numpy(w.lens).to(dev), torch.from_numpy(w.rewards).to(dev)) for w in batches]
+    seqs, lens, rewards = (torch.empty_like(x) for x in host[0])
+    G, N, stride = seqs.shape
+    stop, zv = (torch.empty(G, dtype=torch.uint8, device=dev) for _ in range(2))
+    adv = torch.empty((G, N), device=dev)
+    index, count = torch.zeros(G, dtype=torch.int32, device=dev), torch.zeros(1, dtype=torch.int32, device=dev)
+    ws = torch.empty(max(sr.sr_gate_workspace_bytes(G, N, stride, K), 1), dtype=torch.uint8, device=dev)
+    kws = torch.empty(sr.sr_kept_groups_workspace_bytes(G), dtype=torch.uint8, device=dev)
+
+    def step():
+        sr.sr_gate(seqs, lens, K, threshold, stop=stop, workspace=ws)
+        sr.sr_grpo_advantage(rewards, stop, 1e-6, adv=adv, zero_var=zv)
+        sr.sr_kept_groups(stop, zv, index=index, count=count, workspace=kws)
+
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        run = step
+        if captured:
+            step()
+            stream.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                step()
+            run = graph.replay
+        got = []
+        for k in range(24):
+            for dst, src in zip((seqs, lens, rewards), host[k % 4]):
+                dst.copy_(src)
+            run()
+            got.append([x.clone() for x in (stop, zv, adv, index, count)])
+    torch.cuda.synchronize()
+    want = []
+    for w in batches:
+        ostop = oracle.gate(w.seqs, w.lens, K, threshold, threads=8)[3]
+        oadv, ozv = oracle.advantage(w.rewards, ostop, 1e-6)
+        want.append((ostop, ozv, oadv, oracle.kept_groups(ostop, ozv)))
+    for k, (s, z, a, i, c) in enumerate(got):
+        ostop, ozv, oadv, oidx = want[k % 4]
+        assert np.array_equal(s.cpu().numpy(), ostop) and np.array_equal(z.cpu().numpy(), ozv), k
+        assert np.allclose(a.cpu().numpy(), oadv, rtol=1e-6, atol=0), k
+        assert int(c) == len(oidx) and np.array_equal(i.cpu().numpy()[:int(c)], oidx), k
