@@ -13,36 +13,30 @@
 //            the pattern (0x7FFF: absent).  A block's match word is then just
 //            1 << (loc - first_row_of_block), no table lookup.  A symbol with several
 //            occurrences gets a row of match words instead, and the stream names the row.
-//            Also bins the pairs by (team shape, text length).
+//            Bounds of the pair's distance fall out of the look-ups: the columns without any
+//            match in the pattern from below, the differing positions from above.
+//   bin      team shape of every pair (what the band of its bounds costs at least, see
+//            shape_of_pair) and bin counts.
 //   order    counting sort of the pairs by bin: longest warp tasks first, one team
-//            shape and similar text lengths per bin; warp-task table.
+//            shape and similar durations per bin; warp-task table.  (One launch does both for
+//            batches of up to a thousand pairs.)
 //   dp       persistent warps pull tasks.  A task is a warp of 32/T teams; a team of
-//            T lanes (T in {1, 2, 4, 8}; up to 32 in small batches) owns one pair, lane l
-//            holding R <= 6 consecutive blocks (32*R rows) in registers.  Lanes are skewed by four columns; the
-//            delta words of a lane's last block reach the next lane by warp shuffles.
+//            T lanes owns one pair, a lane holding R <= 4 consecutive blocks (32*R rows) in
+//            registers.  Lanes are skewed by four columns; the
+//            delta bits of a lane's last block reach the next lane by warp shuffles.
 //            All pairs of a task share (T, R) and have similar lengths, so the warp's
 //            lanes stay busy.
-//   finish   one thread per group: ordered fp64 sum of the normalised terms,
-//            threshold, outputs.
+//   finish   one thread per pair for the terms, one per group: ordered fp64 sum of the normalised
+//            terms, threshold, outputs.
 //
-// Band (decide mode).  There prep also counts, per pair, the positions at which the two
-// prefixes differ (after the common prefix): that count plus the length difference is an
-// UPPER bound of the distance (substitute the differing positions, insert or delete the
-// rest), and the threshold caps how large a distance can still matter.  An optimal
-// alignment of distance <= ub never leaves the diagonals d = row - column with
-// |d| + |(m - n) - d| <= ub (Ukkonen's cut-off), so pairs whose bound is small run a
-// banded task, served by CTAs of their own within the dp launch: the pattern's 32-row
-// blocks are grouped in stripes of R blocks, stripe g lives on lane g mod T of a ring of
-// T lanes and is advanced only over the columns where the band crosses it; a stripe the
-// band enters starts from +1 vertical deltas below the stripe above it and a stripe whose
-// upper neighbour the band has left takes +1 horizontal deltas from above -- both
-// over-estimates of cells outside the band, which leave every cell on an optimal path
-// exact.  The distance is read from a running score
-// at the bottom of the last stripe.  A result within the bound is the exact distance; a
-// result above it only says "more than the bound".  (Banding the exact mode from the
-// mismatch count alone was built as well: 41 % fewer block-columns on the token-level
-// batch, but with the banded task bodies next to the six full ones the dp kernel no
-// longer fits the instruction caches and the launch got slower, not faster.)
+// Band.  With bounds lb <= d <= ub of a pair's distance an optimal alignment stays on a band of
+// diagonals (band_of), and where the bounds meet nothing is left to compute.  Rollouts that have
+// converged differ in few positions: their bands are narrow, and the T lanes of a team form a ring that
+// follows the band down the pattern instead of covering all of it.  Cells outside the band are
+// over-estimated at its edges, which leaves every cell on an optimal path exact (the banded block
+// scheme of Sosic and Sikic 2017).  In decide mode the threshold caps how large a distance can
+// still matter, and the pair's upper bound with it: a result within the bound is the exact
+// distance, a result above it only says "more than the bound".
 //
 // Which rollout of a pair is the pattern is fixed by a round-robin tournament on the
 // indices, so that every pattern CTA of `prep` serves the same number of texts.
@@ -52,10 +46,11 @@ namespace sr {
 namespace {
 
 constexpr int kPrepThreads = 256;
-constexpr int kMaxR = 8;            // blocks (32 rows each) per lane
-constexpr int kNumClasses = 32;     // team shapes (T lanes x R blocks), see class_of
-constexpr int kLenBuckets = 32;     // buckets of estimated task duration
-constexpr int kNumBins = kNumClasses * kLenBuckets;
+constexpr int kNumClasses = 21;     // team shapes (T lanes x R blocks), see class_of
+constexpr int kTimeBuckets = 96;    // buckets of estimated task duration
+constexpr int kNumBins = 2048;      // kTimeBuckets * kNumClasses of them used
+constexpr int kOrderThreads = 1024;
+constexpr int kAlonePairs = 1024;   // batches of up to this many pairs are ordered by one CTA
 constexpr uint32_t kLocNone = 0x7FFFu;    // bit 15 clear, far above any row: shifts to 0
 constexpr uint32_t kLocRow = 0x8000u;     // | index of the symbol's mask row
 constexpr uint32_t kLocChain = 0xC000u;   // | first position of the symbol's occurrence chain
@@ -63,31 +58,34 @@ constexpr uint32_t kChainEnd = 0xFFFFu;
 constexpr int kRepeatedFlag = 0x10000;    // a text's stream holds row or chain entries
 constexpr int kPosPerThread = SR_MAX_K / kPrepThreads;
 constexpr int kDpWarpsPerCta = 4;
-constexpr uint32_t kBinMask = 0x3FFu;
+constexpr uint32_t kBinMask = 0x7FFu;
+constexpr uint32_t kHasChains = 0x40000000u;
 constexpr int32_t kCappedFlag = 0x40000000;   // decide mode: the pair's distance exceeds its cap
 constexpr int kStripShift = 12;
 constexpr uint32_t kNeedsDp = 0x80000000u;
-static_assert(kNumBins <= (int)kBinMask + 1, "bin index must fit its field");
+static_assert(kNumBins <= (int)kBinMask + 1 && kTimeBuckets * kNumClasses <= kNumBins, "bin index must fit its field");
 
 struct PairDesc {          // 16 bytes
     uint32_t mn;           // m | n << 16
     uint32_t pat_row;      // g * N + pattern rollout
-    uint32_t bin;          // bits 0..9 bin index; bits 12..21 stripped common prefix (symbols,
-                           // a multiple of 4); bit 31 = pair needs the dp kernel
+    uint32_t bin;          // bits 0..10 bin index; bits 12..21 stripped common prefix (symbols,
+                           // a multiple of 4); bit 30 = the pattern has chains; bit 31 = pair
+                           // needs the dp kernel
     uint32_t lower;        // bits 0..15 a lower bound of the pair's distance (decide mode),
                            // bits 16..31 an upper bound (mismatching positions + length
                            // difference; in decide mode also capped by what the threshold
                            // still allows): the band of the pair follows from it
 };
 
-struct Ctl {               // int32 control block in the workspace
+struct Ctl {               // control block in the workspace
+    unsigned long long work;                   // lane-time of all pairs, about
+    int32_t open;                              // and how many they are
     int32_t hist[kNumBins];
+    int32_t fill[kNumBins];                    // what comes before here starts at zero
     int32_t start[kNumBins];
-    int32_t fill[kNumBins];
     int32_t task_start[kNumBins + 1];          // first warp task of every bin
     int32_t task_counter;
     int32_t total_tasks;
-    int32_t task_counter_band;                 // the banded tasks' own launch
 };
 
 struct MultiWs {
@@ -95,14 +93,14 @@ struct MultiWs {
     int pitch;             // uint16 elements per loc / chain row
     int row_words;         // 32-bit words of a mask row: one per 32 pattern positions
     int row_cap;           // mask rows a pattern may have
-    int min_tlog;          // small batches: teams of at least 2^min_tlog lanes
+    int warps;             // warps the dp kernel keeps resident
 };
 
 MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K) {
     MultiWs w;
     const size_t P = pairs_of(N);
     w.pitch = (K + 7) & ~7;
-    w.min_tlog = 0;
+    w.warps = 1;
     size_t off = 0;
     w.off_ctl = off;   off = align_up(off + sizeof(Ctl), 256);
     w.off_flag = off;  off = align_up(off + (size_t)n_groups, 256);
@@ -113,8 +111,8 @@ MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K) {
     w.off_loc = off;   off = align_up(off + (size_t)n_groups * P * w.pitch * 2, 256);
     // Mask rows for an eighth of the positions: symbols with at least eight occurrences always
     // fit, and 1/rank token frequencies put no more than about K / 10 symbols above one.  A team's
-    // lanes cover up to seven words more than the pattern has: slack after the last row.
-    w.row_words = (K + 31) >> 5;
+    // lanes cover up to fifteen words more than the pattern has: slack after the last row.
+    w.row_words = (K + 3 + 31) >> 5;      // the pattern and what pads its texts to whole quads
     w.row_cap = (K + 7) >> 3;
     w.off_rows = off;
     off = align_up(off + (size_t)n_groups * N * w.row_cap * w.row_words * 4 + 256, 256);
@@ -122,97 +120,99 @@ MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K) {
     return w;
 }
 
-__host__ __device__ inline void team_shape(int m, int min_tlog, int& tlog, int& R) {
-    // T lanes x R blocks per lane >= W blocks of the pattern, with little padding and
-    // R large enough to amortise the per-column work that does not depend on R
-    const int W = (m + 31) >> 5;            // <= 32
-    if (W <= 6) { tlog = 0; R = W; }
-    else if (W <= 12) { tlog = 1; R = (W + 1) >> 1; }
-    else if (W <= 24) { tlog = 2; R = (W + 3) >> 2; }
-    else { tlog = 3; R = (W + 7) >> 3; }
-    // A batch with too few pairs to give every resident warp its tasks spreads a pair over
-    // more lanes (up to the whole warp): shorter tasks, more of them.
-    if (tlog < min_tlog) {
-        int t = tlog;
-        while (t < min_tlog && (1 << t) < W) ++t;
-        tlog = t;
-        R = (W + (1 << t) - 1) >> t;
-    }
-}
-
-// Class of a team shape.  T = 1, 2, 4, 8 with R = 1..6 fill slots log2(T) * 8 + R - 1; the
-// shapes of small batches, T = 16 with R = 1, 2 and T = 32 with R = 1, take slots 6, 7, 14;
-// the banded shapes (ring of T = 4 or 8 lanes, stripes of R = 1..4 blocks) take slots 15, 22,
-// 23, 30, 31.
-__host__ __device__ inline int class_of(int tlog, int R) {
-    if (tlog < 4) return tlog * 8 + (R - 1);
-    return tlog == 4 ? 5 + R : 14;
-}
-__host__ __device__ inline bool is_band_class(int cls) {
-    return cls == 15 || cls == 22 || cls == 23 || cls == 30 || cls == 31;
-}
+// Class of a team shape: T = 1, 2, 4, 8 with R = 1..4, T = 16 with R = 1..3, T = 32 with R = 1, 2.
+// (R = 5 and 6 amortise the work per column over more blocks, but with six bodies of the task
+// loop the instruction cache no longer holds what an SM's warps run side by side.)
+__host__ __device__ inline int max_blocks(int tlog) { return tlog < 4 ? 4 : 7 - tlog; }
+__host__ __device__ inline int class_of(int tlog, int R) { return (tlog < 5 ? 4 * tlog : 19) + R - 1; }
 __host__ __device__ inline void shape_of_class(int cls, int& tlog, int& R) {
-    if ((cls & 7) < 6) { tlog = cls >> 3; R = (cls & 7) + 1; }
-    else if (cls == 6) { tlog = 4; R = 1; }
-    else if (cls == 7) { tlog = 4; R = 2; }
-    else if (cls == 14) { tlog = 5; R = 1; }
-    else if (cls == 15) { tlog = 2; R = 1; }
-    else if (cls == 22) { tlog = 3; R = 1; }
-    else if (cls == 23) { tlog = 3; R = 2; }
-    else if (cls == 30) { tlog = 3; R = 3; }
-    else { tlog = 3; R = 4; }               // 31
-}
-
-// Bins order the pairs by the estimated running time of their warp task (text
-// columns x instructions per column, longest first) and, within one duration
-// bucket, by team shape: all pairs of a bin share the shape and have text lengths
-// within a few percent, and warps that pull tasks in bin order start the longest
-// tasks first, which keeps the finishing times of the warps close together.
-__host__ __device__ inline int bin_of_cost(int cost, int cls) {
-    const int max_cost = (SR_MAX_K + 32) * (14 * kMaxR + 20) + 1;
-    int bucket = (int)(((long long)cost * kLenBuckets) / max_cost);
-    bucket = bucket < 0 ? 0 : (bucket >= kLenBuckets ? kLenBuckets - 1 : bucket);
-    return (kLenBuckets - 1 - bucket) * kNumClasses + cls;
+    tlog = cls < 19 ? cls >> 2 : 5;
+    R = cls - (cls < 19 ? 4 * tlog : 19) + 1;
 }
 
 // Diagonals d = row - column an optimal alignment of an m x n pair can visit when its
-// distance is at most ub: |d| + |(m - n) - d| <= ub.  At least two diagonals wide, so that
-// a stripe always starts while the stripe above it is still running.
-__host__ __device__ inline void band_of(int m, int n, int ub, int& dlo, int& dhi) {
+// distance is at most ub and at least lb.  A path that strays x diagonals beyond those between
+// the corners spends x insertions and x deletions more than the length difference asks for:
+// |m - n| + 2 x <= ub; and lb is a bound of what is spent besides x: lb + x <= ub (with m >= n a
+// path has x insertions and at least as many other edits as lb counts: m - n deletions and one
+// edit per text column without a match; with n > m it has x deletions besides those columns).
+// At least two diagonals wide, so that a stripe always starts while the stripe above it is
+// still running.
+__host__ __device__ inline void band_of(int m, int n, int lb, int ub, int& dlo, int& dhi) {
     const int D = m - n, aD = D < 0 ? -D : D;
     int e = (ub - aD) >> 1;
+    if (ub - lb < e) e = ub - lb;
     if (e < 0) e = 0;
     dlo = (D < 0 ? D : 0) - e;
     dhi = (D > 0 ? D : 0) + e;
     if (dhi == dlo) ++dhi;
 }
 
-// Shape and bin of a pair of m rows x n columns (what is left after the common prefix)
-// whose distance is at most ub.  The banded shapes serve bands of up to 32 R (T - 1)
-// diagonals; one is taken when its estimated lane-time is clearly below that of the full
-// shape (the estimates count instructions per quad of columns and lane).
-__host__ __device__ inline int shape_and_bin(int m, int n, int ub, int min_tlog) {
-    int tlog, R;
-    team_shape(m, min_tlog, tlog, R);
-    const int nq = (n + 3) >> 2;
-    const int full_time = (nq + (1 << tlog) - 1) * (14 * R + 14);
-    const int full_work = full_time << tlog;
+// Cost of an iteration (a quad of columns on R blocks) in units of four issue cycles: measured
+// 26 cycles per block and column with three warps per scheduler, and what does not depend on R.
+__host__ __device__ inline int quad_cost(int R, bool ring) { return 26 * R + (ring ? 30 : 22); }
+
+struct Shape { int tlog, R, time; };
+
+// Team shape of a pair of m rows x n columns (what is left after the common prefix) whose
+// distance lies in lb..ub.  Either the team's lanes hold the whole pattern, or, where the
+// band is narrow enough, they form a ring that follows it: stripe g + T may only enter
+// the band three iterations after stripe g has left it, w + 32 R + 11 < T (32 R + 4) for a band
+// of w + 1 diagonals.  The shape with the least lane-time wins, where one that takes longer than
+// the goal's limit counts for more in the proportion by which it does, and lanes that would be
+// idle otherwise are free.
+struct ShapeGoal { float limit, free_lanes; };
+__device__ inline Shape shape_of_pair(int m, int n, int lb, int ub, ShapeGoal goal) {
+    const int W = (m + 31) >> 5, nq = (n + 3) >> 2;
     int dlo, dhi;
-    band_of(m, n, ub, dlo, dhi);
+    band_of(m, n, lb, ub, dlo, dhi);
     const int w = dhi - dlo;
-    // banded tasks are few and run with the machine half empty, so their shapes favour a
-    // short task (many lanes, few blocks per lane) over the last bit of lane efficiency
-    int bcls = -1;
-    if (w <= 96) bcls = 15; else if (w <= 224) bcls = 22; else if (w <= 448) bcls = 23;
-    else if (w <= 672) bcls = 30; else if (w <= 896) bcls = 31;
-    if (bcls >= 0) {
-        int btl, bR;
-        shape_of_class(bcls, btl, bR);
-        const int G = (((m + 31) >> 5) + bR - 1) / bR;      // stripes
-        const int band_time = (nq + G - 1) * (14 * bR + 20);
-        if ((band_time << btl) * 8 < full_work * 7) return bin_of_cost(4 * band_time, bcls);
+    Shape best{0, 1, 0};
+    float best_score = 3.0e38f;
+#pragma unroll
+    for (int t = 0; t <= 5; ++t) {
+        const int T = 1 << t, room = w + 11 - 4 * T;
+        // all blocks on the team's lanes; a ring of stripes as low as the band allows
+        const int full_R = (W + T - 1) >> t, ring_R = t == 0 ? 99 : (room < 0 ? 1 : room / (32 * (T - 1)) + 1);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int R = k ? ring_R : full_R;
+            if (R > max_blocks(t) || (k && W <= T * R)) continue;
+            // stripes of a ring: ceil(W / R)
+            const int G = (int)((uint32_t)((W + R - 1) * (R == 3 ? 21846 : 65536 >> (R >> 1))) >> 16);
+            const int time = (nq + (k ? G : T) - 1) * quad_cost(R, k);
+            const float score = (float)time * fmaxf((float)T, goal.free_lanes) * fmaxf((float)time, goal.limit);
+            if (score < best_score) {
+                best = Shape{t, R, time};
+                best_score = score;
+            }
+        }
     }
-    return bin_of_cost(4 * full_time, class_of(tlog, R));
+    return best;
+}
+
+// About the lane-time of the pair's cheapest shape.
+__device__ inline int work_of_pair(int m, int n, int lb, int ub) {
+    int dlo, dhi;
+    band_of(m, n, lb, ub, dlo, dhi);
+    return ((n + 3) >> 2) * min((m + 31) >> 5, (dhi - dlo + 128) >> 5) * 36;
+}
+
+// Bins order the pairs by the estimated running time of their warp task, longest first, and,
+// within one duration bucket, by team shape: all pairs of a bin share the shape and have similar
+// text lengths, and warps that pull tasks in bin order start the longest tasks first, which
+// keeps the finishing times of the warps close together.  Buckets are 7 % wide (ten and a half to the octave).
+__device__ inline int bin_of_shape(const Shape& s) {
+    const int bucket = min(max((int)(10.5f * (15.2f - __log2f((float)s.time))), 0), kTimeBuckets - 1);
+    return bucket * kNumClasses + class_of(s.tlog, s.R);
+}
+
+// The pair of a descriptor, rows and columns extended to whole quads.
+struct PairSize { int m, n, lb, ub; };
+__device__ __forceinline__ PairSize size_of_desc(const PairDesc& d) {
+    const int strip = (int)((d.bin >> kStripShift) & 0x3FFu), m = (int)(d.mn & 0xFFFFu), n = (int)(d.mn >> 16);
+    const int pad = -n & 3;                                    // strip is a multiple of four
+    return PairSize{m + pad - strip, n + pad - strip, (int)(d.lower & 0xFFFFu), (int)(d.lower >> 16)};
 }
 
 __device__ __forceinline__ int clamp_len(const int32_t* lens, size_t idx, int K, bool& neg) {
@@ -244,11 +244,21 @@ __device__ __forceinline__ uint32_t pattern_lookup(int32_t sym, uint32_t h, unsi
     return kLocNone;
 }
 
-// kBounds: also count, per text, the columns whose symbol does not occur in the pattern
-// at all.  Each of them costs at least one edit, and so does every unit of length
-// difference: max(|m - n|, absent columns) is a lower bound of the pair's distance that
-// falls out of the look-ups for free.
-template <bool kBounds>
+// Adds the lanes' values to a counter in shared memory; one atomic where they agree on it.
+__device__ __forceinline__ void warp_add(int* counter, int key, int v) {
+    const unsigned live = __activemask();
+    if (__all_sync(live, key == __shfl_sync(live, key, __ffs(live) - 1))) {
+        const int sum = __reduce_add_sync(live, v);
+        if (sum && (threadIdx.x & 31) == __ffs(live) - 1) atomicAdd(counter, sum);
+    } else if (v) {
+        atomicAdd(counter, v);
+    }
+}
+
+// Per text it also counts the columns whose symbol does not occur in the pattern at all and
+// the positions at which text and pattern differ: bounds of the pair's distance that cost next
+// to nothing here.  Where they meet the pair is done.
+template <bool kDecide>
 __global__ void __launch_bounds__(kPrepThreads, 6)
 multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int32_t* dist_out, int g_base) {
     grid_begin();
@@ -437,10 +447,15 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
         const uint32_t l1 = pattern_lookup(sym.y, h1, v1, s_slot, hslots);
         const uint32_t l2 = pattern_lookup(sym.z, h2, v2, s_slot, hslots);
         const uint32_t l3 = pattern_lookup(sym.w, h3, v3, s_slot, hslots);
-        reinterpret_cast<uint2*>(locs + idx * W.pitch)[q] = make_uint2(l0 | (l1 << 16), l2 | (l3 << 16));
-        // columns past the text's end hold whatever the row holds: harmless to count as repeated
-        if (((l0 | l1 | l2 | l3) & kLocRow) && !(s_absent[t] & kRepeatedFlag)) atomicOr(&s_absent[t], kRepeatedFlag);
-        if (kBounds) {
+        // The last quad of a text is filled up with symbols of their own that the pattern is
+        // extended by as well: a common suffix leaves the distance as it is, and the recurrence
+        // always runs whole quads, whose four columns the compiler can then interleave.
+        const uint32_t left = (uint32_t)(s_len[t] - 4 * q);  // columns of this quad that exist (>= 1)
+        const uint32_t w1 = left > 1u ? l1 : (uint32_t)m, w2 = left > 2u ? l2 : (uint32_t)m + 2u - left;
+        const uint32_t w3 = left > 3u ? l3 : (uint32_t)m + 3u - left;
+        reinterpret_cast<uint2*>(locs + idx * W.pitch)[q] = make_uint2(l0 | (w1 << 16), w2 | (w3 << 16));
+        if (((l0 | w1 | w2 | w3) & kLocRow) && !(s_absent[t] & kRepeatedFlag)) atomicOr(&s_absent[t], kRepeatedFlag);
+        {
             // positions below both lengths whose symbol is not the pattern's symbol at the same place
             const int both = min(m, s_len[t]) - 4 * q;       // columns of this quad below both lengths
             int differ = 0;
@@ -449,14 +464,13 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
                 differ = (sym.x != own.x) + (both > 1 && sym.y != own.y) + (both > 2 && sym.z != own.z) +
                          (both > 3 && sym.w != own.w);
             }
-            if (differ) atomicAdd(&s_differ[t], differ);
-            const int left = s_len[t] - 4 * q;           // columns of this quad that exist
-            const int absent = (l0 == kLocNone) + (left > 1 && l1 == kLocNone) +
-                               (left > 2 && l2 == kLocNone) + (left > 3 && l3 == kLocNone);
-            if (absent) atomicAdd(&s_absent[t], absent);
+            warp_add(&s_differ[t], t, differ);
+            const int absent = (l0 == kLocNone) + (w1 == kLocNone) + (w2 == kLocNone) + (w3 == kLocNone);
+            warp_add(&s_absent[t], t, absent);
         }
     }
     __syncthreads();
+    int work = 0;
     if (tid < ntxt) {                                 // descriptors, bins, trivial pairs
         const int j = s_txt[tid], n = s_len[tid];
         // the removed prefix is a multiple of four symbols (the match stream is read in 8-byte
@@ -464,28 +478,39 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
         const int strip = s_cp[tid] < 0 ? -1 : (s_cp[tid] & (s_absent[tid] & kRepeatedFlag ? ~31 : ~3));
         const int lo = min(i, j), hi = max(i, j);
         const size_t idx = (size_t)g * P + pair_index(lo, hi, N);
-        if (strip < 0) {                              // one prefix starts the other (or is empty)
-            dist_out[idx] = abs(m - n);
-            descs[idx] = PairDesc{(uint32_t)m | ((uint32_t)n << 16), (uint32_t)(g * N + i), 0u,
-                                  (uint32_t)abs(m - n) | ((uint32_t)abs(m - n) << 16)};
-        } else {
-            // upper bound: substitute the differing positions, insert / delete the rest (only
-            // the decide mode bands its pairs: 0xFFFF stands for "no bound")
-            const int upper = kBounds ? s_differ[tid] + abs(m - n) : 0xFFFF;
-            const int bin = shape_and_bin(m - strip, n - strip, upper, W.min_tlog);
-            const int lower = kBounds ? max(abs(m - n), s_absent[tid] & (kRepeatedFlag - 1)) : 0;
-            descs[idx] = PairDesc{(uint32_t)m | ((uint32_t)n << 16), (uint32_t)(g * N + i),
-                                  (uint32_t)bin | ((uint32_t)strip << kStripShift) | kNeedsDp,
-                                  (uint32_t)lower | ((uint32_t)upper << 16)};
-            if (kBounds) dist_out[idx] = lower;            // the bound kernel bins the pairs it keeps
-            else atomicAdd(&ctl->hist[bin], 1);
+        // Upper bound of the distance: substitute the differing positions, insert or delete the
+        // rest.  Lower bound: every text column without a match costs an edit, and if the pattern
+        // is at least as long as the text, m - n rows are deleted besides.
+        int lower = abs(m - n), upper = lower;        // one prefix starts the other (or is empty)
+        if (strip >= 0) {
+            const int absent = s_absent[tid] & (kRepeatedFlag - 1);
+            lower = m >= n ? m - n + absent : max(n - m, absent);
+            upper += s_differ[tid];
+        }
+        PairDesc d{(uint32_t)m | ((uint32_t)n << 16), (uint32_t)(g * N + i), 0u, (uint32_t)lower | ((uint32_t)upper << 16)};
+        if (lower < upper) {                          // otherwise that is the distance
+            d.bin = ((uint32_t)strip << kStripShift) | kNeedsDp | (s_repeats[0] > s_repeats[3] ? kHasChains : 0u);
+            if (!kDecide) {                           // decide mode counts the pairs it keeps later
+                const PairSize z = size_of_desc(d);
+                work = work_of_pair(z.m, z.n, z.lb, z.ub);
+            }
+        }
+        descs[idx] = d;
+        if (kDecide || lower == upper) dist_out[idx] = lower;
+    }
+    if (!kDecide && tid < 32) {                       // the texts' threads are those of the first warp
+        const int open = __popc(__ballot_sync(0xFFFFFFFFu, work > 0));
+        work = __reduce_add_sync(0xFFFFFFFFu, work);
+        if (tid == 0 && open) {
+            atomicAdd(&ctl->work, (unsigned long long)work);
+            atomicAdd(&ctl->open, open);
         }
     }
     if (neg && tid == 0 && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
 }
 
 // ----------------------------------------------------------------------- order
-// Exclusive prefix sum over the kNumBins threads of a CTA (one value per thread).
+// Exclusive prefix sum over the kOrderThreads threads of a CTA (one value per thread).
 __device__ __forceinline__ int block_exclusive_scan(int v, int* s_part /* [32] */) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int incl = v;
@@ -512,42 +537,128 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* s_part /* [32] *
     return r;
 }
 
-// Counting sort of the pairs by bin: longest warp tasks first, one team shape and similar
-// text lengths per bin.  Every CTA turns the bin counts into bin starts by itself (a scan
-// of kNumBins values costs less than a launch) and places kNumBins pairs; the first CTA
-// also leaves the tables the dp kernel reads.  `fill` is zeroed by the caller's memset.
-__global__ void __launch_bounds__(kNumBins)
-multi_order_kernel(const PairDesc* descs, int32_t* order, Ctl* ctl, int n_pairs) {
+// The longest a task should take: about what every resident warp has to do on average, so
+// that none is still running long after the others (measured best among 0.6, 1.25 and 2.5 times
+// on token-level batches of 1024 groups).  And how many lanes there are to a pair.
+__device__ __forceinline__ ShapeGoal shape_goal(unsigned long long work, int open, int warps) {
+    const float lanes = 32.0f * (float)warps;
+    return ShapeGoal{1.25f * (float)work / lanes, lanes / (float)max(open, 1)};
+}
+
+// Every pair's shape and bin, and the bin counts.
+__global__ void __launch_bounds__(kOrderThreads)
+multi_bin_kernel(PairDesc* descs, Ctl* ctl, int n_pairs, int warps) {
     grid_begin();
-    __shared__ int s_part[32];
-    __shared__ int32_t s_start[kNumBins];
-    const int t = threadIdx.x;
-    const int own = ctl->hist[t];
-    const int start = block_exclusive_scan(own, s_part);
-    s_start[t] = start;
-    if (blockIdx.x == 0) {
-        // warp tasks per bin (32 / T pairs per task), exclusive prefix over the bins
-        int tl, rr;
-        shape_of_class(t % kNumClasses, tl, rr);
-        const int tpw = 32 >> tl;
-        const int own_tasks = (own + tpw - 1) / tpw;
-        const int task_start = block_exclusive_scan(own_tasks, s_part);
-        ctl->start[t] = start;
-        ctl->task_start[t] = task_start;
-        if (t == kNumBins - 1) {
-            ctl->task_start[kNumBins] = task_start + own_tasks;
-            ctl->total_tasks = task_start + own_tasks;
-            ctl->task_counter = 0;
-            ctl->task_counter_band = 0;
+    __shared__ int32_t s_hist[kNumBins];
+    for (int b = threadIdx.x; b < kNumBins; b += kOrderThreads) s_hist[b] = 0;
+    const ShapeGoal goal = shape_goal(ctl->work, ctl->open, warps);
+    __syncthreads();
+    const int idx = blockIdx.x * kOrderThreads + threadIdx.x;
+    if (idx < n_pairs) {
+        const PairDesc d = descs[idx];
+        if (d.bin & kNeedsDp) {
+            const PairSize z = size_of_desc(d);
+            const int bin = bin_of_shape(shape_of_pair(z.m, z.n, z.lb, z.ub, goal));
+            descs[idx].bin = d.bin | (uint32_t)bin;
+            atomicAdd(&s_hist[bin], 1);
         }
     }
     __syncthreads();
-    const int idx = blockIdx.x * kNumBins + t;
-    if (idx >= n_pairs) return;
-    const uint32_t b = descs[idx].bin;
-    if (!(b & kNeedsDp)) return;
-    const int bin = (int)(b & kBinMask);
-    order[s_start[bin] + atomicAdd(&ctl->fill[bin], 1)] = idx;
+    for (int b = threadIdx.x; b < kNumBins; b += kOrderThreads)
+        if (s_hist[b]) atomicAdd(&ctl->hist[b], s_hist[b]);
+}
+
+// Counting sort of the pairs by bin: longest warp tasks first, one team shape and similar
+// text lengths per bin.  Every CTA turns the bin counts into bin starts by itself (a scan
+// of kNumBins values costs less than a launch) and places kOrderThreads pairs; the first CTA
+// also leaves the tables the dp kernel reads.
+// kAlone: one CTA sorts the whole batch, and bins it first.
+template <bool kAlone>
+__global__ void __launch_bounds__(kOrderThreads)
+multi_order_kernel(PairDesc* descs, int32_t* order, Ctl* ctl, int n_pairs, int warps) {
+    grid_begin();
+    __shared__ int s_part[32];
+    __shared__ int32_t s_start[kNumBins], s_hist[kNumBins];
+    __shared__ unsigned long long s_work;
+    __shared__ int s_open;
+    const int t = threadIdx.x;
+    constexpr int kPer = kAlone ? kAlonePairs / kOrderThreads : 1;
+    uint32_t bins[kPer];
+    if (kAlone) {
+        s_hist[2 * t] = s_hist[2 * t + 1] = 0;
+        if (t == 0) { s_work = 0ull; s_open = 0; }
+        __syncthreads();
+        PairDesc d[kPer];
+        int work = 0, open = 0;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const int idx = k * kOrderThreads + t;
+            d[k].bin = 0u;
+            if (idx < n_pairs) d[k] = descs[idx];
+            if (d[k].bin & kNeedsDp) {
+                const PairSize z = size_of_desc(d[k]);
+                work += work_of_pair(z.m, z.n, z.lb, z.ub);
+                ++open;
+            }
+        }
+        work = __reduce_add_sync(0xFFFFFFFFu, work);
+        open = __reduce_add_sync(0xFFFFFFFFu, open);
+        if ((t & 31) == 0 && open) {
+            atomicAdd(&s_work, (unsigned long long)work);
+            atomicAdd(&s_open, open);
+        }
+        __syncthreads();
+        const ShapeGoal goal = shape_goal(s_work, s_open, warps);
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            bins[k] = d[k].bin;
+            if (d[k].bin & kNeedsDp) {
+                const PairSize z = size_of_desc(d[k]);
+                const int bin = bin_of_shape(shape_of_pair(z.m, z.n, z.lb, z.ub, goal));
+                bins[k] |= (uint32_t)bin;
+                atomicAdd(&s_hist[bin], 1);
+            }
+        }
+        __syncthreads();
+    } else {
+        s_hist[2 * t] = ctl->hist[2 * t];
+        s_hist[2 * t + 1] = ctl->hist[2 * t + 1];
+        const int idx = blockIdx.x * kOrderThreads + t;
+        bins[0] = idx < n_pairs ? descs[idx].bin : 0u;
+    }
+    const int own[2] = {s_hist[2 * t], s_hist[2 * t + 1]};
+    const int start = block_exclusive_scan(own[0] + own[1], s_part);
+    s_start[2 * t] = start;
+    s_start[2 * t + 1] = start + own[0];
+    if (kAlone || blockIdx.x == 0) {
+        // warp tasks per bin (32 / T pairs per task), exclusive prefix over the bins
+        int tasks[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            int tl, rr;
+            shape_of_class((2 * t + k) % kNumClasses, tl, rr);
+            const int tpw = 32 >> tl;
+            tasks[k] = (own[k] + tpw - 1) >> (5 - tl);
+        }
+        const int task_start = block_exclusive_scan(tasks[0] + tasks[1], s_part);
+        ctl->start[2 * t] = start;
+        ctl->start[2 * t + 1] = start + own[0];
+        ctl->task_start[2 * t] = task_start;
+        ctl->task_start[2 * t + 1] = task_start + tasks[0];
+        if (kAlone) { ctl->hist[2 * t] = own[0]; ctl->hist[2 * t + 1] = own[1]; }
+        if (t == kOrderThreads - 1) {
+            ctl->task_start[kNumBins] = task_start + tasks[0] + tasks[1];
+            ctl->total_tasks = task_start + tasks[0] + tasks[1];
+            ctl->task_counter = 0;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if (!(bins[k] & kNeedsDp)) continue;
+        const int bin = (int)(bins[k] & kBinMask), idx = (blockIdx.x * kPer + k) * kOrderThreads + t;
+        order[kAlone ? atomicAdd(&s_start[bin], 1) : s_start[bin] + atomicAdd(&ctl->fill[bin], 1)] = idx;
+    }
 }
 
 // -------------------------------------------------------------------------- dp
@@ -557,38 +668,51 @@ __device__ __forceinline__ uint32_t shl_clamp(uint32_t v, uint32_t s) {
     return r;
 }
 
-// Match words of a quad of text columns for the R blocks a lane owns.  A position becomes a
-// one-hot word; an entry that names a mask row is read from it (`rows` points at the lane's
-// first word of the pattern's first row); a chain is walked.  Runs one quad ahead of the
-// recurrence, so that the loads of the rows are in flight while the previous quad is worked on.
+// Loads a lane's R words of a mask row where `p` is set, without a branch: the recurrence around
+// it stays one block of straight-line code.
 template <int R>
-__device__ __forceinline__ void match_words(uint2 q, uint32_t rowbase, int m, const uint32_t* __restrict__ rows,
-                                            int row_words, const uint16_t* __restrict__ nxt,
-                                            uint32_t (&Eq)[4][R]) {
+__device__ __forceinline__ void load_row_if(uint32_t p, const uint32_t* row, uint32_t (&Eq)[R]) {
+    static_assert(R >= 1 && R <= 4, "");
+    if constexpr (R == 1)
+        asm("{ .reg .pred p; setp.ne.u32 p, %1, 0; @p ld.global.nc.u32 %0, [%2]; }" : "+r"(Eq[0]) : "r"(p), "l"(row));
+    else if constexpr (R == 2)
+        asm("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p ld.global.nc.u32 %0, [%3]; @p ld.global.nc.u32 %1, [%3 + 4]; }"
+            : "+r"(Eq[0]), "+r"(Eq[1]) : "r"(p), "l"(row));
+    else if constexpr (R == 3)
+        asm("{ .reg .pred p; setp.ne.u32 p, %3, 0; @p ld.global.nc.u32 %0, [%4]; @p ld.global.nc.u32 %1, [%4 + 4]; "
+            "@p ld.global.nc.u32 %2, [%4 + 8]; }"
+            : "+r"(Eq[0]), "+r"(Eq[1]), "+r"(Eq[2]) : "r"(p), "l"(row));
+    else
+        asm("{ .reg .pred p; setp.ne.u32 p, %4, 0; @p ld.global.nc.u32 %0, [%5]; @p ld.global.nc.u32 %1, [%5 + 4]; "
+            "@p ld.global.nc.u32 %2, [%5 + 8]; @p ld.global.nc.u32 %3, [%5 + 12]; }"
+            : "+r"(Eq[0]), "+r"(Eq[1]), "+r"(Eq[2]), "+r"(Eq[3]) : "r"(p), "l"(row));
+}
+
+// Match words of a text column for the R blocks a lane owns.  A position becomes a
+// one-hot word; an entry that names a mask row is read from it (`words` points at the lane's
+// first word of the pattern's first row).
+template <int R>
+__device__ __forceinline__ void match_words(uint32_t loc, uint32_t rowbase, const uint32_t* __restrict__ words,
+                                            int row_words, uint32_t (&Eq)[R]) {
+    const uint32_t d0 = loc - rowbase;
+#pragma unroll
+    for (int r = 0; r < R; ++r) Eq[r] = shl_clamp(1u, d0 - 32u * r);     // 0 for rows and chains
+    load_row_if<R>((loc & kLocChain) == kLocRow, words + (loc & 0x3FFFu) * (uint32_t)row_words, Eq);
+}
+
+// The columns of a quad whose symbol is left as a chain of positions: walk it.
+template <int R>
+__device__ __forceinline__ void add_chains(uint2 q, uint32_t rowbase, const uint16_t* __restrict__ nxt, uint32_t (&Eq)[4][R]) {
     const uint32_t loc[4] = {q.x & 0xFFFFu, q.x >> 16, q.y & 0xFFFFu, q.y >> 16};
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const uint32_t d0 = loc[u] - rowbase;
+        if (loc[u] < kLocChain) continue;
+        uint32_t p = loc[u] & 0x3FFFu;
+        for (int hop = 0; hop < SR_MAX_K && p < (uint32_t)SR_MAX_K; ++hop) {   // a chain ends at 0xFFFF
+            const uint32_t dd = p - rowbase;
 #pragma unroll
-        for (int r = 0; r < R; ++r) Eq[u][r] = shl_clamp(1u, d0 - 32u * r);
-    }
-    if ((q.x | q.y) & (kLocRow | (kLocRow << 16))) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (!(loc[u] & kLocRow)) continue;
-            if ((loc[u] & kLocChain) == kLocRow) {
-                const uint32_t* row = rows + (loc[u] & 0x3FFFu) * (uint32_t)row_words;
-#pragma unroll
-                for (int r = 0; r < R; ++r) Eq[u][r] = __ldg(row + r);
-            } else {
-                uint32_t p = loc[u] & 0x3FFFu;
-                for (int hop = 0; hop < SR_MAX_K && p < (uint32_t)m; ++hop) {   // chain ends at 0xFFFF
-                    const uint32_t dd = p - rowbase;
-#pragma unroll
-                    for (int r = 0; r < R; ++r) Eq[u][r] |= shl_clamp(1u, dd - 32u * r);
-                    p = __ldg(nxt + p);
-                }
-            }
+            for (int r = 0; r < R; ++r) Eq[u][r] |= shl_clamp(1u, dd - 32u * r);
+            p = __ldg(nxt + p);
         }
     }
 }
@@ -605,31 +729,41 @@ __device__ __forceinline__ void column_step(const uint32_t (&Eq)[R],
     for (int r = 0; r < R; ++r) {
         const uint32_t pv = Pv[r], mv = Mv[r];
         const uint32_t hm = inM >> 31;
-        const uint32_t Xv = Eq[r] | mv;
-        const uint32_t Eh = Eq[r] | hm;
-        const uint32_t Xh = (((Eh & pv) + pv) ^ pv) | Eh;
-        const uint32_t Ph = mv | ~(Xh | pv);
-        const uint32_t Mh = pv & Xh;
+        // D0: the cells whose value equals that of their upper left neighbour
+        const uint32_t D0 = ((((Eq[r] | hm) & pv) + pv) ^ pv) | (Eq[r] | mv | hm);
+        const uint32_t Ph = mv | ~(D0 | pv);
+        const uint32_t Mh = pv & D0;
         const uint32_t Phs = __funnelshift_l(inP, Ph, 1);
         // `two` holds 2 but is a run-time value, so this shift-and-insert is a multiply-add:
         // it issues on the FMA pipe and leaves the integer ALU, the bottleneck, one
         // instruction lighter per block (measured: 8 % faster than a second funnel shift)
         const uint32_t Mhs = Mh * two + hm;              // (Mh << 1) | hm
-        Pv[r] = Mhs | ~(Xv | Phs);
-        Mv[r] = Phs & Xv;
+        Pv[r] = Mhs | ~(D0 | Phs);
+        Mv[r] = Phs & D0;
         inP = Ph;
         inM = Mh;
     }
 }
 
-// A warp task: 32/T teams of T lanes, one pair per team, lane l of a team holding
-// rows [32*R*l, 32*R*(l+1)) of the pattern.  Lanes are skewed by one QUAD of text
-// columns: in iteration j lane l works on columns 4(j-l) .. 4(j-l)+3.  The four
+// A warp task: 32/T teams of T lanes, one pair per team.  The pattern's blocks are grouped in
+// stripes of R blocks, stripe g on lane g mod T.  Lanes are skewed by one QUAD of text columns:
+// in iteration j stripe g works on columns 4(j-g) .. 4(j-g)+3.  The four
 // columns are unrolled, so (a) a lane fetches its four stream entries with one
-// 8-byte load, one iteration ahead, (b) the delta words a lane needs from the lane
-// above were produced a whole iteration earlier, so the shuffles never wait, and (c)
+// 8-byte load, ahead of their use, (b) the deltas a lane needs from the stripe
+// above (one +1 and one -1 bit per column, packed in two words) were produced a whole
+// iteration earlier, so the shuffles never wait, and (c)
 // the blocks of consecutive columns overlap in the pipeline.
-// (Not inlined on purpose: as eight separate functions the instantiations are
+//
+// Where the team has a lane for every stripe, each runs over all columns.  Otherwise (G > T) the
+// lanes form a ring that follows the band of the pair's bound: a stripe is run over the quads in
+// which the band crosses it, and when the band has left it its lane takes the stripe T places
+// further down, which starts from +1 vertical deltas below the stripe above; a stripe whose upper
+// neighbour the band has left takes +1 horizontal deltas from above.  The distance is then the sum
+// of the deltas along a path of cells that are all inside the band: down the first column of
+// every stripe it enters, along a stripe's bottom row until the next stripe begins, at the end less the
+// vertical deltas of the rows beyond the pattern's end.  A result above the pair's bound is
+// reported as bound + 1 with kCappedFlag.
+// (Not inlined on purpose: as separate functions the instantiations are
 // scheduled independently, which measured 8 % faster than one merged kernel body.)
 template <int R>
 __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDesc* descs,
@@ -639,99 +773,11 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
     const int lane = threadIdx.x & 31;
     const int T = 1 << tlog;
     const int lt = lane & (T - 1);
-    // m_all: the whole pattern (bounds the occurrence chains); m, n: rows and columns left
-    // after the common prefix of `strip` symbols, which neither side runs through
-    int idx = 0, m_all = 0, m = 0, n = 0, strip = 0;
-    const uint2* loc4 = reinterpret_cast<const uint2*>(locs);
-    const uint16_t* nxt = nexts;
-    const uint32_t* rows = masks;
-    if (valid) {
-        idx = order[pos];
-        const PairDesc d = descs[idx];
-        strip = (int)((d.bin >> kStripShift) & 0x3FFu);
-        m_all = (int)(d.mn & 0xFFFFu);
-        m = m_all - strip;
-        n = (int)(d.mn >> 16) - strip;
-        // rows are 16-byte aligned and strip is a multiple of 4 entries: 8-byte loads
-        loc4 = reinterpret_cast<const uint2*>(locs + (size_t)idx * W.pitch + strip);
-        nxt = nexts + (size_t)d.pat_row * W.pitch;
-        rows = masks + (size_t)d.pat_row * (W.row_cap * W.row_words) + (strip >> 5) + lt * R;
-    }
-    const uint32_t rowbase = (uint32_t)(lt * R * 32);
-    const uint32_t rowabs = rowbase + (uint32_t)strip;          // first pattern position of this lane
-    const int nq = (n + 3) >> 2;                       // quads of text columns
-    int iters = valid ? nq + T - 1 : 0;
-    iters = __reduce_max_sync(0xFFFFFFFFu, iters);
-    const bool top = lt == 0;
-
-    uint32_t Pv[R], Mv[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) { Pv[r] = 0xFFFFFFFFu; Mv[r] = 0u; }
-    uint32_t outP[4] = {0u, 0u, 0u, 0u}, outM[4] = {0u, 0u, 0u, 0u};
-    const uint2 none = make_uint2(kLocNone | (kLocNone << 16), kLocNone | (kLocNone << 16));
-    uint2 q_next = valid ? (top ? __ldg(loc4) : none) : none;
-    uint32_t Eq[4][R];
-    match_words<R>(q_next, rowabs, m_all, rows, W.row_words, nxt, Eq);
-    q_next = (valid && 1 - lt >= 0 && 1 - lt < nq) ? __ldg(loc4 + 1 - lt) : none;
-
-    for (int j = 0; j < iters; ++j) {
-        const int qi = j - lt;
-        const bool active = valid && qi >= 0 && qi < nq;
-        const uint2 q = q_next;                         // the quad after this one
-        q_next = (valid && qi + 2 >= 0 && qi + 2 < nq) ? __ldg(loc4 + qi + 2) : none;
-        // delta words leaving the lane above for this quad (it worked on it last iteration)
-        uint32_t inP[4], inM[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            inP[u] = __shfl_up_sync(0xFFFFFFFFu, outP[u], 1);
-            inM[u] = __shfl_up_sync(0xFFFFFFFFu, outM[u], 1);
-            if (top) { inP[u] = 0x80000000u; inM[u] = 0u; }   // row 0: D[0][c] - D[0][c-1] = +1
-        }
-        if (active) {
-            const int left = n - 4 * qi;               // columns of this quad that exist (>= 1)
-            column_step<R>(Eq[0], Pv, Mv, inP[0], inM[0], two);
-            if (left > 1) column_step<R>(Eq[1], Pv, Mv, inP[1], inM[1], two);
-            if (left > 2) column_step<R>(Eq[2], Pv, Mv, inP[2], inM[2], two);
-            if (left > 3) column_step<R>(Eq[3], Pv, Mv, inP[3], inM[3], two);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) { outP[u] = inP[u]; outM[u] = inM[u]; }
-        }
-        match_words<R>(q, rowabs, m_all, rows, W.row_words, nxt, Eq);
-    }
-    // D[m][n] = n + (sum of the vertical deltas of the last column over rows 1..m)
-    int part = 0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int rows = min(max(m - (int)(rowbase + 32 * r), 0), 32);
-        const uint32_t msk = low_mask(rows);
-        part += __popc(Pv[r] & msk) - __popc(Mv[r] & msk);
-    }
-    for (int off = 1; off < T; off <<= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, off);
-    if (valid && top) dist_out[idx] = n + part;
-}
-
-// A banded warp task: 32/T teams, one pair per team, the team's T lanes a ring.  The
-// pattern's blocks are grouped in stripes of R blocks; stripe g runs on lane g mod T over
-// the quads of text columns in which the band crosses it, one iteration behind stripe
-// g - 1, exactly like the lanes of the full task; when the band has left a stripe its lane
-// takes the stripe T places further down, which starts from +1 vertical deltas below the
-// stripe above; a stripe whose upper neighbour the band has left takes +1 horizontal
-// deltas from above.  A lane keeps the score at the bottom row of its stripe (started from
-// the stripe above plus the +1 deltas it is initialised with, then advanced by the
-// horizontal delta that leaves the stripe in every column); the pair's distance is that
-// score of the last stripe after the last column, less the vertical deltas of the rows
-// beyond the pattern's end.  A result above the pair's bound is reported as bound + 1 with
-// kCappedFlag.
-template <int R>
-__device__ __noinline__ void dp_task_band(int tlog, int pos, bool valid, const PairDesc* descs,
-                                             const int32_t* order, const uint16_t* locs,
-                                             const uint16_t* nexts, const uint32_t* masks, MultiWs W,
-                                             int32_t* dist_out, uint32_t two) {
-    const int lane = threadIdx.x & 31;
-    const int T = 1 << tlog;
-    const int lt = lane & (T - 1);
     const int src = (lane & ~(T - 1)) | ((lt - 1) & (T - 1));      // the lane of the stripe above
-    int idx = 0, m_all = 0, m = 0, n = 0, strip = 0, ub = 0;
+    // m, n: rows and columns left after the common prefix of `strip` symbols, which neither
+    // side runs through
+    bool chains = false;
+    int idx = 0, m = 0, n = 0, strip = 0, lb = 0, ub = 0;
     const uint2* loc4 = reinterpret_cast<const uint2*>(locs);
     const uint16_t* nxt = nexts;
     const uint32_t* rows = masks;
@@ -739,128 +785,133 @@ __device__ __noinline__ void dp_task_band(int tlog, int pos, bool valid, const P
         idx = order[pos];
         const PairDesc d = descs[idx];
         strip = (int)((d.bin >> kStripShift) & 0x3FFu);
-        m_all = (int)(d.mn & 0xFFFFu);
-        m = m_all - strip;
+        chains = d.bin & kHasChains;
         n = (int)(d.mn >> 16) - strip;
+        m = (int)(d.mn & 0xFFFFu) - strip + (-n & 3);  // both extended to whole quads of columns
+        n = (n + 3) & ~3;
+        lb = (int)(d.lower & 0xFFFFu);
         ub = (int)(d.lower >> 16);
+        // rows are 16-byte aligned and strip is a multiple of 4 entries: 8-byte loads
         loc4 = reinterpret_cast<const uint2*>(locs + (size_t)idx * W.pitch + strip);
         nxt = nexts + (size_t)d.pat_row * W.pitch;
         rows = masks + (size_t)d.pat_row * (W.row_cap * W.row_words) + (strip >> 5);
     }
-    int dlo, dhi;
-    band_of(m, n, ub, dlo, dhi);
-    const int nq = (n + 3) >> 2;                       // quads of text columns
-    const int G = valid ? (((m + 31) >> 5) + R - 1) / R : 0;       // stripes
-    int iters = valid ? nq + G - 1 : 0;
-    iters = __reduce_max_sync(0xFFFFFFFFu, iters);
-    // quads in which the band crosses stripe g: columns 32 R g - dhi .. 32 R (g + 1) - 1 - dlo
-    auto first_quad = [&](int g) { const int c = 32 * R * g - dhi; return c <= 0 ? 0 : c >> 2; };
-    auto last_quad = [&](int g) { return min((32 * R * (g + 1) - 1 - dlo) >> 2, nq - 1); };
-
+    constexpr int H = 32 * R;                          // rows of a stripe
+    const int nq = n >> 2;                             // quads of text columns
+    const int G = (m + H - 1) / H;                     // stripes (0: no pair)
+    const bool ring = G > T;
+    const bool any_ring = __any_sync(0xFFFFFFFFu, ring), any_chains = __any_sync(0xFFFFFFFFu, chains);
+    const int iters = __reduce_max_sync(0xFFFFFFFFu, G ? nq + G - 1 : 0);
+    // Stripe g crosses the band in columns H g - dhi .. H (g + 1) - 1 - dlo: quads first .. last,
+    // before they are clipped to the matrix.
+    int dlo = -2 * SR_MAX_K, dhi = 2 * SR_MAX_K;
+    if (ring) band_of(m, n, lb, ub, dlo, dhi);
     int g = lt;                                        // the stripe this lane holds
-    int js = 0x7FFFFFFF, je = -1, above_end = -1;      // its iterations; last quad of the stripe above
-    if (g < G) {
-        js = first_quad(g) + g;
-        je = last_quad(g) + g;
-        above_end = g > 0 ? last_quad(g - 1) : -1;
-    }
+    int first = (H * g - dhi) >> 2, last = (H * (g + 1) - 1 - dlo) >> 2;
+    // its first iteration and how many follow, the last iteration in which the stripe above feeds
+    // it and in which its bottom row is part of the path, its first pattern position, and
+    // where its stream (by iteration) and the mask rows' words begin
+    int js, above_until, acc_until;
+    uint32_t span, rowbase = (uint32_t)(strip + H * g);
+    const uint2* stream = loc4 - g;
+    const uint32_t* words = rows + R * g;
+    auto enter = [&]() {
+        js = max(first, 0) + g;
+        span = (uint32_t)(min(last, nq - 1) + g - js);
+        above_until = g > 0 ? last - H / 4 + g : -1;
+        acc_until = (g == G - 1 ? nq : max(first + H / 4, 0)) + g - 1;
+        if (g >= G) { js = 0x40000000; span = 0u; acc_until = -1; }
+    };
+    enter();
     uint32_t Pv[R], Mv[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) { Pv[r] = 0xFFFFFFFFu; Mv[r] = 0u; }
-    uint32_t outP[4] = {0u, 0u, 0u, 0u}, outM[4] = {0u, 0u, 0u, 0u};
-    uint32_t up = 0u, down = 0u;                       // +1 / -1 horizontal deltas seen at the stripe's bottom
-    int base = 0, before = 0;                          // score = base + up - down; score before the last quad
+    uint32_t outP = 0u, outM = 0u;                     // deltas leaving the stripe, latest column in bit 0
+    int acc = 0;
     const uint2 none = make_uint2(kLocNone | (kLocNone << 16), kLocNone | (kLocNone << 16));
-    uint2 q_next = none;
+    auto fetch = [&](int j) { return (uint32_t)(j - js) <= span ? __ldg(stream + j) : none; };
+    uint32_t Eq[4][R];
+    {
+        const uint2 q = fetch(0);
+        const uint32_t loc[4] = {q.x & 0xFFFFu, q.x >> 16, q.y & 0xFFFFu, q.y >> 16};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) match_words<R>(loc[u], rowbase, words, W.row_words, Eq[u]);
+        if (any_chains) add_chains<R>(q, rowbase, nxt, Eq);
+    }
+    uint2 q1 = fetch(1);
 
+    // The body is one block of straight-line code, so that the compiler can fill the latencies of
+    // one column's chain of operations with the others' and with the next quad's match words:
+    // a lane outside its stripe's quads runs along.  Before them it leaves its words alone by
+    // itself (no matches, nothing coming in from above: all-ones stay all-ones); after them its
+    // words are kept.
     for (int j = 0; j < iters; ++j) {
-        // delta words and score of the stripe above, as its lane left them one iteration ago
-        uint32_t inP[4], inM[4];
+        const uint2 q = q1;                            // the quad after this one
+        q1 = fetch(j + 2);
+        const bool active = (uint32_t)(j - js) <= span;
+        // deltas leaving the stripe above for this quad (it worked on it last iteration)
+        uint32_t wP = __shfl_sync(0xFFFFFFFFu, outP, src) << 28, wM = __shfl_sync(0xFFFFFFFFu, outM, src) << 28;
+        if (j > above_until) { wP = 0xF0000000u; wM = 0u; }    // row 0, or the band left the stripe above: +1 everywhere
+        if (!active) wP = wM = 0u;
+        uint32_t oldP[R], oldM[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) { oldP[r] = Pv[r]; oldM[r] = Mv[r]; }
+        const uint32_t loc[4] = {q.x & 0xFFFFu, q.x >> 16, q.y & 0xFFFFu, q.y >> 16};
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            inP[u] = __shfl_sync(0xFFFFFFFFu, outP[u], src);
-            inM[u] = __shfl_sync(0xFFFFFFFFu, outM[u], src);
+            uint32_t cP = wP, cM = wM;
+            column_step<R>(Eq[u], Pv, Mv, cP, cM, two);
+            outP = __funnelshift_l(cP, outP, 1);
+            outM = __funnelshift_l(cM, outM, 1);
+            wP *= two;                                 // shifts on the FMA pipe
+            wM *= two;
+            match_words<R>(loc[u], rowbase, words, W.row_words, Eq[u]);
         }
-        const int above_before = __shfl_sync(0xFFFFFFFFu, before, src);
-        if (j > je && g < G) {                         // the band has left this stripe: take the next one
-            g += T;
-            if (g < G) {
-                js = first_quad(g) + g;
-                je = last_quad(g) + g;
-                above_end = last_quad(g - 1);
+#pragma unroll
+        for (int r = 0; r < R; ++r) { Pv[r] = active ? Pv[r] : oldP[r]; Mv[r] = active ? Mv[r] : oldM[r]; }
+        if (any_chains) add_chains<R>(q, rowbase, nxt, Eq);
+        if (any_ring && active) {
+            if (ring && j <= acc_until) acc += __popc(outP & 0xFu) - __popc(outM & 0xFu);
+            if (g + T < G && (uint32_t)(j - js) == span) {   // the band has left this stripe
+                acc += H;
+                g += T;
+                first += T * (H / 4);
+                last += T * (H / 4);
+                rowbase += T * H;
+                stream -= T;
+                words += T * R;
+                enter();
 #pragma unroll
                 for (int r = 0; r < R; ++r) { Pv[r] = 0xFFFFFFFFu; Mv[r] = 0u; }
-            } else {
-                js = 0x7FFFFFFF;
-                je = -1;
             }
         }
-        if (j >= js && j <= je) {
-            const int qi = j - g;
-            uint2 q = q_next;
-            if (j == js) {
-                // first quad of the stripe: the rows start one apart below the stripe above
-                // (or below the matrix's first column)
-                q = __ldg(loc4 + qi);
-                base = qi > 0 ? above_before + 32 * R : 32 * R * (g + 1);
-                up = 0u;
-                down = 0u;
-            }
-            if (g == 0 || qi > above_end) {            // nothing above: row 0, or the band left it
-#pragma unroll
-                for (int u = 0; u < 4; ++u) { inP[u] = 0x80000000u; inM[u] = 0u; }
-            }
-            before = base + (int)up - (int)down;
-            const uint32_t rowabs = (uint32_t)(strip + 32 * R * g);
-            const int left = n - 4 * qi;               // columns of this quad that exist (>= 1)
-            uint32_t Eq[4][R];
-            match_words<R>(q, rowabs, m_all, rows + R * g, W.row_words, nxt, Eq);
-            column_step<R>(Eq[0], Pv, Mv, inP[0], inM[0], two);
-            up = __umulhi(inP[0], two) + up;           // top bit of the word: the delta leaving the stripe
-            down = __umulhi(inM[0], two) + down;
-            if (left > 1) {
-                column_step<R>(Eq[1], Pv, Mv, inP[1], inM[1], two);
-                up = __umulhi(inP[1], two) + up;
-                down = __umulhi(inM[1], two) + down;
-            }
-            if (left > 2) {
-                column_step<R>(Eq[2], Pv, Mv, inP[2], inM[2], two);
-                up = __umulhi(inP[2], two) + up;
-                down = __umulhi(inM[2], two) + down;
-            }
-            if (left > 3) {
-                column_step<R>(Eq[3], Pv, Mv, inP[3], inM[3], two);
-                up = __umulhi(inP[3], two) + up;
-                down = __umulhi(inM[3], two) + down;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) { outP[u] = inP[u]; outM[u] = inM[u]; }
-            if (g == G - 1 && qi == nq - 1) {
-                // the score at the stripe's bottom row, less the vertical deltas of the rows
-                // past the pattern's end
-                int d = base + (int)up - (int)down;
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int rows = min(max(m - 32 * (R * g + r), 0), 32);
-                    const uint32_t past = ~low_mask(rows);
-                    d -= __popc(Pv[r] & past) - __popc(Mv[r] & past);
-                }
-                dist_out[idx] = d > ub ? ((ub + 1) | kCappedFlag) : d;
-            }
-        }
-        q_next = (j + 1 > js && j + 1 <= je) ? __ldg(loc4 + (j + 1 - g)) : none;
     }
+    if (!ring) {
+        // D[m][n] = n + (sum of the vertical deltas of the last column over rows 1..m)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const uint32_t msk = low_mask(min(max(m - (H * lt + 32 * r), 0), 32));
+            acc += __popc(Pv[r] & msk) - __popc(Mv[r] & msk);
+        }
+        if (lt == 0) acc += n;
+    } else if (g < G) {                                // the lane's last stripe
+        acc += H;
+        if (g == G - 1) {                              // rows past the pattern's end
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const uint32_t past = ~low_mask(min(max(m - (H * g + 32 * r), 0), 32));
+                acc -= __popc(Pv[r] & past) - __popc(Mv[r] & past);
+            }
+        }
+    }
+    for (int off = 1; off < T; off <<= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
+    if (valid && lt == 0) dist_out[idx] = ring && acc > ub ? ((ub + 1) | kCappedFlag) : acc;
 }
 
-// Persistent warps pull warp tasks, longest first, from the bins' task list.  kBoth: the
-// batch has banded tasks as well (decide mode); CTAs with an odd index then serve those,
-// from a task counter of their own, and the even CTAs the full tasks, so that the two
-// kinds -- neither of which fills the machine -- run side by side.
-template <bool kBoth>
+// Persistent warps pull warp tasks, longest first, from the bins' task list.
 __global__ void __launch_bounds__(kDpWarpsPerCta * 32)
 multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
     grid_begin();
-    const bool kBand = kBoth && (blockIdx.x & 1);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
     const PairDesc* descs = reinterpret_cast<const PairDesc*>(ws + W.off_desc);
     const int32_t* order = reinterpret_cast<const int32_t*>(ws + W.off_order);
@@ -869,10 +920,9 @@ multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
     const uint32_t* masks = reinterpret_cast<const uint32_t*>(ws + W.off_rows);
     const int lane = threadIdx.x & 31;
     const int total = ctl->total_tasks;
-    int32_t* counter = kBand ? &ctl->task_counter_band : &ctl->task_counter;
     while (true) {
         int task = 0;
-        if (lane == 0) task = atomicAdd(counter, 1);
+        if (lane == 0) task = atomicAdd(&ctl->task_counter, 1);
         task = __shfl_sync(0xFFFFFFFFu, task, 0);
         if (task >= total) break;
         int k = 0, hi = kNumBins;                     // last bin whose first task is <= task
@@ -880,28 +930,16 @@ multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
             const int mid = (k + hi) >> 1;
             if (ctl->task_start[mid] <= task) k = mid; else hi = mid;
         }
-        if (is_band_class(k % kNumClasses) != kBand) continue;
         int tlog, R;
         shape_of_class(k % kNumClasses, tlog, R);
         const int tpw = 32 >> tlog;
         const int pos = ctl->start[k] + (task - ctl->task_start[k]) * tpw + (lane >> tlog);
-        const bool valid = pos < ctl->start[k] + ctl->fill[k];     // fill = pairs in the bin
-        if (kBand) {
-            switch (R) {
-                case 1: dp_task_band<1>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
-                case 2: dp_task_band<2>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
-                case 3: dp_task_band<3>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
-                default: dp_task_band<4>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
-            }
-        } else {
-            switch (R) {
-                case 1: dp_task<1>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
-                case 2: dp_task<2>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
-                case 3: dp_task<3>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
-                case 4: dp_task<4>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
-                case 5: dp_task<5>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
-                default: dp_task<6>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
-            }
+        const bool valid = pos < ctl->start[k] + ctl->hist[k];
+        switch (R) {
+            case 1: dp_task<1>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+            case 2: dp_task<2>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+            case 3: dp_task<3>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
+            default: dp_task<4>(tlog, pos, valid, descs, order, locs, nexts, masks, W, dist_out, two); break;
         }
     }
 }
@@ -918,123 +956,117 @@ multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
 // (L_p the longer prefix, 1 for raw distances).  The pair's band is cut to that cap (plus a
 // margin of two that swamps the rounding of this estimate); a pair whose banded result
 // exceeds its cap is reported as "more than the cap", which is all Eq. 2 needs to know.
-__global__ void __launch_bounds__(128)
-multi_bound_kernel(GateArgs a, PairDesc* descs, Ctl* ctl, uint8_t* flag, uint8_t* exact, int min_tlog) {
+// One thread per pair, gpb groups per CTA (more pairs than threads: several per thread); one
+// thread per group for the ordered sums.
+constexpr int kGroupThreads = 256;
+constexpr int kMaxPairs = SR_MAX_N * (SR_MAX_N - 1) / 2;       // pairs of a CTA: 256, or one group's
+
+__global__ void __launch_bounds__(kGroupThreads)
+multi_bound_kernel(GateArgs a, PairDesc* descs, Ctl* ctl, uint8_t* flag, uint8_t* exact, int gpb) {
     grid_begin();
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= a.n_groups) return;
-    const int N = a.N, P = pairs_of(N);
-    PairDesc* d = descs + (size_t)g * P;
-    double s = 0.0;
-    int isum = 0;
-    for (int p = 0; p < P; ++p) {
-        const int m = (int)(d[p].mn & 0xFFFFu), n = (int)(d[p].mn >> 16);
-        const int lb = (int)(d[p].lower & 0xFFFFu);
-        isum += lb;
-        s = __dadd_rn(s, pair_term(lb, m, n, a.norm_mode));      // max(m, n) is symmetric in the roles
+    __shared__ double s_term[kMaxPairs], s_sum[kGroupThreads];
+    __shared__ int s_lower[kMaxPairs], s_work, s_open;
+    const int P = pairs_of(a.N), tid = threadIdx.x;
+    const int g0 = blockIdx.x * gpb, ng = min(gpb, a.n_groups - g0);
+    PairDesc* d = descs + (size_t)g0 * P;
+    if (tid == 0) s_work = s_open = 0;
+    for (int e = tid; e < ng * P; e += kGroupThreads) {
+        const int m = (int)(d[e].mn & 0xFFFFu), n = (int)(d[e].mn >> 16);
+        s_lower[e] = (int)(d[e].lower & 0xFFFFu);
+        s_term[e] = pair_term(s_lower[e], m, n, a.norm_mode);        // max(m, n) is symmetric in the roles
     }
-    const double dk = __ddiv_rn(s, (double)P);
-    const bool open = dk < a.threshold;                  // the bound alone cannot decide
-    flag[g] = open ? 1 : 0;
-    if (exact) exact[g] = open ? 1 : 0;
-    if (open) {
-        const double budget = (double)P * a.threshold;
+    __syncthreads();
+    if (tid < ng) {
+        const int g = g0 + tid;
+        double s = 0.0;
+        int isum = 0;
         for (int p = 0; p < P; ++p) {
-            if (!(d[p].bin & kNeedsDp)) continue;
-            const int m = (int)(d[p].mn & 0xFFFFu), n = (int)(d[p].mn >> 16);
-            const int lb = (int)(d[p].lower & 0xFFFFu);
-            int ub = (int)(d[p].lower >> 16);
-            const double longer = a.norm_mode == SR_NORM_NONE ? 1.0 : (double)max(m, n);
-            const double room = (budget - (s - pair_term(lb, m, n, a.norm_mode))) * longer;
-            // room < 2^31 here: an open group has s < budget, so room <= (budget + term) * longer
-            const int cap = max(lb, (int)fmin(room, 1.0e9)) + 2;
-            ub = min(ub, cap);
-            const int strip = (int)((d[p].bin >> kStripShift) & 0x3FFu);
-            const int bin = shape_and_bin(m - strip, n - strip, ub, min_tlog);
-            d[p].bin = (uint32_t)bin | ((uint32_t)strip << kStripShift) | kNeedsDp;
-            d[p].lower = (uint32_t)lb | ((uint32_t)ub << 16);
-            atomicAdd(&ctl->hist[bin], 1);
+            isum += s_lower[tid * P + p];
+            s = __dadd_rn(s, s_term[tid * P + p]);
         }
-    } else {
-        for (int p = 0; p < P; ++p) d[p].bin &= ~kNeedsDp;
-        if (a.pair_sum) a.pair_sum[g] = isum;
-        if (a.mean) a.mean[g] = dk;
-        a.stop[g] = 0;
+        const double dk = __ddiv_rn(s, (double)P);
+        const bool open = dk < a.threshold;                  // the bound alone cannot decide
+        flag[g] = open ? 1 : 0;
+        if (exact) exact[g] = open ? 1 : 0;
+        s_sum[tid] = open ? s : __longlong_as_double(-1LL);  // NaN: settled
+        if (!open) {
+            if (a.pair_sum) a.pair_sum[g] = isum;
+            if (a.mean) a.mean[g] = dk;
+            a.stop[g] = 0;
+        }
+    }
+    __syncthreads();
+    const double budget = (double)P * a.threshold;
+    int work = 0, open = 0;
+    for (int e = tid; e < ng * P; e += kGroupThreads) {
+        PairDesc x = d[e];
+        if (!(x.bin & kNeedsDp)) continue;
+        const double s = s_sum[e / P];
+        if (s != s) {
+            d[e].bin = x.bin & ~kNeedsDp;
+            continue;
+        }
+        const int m = (int)(x.mn & 0xFFFFu), n = (int)(x.mn >> 16), lb = s_lower[e];
+        const double longer = a.norm_mode == SR_NORM_NONE ? 1.0 : (double)max(m, n);
+        const double room = (budget - (s - s_term[e])) * longer;
+        // room < 2^31 here: an open group has s < budget, so room <= (budget + term) * longer
+        const int ub = min((int)(x.lower >> 16), max(lb, (int)fmin(room, 1.0e9)) + 2);
+        x.lower = (uint32_t)lb | ((uint32_t)ub << 16);
+        d[e].lower = x.lower;
+        const PairSize z = size_of_desc(x);
+        work += work_of_pair(z.m, z.n, z.lb, z.ub);
+        ++open;
+    }
+    if (open) {
+        atomicAdd(&s_work, work);
+        atomicAdd(&s_open, open);
+    }
+    __syncthreads();
+    if (tid == 0 && s_open) {
+        atomicAdd(&ctl->work, (unsigned long long)s_work);
+        atomicAdd(&ctl->open, s_open);
     }
 }
 
 // ---------------------------------------------------------------------- finish
 // One thread per pair turns its distance into a term of d_K (the loads and divisions of a
 // group run side by side); one thread per group then adds the terms in pair order.
-constexpr int kFinishThreads = 256;
-
-__global__ void __launch_bounds__(kFinishThreads)
+__global__ void __launch_bounds__(kGroupThreads)
 multi_finish_kernel(GateArgs a, int32_t* dist, const uint8_t* flag, uint8_t* exact, int gpb) {
     grid_begin();
-    __shared__ double s_term[kFinishThreads];
-    __shared__ int32_t s_dist[kFinishThreads];
-    const int N = a.N, P = pairs_of(N);
-    const int tid = threadIdx.x;
-    const int g0 = blockIdx.x * gpb;
-    const int ng = min(gpb, a.n_groups - g0);
-    if (P <= kFinishThreads) {
-        if (tid < ng * P) {
-            const int g = tid / P, p = tid - g * P;
-            int i, j;
-            pair_from_index(p, N, i, j);
-            bool neg = false;
-            const int mi = clamp_len(a.lens, (size_t)(g0 + g) * N + i, a.K, neg);
-            const int mj = clamp_len(a.lens, (size_t)(g0 + g) * N + j, a.K, neg);
-            // decide mode marks a distance beyond its pair's cap: the value is then a lower bound
-            const int raw = dist[(size_t)g0 * P + tid];
-            const int d = raw & ~kCappedFlag;
-            if (raw != d) dist[(size_t)g0 * P + tid] = d;
-            s_dist[tid] = raw;
-            s_term[tid] = pair_term(d, mi, mj, a.norm_mode);
-        }
-        __syncthreads();
-        if (tid < ng) {
-            const int g = g0 + tid;
-            if (flag && flag[g] == 0) return;                // decided from the bounds
-            double s = 0.0;
-            int isum = 0, capped = 0;
-            for (int p = 0; p < P; ++p) {
-                s = __dadd_rn(s, s_term[tid * P + p]);
-                isum += s_dist[tid * P + p] & ~kCappedFlag;
-                capped |= s_dist[tid * P + p] & kCappedFlag;
-            }
-            const double dk = __ddiv_rn(s, (double)P);
-            if (a.pair_sum) a.pair_sum[g] = isum;
-            if (a.mean) a.mean[g] = dk;
-            a.stop[g] = dk < a.threshold ? 1 : 0;
-            if (capped && exact) exact[g] = 0;          // some distances are lower bounds
-        }
-        return;
+    __shared__ double s_term[kMaxPairs];
+    __shared__ int32_t s_dist[kMaxPairs];
+    const int N = a.N, P = pairs_of(N), tid = threadIdx.x;
+    const int g0 = blockIdx.x * gpb, ng = min(gpb, a.n_groups - g0);
+    for (int e = tid; e < ng * P; e += kGroupThreads) {
+        const int g = e / P, pr = kPairs.v[N][e - g * P];
+        bool neg = false;
+        const int mi = clamp_len(a.lens, (size_t)(g0 + g) * N + (pr & 0xFF), a.K, neg);
+        const int mj = clamp_len(a.lens, (size_t)(g0 + g) * N + (pr >> 8), a.K, neg);
+        // decide mode marks a distance beyond its pair's cap: the value is then a lower bound
+        const int raw = dist[(size_t)g0 * P + e];
+        const int d = raw & ~kCappedFlag;
+        if (raw != d) dist[(size_t)g0 * P + e] = d;
+        s_dist[e] = raw;
+        s_term[e] = pair_term(d, mi, mj, a.norm_mode);
     }
-    // groups of more than 23 rollouts (more pairs than threads): one thread per group
-    if (tid != 0) return;
-    const int g = g0;
-    if (flag && flag[g] == 0) return;
-    bool neg = false;
+    __syncthreads();
+    if (tid >= ng) return;
+    const int g = g0 + tid;
+    if (flag && flag[g] == 0) return;                        // decided from the bounds
     double s = 0.0;
-    int isum = 0, p = 0, capped = 0;
-    for (int i = 0; i < N; ++i) {
-        const int mi = clamp_len(a.lens, (size_t)g * N + i, a.K, neg);
-        for (int j = i + 1; j < N; ++j, ++p) {
-            const int mj = clamp_len(a.lens, (size_t)g * N + j, a.K, neg);
-            const int raw = dist[(size_t)g * P + p];
-            const int d = raw & ~kCappedFlag;
-            if (raw != d) dist[(size_t)g * P + p] = d;
-            capped |= raw & kCappedFlag;
-            isum += d;
-            s = __dadd_rn(s, pair_term(d, mi, mj, a.norm_mode));
-        }
+    int isum = 0, capped = 0;
+#pragma unroll 4
+    for (int p = 0; p < P; ++p) {
+        s = __dadd_rn(s, s_term[tid * P + p]);
+        isum += s_dist[tid * P + p] & ~kCappedFlag;
+        capped |= s_dist[tid * P + p] & kCappedFlag;
     }
     const double dk = __ddiv_rn(s, (double)P);
     if (a.pair_sum) a.pair_sum[g] = isum;
     if (a.mean) a.mean[g] = dk;
     a.stop[g] = dk < a.threshold ? 1 : 0;
-    if (capped && exact) exact[g] = 0;
+    if (capped && exact) exact[g] = 0;                       // some distances are lower bounds
 }
 
 }  // namespace
@@ -1057,16 +1089,10 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     int dev = 0, sms = 0;
     SR_CUDA_TRY(cudaGetDevice(&dev));
     SR_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // fewer than two pairs per resident warp (12 warps per SM): widen the teams until there
-    // are about eight lanes' worth of pairs per warp (measured on token-level batches of 16 to
-    // 256 groups: -40 % at 16 groups, -22 % at 64, nothing to gain from 128 on)
-    const long long warps = 12LL * sms;
-    if (n_pairs_ll < 2 * warps)
-        while (W.min_tlog < 5 && (n_pairs_ll << W.min_tlog) < 8 * warps) ++W.min_tlog;
-    // decide mode: what is left after the bounds is little work in a few long tasks, so the
-    // launch lasts as long as its longest pair: spread every pair over as many lanes as it
-    // has blocks (up to the whole warp), which shortens that pair fourfold
-    if (decide) W.min_tlog = 5;
+    // the dp kernel's persistent grid: 3 CTAs of 4 warps per SM (3 warps per scheduler): enough to
+    // keep the integer pipe busy, few enough that most tasks are pulled dynamically, longest
+    // first (measured best among 2..6 warps per scheduler)
+    W.warps = 3 * kDpWarpsPerCta * sms;
     const int n_pairs = (int)n_pairs_ll;
     int32_t* dist = a.pair_dist ? a.pair_dist : reinterpret_cast<int32_t*>(ws + W.off_dist);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
@@ -1076,9 +1102,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const int prep_smem = hslots * 8 + W.pitch * 4;
 
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[0], s));
-    // bin counts (filled by prep) and fill counters (used by the ordering kernel) start at zero
-    static_assert(offsetof(Ctl, fill) + sizeof(Ctl::fill) == 3 * kNumBins * sizeof(int32_t), "hist, start, fill lead Ctl");
-    SR_CUDA_TRY(cudaMemsetAsync(ctl, 0, 3 * kNumBins * sizeof(int32_t), s));
+    // what the kernels add up starts at zero (one CTA that orders the batch alone needs nothing)
+    const bool alone = n_pairs <= kAlonePairs;
+    if (!alone || decide) SR_CUDA_TRY(cudaMemsetAsync(ctl, 0, offsetof(Ctl, start), s));
     uint8_t* flag = decide ? ws + W.off_flag : nullptr;
     // The match-stream pass works group by group, so when the groups arrive in pieces it runs
     // piece by piece: `feed->before` enqueues whatever makes groups [g0, g1) ready on `s`.
@@ -1096,28 +1122,25 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
         else
             SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<false>, (g1 - g0) * a.N, kPrepThreads, prep_smem, s, a, ws, W, hslots, dist, g0);
     }
+    const int gpb = P <= kGroupThreads ? kGroupThreads / P : 1;
+    PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
+    int32_t* order = reinterpret_cast<int32_t*>(ws + W.off_order);
     if (decide) {
-        SR_LAUNCH("multi_bound_kernel", multi_bound_kernel, (a.n_groups + 127) / 128, 128, 0, s,  a, reinterpret_cast<PairDesc*>(ws + W.off_desc), ctl, flag, exact, W.min_tlog);
+        SR_LAUNCH("multi_bound_kernel", multi_bound_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, descs, ctl, flag, exact, gpb);
     }
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[1], s));
-    SR_LAUNCH("multi_order_kernel", multi_order_kernel, (n_pairs + kNumBins - 1) / kNumBins, kNumBins, 0, s,  reinterpret_cast<const PairDesc*>(ws + W.off_desc), reinterpret_cast<int32_t*>(ws + W.off_order), ctl, n_pairs);
+    const int order_blocks = alone ? 1 : (n_pairs + kOrderThreads - 1) / kOrderThreads;
+    if (!alone) SR_LAUNCH("multi_bin_kernel", multi_bin_kernel, order_blocks, kOrderThreads, 0, s, descs, ctl, n_pairs, W.warps);
+    SR_LAUNCH("multi_order_kernel", alone ? multi_order_kernel<true> : multi_order_kernel<false>, order_blocks, kOrderThreads, 0, s, descs, order, ctl, n_pairs, W.warps);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[2], s));
-    // persistent grid: a multiple of the SM count; warps pull tasks until none is left
-    long long want = (n_pairs_ll + kDpWarpsPerCta - 1) / kDpWarpsPerCta;
-    // 3 CTAs of 4 warps per SM (3 warps per scheduler): enough to keep the integer pipe
-    // busy, few enough that most tasks are pulled dynamically, longest first (measured
-    // best among 2..6 warps per scheduler)
-    long long cap = (long long)sms * 3;
-    int blocks = (int)(want < cap ? want : cap);
-    if (blocks < 1) blocks = 1;
+    const long long want = (n_pairs_ll + kDpWarpsPerCta - 1) / kDpWarpsPerCta;
+    const int blocks = (int)(want < 3LL * sms ? want : 3LL * sms);
     // (an ordinary launch: CTAs made resident while the tail of prep still fills some SMs would
     // crowd onto the others, 478 us instead of 434 for the token-level batch of 1024 groups)
-    const int rc = decide ? launch_as(false, "multi_dp_kernel", multi_dp_kernel<true>, 2 * blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u)
-                          : launch_as(false, "multi_dp_kernel", multi_dp_kernel<false>, blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u);
+    const int rc = launch_as(false, "multi_dp_kernel", multi_dp_kernel, blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u);
     if (rc != SR_OK) return rc;
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[3], s));
-    const int fin_gpb = P <= kFinishThreads ? kFinishThreads / P : 1;
-    SR_LAUNCH("multi_finish_kernel", multi_finish_kernel, (a.n_groups + fin_gpb - 1) / fin_gpb, kFinishThreads, 0, s, a, dist, flag, exact, fin_gpb);
+    SR_LAUNCH("multi_finish_kernel", multi_finish_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, dist, flag, exact, gpb);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[4], s));
     return SR_OK;
 }
