@@ -52,10 +52,10 @@ constexpr int kNumBins = 2048;      // kTimeBuckets * kNumClasses of them used
 constexpr int kOrderThreads = 1024;
 constexpr int kAlonePairs = 1024;   // batches of up to this many pairs are ordered by one CTA
 constexpr uint32_t kLocNone = 0x7FFFu;    // bit 15 clear, far above any row: shifts to 0
+constexpr uint32_t kLocOpen = 0xFFFFFFFFu;   // look-up not finished
 constexpr uint32_t kLocRow = 0x8000u;     // | index of the symbol's mask row
 constexpr uint32_t kLocChain = 0xC000u;   // | first position of the symbol's occurrence chain
 constexpr uint32_t kChainEnd = 0xFFFFu;
-constexpr int kRepeatedFlag = 0x10000;    // a text's stream holds row or chain entries
 constexpr int kPosPerThread = SR_MAX_K / kPrepThreads;
 constexpr int kDpWarpsPerCta = 4;
 constexpr uint32_t kBinMask = 0x7FFu;
@@ -222,76 +222,85 @@ __device__ __forceinline__ int clamp_len(const int32_t* lens, size_t idx, int K,
 }
 
 // ------------------------------------------------------------------------ prep
-// A slot of the pattern's hash table: symbol in the high word, position of the
-// claiming occurrence + 1 in the low word (0 = empty slot), so that one 8-byte
-// shared-memory load answers "empty, this symbol, or another symbol".
-__device__ __forceinline__ unsigned long long make_slot(int32_t sym, uint32_t pos_plus_1) {
-    return ((unsigned long long)(uint32_t)sym << 32) | pos_plus_1;
-}
+// Hash table of a pattern's symbols in shared memory.  A symbol times an odd constant is a
+// one-to-one map of the 32-bit words, so the upper bits of the product (the home bucket) and the lower
+// ones (the tag) name the symbol, and a slot of 32 bits can say all there is to know:
+//     tag | how many buckets from its home (0..2; 3: empty) | position of the symbol's first claimant
+// With four buckets of two slots per position these fields fill a word exactly.  A bucket is one
+// 8-byte load, and in 97 look-ups of a hundred the only one.  (Single slots, eight per position, sent
+// 8 % of the look-ups to a second slot, and so nearly every warp through a loop of three or four probes:
+// 370 instructions for four columns of a warp; slots of 64 bits with the whole symbol, four per
+// position, took the same space and collided as often.)
+// A symbol that finds no slot in its three buckets is left out and its positions are listed: a
+// look-up that runs into six foreign symbols searches the list, or the pattern itself where the
+// list was too short.
+constexpr int kMaxTexts = SR_MAX_N / 2;        // texts a pattern is paired with
+constexpr uint32_t kHashMul = 0x9E3779B1u;
+constexpr uint32_t kSlotEmpty = 0xFFFFFFFFu;
+constexpr uint32_t kMaxProbe = 2u;
+constexpr int kMaxListed = 8;
 
-// Stream entry of `sym` (its position, mask row or chain in the pattern hashed in shared
-// memory), given the content `v` of its home slot `h` (read by the caller, so that the first
-// probes of the four look-ups of a quad are in flight together).
-__device__ __forceinline__ uint32_t pattern_lookup(int32_t sym, uint32_t h, unsigned long long v,
-                                                   const unsigned long long* s_slot, int hslots) {
-    for (int probe = 0; probe < hslots; ++probe) {     // an empty slot always exists
-        const uint32_t o = (uint32_t)v;
-        if (o == 0u) break;
-        if ((int32_t)(v >> 32) == sym) return o - 1u;
-        h = (h + 1u) & (uint32_t)(hslots - 1);
-        v = s_slot[h];
+struct PatternTable {
+    uint32_t* slot;                    // [4 << pos_bits and kMaxProbe more][2]
+    int pos_bits, log_buckets;         // log_buckets = 2 + pos_bits
+    uint32_t pos_mask;
+    __device__ __forceinline__ uint32_t home(uint32_t x) const { return x >> (32 - log_buckets); }
+    __device__ __forceinline__ uint32_t tag(uint32_t x, uint32_t d) const { return (x << log_buckets) | (d << pos_bits); }
+    __device__ __forceinline__ bool holds(uint32_t e, uint32_t want) const { return ((e ^ want) & ~pos_mask) == 0u; }
+    __device__ __forceinline__ uint32_t position(uint32_t e) const { return e & pos_mask; }
+    // what a bucket says about a symbol: its position, not here nor further on, or neither
+    __device__ __forceinline__ uint32_t look(uint2 b, uint32_t want) const {
+        const bool first = holds(b.x, want);
+        uint32_t r = b.y == kSlotEmpty ? kLocNone : kLocOpen;
+        if (first || holds(b.y, want)) r = position(first ? b.x : b.y);
+        return r;
     }
-    return kLocNone;
-}
+};
 
-// Adds the lanes' values to a counter in shared memory; one atomic where they agree on it.
-__device__ __forceinline__ void warp_add(int* counter, int key, int v) {
-    const unsigned live = __activemask();
-    if (__all_sync(live, key == __shfl_sync(live, key, __ffs(live) - 1))) {
-        const int sum = __reduce_add_sync(live, v);
-        if (sum && (threadIdx.x & 31) == __ffs(live) - 1) atomicAdd(counter, sum);
-    } else if (v) {
-        atomicAdd(counter, v);
+// Position of the first `sym` among those left out of the table, m if there is none.
+__device__ __noinline__ uint32_t first_left_out(const int32_t* __restrict__ pat, int32_t sym, int m,
+                                                const uint16_t* s_list, int n_list) {
+    uint32_t first = (uint32_t)m;
+    if (n_list <= kMaxListed) {
+        for (int k = 0; k < n_list; ++k)
+            if (__ldg(pat + s_list[k]) == sym) first = min(first, (uint32_t)s_list[k]);
+    } else {
+        for (first = 0u; first < (uint32_t)m && __ldg(pat + first) != sym; ) ++first;
     }
+    return first;
 }
 
-// Per text it also counts the columns whose symbol does not occur in the pattern at all and
-// the positions at which text and pattern differ: bounds of the pair's distance that cost next
-// to nothing here.  Where they meet the pair is done.
+// One CTA per pattern.  Per text it also counts the columns whose symbol does not occur in the
+// pattern at all and the positions at which text and pattern differ: bounds of the pair's distance that
+// cost next to nothing here.  Where they meet the pair is done.
 template <bool kDecide>
 __global__ void __launch_bounds__(kPrepThreads, 6)
-multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int32_t* dist_out, int g_base) {
+multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base) {
     grid_begin();
     extern __shared__ __align__(16) unsigned char smem[];
-    unsigned long long* s_slot = reinterpret_cast<unsigned long long*>(smem);    // [hslots_max]
-    uint32_t* s_info = reinterpret_cast<uint32_t*>(s_slot + hslots_max);         // [pitch]
-    __shared__ int s_txt[SR_MAX_N], s_len[SR_MAX_N], s_qstart[SR_MAX_N + 1], s_absent[SR_MAX_N];
-    __shared__ int s_cp[SR_MAX_N], s_differ[SR_MAX_N];
+    uint32_t* s_info = reinterpret_cast<uint32_t*>(smem);         // [pitch] see below
+    uint32_t* s_slot = s_info + W.pitch;                          // [slots]
+    // (At K = 1024 the 36 KB of dynamic plus the static shared memory sit just under the size
+    // at which six CTAs share an SM.)
+    __shared__ int64_t s_text[kMaxTexts], s_stream[kMaxTexts];    // where a text's symbols and stream begin
+    __shared__ int s_txt[kMaxTexts], s_len[kMaxTexts], s_qstart[kMaxTexts + 1], s_cp[kMaxTexts];
+    __shared__ uint32_t s_count[kMaxTexts];  // differing positions | absent columns << 16
+    __shared__ uint32_t s_flag[kMaxTexts];   // the stream holds row or chain entries
     __shared__ int s_repeats[4];     // symbols with >= 2, 3, 4 occurrences; mask rows handed out
-    // (At K = 1024 the 36 KB of dynamic plus these 656 bytes of static shared memory sit just
-    // under the size at which six CTAs share an SM: 512 bytes more were measured to cost one
-    // CTA per SM and a fifth of the kernel's speed.  Smaller tables with more CTAs per SM are
-    // slower too: the probe length matters more than the residency.  Six CTAs of 256 threads
-    // leave 40 registers per thread, which the launch bounds grant: capped at 32 the kernel's
-    // time jumped by 10 % on changes as small as one more parameter.)
+    __shared__ int s_over;           // positions left out of the table, and the first of them
+    __shared__ uint16_t s_list[kMaxListed];
 
     const int N = a.N, K = a.K, P = pairs_of(N);
-    const int g = g_base + blockIdx.x / N, i = blockIdx.x % N;
-    const int tid = threadIdx.x;
-    const int M = (N & 1) ? N : N - 1;
-    if (i >= M) return;                               // the last rollout of an even group is never a pattern
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int M = (N & 1) ? N : N - 1;                // the last rollout of an even group is never a pattern
+    const int g = g_base + blockIdx.x / M, i = blockIdx.x % M;
     bool neg = false;
     const int m = clamp_len(a.lens, (size_t)g * N + i, K, neg);
-    // the table holds at least four times as many slots as the pattern has symbols:
-    // short probe sequences matter more than shared memory here (lanes wait for the
-    // longest probe of their warp)
-    int hslots = 64;
-    while (hslots < 4 * m) hslots <<= 1;
-    const int hshift = __clz(hslots) + 1;             // 32 - log2(hslots)
-    for (int q = tid; 4 * q < m; q += kPrepThreads)
-        reinterpret_cast<uint4*>(s_info)[q] = make_uint4(0u, 0u, 0u, 0u);
+    const int pos_bits = max(6, 32 - __clz(max(m, 1) - 1));       // of positions 0 .. m - 1
+    const PatternTable table{s_slot, pos_bits, 2 + pos_bits, (1u << pos_bits) - 1u};
+    const int slots = (8 << pos_bits) + 8;
     if (tid < 4) s_repeats[tid] = 0;
-    for (int h = tid; h < hslots; h += kPrepThreads) s_slot[h] = 0ull;
+    if (tid == 4) s_over = 0;
     // The texts this pattern is paired with, one warp per text.  The warp also measures the
     // common prefix of pattern and text (128 positions per trip, stopping at the first
     // mismatch): rollouts of one group start from the same state and often agree on their
@@ -299,6 +308,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
     // after a common prefix is removed, so those rows and columns are never looked up nor
     // run through the recurrence.
     const int32_t* pat = a.seqs + ((size_t)g * N + i) * a.stride;
+    const int4* pat4 = reinterpret_cast<const int4*>(pat);
     // Which rollout of a pair is the pattern follows a round-robin tournament: with M = N
     // for odd N and N - 1 otherwise, rollout i < M is the pattern against the `half` rollouts
     // after it (cyclically among the first M) and, for even N, against the last rollout,
@@ -308,45 +318,49 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
     const int half = (M - 1) / 2;
     const int n_before = max(0, i - half), n_after = min(i + half, M - 1) - i;
     const int ntxt = n_before + n_after + ((N & 1) ? 0 : 1);
-    {
-        const int lane = tid & 31;
-        for (int t = tid >> 5; t < ntxt; t += kPrepThreads / 32) {
-            const int j = t < n_before ? t : (t < n_before + n_after ? i + 1 + (t - n_before) : N - 1);
-            bool neg_t = false;
-            const int n = clamp_len(a.lens, (size_t)g * N + j, K, neg_t);
-            const int32_t* txt = a.seqs + ((size_t)g * N + j) * a.stride;
-            const int lo = min(m, n);
-            int cp = lo;                              // first mismatch; min(m, n) = none found
-            for (int base = 0; base < lo && cp == lo; base += 128) {
-                bool ne[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int p = base + 32 * u + lane;
-                    ne[u] = p < lo && __ldg(pat + p) != __ldg(txt + p);
-                }
-#pragma unroll
-                for (int u = 3; u >= 0; --u) {
-                    const unsigned b = __ballot_sync(0xFFFFFFFFu, ne[u]);
-                    if (b) cp = base + 32 * u + __ffs(b) - 1;
-                }
+    // the clears fall to the warps without a text, or to all if each has one
+    const int clearing = ntxt < kPrepThreads / 32 ? kPrepThreads - 32 * ntxt : kPrepThreads;
+    if (const int q = kPrepThreads - 1 - tid; q < clearing) {
+        for (int e = q; 4 * e < m; e += clearing) reinterpret_cast<uint4*>(s_info)[e] = make_uint4(0u, 0u, 0u, 0u);
+        for (int e = q; 4 * e < slots; e += clearing)
+            reinterpret_cast<uint4*>(s_slot)[e] = make_uint4(kSlotEmpty, kSlotEmpty, kSlotEmpty, kSlotEmpty);
+    }
+    for (int t = tid >> 5; t < ntxt; t += kPrepThreads / 32) {
+        const int j = t < n_before ? t : (t < n_before + n_after ? i + 1 + (t - n_before) : N - 1);
+        bool neg_t = false;
+        const int n = clamp_len(a.lens, (size_t)g * N + j, K, neg_t);
+        const int64_t row = ((int64_t)g * N + j) * a.stride;
+        const int4* txt4 = reinterpret_cast<const int4*>(a.seqs + row);
+        const int lo = min(m, n);
+        int cp = lo;                                  // first mismatch; min(m, n) = none found
+        for (int base = 0; base < lo && cp == lo; base += 128) {
+            const int at = base + 4 * lane;
+            int eq = 4;                               // symbols of the lane's quad that agree
+            if (at < lo) {
+                const int4 u = __ldg(pat4 + (at >> 2)), v = __ldg(txt4 + (at >> 2));
+                eq = u.x != v.x ? 0 : (u.y != v.y ? 1 : (u.z != v.z ? 2 : (u.w != v.w ? 3 : 4)));
             }
-            if (lane == 0) {
-                s_txt[t] = j;
-                s_len[t] = n;
-                s_absent[t] = 0;
-                s_differ[t] = 0;
-                s_cp[t] = cp;
-                if (neg_t && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
+            const unsigned b = __ballot_sync(0xFFFFFFFFu, eq < 4);
+            if (b) {
+                const int first = __ffs(b) - 1;
+                cp = min(base + 4 * first + __shfl_sync(0xFFFFFFFFu, eq, first), lo);
             }
+        }
+        if (lane == 0) {
+            s_txt[t] = j;
+            s_len[t] = n;
+            s_text[t] = row;
+            s_stream[t] = ((int64_t)g * P + pair_index(min(i, j), max(i, j), N)) * W.pitch;
+            s_count[t] = 0u;
+            s_flag[t] = 0u;
+            s_cp[t] = cp >= lo ? -1 : cp;             // -1: one prefix is the start of the other, nothing is left to do
+            if (neg_t && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
         }
     }
     __syncthreads();
     if (tid == 0) {
         int quads = 0;
         for (int t = 0; t < ntxt; ++t) {
-            const int lo = min(m, s_len[t]);
-            // if one prefix is the start of the other nothing is left to do
-            if (s_cp[t] >= lo) s_cp[t] = -1;
             s_qstart[t] = quads;
             quads += s_cp[t] < 0 ? 0 : (s_len[t] - (s_cp[t] & ~31) + 3) >> 2;
         }
@@ -354,38 +368,61 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
     }
     // Every position claims the slot of its symbol or counts itself as a further occurrence
     // with the position that did (s_info[claimant]).
-    uint32_t my_slot[kPosPerThread], my_first[kPosPerThread];
-    bool repeated = false;
+    uint32_t my_first[kPosPerThread];
+    bool repeated = false;           // or left out
 #pragma unroll
     for (int k = 0; k < kPosPerThread; ++k) {
-        const int p = tid + k * kPrepThreads;
-        my_slot[k] = 0u;
-        my_first[k] = (uint32_t)p;
-        if (p >= m) continue;
-        const int32_t sym = __ldg(pat + p);
-        uint32_t h = ((uint32_t)sym * 0x9E3779B1u) >> hshift;
-        const unsigned long long mine = make_slot(sym, (uint32_t)p + 1u);
-        for (int probe = 0; probe < hslots; ++probe) {
-            unsigned long long v = s_slot[h];
-            if ((uint32_t)v == 0u) v = atomicCAS(&s_slot[h], 0ull, mine);
-            if ((uint32_t)v == 0u) break;
-            if ((int32_t)(v >> 32) == sym) {
-                my_first[k] = (uint32_t)v - 1u;
-                atomicAdd(&s_info[my_first[k]], 1u);
-                repeated = true;
-                break;
+        const uint32_t p = tid + k * kPrepThreads;
+        my_first[k] = p;
+        if (p >= (uint32_t)m) continue;
+        const uint32_t x = (uint32_t)__ldg(pat + p) * kHashMul, h = table.home(x);
+        bool placed = false;
+        for (uint32_t d = 0; !placed && d <= kMaxProbe; ++d) {
+            const uint32_t want = table.tag(x, d);
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t* at = &s_slot[2u * (h + d) + half];
+                uint32_t e = *at;
+                if (e == kSlotEmpty) e = atomicCAS(at, kSlotEmpty, want | p);
+                if (e == kSlotEmpty) { placed = true; break; }
+                if (table.holds(e, want)) {
+                    my_first[k] = table.position(e);
+                    placed = true;
+                    break;
+                }
             }
-            h = (h + 1u) & (uint32_t)(hslots - 1);
         }
-        my_slot[k] = h;
+        if (!placed) {
+            const int at = atomicAdd(&s_over, 1);
+            if (at < kMaxListed) s_list[at] = (uint16_t)p;
+            my_first[k] = kLocOpen;
+            repeated = true;
+        } else if (my_first[k] != p) {
+            atomicAdd(&s_info[my_first[k]], 1u);
+            repeated = true;
+        }
     }
     if (__syncthreads_or(repeated)) {
+        if (s_over) {
+#pragma unroll
+            for (int k = 0; k < kPosPerThread; ++k) {
+                const uint32_t p = tid + k * kPrepThreads;
+                if (my_first[k] != kLocOpen) continue;
+                my_first[k] = first_left_out(pat, __ldg(pat + p), m, s_list, s_over);
+                if (my_first[k] != p) atomicAdd(&s_info[my_first[k]], 1u);
+            }
+            __syncthreads();
+        }
         // Symbols with several occurrences.  In written language a few tokens make up much of
         // every rollout (a third of the columns of such a text meet a symbol that occurs more
         // than once, the most common one dozens of times), so these get a row of match words,
-        // one per 32 positions, which the recurrence reads in place of its one-hot word.  The
-        // pool has room for every symbol with at least eight occurrences; what does not fit
+        // one per 32 positions, which the recurrence reads in place of its one-hot word.  (Walking
+        // a chain of occurrences per column made the recurrence wait for the longest chain of the
+        // warp: 16 groups of 8 such texts of up to 1024 tokens took 2.2 ms, with the rows 0.16 ms.)
+        // The pool has room for every symbol with at least eight occurrences; what does not fit
         // (the rarest of the repeated ones) is left as a chain of at most seven positions.
+        // From here on the lower half of s_info[claimant] is the symbol's stream entry, the upper half
+        // the head of the chain of its further positions.
 #pragma unroll
         for (int k = 0; k < kPosPerThread; ++k) {
             const int p = tid + k * kPrepThreads;
@@ -400,10 +437,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
             const int p = tid + k * kPrepThreads;
             if (p >= m || my_first[k] != (uint32_t)p) continue;
             const uint32_t more = s_info[p];
-            if (more == 0u) continue;
-            const uint32_t code = more >= need ? kLocRow | (uint32_t)atomicAdd(&s_repeats[3], 1) : kLocChain | (uint32_t)p;
-            s_info[p] = more >= need ? code : kChainEnd;
-            s_slot[my_slot[k]] = make_slot(__ldg(pat + p), code + 1u);
+            s_info[p] = more == 0u ? (uint32_t)p : (more >= need ? kLocRow | (uint32_t)atomicAdd(&s_repeats[3], 1) : (kChainEnd << 16) | kLocChain | (uint32_t)p);
         }
         __syncthreads();
         uint32_t* rows = reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * N + i) * W.row_cap * W.row_words;
@@ -414,91 +448,133 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int hslots_max, int3
             const int p = tid + k * kPrepThreads;
             if (p >= m) continue;
             const uint32_t f = my_first[k], info = s_info[f];
-            if ((info & kLocChain) == kLocRow)         // not a chain's end (all bits set) nor a count or position
+            if ((info & kLocChain) == kLocChain) {
+                if (f != (uint32_t)p) s_info[p] = atomicExch(&s_info[f], ((uint32_t)p << 16) | kLocChain | f);
+            } else if (info & kLocRow) {
                 atomicOr(&rows[(info & 0x3FFFu) * W.row_words + (p >> 5)], 1u << (p & 31));
-            else if (f != (uint32_t)p)
-                s_info[p] = atomicExch(&s_info[f], (uint32_t)p);
+            }
         }
         if (s_repeats[0] > s_repeats[3]) {             // some chains: leave them for the recurrence
             __syncthreads();
             uint16_t* g_next = reinterpret_cast<uint16_t*>(ws + W.off_next) + ((size_t)g * N + i) * W.pitch;
-            for (int p = tid; p < m; p += kPrepThreads) g_next[p] = (uint16_t)s_info[p];
+            for (int p = tid; p < m; p += kPrepThreads) g_next[p] = (uint16_t)(s_info[p] >> 16);
         }
     }
+    const bool named = s_repeats[0] > 0;
+    const int left_out = s_over;
 
-    PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
+    // Match streams of all texts, four columns per thread and trip: one 16-byte load of
+    // symbols, four independent look-ups, one 8-byte store.
     uint16_t* locs = reinterpret_cast<uint16_t*>(ws + W.off_loc);
-    Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
-    // match streams of all texts, four columns per thread and trip: one 16-byte load
-    // of symbols, four independent look-ups, one 8-byte store
     const int total_quads = s_qstart[ntxt];
-    for (int item = tid; item < total_quads; item += kPrepThreads) {
+    for (int base = tid - lane; base < total_quads; base += kPrepThreads) {
+        const int item = min(base + lane, total_quads - 1);        // lanes past the end run along
+        const bool live = base + lane < total_quads;
         int t = 0;
         while (item >= s_qstart[t + 1]) ++t;
         const int q = ((s_cp[t] & ~31) >> 2) + item - s_qstart[t];      // quad index within the text
-        const int j = s_txt[t];
-        const int lo = min(i, j), hi = max(i, j);
-        const size_t idx = (size_t)g * P + pair_index(lo, hi, N);
-        const int4 sym = __ldg(reinterpret_cast<const int4*>(a.seqs + ((size_t)g * N + j) * a.stride) + q);
-        const uint32_t h0 = ((uint32_t)sym.x * 0x9E3779B1u) >> hshift, h1 = ((uint32_t)sym.y * 0x9E3779B1u) >> hshift;
-        const uint32_t h2 = ((uint32_t)sym.z * 0x9E3779B1u) >> hshift, h3 = ((uint32_t)sym.w * 0x9E3779B1u) >> hshift;
-        const unsigned long long v0 = s_slot[h0], v1 = s_slot[h1], v2 = s_slot[h2], v3 = s_slot[h3];
-        const uint32_t l0 = pattern_lookup(sym.x, h0, v0, s_slot, hslots);
-        const uint32_t l1 = pattern_lookup(sym.y, h1, v1, s_slot, hslots);
-        const uint32_t l2 = pattern_lookup(sym.z, h2, v2, s_slot, hslots);
-        const uint32_t l3 = pattern_lookup(sym.w, h3, v3, s_slot, hslots);
+        const int4 sym4 = __ldg(reinterpret_cast<const int4*>(a.seqs + s_text[t]) + q);
+        const int32_t sym[4] = {sym4.x, sym4.y, sym4.z, sym4.w};
+        uint32_t home[4], want[4], l[4];
+        uint2 e[4];
+        bool more = false;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t x = (uint32_t)sym[u] * kHashMul;
+            home[u] = table.home(x);
+            want[u] = table.tag(x, 0u);
+            e[u] = reinterpret_cast<const uint2*>(s_slot)[home[u]];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            l[u] = table.look(e[u], want[u]);
+            more |= l[u] == kLocOpen;
+        }
+        for (uint32_t d = 1; more && d <= kMaxProbe; ++d) {        // the home bucket holds two foreign symbols
+            more = false;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (l[u] != kLocOpen) continue;
+                l[u] = table.look(reinterpret_cast<const uint2*>(s_slot)[home[u] + d], want[u] | (d << pos_bits));
+                more |= l[u] == kLocOpen;
+            }
+        }
+        if (more) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (l[u] != kLocOpen) continue;
+                l[u] = kLocNone;
+                if (left_out) {
+                    const uint32_t p = first_left_out(pat, sym[u], m, s_list, left_out);
+                    if (p < (uint32_t)m) l[u] = p;
+                }
+            }
+        }
+        if (named) {                                   // positions to stream entries
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (l[u] != kLocNone) l[u] = reinterpret_cast<const uint16_t*>(s_info)[2u * l[u]];
+        }
         // The last quad of a text is filled up with symbols of their own that the pattern is
         // extended by as well: a common suffix leaves the distance as it is, and the recurrence
         // always runs whole quads, whose four columns the compiler can then interleave.
-        const uint32_t left = (uint32_t)(s_len[t] - 4 * q);  // columns of this quad that exist (>= 1)
-        const uint32_t w1 = left > 1u ? l1 : (uint32_t)m, w2 = left > 2u ? l2 : (uint32_t)m + 2u - left;
-        const uint32_t w3 = left > 3u ? l3 : (uint32_t)m + 3u - left;
-        reinterpret_cast<uint2*>(locs + idx * W.pitch)[q] = make_uint2(l0 | (w1 << 16), w2 | (w3 << 16));
-        if (((l0 | w1 | w2 | w3) & kLocRow) && !(s_absent[t] & kRepeatedFlag)) atomicOr(&s_absent[t], kRepeatedFlag);
-        {
-            // positions below both lengths whose symbol is not the pattern's symbol at the same place
-            const int both = min(m, s_len[t]) - 4 * q;       // columns of this quad below both lengths
-            int differ = 0;
-            if (both > 0) {
-                const int4 own = __ldg(reinterpret_cast<const int4*>(pat) + q);
-                differ = (sym.x != own.x) + (both > 1 && sym.y != own.y) + (both > 2 && sym.z != own.z) +
-                         (both > 3 && sym.w != own.w);
-            }
-            warp_add(&s_differ[t], t, differ);
-            const int absent = (l0 == kLocNone) + (w1 == kLocNone) + (w2 == kLocNone) + (w3 == kLocNone);
-            warp_add(&s_absent[t], t, absent);
+        const int left = s_len[t] - 4 * q;             // columns of this quad that exist (>= 1)
+#pragma unroll
+        for (int u = 1; u < 4; ++u)
+            if (u >= left) l[u] = (uint32_t)(m + u - left);
+        if (live) reinterpret_cast<uint2*>(locs + s_stream[t])[q] = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
+        if (named && ((l[0] | l[1] | l[2] | l[3]) & kLocRow)) s_flag[t] = 1u;
+        // positions below both lengths whose symbol is not the pattern's symbol at the same place,
+        // and columns without any match
+        uint32_t count = 0u;
+        const int both = min(m, s_len[t]) - 4 * q;     // columns of this quad below both lengths
+        if (both > 0) {
+            const int4 own = __ldg(pat4 + q);
+            count = (sym[0] != own.x) + (both > 1 && sym[1] != own.y) + (both > 2 && sym[2] != own.z) +
+                    (both > 3 && sym[3] != own.w);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) count += l[u] == kLocNone ? 0x10000u : 0u;
+        if (!live) count = 0u;
+        // quads of a warp follow one another, so most warps work on one text
+        const int t_first = __shfl_sync(0xFFFFFFFFu, t, 0);
+        if (t_first == __shfl_sync(0xFFFFFFFFu, t, 31)) {
+            count = __reduce_add_sync(0xFFFFFFFFu, count);
+            if (lane == 0) atomicAdd(&s_count[t], count);
+        } else if (count) {
+            atomicAdd(&s_count[t], count);
         }
     }
     __syncthreads();
+    if (tid >= 32) return;                             // descriptors: the texts' threads are in the first warp
+    PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
+    Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
     int work = 0;
-    if (tid < ntxt) {                                 // descriptors, bins, trivial pairs
+    if (tid < ntxt) {
         const int j = s_txt[tid], n = s_len[tid];
         // the removed prefix is a multiple of four symbols (the match stream is read in 8-byte
         // quads), and of 32 where the stream refers to mask rows (whose words start there)
-        const int strip = s_cp[tid] < 0 ? -1 : (s_cp[tid] & (s_absent[tid] & kRepeatedFlag ? ~31 : ~3));
-        const int lo = min(i, j), hi = max(i, j);
-        const size_t idx = (size_t)g * P + pair_index(lo, hi, N);
+        const int strip = s_cp[tid] < 0 ? -1 : (s_cp[tid] & (s_flag[tid] ? ~31 : ~3));
+        const size_t idx = (size_t)g * P + pair_index(min(i, j), max(i, j), N);
         // Upper bound of the distance: substitute the differing positions, insert or delete the
         // rest.  Lower bound: every text column without a match costs an edit, and if the pattern
         // is at least as long as the text, m - n rows are deleted besides.
         int lower = abs(m - n), upper = lower;        // one prefix starts the other (or is empty)
         if (strip >= 0) {
-            const int absent = s_absent[tid] & (kRepeatedFlag - 1);
+            const int absent = (int)(s_count[tid] >> 16);
             lower = m >= n ? m - n + absent : max(n - m, absent);
-            upper += s_differ[tid];
+            upper += (int)(s_count[tid] & 0xFFFFu);
         }
         PairDesc d{(uint32_t)m | ((uint32_t)n << 16), (uint32_t)(g * N + i), 0u, (uint32_t)lower | ((uint32_t)upper << 16)};
         if (lower < upper) {                          // otherwise that is the distance
             d.bin = ((uint32_t)strip << kStripShift) | kNeedsDp | (s_repeats[0] > s_repeats[3] ? kHasChains : 0u);
-            if (!kDecide) {                           // decide mode counts the pairs it keeps later
-                const PairSize z = size_of_desc(d);
-                work = work_of_pair(z.m, z.n, z.lb, z.ub);
-            }
+            const PairSize z = size_of_desc(d);
+            work = work_of_pair(z.m, z.n, z.lb, z.ub);
         }
         descs[idx] = d;
         if (kDecide || lower == upper) dist_out[idx] = lower;
     }
-    if (!kDecide && tid < 32) {                       // the texts' threads are those of the first warp
+    if (!kDecide) {                                   // decide mode counts the pairs it keeps later
         const int open = __popc(__ballot_sync(0xFFFFFFFFu, work > 0));
         work = __reduce_add_sync(0xFFFFFFFFu, work);
         if (tid == 0 && open) {
@@ -1097,9 +1173,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     int32_t* dist = a.pair_dist ? a.pair_dist : reinterpret_cast<int32_t*>(ws + W.off_dist);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
 
-    int hslots = 64;
-    while (hslots < 4 * a.K) hslots <<= 1;
-    const int prep_smem = hslots * 8 + W.pitch * 4;
+    int pos_bits = 6;
+    while ((1 << pos_bits) < a.K) ++pos_bits;
+    const int prep_smem = (W.pitch + (8 << pos_bits) + 8) * 4, patterns = (a.N & 1) ? a.N : a.N - 1;
 
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[0], s));
     // what the kernels add up starts at zero (one CTA that orders the batch alone needs nothing)
@@ -1118,9 +1194,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
             if (rc != SR_OK) return rc;
         }
         if (decide)
-            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<true>, (g1 - g0) * a.N, kPrepThreads, prep_smem, s, a, ws, W, hslots, dist, g0);
+            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<true>, (g1 - g0) * patterns, kPrepThreads, prep_smem, s, a, ws, W, dist, g0);
         else
-            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<false>, (g1 - g0) * a.N, kPrepThreads, prep_smem, s, a, ws, W, hslots, dist, g0);
+            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<false>, (g1 - g0) * patterns, kPrepThreads, prep_smem, s, a, ws, W, dist, g0);
     }
     const int gpb = P <= kGroupThreads ? kGroupThreads / P : 1;
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);

@@ -24,3 +24,20 @@ def test_symbols_with_a_given_number_of_occurrences(K, times):
     lens[0] = K
     want = oracle.gate(seqs, lens, K, 0.4, threads=8)
     assert_gate_matches(gate_gpu(seqs, lens, K, 0.4), want, f"K={K}, {times} occurrences")
+
+
+@pytest.mark.parametrize("K", [64, 300, 1024])
+def test_symbols_that_crowd_one_slot_of_the_table(K):
+    """IDs chosen so that dozens of them hash to the same home slot: more than its neighbourhood holds."""
+    rng = np.random.default_rng(K)
+    inverse = pow(0x9E3779B1, -1, 1 << 32)
+    crowd = (np.array([5 << 25], dtype=np.uint64) + np.arange(40, dtype=np.uint64)) * np.uint64(inverse) % np.uint64(1 << 32)
+    crowd = crowd.astype(np.uint32).view(np.int32)
+    G, N, stride = 5, 6, (K + 3) // 4 * 4
+    seqs = rng.integers(-2 ** 31, 2 ** 31, size=(G, N, stride)).astype(np.int32)
+    pick = rng.random((G, N, stride)) < np.array([0.05, 0.3, 0.9, 0.9, 0.5]).reshape(G, 1, 1)
+    seqs[pick] = rng.choice(crowd, size=int(pick.sum()))
+    seqs[3, 1:] = np.where(rng.random((N - 1, stride)) < 0.1, seqs[3, 1:], seqs[3, :1])
+    lens = rng.integers(K // 2 + 1, K + 1, size=(G, N)).astype(np.int32)
+    want = oracle.gate(seqs, lens, K, 0.4, threads=8)
+    assert_gate_matches(gate_gpu(seqs, lens, K, 0.4), want, f"K={K}")
