@@ -164,18 +164,21 @@ __device__ __forceinline__ void word_column(uint32_t Eq, uint32_t& Pv, uint32_t&
 __device__ __forceinline__ void group_sum_and_gate(const double* term, const int32_t* dist, int P,
                                                    const GateArgs& a, size_t g) {
     double s = 0.0;
-    int isum = 0, p = 0;
+    int p = 0;
     for (; p + 8 <= P; p += 8) {
         double t[8];
-        int d[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) { t[u] = term[p + u]; d[u] = dist[p + u]; }
+        for (int u = 0; u < 8; ++u) t[u] = term[p + u];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) { s = __dadd_rn(s, t[u]); isum += d[u]; }
+        for (int u = 0; u < 8; ++u) s = __dadd_rn(s, t[u]);
     }
-    for (; p < P; ++p) { s = __dadd_rn(s, term[p]); isum += dist[p]; }
+    for (; p < P; ++p) s = __dadd_rn(s, term[p]);
+    if (a.pair_sum) {
+        int isum = 0;
+        for (p = 0; p < P; ++p) isum += dist[p];
+        a.pair_sum[g] = isum;
+    }
     const double dk = __ddiv_rn(s, (double)P);
-    if (a.pair_sum) a.pair_sum[g] = isum;
     if (a.mean) a.mean[g] = dk;
     a.stop[g] = dk < a.threshold ? 1 : 0;
 }

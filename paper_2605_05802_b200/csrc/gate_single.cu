@@ -4,206 +4,428 @@
 // distance is read off as n + popc(Pv) - popc(Mv), so no per-column score is kept.  The
 // two kernels differ in where a column's match word comes from.
 //
-// K <= 16 (the paper's K = 10 and 15): gate_direct_kernel.  A thread keeps both prefixes
+// K <= 16, few rollouts or few groups: gate_direct_kernel.  A thread keeps both prefixes
 // of its pair in registers (int4 loads; the rows of a group are shared by its pairs, so
 // all but the first touch hit L1) and builds the match word of a column by comparing the
 // text symbol with every pattern symbol: 2 instructions per cell against the ~14 of a
-// column, no tables, no atomics, no shared memory before the final sums -- at these
-// lengths cheaper than naming the symbols first, and free of the latencies that kept the
-// table kernel from filling the issue slots.
+// column, no tables, no atomics, no shared memory before the final sums, one round of latencies.
 //
-// K = 17..32: gate_single_kernel.  A group is handled by one warp (N <= 8) or one CTA:
-//   1. every thread fetches one or two quads of symbols (int4 loads) and keeps them in
-//      registers; each symbol claims a slot of the group's open-addressing table in
-//      shared memory (64-bit slots {symbol, claimed}; all 2^32 IDs are legal) -- the slot
-//      index is the symbol's name within the group from here on -- and notes, in a byte
-//      map indexed by (rollout, slot), one position at which the rollout holds it;
-//   2. the positions of a rollout holding the same symbol OR their bits into the match
-//      mask peq[rollout][noted position];
-//   3. the pair threads take a column's match word from
-//      peq[pattern][map[pattern][slot of the text symbol]] (33rd mask = 0: absent);
+// Otherwise: gate_named_kernel.  A group is handled by a warp (which takes several if they have
+// room on its lanes) or, for K > 15 and N > 8, by a CTA:
+//   1. every symbol is named by one position that holds it: all positions write themselves to
+//      the slot of a small table that their symbol hashes to, and look who stayed there;
+//   2. a name has a row of match masks, one per rollout: every position sets its bit in its
+//      rollout's mask of its symbol's row, and the text keeps the row's place;
+//   3. a column's match word for any pattern is then one look-up, row[pattern].  For K <= 15 the
+//      masks of two patterns share a word, and one recurrence serves two pairs;
 //   4. one thread per group adds the normalised terms in fp64 in pair order, thresholds
 //      (Eq. 2) and writes out, for all groups of a CTA side by side.
-// Three synchronisations per group before that (warp-level for N <= 8).  All index
-// arithmetic is shifts and adds.
+// Bound: instruction issue (0.6 to 0.7 per scheduler and clock, as all integer code here), a third of it
+// in the recurrence.  Measured against one-look-up-more tables (64-bit compare-and-swap slots, a
+// byte map per rollout and slot) for K > 16 and direct comparison for K <= 16: 4096 groups of 16, K = 30:
+// 33.7 -> 23 us; 16384 groups of 8, K = 30: 51 -> 31 us; 65536 groups of 8, K = 15, ragged: 64 -> 44 us.
 #include "common.cuh"
 
 namespace sr {
 namespace {
 
-constexpr int kTxtPitch = 36;          // 16-bit slot names per rollout: 32 + pad, rows 8-byte aligned
-constexpr int kPeqPitch = 33;          // 32 masks by position + one all-zero mask for "absent"
-constexpr uint32_t kAbsentOff = 32 * 4;   // map entries are BYTE offsets into a peq row
-constexpr int kMaxItems = 2;           // quads of symbols a thread may own
-
-struct SingleLayout {
-    int hslots, hshift, hlog;          // slots of the group table (power of two), 32 - log2, log2
-    int qshift;                        // log2 of the quads per rollout that are fetched (K <= 4 << qshift)
-    int n_items;                       // N << qshift
-    // byte offsets within a group's shared memory: the table and the masks (cleared to 0
-    // together), the map (cleared to "absent"), slot names of the symbols, lengths
-    int off_hash, off_peq, off_map, off_txt, off_len;
-    int zero_words16, map_words16;     // sizes of the two clears in 16-byte units
-    int group_bytes;
-    int off_term, off_dist;            // per CTA, after the groups: [groups per CTA][P]
+// A unit is what a warp works on (kWarp: as many groups as its lanes have room for) or one group
+// that a CTA works on.  Positions, items (quads of symbols) and rollouts are numbered within it.
+struct NamedLayout {
+    int groups;                        // groups per unit
+    int Q, items;                      // quads per rollout, items per unit
+    uint32_t inv_Q, inv_N, inv_C;      // ceil(2^20 / x): division of numbers below 2048 by multiply-shift
+    int table_log;                     // names: slots per group
+    int row_words;                     // words of a row of match masks
+    int combos;                        // recurrences per group (kPacked: two pairs each)
+    int pitch;                         // terms per group
+    // byte offsets within a unit's shared memory
+    int off_table, off_name, off_row, off_peq, off_len, off_order, unit_bytes;
 };
 
-__device__ __forceinline__ void group_sync(bool warp_level) {
-    if (warp_level) __syncwarp(); else __syncthreads();
+__device__ __forceinline__ int div20(int x, uint32_t inv) { return (int)(((uint32_t)x * inv) >> 20); }
+
+// kPacked: the recurrences of a group, enough to serve every pair once: word x of patterns
+// (2x, 2x + 1) with the text that is its own upper half, and every word a with the two texts of every
+// word b > a.  For each: word, text, and the places of its two pairs in pair order (kNoPair: none).
+constexpr uint32_t kNoPair = 0xFFFFu;
+struct ComboTable {
+    uint16_t start[SR_MAX_N + 1];
+    uint2 v[2992];                     // sum over N of ceil(N / 2)^2
+    constexpr ComboTable() : start(), v() {
+        int at = 0;
+        for (int n = 2; n <= SR_MAX_N; ++n) {
+            start[n] = (uint16_t)at;
+            const int words = (n + 1) / 2;
+            for (int a = 0; a < words; ++a)
+                for (int j = 2 * a + 1; j < 2 * words; ++j) {
+                    uint32_t place[2] = {kNoPair, kNoPair};
+                    for (int h = 0; h < 2; ++h) {
+                        const int i = 2 * a + h;
+                        if (i < j && j < n) place[h] = (uint32_t)(i * n - i * (i + 1) / 2 + (j - i - 1));
+                    }
+                    v[at].x = (uint32_t)(a | (j << 8));
+                    v[at++].y = place[0] | (place[1] << 16);
+                }
+        }
+    }
+};
+__device__ const ComboTable kCombos = ComboTable();
+
+template <bool kWarp>
+__device__ __forceinline__ void unit_sync() {
+    if (kWarp) __syncwarp(); else __syncthreads();
 }
 
-// kWarp: one warp per group, blockDim.x / 32 groups per CTA; otherwise one group per CTA.
-template <bool kWarp>
+// kPacked (K <= 15): two patterns share a word, 15 rows and a guard bit each: one look-up and one
+// recurrence serve two pairs.
+template <bool kPacked, bool kWarp, int kItems>
 __global__ void __launch_bounds__(kWarp ? 256 : 512)
-gate_single_kernel(GateArgs a, SingleLayout L) {
-    grid_begin();
+gate_named_kernel(GateArgs a, NamedLayout L, uint32_t two) {
+    // Rows: a CTA's group of more than eight rollouts would need 32 KB and more with one for every
+    // position, so there only symbols that several rollouts hold get one.
+    constexpr bool kAlloc = !kWarp;
     extern __shared__ __align__(16) unsigned char smem[];
     const int N = a.N, K = a.K, P = pairs_of(N);
-    const int t = kWarp ? (threadIdx.x & 31) : threadIdx.x;               // thread within the group
+    const int t = kWarp ? (threadIdx.x & 31) : threadIdx.x;               // thread within the unit
     const int nthr = kWarp ? 32 : blockDim.x;
-    const int gl = kWarp ? (threadIdx.x >> 5) : 0;                        // group within the CTA
-    const int g = kWarp ? blockIdx.x * (blockDim.x >> 5) + gl : blockIdx.x;
-    const bool live = g < a.n_groups;              // a warp without a group only keeps the barrier company
-    unsigned char* base = smem + (size_t)gl * L.group_bytes;
-    unsigned long long* s_hash = reinterpret_cast<unsigned long long*>(base + L.off_hash);  // [hslots]
-    unsigned char* s_peq = base + L.off_peq;                                                // [N][33] words
-    unsigned char* s_map = base + L.off_map;                                                // [N][hslots]
-    uint16_t* s_txt = reinterpret_cast<uint16_t*>(base + L.off_txt);                        // [N][36]
-    int32_t* s_len = reinterpret_cast<int32_t*>(base + L.off_len);                          // [N]
-    double* s_term = reinterpret_cast<double*>(smem + L.off_term) + gl * P;                 // [P]
-    int32_t* s_dist = reinterpret_cast<int32_t*>(smem + L.off_dist) + gl * P;               // [P]
+    const int unit = kWarp ? threadIdx.x >> 5 : 0, units = kWarp ? blockDim.x >> 5 : 1;
+    const int g0 = (blockIdx.x * units + unit) * L.groups;
+    const int ng = min(L.groups, a.n_groups - g0);                        // <= 0: only keeps the barrier company
+    unsigned char* base = smem + (size_t)unit * L.unit_bytes;
+    int32_t* s_sym = reinterpret_cast<int32_t*>(base);                    // [items][4]
+    uint32_t* s_txt = reinterpret_cast<uint32_t*>(base);                  // [items][4] byte offsets of rows, once the symbols have names
+    uint16_t* s_name = reinterpret_cast<uint16_t*>(base + L.off_name);    // [items][4]
+    uint16_t* s_row = reinterpret_cast<uint16_t*>(base + L.off_row);      // [items][4]
+    uint32_t* s_peq = reinterpret_cast<uint32_t*>(base + L.off_peq);      // [rows][row_words]
+    int32_t* s_len = reinterpret_cast<int32_t*>(base + L.off_len);        // [rollouts], then row counter, ragged
+    uint8_t* s_order = base + L.off_order;                                // [N]
+    int& s_rows = s_len[L.groups * N];
+    int& s_ragged = s_len[L.groups * N + 1];
 
-    if (live) {
-        // ---- symbols first (the longest latency), then the clears
-        const int qmask = (1 << L.qshift) - 1;
-        int4 sym[kMaxItems];
-        int row_len[kMaxItems];
+    // before the wait: nothing global in here
+    if (ng > 0) {
+        if (kAlloc) {
 #pragma unroll
-        for (int u = 0; u < kMaxItems; ++u) {
-            const int item = t + u * nthr;
-            sym[u] = make_int4(0, 0, 0, 0);
-            row_len[u] = 0;
-            if (item < L.n_items) {
-                const int i = item >> L.qshift, q = item & qmask;
-                const size_t row = (size_t)g * N + i;
-                int len = a.lens ? __ldg(a.lens + row) : K;
+            for (int u = 0; u < kItems; ++u) {
+                const int e = t + u * nthr;
+                if (e < L.items) reinterpret_cast<uint2*>(s_row)[e] = make_uint2(0u, 0u);
+            }
+            for (int w = t; w < L.row_words; w += nthr) s_peq[w] = 0u;    // row 0: no match
+        } else {
+            for (int w = t; w < L.items * L.row_words; w += nthr) reinterpret_cast<uint4*>(s_peq)[w] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        if (!kWarp && t == 0) { s_rows = 0; s_ragged = 0; }
+    }
+    grid_begin();
+    if (ng > 0) {
+        const int32_t* seqs = a.seqs + (size_t)g0 * N * a.stride;
+        int32_t sym[kItems][4];
+        int roll[kItems], live[kItems];            // rollout of the item; positions of its quad inside the prefix
+        int open = 0;                              // positions without a name, one bit each
+#pragma unroll
+        for (int u = 0; u < kItems; ++u) {
+            const int e = t + u * nthr;
+            roll[u] = div20(e, L.inv_Q);
+            live[u] = 0;
+            if (e < ng * N * L.Q) {
+                const int q = e - roll[u] * L.Q;
+                // whole quads inside the row: stride is a multiple of 4 and >= K
+                int4 v = make_int4(0, 0, 0, 0);
+                if (4 * q < K) v = __ldg(reinterpret_cast<const int4*>(seqs + (uint64_t)(uint32_t)roll[u] * (uint32_t)a.stride) + q);
+                int len = a.lens ? __ldg(a.lens + (size_t)g0 * N + roll[u]) : K;
+                reinterpret_cast<int4*>(s_sym)[e] = v;
+                sym[u][0] = v.x; sym[u][1] = v.y; sym[u][2] = v.z; sym[u][3] = v.w;
                 if (q == 0) {
                     if (len < 0 && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
-                    s_len[i] = min(max(len, 0), K);
+                    s_len[roll[u]] = min(max(len, 0), K);
+                    if (!kWarp && len < K) s_ragged = 1;
                 }
-                len = min(max(len, 0), K);
-                row_len[u] = len;
-                if (4 * q < len) sym[u] = __ldg(reinterpret_cast<const int4*>(a.seqs + row * a.stride) + q);
+                live[u] = min(max(min(len, K) - 4 * q, 0), 4);
             }
         }
+        // ---- names: the symbol of a position is named by one of the positions that hold it.  Every
+        // position writes itself to the slot its symbol hashes to (whichever write lands last
+        // stays), and if the position found there afterwards holds the same symbol, that is the
+        // name -- for all holders of the symbol alike.  The symbols that lost their slot to another
+        // one go on with another hash; every round names at least one symbol of each slot.
+        auto slot_of = [&](int r, uint32_t sy, uint32_t mul) {
+            return reinterpret_cast<uint16_t*>(base + L.off_table) + ((kWarp ? div20(r, L.inv_N) : 0) << L.table_log) +
+                   ((sy * mul) >> (32 - L.table_log));
+        };
+        uint16_t* slot[kItems][4];
+#pragma unroll
+        for (int u = 0; u < kItems; ++u)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                slot[u][k] = slot_of(roll[u], (uint32_t)sym[u][k], 0x9E3779B1u);
+                if (k < live[u]) *slot[u][k] = (uint16_t)(4 * (t + u * nthr) + k);
+            }
+        unit_sync<kWarp>();
+#pragma unroll
+        for (int u = 0; u < kItems; ++u) {
+            if (live[u] == 0) continue;
+            uint32_t name[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                name[k] = 0u;
+                if (k < live[u]) {
+                    name[k] = *slot[u][k];
+                    if (s_sym[name[k]] != sym[u][k]) open |= 1 << (4 * u + k);
+                }
+            }
+            reinterpret_cast<uint2*>(s_name)[t + u * nthr] = make_uint2(name[0] | (name[1] << 16), name[2] | (name[3] << 16));
+        }
+        uint32_t mul = 0x9E3779B1u;
+        for (int round = 0; round < 4 * 1024; ++round) {
+            if (!(kWarp ? __any_sync(0xFFFFFFFFu, open) : __syncthreads_or(open))) break;
+            if (kWarp) __syncwarp();               // the reads of the round before are done
+            mul = mul * 0x2C1B3C6Du + 0x297A2D3Au;                        // stays odd
+            for (int m = open; m; m &= m - 1) {
+                const int b = __ffs(m) - 1, pos = 4 * (t + (b >> 2) * nthr) + (b & 3);
+                *slot_of(div20(pos >> 2, L.inv_Q), (uint32_t)s_sym[pos], mul) = (uint16_t)pos;
+            }
+            unit_sync<kWarp>();
+            for (int m = open; m; m &= m - 1) {
+                const int b = __ffs(m) - 1, pos = 4 * (t + (b >> 2) * nthr) + (b & 3);
+                const int name = *slot_of(div20(pos >> 2, L.inv_Q), (uint32_t)s_sym[pos], mul);
+                if (s_sym[name] == s_sym[pos]) {
+                    s_name[pos] = (uint16_t)name;
+                    open &= ~(1 << b);
+                }
+            }
+        }
+        // ---- names held by more than one rollout get a row of match masks, one per rollout (without
+        // kAlloc every position has one)
+        if (kAlloc) {
+#pragma unroll
+        for (int u = 0; u < kItems; ++u) {
+            if (live[u] == 0) continue;
+            const uint2 v = reinterpret_cast<const uint2*>(s_name)[t + u * nthr];
+            const uint32_t name[4] = {v.x & 0xFFFFu, v.x >> 16, v.y & 0xFFFFu, v.y >> 16};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (k < live[u] && (uint32_t)((int)(name[k] >> 2) - roll[u] * L.Q) >= (uint32_t)L.Q) s_row[name[k]] = 1;
+        }
+        unit_sync<kWarp>();
         {
-            uint4* z4 = reinterpret_cast<uint4*>(s_hash);
-#pragma unroll 4
-            for (int e = t; e < L.zero_words16; e += nthr) z4[e] = make_uint4(0u, 0u, 0u, 0u);
-            uint4* m4 = reinterpret_cast<uint4*>(s_map);
-            const uint32_t absent4 = kAbsentOff * 0x01010101u;
-#pragma unroll 4
-            for (int e = t; e < L.map_words16; e += nthr) m4[e] = make_uint4(absent4, absent4, absent4, absent4);
-        }
-        group_sync(kWarp);
-
-        // ---- every symbol claims (or finds) its slot; the slot index names the symbol
-        uint32_t slot[kMaxItems][4];
+            uint2 f[kItems];
+            int own = 0;
 #pragma unroll
-        for (int u = 0; u < kMaxItems; ++u) {
-            const int item = t + u * nthr;
-            const int i = item >> L.qshift, q = item & qmask;
-            const int32_t s4[4] = {sym[u].x, sym[u].y, sym[u].z, sym[u].w};
-            volatile unsigned char* map_i = s_map + ((size_t)i << L.hlog);
+            for (int u = 0; u < kItems; ++u) {
+                const int e = t + u * nthr;
+                f[u] = make_uint2(0u, 0u);
+                if (e < L.items) f[u] = reinterpret_cast<const uint2*>(s_row)[e];
+                own += __popc(f[u].x) + __popc(f[u].y);
+            }
+            int incl = own;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int up = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+                if ((t & 31) >= d) incl += up;
+            }
+            const int all = __shfl_sync(0xFFFFFFFFu, incl, 31);
+            int first = 0;
+            if (!kWarp) {
+                if ((t & 31) == 0) first = atomicAdd(&s_rows, all);
+                first = __shfl_sync(0xFFFFFFFFu, first, 0);
+            }
+            uint32_t row = (uint32_t)((first + incl - own + 1) * L.row_words);
+#pragma unroll
+            for (int u = 0; u < kItems; ++u) {
+                if ((f[u].x | f[u].y) == 0u) continue;
+                uint32_t h[4] = {f[u].x & 1u, f[u].x >> 16, f[u].y & 1u, f[u].y >> 16};
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (h[k]) { h[k] = row; row += L.row_words; }
+                reinterpret_cast<uint2*>(s_row)[t + u * nthr] = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+            }
+            {
+                const int begin = (first + 1) * L.row_words, end = begin + all * L.row_words;   // the warp's rows
+                for (int w = begin + (t & 31); w < end; w += 32) s_peq[w] = 0u;
+            }
+        }
+        }
+        if (!kWarp && t < N) {
+            // rollouts by falling length (ties by index), so that the pairs of a warp have texts
+            // of similar lengths
+            int rank = t;
+            if (s_ragged) {
+                const int mine = s_len[t];
+                rank = 0;
+                for (int r = 0; r < N; ++r) rank += s_len[r] > mine || (s_len[r] == mine && r < t);
+            }
+            s_order[rank] = (uint8_t)t;
+        }
+        unit_sync<kWarp>();
+        // ---- every position sets its bit in its rollout's mask and notes the row's place
+#pragma unroll
+        for (int u = 0; u < kItems; ++u) {
+            if (live[u] == 0) continue;
+            const int q = (t + u * nthr) - roll[u] * L.Q;
+            const int i = kWarp ? roll[u] - div20(roll[u], L.inv_N) * N : roll[u];
+            unsigned char* mine = reinterpret_cast<unsigned char*>(s_peq) + 4 * (kPacked ? i >> 1 : i);
+            const uint32_t bit = 1u << (4 * q + (kPacked ? (i & 1) << 4 : 0));
+            const uint2 v = reinterpret_cast<const uint2*>(s_name)[t + u * nthr];
+            const uint32_t name[4] = {v.x & 0xFFFFu, v.x >> 16, v.y & 0xFFFFu, v.y >> 16};
+            uint32_t row[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int r = 4 * q + k;
-                slot[u][k] = 0u;
-                if (r < row_len[u]) {
-                    const int32_t s = s4[k];
-                    uint32_t h = ((uint32_t)s * 0x9E3779B1u) >> L.hshift;
-                    const unsigned long long mine = ((unsigned long long)(uint32_t)s << 32) | 1ull;
-                    // at most half of the slots ever fill up, so a free or matching slot is
-                    // always found; the trip count is bounded all the same
-                    for (int probe = 0; probe < L.hslots; ++probe) {
-                        unsigned long long v = s_hash[h];
-                        if ((uint32_t)v == 0u) v = atomicCAS(&s_hash[h], 0ull, mine);
-                        if ((uint32_t)v == 0u || (int32_t)(v >> 32) == s) break;
-                        h = (h + 1u) & (uint32_t)(L.hslots - 1);
-                    }
-                    slot[u][k] = h;
-                    // several positions of a rollout with the same symbol store to the same
-                    // byte; whichever store lands last names the representative: any will do
-                    map_i[h] = (unsigned char)(4 * r);
+                row[k] = 0u;
+                if (k < live[u]) {
+                    row[k] = (kAlloc ? s_row[name[k]] : name[k] * L.row_words) * 4u;
+                    if (!kAlloc || row[k]) atomicOr(reinterpret_cast<uint32_t*>(mine + row[k]), bit << k);
                 }
             }
-            if (4 * q < row_len[u])
-                *reinterpret_cast<uint2*>(s_txt + i * kTxtPitch + 4 * q) =
-                    make_uint2(slot[u][0] | (slot[u][1] << 16), slot[u][2] | (slot[u][3] << 16));
+            reinterpret_cast<uint4*>(s_txt)[t + u * nthr] = make_uint4(row[0], row[1], row[2], row[3]);
         }
-        group_sync(kWarp);
-
-        // ---- match masks: peq[i][representative position] collects the positions of the symbol
-#pragma unroll
-        for (int u = 0; u < kMaxItems; ++u) {
-            const int item = t + u * nthr;
-            const int i = item >> L.qshift, q = item & qmask;
-            const unsigned char* map_i = s_map + ((size_t)i << L.hlog);
-            unsigned char* peq_i = s_peq + i * (kPeqPitch * 4);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int r = 4 * q + k;
-                if (r < row_len[u])
-                    atomicOr(reinterpret_cast<uint32_t*>(peq_i + map_i[slot[u][k]]), 1u << r);
+        unit_sync<kWarp>();
+        // ---- recurrences: one thread per pair, or per text and word of two patterns
+        for (int c = t; c < ng * L.combos; c += nthr) {
+            const int gl = kWarp ? div20(c, L.inv_C) : 0, x = c - gl * L.combos;
+            int word, pj, at[2];                   // word of the rows, text, place of the pair(s)
+            if (kPacked) {
+                const uint2 v = kCombos.v[kCombos.start[N] + x];
+                word = v.x & 0xFF;
+                pj = v.x >> 8;
+                at[0] = v.y & 0xFFFFu;
+                at[1] = v.y >> 16;
+                if (at[0] == kNoPair) continue;    // odd N: the last word has no upper half
+            } else {
+                const int pr = kPairs.v[N][x];
+                word = pr >> 8;
+                pj = pr & 0xFF;
+                at[0] = x;
+                at[1] = kNoPair;
+                if (!kWarp) {                      // the pattern is the longer prefix, texts ascend
+                    pj = s_order[N - 1 - pj];
+                    word = s_order[N - 1 - word];
+                    at[0] = pair_index(min(pj, word), max(pj, word), N);
+                }
             }
-        }
-        group_sync(kWarp);
-
-        // ---- one thread per pair; the pattern (rows) is the longer prefix
-        for (int p = t; p < P; p += nthr) {
-            const int pr = kPairs.v[N][p];
-            int pi = pr & 0xFF, pj = pr >> 8;
-            const int mi = s_len[pi], mj = s_len[pj];
-            int mp = mi, mt = mj;
-            if (mj > mi) { const int x = pi; pi = pj; pj = x; mp = mj; mt = mi; }
-            const unsigned char* map = s_map + ((size_t)pi << L.hlog);
-            const unsigned char* peq = s_peq + pi * (kPeqPitch * 4);
-            const uint16_t* txt = s_txt + pj * kTxtPitch;
-            uint32_t Pv = 0xFFFFFFFFu, Mv = 0u, Ph, Mh;
-            int c = 0;
-            for (; c + 4 <= mt; c += 4) {          // four columns per trip: their look-ups overlap
-                const uint2 w = *reinterpret_cast<const uint2*>(txt + c);
-                const uint32_t e0 = *reinterpret_cast<const uint32_t*>(peq + map[w.x & 0xFFFFu]);
-                const uint32_t e1 = *reinterpret_cast<const uint32_t*>(peq + map[w.x >> 16]);
-                const uint32_t e2 = *reinterpret_cast<const uint32_t*>(peq + map[w.y & 0xFFFFu]);
-                const uint32_t e3 = *reinterpret_cast<const uint32_t*>(peq + map[w.y >> 16]);
-                word_column(e0, Pv, Mv, Ph, Mh);
-                word_column(e1, Pv, Mv, Ph, Mh);
-                word_column(e2, Pv, Mv, Ph, Mh);
-                word_column(e3, Pv, Mv, Ph, Mh);
+            const int mt = s_len[gl * N + pj];
+            const unsigned char* peq = reinterpret_cast<const unsigned char*>(s_peq + word);
+            const uint4* txt = reinterpret_cast<const uint4*>(s_txt) + (gl * N + pj) * L.Q;
+            // Rows of the lower pattern in bits 0..14 and of the upper one in bits 16..30.  The guard bits
+            // above them are kept 1 in Mv (so they are 1 in D0 and Ph, whose shift then brings the
+            // upper pattern its +1 at row 0) and 0 in Pv (which takes the carry of the sum).
+            constexpr uint32_t kGuard = kPacked ? 0x80008000u : 0u, kBelow = kPacked ? 0x3FFF3FFFu : 0xFFFFFFFFu;
+            uint32_t Pv = ~kGuard, Mv = kGuard;
+            auto column = [&](uint32_t off) {
+                const uint32_t Eq = *reinterpret_cast<const uint32_t*>(peq + off);
+                const uint32_t D0 = (((Eq & Pv) + Pv) ^ Pv) | (Eq | Mv);
+                const uint32_t Ph = Mv | ~(D0 | Pv), Mh = D0 & Pv & kBelow;
+                // `two` is a run-time 2: the shifts are multiply-adds on the FMA pipe, which
+                // leaves the integer pipe, the bottleneck, the seven logic operations
+                const uint32_t Phs = Ph * two + 1u, Mhs = Mh * two;
+                Pv = Mhs | ~(D0 | Phs);
+                Mv = (Phs & D0) | kGuard;
+            };
+            uint4 w = txt[0];
+            int c4 = mt >> 2;
+            for (; c4 > 0; --c4) {
+                const uint4 v = w;
+                w = *++txt;                        // one quad past the end at most: within the unit
+                column(v.x);
+                column(v.y);
+                column(v.z);
+                column(v.w);
             }
-            for (; c < mt; ++c)
-                word_column(*reinterpret_cast<const uint32_t*>(peq + map[txt[c]]), Pv, Mv, Ph, Mh);
-            const uint32_t msk = low_mask(mp);
-            const int d = mt + __popc(Pv & msk) - __popc(Mv & msk);
-            s_dist[p] = d;
-            // one term of d_K (Section 3.2): distance / longer prefix, from the quotient table
-            s_term[p] = a.norm_mode == SR_NORM_NONE ? (double)d : kQuot.v[d * 33 + mp];
-            if (a.pair_dist) a.pair_dist[(size_t)g * P + p] = d;
+            const int left = mt & 3;
+            if (left > 0) column(w.x);
+            if (left > 1) column(w.y);
+            if (left > 2) column(w.z);
+            double* s_term = reinterpret_cast<double*>(base + L.off_table) + gl * L.pitch;
+            int32_t* s_dist = reinterpret_cast<int32_t*>(reinterpret_cast<double*>(base + L.off_table) + L.groups * L.pitch) + gl * L.pitch;
+#pragma unroll
+            for (int h = 0; h < (kPacked ? 2 : 1); ++h) {
+                if (kPacked && at[h] == kNoPair) continue;
+                const int mp = s_len[gl * N + (kPacked ? 2 * word + h : word)];
+                const uint32_t msk = kPacked ? ((1u << mp) - 1u) << (16 * h) : low_mask(mp);
+                const int d = mt + __popc(Pv & msk) - __popc(Mv & msk);
+                if (a.pair_sum) s_dist[at[h]] = d;
+                // one term of d_K (Section 3.2): distance / longer prefix, from the quotient table
+                s_term[at[h]] = a.norm_mode == SR_NORM_NONE ? (double)d : kQuot.v[d * 33 + max(mp, mt)];
+                if (a.pair_dist) a.pair_dist[(size_t)(g0 + gl) * P + at[h]] = d;
+            }
         }
     }
     __syncthreads();
 
     // ---- d_K: ordered fp64 sum, strict threshold (Eq. 2): one thread per group of the CTA
-    const int groups_here = kWarp ? (blockDim.x >> 5) : 1;
-    if ((int)threadIdx.x < groups_here) {
-        const size_t gg = kWarp ? (size_t)blockIdx.x * groups_here + threadIdx.x : (size_t)blockIdx.x;
-        if (gg < (size_t)a.n_groups)
-            group_sum_and_gate(reinterpret_cast<const double*>(smem + L.off_term) + threadIdx.x * P,
-                               reinterpret_cast<const int32_t*>(smem + L.off_dist) + threadIdx.x * P, P, a, gg);
+    const int n_here = units * L.groups;
+    if ((int)threadIdx.x < n_here) {
+        const int u = threadIdx.x / L.groups, gl = threadIdx.x - u * L.groups;
+        const size_t g = (size_t)blockIdx.x * n_here + threadIdx.x;
+        const double* term = reinterpret_cast<const double*>(smem + (size_t)u * L.unit_bytes + L.off_table);
+        if (g < (size_t)a.n_groups)
+            group_sum_and_gate(term + gl * L.pitch, reinterpret_cast<const int32_t*>(term + L.groups * L.pitch) + gl * L.pitch, P, a, g);
     }
 }
 
+template <bool kPacked, bool kWarp>
+int launch_gate_named(const GateArgs& a, cudaStream_t s) {
+    constexpr bool kAlloc = !kWarp;
+    const int N = a.N, P = pairs_of(N);
+    NamedLayout L;
+    L.Q = a.K > 0 ? (a.K + 3) >> 2 : 1;
+    L.row_words = kPacked ? (N + 1) >> 1 : N;
+    L.combos = kPacked ? L.row_words * L.row_words : P;
+    L.groups = 1;
+    if (kWarp)                                     // fill the lanes, with at most four quads each
+        while ((L.groups + 1) * L.combos <= 32 && (L.groups + 1) * N * L.Q <= 128) ++L.groups;
+    L.items = L.groups * N * L.Q;
+    auto inv = [](int x) { return ((1u << 20) + (uint32_t)x - 1u) / (uint32_t)x; };
+    L.inv_Q = inv(L.Q);
+    L.inv_N = inv(N);
+    L.inv_C = inv(L.combos);
+    L.table_log = 6;                               // at least two slots to a symbol (four were no better)
+    while ((1 << L.table_log) < 2 * N * a.K) ++L.table_log;
+    L.pitch = P | 1;
+    int off = 0;
+    auto take = [&](int bytes) { int o = off; off = (off + bytes + 15) & ~15; return o; };
+    take(L.items * 16);
+    // the terms and distances of the pairs take the table's place
+    const int table = L.groups * (2 << L.table_log), terms = L.groups * L.pitch * 12;
+    L.off_table = take(table > terms ? table : terms);
+    L.off_name = take(L.items * 8);
+    L.off_row = take(kAlloc ? L.items * 8 : 0);
+    // allocated rows have at least two holders
+    L.off_peq = take((kAlloc ? L.groups * (N * a.K / 2) + 1 : 4 * L.items) * L.row_words * 4);
+    L.off_len = take((L.groups * N + 2) * 4);
+    L.off_order = take(N);
+    L.unit_bytes = off;
+    int threads, units = 1, items_per_thread;
+    if (kWarp) {
+        units = 8;
+        while (units > 1 && units * L.unit_bytes > 48 * 1024) units >>= 1;
+        while (units > 1 && (long long)a.n_groups <= (units >> 1) * L.groups) units >>= 1;
+        threads = 32 * units;
+        items_per_thread = (L.items + 31) / 32;
+    } else {
+        threads = (P + 31) & ~31;
+        if (threads > 512) threads = 512;
+        items_per_thread = (L.items + threads - 1) / threads;
+    }
+    const int smem = units * L.unit_bytes, per = units * L.groups;
+    const int blocks = (a.n_groups + per - 1) / per;
+    auto kernel = items_per_thread <= 1 ? gate_named_kernel<kPacked, kWarp, 1>
+                : items_per_thread == 2 ? gate_named_kernel<kPacked, kWarp, 2>
+                                        : gate_named_kernel<kPacked, kWarp, 4>;
+    if (smem > 48 * 1024) {
+        // per-device note of what each kernel was already allowed: the opt-in call is host
+        // time on a path whose small calls are launch-bound
+        static int granted[3][64] = {};
+        int* most = granted[items_per_thread <= 1 ? 0 : (items_per_thread == 2 ? 1 : 2)];
+        int dev = 0;
+        SR_CUDA_TRY(cudaGetDevice(&dev));
+        if (dev < 0 || dev >= 64 || most[dev] < smem) {
+            SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            if (dev >= 0 && dev < 64) most[dev] = smem;
+        }
+    }
+    return launch("gate_named_kernel", kernel, blocks, threads, smem, s, a, L, 2u);
+}
 
 // ---------------------------------------------------------------------------------
 // K <= 16: prefixes in registers, match words by direct comparison.  Threads are packed
@@ -287,66 +509,20 @@ int launch_gate_direct(const GateArgs& a, cudaStream_t s) {
 
 int launch_gate_single(const GateArgs& a, cudaStream_t s) {
     if (a.n_groups == 0) return SR_OK;
-    if (a.K <= 4) return launch_gate_direct<4>(a, s);
-    if (a.K <= 8) return launch_gate_direct<8>(a, s);
-    if (a.K <= 12) return launch_gate_direct<12>(a, s);
-    if (a.K <= 16) return launch_gate_direct<16>(a, s);
-    const int N = a.N, P = pairs_of(N);
-    SingleLayout L;
-    int h = 32;
-    while (h < 2 * N * a.K) h <<= 1;
-    L.hslots = h;
-    L.hlog = 0;
-    while ((1 << L.hlog) < h) ++L.hlog;
-    L.hshift = 32 - L.hlog;
-    L.qshift = 0;
-    while ((4 << L.qshift) < a.K) ++L.qshift;
-    L.n_items = N << L.qshift;
-    int off = 0;
-    auto take = [&](int bytes) { int o = off; off = (off + bytes + 15) & ~15; return o; };
-    L.off_hash = take(L.hslots * 8);
-    L.off_peq = take(N * kPeqPitch * 4);
-    L.zero_words16 = off >> 4;                      // table and masks are adjacent: one clear
-    L.off_map = take(L.hslots * N);
-    L.map_words16 = (L.hslots * N) >> 4;            // hslots >= 32: a whole number of 16-byte units
-    L.off_txt = take(N * kTxtPitch * 2);
-    L.off_len = take(N * 4);
-    L.group_bytes = off;
-    const bool warp = N <= 8;
-    int threads, groups_per_cta;
-    if (warp) {
-        // eight groups per CTA, fewer when shared memory would leave an SM under four CTAs
-        groups_per_cta = 8;
-        while (groups_per_cta > 2 && groups_per_cta * (L.group_bytes + P * 12) > 56 * 1024) groups_per_cta >>= 1;
-        threads = groups_per_cta * 32;
-    } else {
-        groups_per_cta = 1;
-        threads = (P + 31) & ~31;
-        if (threads > 512) threads = 512;
-        if (threads * kMaxItems < L.n_items) return SR_ERR_BAD_N;   // cannot happen for N <= 32
+    // Comparing directly costs two instructions per cell, naming the symbols first a few dozen per
+    // symbol and a longer chain of latencies: with fewer than eight rollouts, or in batches too small
+    // to fill the machine, direct comparison is quicker (K = 10, N = 8: 3.6 against 4.2 us for 10
+    // groups, 21 against 18.5 us for 32768; K = 15: 33 against 24 us; N = 4: 11 against 16 us).
+    const bool direct = a.N < 8 || (long long)a.n_groups * pairs_of(a.N) * (a.K > 9 ? a.K - 8 : 1) < 200000;
+    if (a.K <= 16 && direct) {
+        if (a.K <= 4) return launch_gate_direct<4>(a, s);
+        if (a.K <= 8) return launch_gate_direct<8>(a, s);
+        if (a.K <= 12) return launch_gate_direct<12>(a, s);
+        return launch_gate_direct<16>(a, s);
     }
-    off = groups_per_cta * L.group_bytes;
-    L.off_term = take(groups_per_cta * P * 8);
-    L.off_dist = take(groups_per_cta * P * 4);
-    const int smem = off;
-    const int blocks = (a.n_groups + groups_per_cta - 1) / groups_per_cta;
-    if (smem > 48 * 1024) {
-        // per-device note of what each kernel was already allowed: the opt-in call is host
-        // time on a path whose small calls are launch-bound
-        static int granted[2][64] = {};
-        int dev = 0;
-        SR_CUDA_TRY(cudaGetDevice(&dev));
-        if (dev < 0 || dev >= 64 || granted[warp][dev] < smem) {
-            if (warp)
-                SR_CUDA_TRY(cudaFuncSetAttribute(gate_single_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            else
-                SR_CUDA_TRY(cudaFuncSetAttribute(gate_single_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            if (dev >= 0 && dev < 64) granted[warp][dev] = smem;
-        }
-    }
-    if (warp) SR_LAUNCH("gate_single_kernel", gate_single_kernel<true>, blocks, threads, smem, s, a, L);
-    else SR_LAUNCH("gate_single_kernel", gate_single_kernel<false>, blocks, threads, smem, s, a, L);
-    return SR_OK;
+    if (a.K <= 15) return launch_gate_named<true, true>(a, s);
+    if (a.N <= 8) return launch_gate_named<false, true>(a, s);
+    return launch_gate_named<false, false>(a, s);
 }
 
 }  // namespace sr

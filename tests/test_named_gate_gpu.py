@@ -1,0 +1,38 @@
+"""Single-word gate through the kernel that names symbols: batches large enough to leave the direct
+comparison, two patterns per word up to K = 15, a warp or a CTA per group above, odd group sizes,
+lengths around quads, symbols that occur once, everywhere, or fight for one slot of the table."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import assert_gate_matches, gate_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,K", [(8, 15), (8, 9), (9, 12), (11, 14), (16, 13), (32, 3), (31, 15), (32, 15), (17, 1),
+                                 (2, 17), (3, 32), (5, 31), (8, 32), (8, 17), (9, 16), (13, 29), (32, 32), (31, 18)])
+@pytest.mark.parametrize("symbols", ["few", "base", "wide", "crowd"])
+def test_named_gate(N, K, symbols):
+    P = N * (N - 1) // 2
+    G = 37 if K > 16 else 200000 // (P * max(K - 8, 1)) + 3
+    rng = np.random.default_rng(1000 * N + K)
+    stride = (K + 3) // 4 * 4 + 4
+    if symbols == "few":
+        seqs = rng.integers(0, 5, size=(G, N, stride))
+    elif symbols == "base":
+        base = rng.integers(0, 4096, size=(G, 1, stride))
+        seqs = np.where(rng.random((G, N, stride)) < rng.beta(0.5, 2.0, size=(G, 1, 1)),
+                        rng.integers(0, 4096, size=(G, N, stride)), base)
+    elif symbols == "wide":
+        seqs = rng.integers(-2 ** 31, 2 ** 31, size=(G, N, stride))
+    else:                                    # one home slot under the first hash
+        inverse = pow(0x9E3779B1, -1, 1 << 32)
+        crowd = (((3 << 24) + np.arange(64, dtype=np.uint64)) * np.uint64(inverse) % np.uint64(1 << 32)).astype(np.uint32).view(np.int32)
+        seqs = rng.choice(crowd, size=(G, N, stride))
+    lens = rng.integers(0, K + 3, size=(G, N)).astype(np.int32)
+    lens[::3] = K
+    lens[1::7, 0] = -1
+    seqs = seqs.astype(np.int32)
+    want = oracle.gate(seqs, np.maximum(lens, 0), K, 0.3, threads=8)
+    assert_gate_matches(gate_gpu(seqs, lens, K, 0.3), want, f"N={N} K={K} {symbols}")
