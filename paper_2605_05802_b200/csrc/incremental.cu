@@ -7,10 +7,11 @@
 //   VP / VN : bit r-1 set iff D[r][n] - D[r-1][n] is +1 / -1   (last column)
 //   HP / HN : bit c-1 set iff D[m][c] - D[m][c-1] is +1 / -1   (last row)
 // and D[m][n] = n + popc(VP) - popc(VN) is never stored.  When j appends y, one
-// bit-parallel column step over the rows gives the new last column and the
-// horizontal delta of the bottom row; when i appends x, the same step on the
-// transposed roles gives the new last row; when both append, both steps start from
-// the OLD state and the new corner D[m+1][n+1] is the usual three-way minimum.
+// bit-parallel column step over the rows gives the new last column, and the
+// horizontal delta of the bottom row is appended to the last row; when i appends x, the
+// same step on the transposed roles gives the new last row, and the vertical delta that leaves
+// it is appended to the last column.  When both append, the row comes first, so that the
+// column step already runs over m + 1 rows and its last cell is the new corner.
 //
 // State buffer layout (position independent, byte-copyable):
 //   [0, 256)        header: magic, n_groups, N, max_steps, steps taken so far (an upper
@@ -73,17 +74,24 @@ __global__ void incr_init_kernel(unsigned char* state, IncrLayout L, int n_group
         pairs[e] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// One bit-parallel column step over `m` rows (m >= 1) with horizontal input +1 at
-// row 0; returns the horizontal delta leaving the bottom row.  Bits of Eq at or above m
-// are harmless: carries and shifts only move upwards, and the result is masked.
-__device__ __forceinline__ int column_step(uint32_t Eq, uint32_t& Pv, uint32_t& Mv, int m) {
+// The bit-parallel column step on the last column (P, M) of `len` cells, whose match bits are `Eq`
+// (bits at or above len are harmless: carries and shifts only move upwards, and the result is
+// masked with `below`, the bits under len); `last` is bit len - 1.  The delta that leaves the last
+// cell (+1 where there is none) is appended to the crossing vector (cP, cM) as bit `at`.
+__device__ __forceinline__ void append_step(uint32_t Eq, uint32_t& P, uint32_t& M, int len, uint32_t last,
+                                            uint32_t below, uint32_t& cP, uint32_t& cM, uint32_t at) {
     uint32_t Ph, Mh;
-    word_column(Eq, Pv, Mv, Ph, Mh);
-    const int hout = (int)((Ph >> (m - 1)) & 1u) - (int)((Mh >> (m - 1)) & 1u);
-    const uint32_t msk = low_mask(m);
-    Pv &= msk;
-    Mv &= msk;
-    return hout;
+    word_column(Eq, P, M, Ph, Mh);
+    P &= below;
+    M &= below;
+    if ((Ph & last) != 0u || len == 0) cP |= at;
+    if ((Mh & last) != 0u) cM |= at;
+}
+
+__device__ __forceinline__ uint32_t bit_of(int k) {     // 1 << k for 0 <= k < 32, otherwise 0
+    uint32_t r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(k));
+    return r;
 }
 
 struct IncrArgs {
@@ -154,10 +162,12 @@ __device__ __forceinline__ void match_masks(const int4* quads, int N, int ri, in
 template <int kN>
 __global__ void __launch_bounds__(512, 3)
 incr_step_kernel(IncrArgs a) {
-    grid_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     const int N = kN ? kN : a.N, P = pairs_of(N);
     const int tid = threadIdx.x;
+    const int grp = (int)(((uint32_t)tid * a.inv_P) >> 20);
+    const int pr = kPairs.v[N][min(tid - grp * P, P - 1)];     // a table: no need to wait for it
+    grid_begin();
     const int g0 = blockIdx.x * a.gpb;
     const int ng = min(a.gpb, a.n_groups - g0);
     int32_t* s_dist = reinterpret_cast<int32_t*>(smem + a.off_dist);    // [gpb][P]
@@ -184,11 +194,9 @@ incr_step_kernel(IncrArgs a) {
         reinterpret_cast<uint32_t*>(a.state)[4] = steps_taken + 1u;
     const bool is_pair = tid < ng * P;
     uint4 st = make_uint4(0u, 0u, 0u, 0u);
-    int ri = 0, rj = 0, m = 0, n = 0, grp = 0;
+    int ri = 0, rj = 0, m = 0, n = 0;
     int32_t x = SR_NO_ACTION, y = SR_NO_ACTION;
     if (is_pair) {
-        grp = (int)(((uint32_t)tid * a.inv_P) >> 20);
-        const int pr = kPairs.v[N][tid - grp * P];
         ri = pr & 0xFF;
         rj = pr >> 8;
         st = g_pairs[tid];
@@ -225,13 +233,6 @@ incr_step_kernel(IncrArgs a) {
         if (a.status) atomicOr(a.status, SR_STATUS_STEP_OVERFLOW);
     }
 
-    const bool ai = x != SR_NO_ACTION, aj = y != SR_NO_ACTION;
-    int hout = 1, vout = 1;
-    uint32_t VP2 = st.x, VN2 = st.y, HP2 = st.z, HN2 = st.w;
-    if (is_pair) {
-        if (aj && m > 0) hout = column_step(eq_y, VP2, VN2, m);
-        if (ai && n > 0) vout = column_step(eq_x, HP2, HN2, n);
-    }
     __syncthreads();       // every thread has read the lengths (and the stored actions) before the appends
     if (is_roll && my_act != SR_NO_ACTION) {
         const int g = (int)(((uint32_t)tid * a.inv_N) >> 20), i = tid - g * N;
@@ -240,33 +241,25 @@ incr_step_kernel(IncrArgs a) {
     }
     if (is_pair) {
         uint32_t VP = st.x, VN = st.y, HP = st.z, HN = st.w;
-        const int c = n + __popc(VP) - __popc(VN);
-        int d = c, mi = m, mj = n;
-        if (ai && aj) {
-            const int left = c + vout, up = c + hout;
-            d = min(min(c + (x != y ? 1 : 0), up + 1), left + 1);
-            const int vd = d - up, hd = d - left;
-            VP = VP2 | (vd > 0 ? 1u << m : 0u);
-            VN = VN2 | (vd < 0 ? 1u << m : 0u);
-            HP = HP2 | (hd > 0 ? 1u << n : 0u);
-            HN = HN2 | (hd < 0 ? 1u << n : 0u);
-            mi = m + 1; mj = n + 1;
-        } else if (aj) {
-            d = c + hout;
-            VP = VP2; VN = VN2;
-            HP |= hout > 0 ? 1u << n : 0u;
-            HN |= hout < 0 ? 1u << n : 0u;
-            mj = n + 1;
-        } else if (ai) {
-            d = c + vout;
-            HP = HP2; HN = HN2;
-            VP |= vout > 0 ? 1u << m : 0u;
-            VN |= vout < 0 ? 1u << m : 0u;
-            mi = m + 1;
+        const bool ai = x != SR_NO_ACTION, aj = y != SR_NO_ACTION;
+        const uint32_t bm = bit_of(m), bn = bit_of(n);         // 0 at 32: the rollout is full
+        uint32_t last = bit_of(m - 1), below = bm - 1u;
+        if (ai) {
+            append_step(eq_x, HP, HN, n, bit_of(n - 1), bn - 1u, VP, VN, bm);
+            eq_y &= below;                                     // the new row's match bit is x == y
+            if (x == y) eq_y |= bm;
+            last = bm;
+            below = 2u * bm - 1u;
+            ++m;
         }
+        if (aj) {
+            append_step(eq_y, VP, VN, m, last, below, HP, HN, bn);
+            ++n;
+        }
+        const int d = n + __popc(VP) - __popc(VN);
         if (ai || aj) g_pairs[tid] = make_uint4(VP, VN, HP, HN);
-        s_dist[tid] = d;
-        s_term[tid] = a.norm_mode == SR_NORM_NONE ? (double)d : kQuot.v[d * 33 + max(mi, mj)];
+        if (a.pair_sum) s_dist[tid] = d;
+        s_term[tid] = a.norm_mode == SR_NORM_NONE ? (double)d : kQuot.v[d * 33 + max(m, n)];
         if (a.pair_dist) a.pair_dist[(size_t)g0 * P + tid] = d;
     }
     __syncthreads();
