@@ -33,6 +33,8 @@ namespace {
 
 constexpr uint32_t kMagic = 0x53524731u;   // "SRG1"
 constexpr int kHistPitch = 32;
+constexpr int kRollThreads = 128;
+constexpr int kAhead = 4;          // pair states in flight per thread
 
 struct IncrLayout {
     size_t off_lens, off_hist, off_pairs, total;
@@ -108,9 +110,11 @@ struct IncrArgs {
     int32_t* status;
     int gpb;                                               // groups per CTA
     uint32_t inv_P, inv_N;                                 // ceil(2^20 / P), ceil(2^20 / N): thread -> group by multiply-shift (exact below 512)
-    int off_dist, off_term;                                // shared-memory offsets
+    int off_dist, off_term, off_roll, off_eq;              // shared-memory offsets
     uint32_t one;                                          // 1, as a run-time value
 };
+
+__device__ __forceinline__ int div20(int x, uint32_t inv) { return (int)(((uint32_t)x * inv) >> 20); }
 
 // Match masks of a pair's two new actions against the stored actions of the other
 // rollout: bit r of eq_y set iff action r of rollout ri equals y, bit c of eq_x set iff
@@ -148,7 +152,29 @@ __device__ __forceinline__ void match_masks(const int4* quads, int N, int ri, in
     }
 }
 
-// One thread per pair, `gpb` groups per CTA.  The header (hot in L2: every CTA reads it)
+// Appends to one pair (x by rollout i, y by rollout j, where ai / aj), stores its state and returns its
+// distance; m and n become the new lengths.
+__device__ __forceinline__ int step_pair(uint4 st, bool ai, bool aj, int32_t x, int32_t y, uint32_t eq_x, uint32_t eq_y,
+                                         int& m, int& n, uint4* where) {
+    const uint32_t bm = bit_of(m), bn = bit_of(n);         // 0 at 32: the rollout is full
+    uint32_t last = bit_of(m - 1), below = bm - 1u;
+    if (ai) {
+        append_step(eq_x, st.z, st.w, n, bit_of(n - 1), bn - 1u, st.x, st.y, bm);
+        eq_y &= below;                                     // the new row's match bit is x == y
+        if (x == y) eq_y |= bm;
+        last = bm;
+        below = 2u * bm - 1u;
+        ++m;
+    }
+    if (aj) {
+        append_step(eq_y, st.x, st.y, m, last, below, st.z, st.w, bn);
+        ++n;
+    }
+    if (ai || aj) *where = st;
+    return n + __popc(st.x) - __popc(st.y);
+}
+
+// Small batches: one thread per pair, `gpb` groups per CTA.  The header (hot in L2: every CTA reads it)
 // says how many steps the state has taken, which bounds every length; with that, all a
 // pair needs -- its state, the two lengths, the two new actions AND the stored actions of
 // both rollouts -- is requested in ONE round of independent loads instead of waiting for
@@ -240,28 +266,127 @@ incr_step_kernel(IncrArgs a) {
         g_len[tid] = my_len + 1;
     }
     if (is_pair) {
-        uint32_t VP = st.x, VN = st.y, HP = st.z, HN = st.w;
-        const bool ai = x != SR_NO_ACTION, aj = y != SR_NO_ACTION;
-        const uint32_t bm = bit_of(m), bn = bit_of(n);         // 0 at 32: the rollout is full
-        uint32_t last = bit_of(m - 1), below = bm - 1u;
-        if (ai) {
-            append_step(eq_x, HP, HN, n, bit_of(n - 1), bn - 1u, VP, VN, bm);
-            eq_y &= below;                                     // the new row's match bit is x == y
-            if (x == y) eq_y |= bm;
-            last = bm;
-            below = 2u * bm - 1u;
-            ++m;
-        }
-        if (aj) {
-            append_step(eq_y, VP, VN, m, last, below, HP, HN, bn);
-            ++n;
-        }
-        const int d = n + __popc(VP) - __popc(VN);
-        if (ai || aj) g_pairs[tid] = make_uint4(VP, VN, HP, HN);
+        const int d = step_pair(st, x != SR_NO_ACTION, y != SR_NO_ACTION, x, y, eq_x, eq_y, m, n, g_pairs + tid);
         if (a.pair_sum) s_dist[tid] = d;
         s_term[tid] = a.norm_mode == SR_NORM_NONE ? (double)d : kQuot.v[d * 33 + max(m, n)];
         if (a.pair_dist) a.pair_dist[(size_t)g0 * P + tid] = d;
     }
+    __syncthreads();
+    if (tid < ng) {
+        GateArgs out{};
+        out.pair_sum = a.pair_sum; out.mean = a.mean; out.stop = a.stop; out.threshold = a.threshold;
+        group_sum_and_gate(s_term + tid * P, s_dist + tid * P, P, out, (size_t)g0 + tid);
+    }
+}
+
+// Large batches: one thread per rollout for the match masks, then one per pair for the steps, in a loop.
+// A rollout's stored actions are read once, by one thread, and compared with the new actions
+// of the group's other rollouts (kMasks at a time); the masks go to the pairs through shared memory.  A
+// thread per pair that does its own comparing reads every stored action N - 1 times: the
+// return path of L1 (16 bytes a lane and load) and the indices of its loads were half of that kernel.
+// 30 steps: 65536 groups of 8 792 -> 706 us, 16384 groups of 16 1033 -> 738 us.
+template <int kMasks>
+__global__ void __launch_bounds__(kRollThreads)
+incr_rollout_kernel(IncrArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int N = a.N, P = pairs_of(N), tid = threadIdx.x;
+    double* s_term = reinterpret_cast<double*>(smem + a.off_term);      // [gpb][P]
+    int32_t* s_dist = reinterpret_cast<int32_t*>(smem + a.off_dist);    // [gpb][P]
+    int2* s_roll = reinterpret_cast<int2*>(smem + a.off_roll);          // [gpb * N] length before, action or none
+    uint32_t* s_eq = reinterpret_cast<uint32_t*>(smem + a.off_eq);      // [gpb * N][N - 1]
+    const int g = div20(tid, a.inv_N), i = tid - g * N;
+    grid_begin();
+    const int g0 = blockIdx.x * a.gpb;
+    const int ng = min(a.gpb, a.n_groups - g0);
+    const uint4 hdr = *reinterpret_cast<const uint4*>(a.state);         // magic, n_groups, N, max_steps
+    const uint32_t steps_taken = reinterpret_cast<const uint32_t*>(a.state)[4];
+    int32_t* g_len = reinterpret_cast<int32_t*>(a.state + a.L.off_lens) + (size_t)g0 * N;
+    int32_t* g_hist = reinterpret_cast<int32_t*>(a.state + a.L.off_hist) + (size_t)g0 * N * kHistPitch;
+    uint4* g_pairs = reinterpret_cast<uint4*>(a.state + a.L.off_pairs) + (size_t)g0 * P;
+    const int32_t* g_new = a.new_actions + (size_t)g0 * N;
+
+    const bool is_roll = tid < ng * N;
+    int my_len = 0;
+    int32_t my_act = SR_NO_ACTION;
+    if (is_roll) { my_len = g_len[tid]; my_act = __ldg(g_new + tid); }
+    // the first pairs' states are on their way while the masks are made
+    uint4 st[kAhead];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k)
+        if (tid + k * kRollThreads < ng * P) st[k] = g_pairs[tid + k * kRollThreads];
+    const bool bad = hdr.x != kMagic || hdr.y != (uint32_t)a.n_groups || hdr.z != (uint32_t)N;
+    if (bad) {                                     // uniform over the grid: nothing is touched
+        if (tid == 0 && a.status) atomicOr(a.status, SR_STATUS_BAD_STATE);
+        return;
+    }
+    const int max_steps = (int)hdr.w;
+    // quads of stored actions any rollout can hold by now (or one more where a CTA already
+    // sees this step's own count)
+    const int nq = (min((uint32_t)max_steps, steps_taken) + 3u) >> 2;
+    if (blockIdx.x == 0 && tid == 0 && steps_taken < 0x7FFFFFFFu)
+        reinterpret_cast<uint32_t*>(a.state)[4] = steps_taken + 1u;
+
+    if (is_roll) {
+        if (my_act != SR_NO_ACTION && my_len >= max_steps) {
+            my_act = SR_NO_ACTION;
+            if (a.status) atomicOr(a.status, SR_STATUS_STEP_OVERFLOW);
+        }
+        s_roll[tid] = make_int2(my_len, my_act);
+        const int4* quads = reinterpret_cast<const int4*>(g_hist) + g * 8 * N + i;
+        uint32_t* eq_out = s_eq + tid * (N - 1);
+        for (int d0 = 0; d0 < N - 1; d0 += kMasks) {           // rollouts i + 1 + d0 ... , cyclically
+            int32_t y[kMasks];
+            uint32_t eq[kMasks];
+#pragma unroll
+            for (int k = 0; k < kMasks; ++k) {
+                int j = i + 1 + min(d0 + k, N - 2);
+                if (j >= N) j -= N;
+                y[k] = __ldg(g_new + g * N + j);
+                eq[k] = 0u;
+            }
+            uint32_t bit = a.one;
+#pragma unroll 2
+            for (int q = 0; q < nq; ++q) {
+                const int4 v = quads[q * N];
+                const uint32_t b1 = 2u * bit, b2 = 4u * bit, b3 = 8u * bit;
+#pragma unroll
+                for (int k = 0; k < kMasks; ++k)
+                    // `one` holds 1 but is a run-time value: the bits are set by multiply-adds, which
+                    // issue on the FMA pipe while the comparisons keep the integer ALU busy
+                    asm("{ .reg .pred e0, e1, e2, e3;\n\t"
+                        "setp.eq.s32 e0, %1, %5; setp.eq.s32 e1, %2, %5; setp.eq.s32 e2, %3, %5; setp.eq.s32 e3, %4, %5;\n\t"
+                        "@e0 mad.lo.u32 %0, %10, %6, %0; @e1 mad.lo.u32 %0, %10, %7, %0;\n\t"
+                        "@e2 mad.lo.u32 %0, %10, %8, %0; @e3 mad.lo.u32 %0, %10, %9, %0; }"
+                        : "+r"(eq[k])
+                        : "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(y[k]), "r"(bit), "r"(b1), "r"(b2), "r"(b3), "r"(a.one));
+                bit = 16u * bit;
+            }
+#pragma unroll
+            for (int k = 0; k < kMasks; ++k)
+                if (d0 + k < N - 1) eq_out[d0 + k] = eq[k];
+        }
+        // nobody else reads this rollout's stored actions or length
+        if (my_act != SR_NO_ACTION) {
+            g_hist[((g * 8 + (my_len >> 2)) * N + i) * 4 + (my_len & 3)] = my_act;
+            g_len[tid] = my_len + 1;
+        }
+    }
+    __syncthreads();
+    auto pair = [&](int e, const uint4& state) {
+        const int pg = div20(e, a.inv_P), pr = kPairs.v[N][e - pg * P];
+        const int ri = pr & 0xFF, rj = pr >> 8, gi = pg * N + ri, gj = pg * N + rj;
+        const int2 A = s_roll[gi], B = s_roll[gj];
+        int m = A.x, n = B.x;
+        const uint32_t eq_y = s_eq[gi * (N - 1) + (rj - ri - 1)], eq_x = s_eq[gj * (N - 1) + (ri - rj + N - 1)];
+        const int d = step_pair(state, A.y != SR_NO_ACTION, B.y != SR_NO_ACTION, A.y, B.y, eq_x, eq_y, m, n, g_pairs + e);
+        if (a.pair_sum) s_dist[e] = d;
+        s_term[e] = a.norm_mode == SR_NORM_NONE ? (double)d : kQuot.v[d * 33 + max(m, n)];
+        if (a.pair_dist) a.pair_dist[(size_t)g0 * P + e] = d;
+    };
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k)
+        if (tid + k * kRollThreads < ng * P) pair(tid + k * kRollThreads, st[k]);
+    for (int e = tid + kAhead * kRollThreads; e < ng * P; e += kRollThreads) pair(e, g_pairs[e]);
     __syncthreads();
     if (tid < ng) {
         GateArgs out{};
@@ -304,16 +429,28 @@ int launch_incr_step(void* state, size_t bytes, const int32_t* new_actions, int3
     a.threshold = threshold; a.norm_mode = norm_mode;
     a.pair_dist = pair_dist; a.pair_sum = pair_sum; a.mean = mean; a.stop = stop; a.status = status;
     const int P = pairs_of(N);
-    int gpb = 256 / P;
-    if (gpb < 1) gpb = 1;
-    if (gpb > 32) gpb = 32;
-    while (gpb > 1 && gpb * N > 256) --gpb;      // one appending thread per rollout
-    a.gpb = gpb;
     a.one = 1u;
     a.inv_P = ((1u << 20) + (uint32_t)P - 1u) / (uint32_t)P;
     a.inv_N = ((1u << 20) + (uint32_t)N - 1u) / (uint32_t)N;
     int off = 0;
     auto take = [&](int b) { int o = off; off = (off + b + 15) & ~15; return o; };
+    // the thread-per-rollout form has the longer chain per thread and pays off once several CTAs of it
+    // share every SM (N = 8: even at 25000 groups; N = 16: at 6000)
+    if ((long long)n_groups * P >= 700000) {
+        a.gpb = kRollThreads / N;
+        a.off_dist = take(pair_sum ? a.gpb * P * 4 : 0);
+        a.off_term = take(a.gpb * P * 8);
+        a.off_roll = take(a.gpb * N * 8);
+        a.off_eq = take(a.gpb * N * (N - 1) * 4);
+        auto kernel = N <= 5 ? incr_rollout_kernel<4> : (N <= 8 ? incr_rollout_kernel<7> : incr_rollout_kernel<8>);
+        SR_LAUNCH("incr_rollout_kernel", kernel, (n_groups + a.gpb - 1) / a.gpb, kRollThreads, off, s, a);
+        return SR_OK;
+    }
+    int gpb = 256 / P;
+    if (gpb < 1) gpb = 1;
+    if (gpb > 32) gpb = 32;
+    while (gpb > 1 && gpb * N > 256) --gpb;      // one appending thread per rollout
+    a.gpb = gpb;
     a.off_dist = take(gpb * P * 4);
     a.off_term = take(gpb * P * 8);
     int threads = (gpb * P + 31) & ~31;
