@@ -322,7 +322,7 @@ int sr_grpo_advantage(const float* rewards, const uint8_t* drop_mask, int32_t n_
  *
  * seqs / lens / stride / K as for sr_gate, with K <= 32 (action-level prefixes).  The
  * ratios and the Jaccard mean are exact to the last bit of their definition; the entropy
- * goes through the device logarithm and agrees with a host libm to a few ulp.
+ * uses the host's logarithm and agrees with other libms to a few ulp.
  * (Not computed: obs_unique_ratio, which needs the environment's observations.)
  */
 int sr_group_signals(const int32_t* seqs, const int32_t* lens, int32_t n_groups, int32_t N,

@@ -40,18 +40,25 @@ void note_cuda_error(cudaError_t e, const char* where);
 // kernel implies that of all before it.  (early = false: an ordinary launch, for a persistent
 // kernel whose CTAs must spread evenly over SMs that the kernel before it no longer occupies.)
 template <typename... Params, typename... Args>
-int launch_as(bool early, const char* name, void (*kernel)(Params...), int blocks, int threads, size_t smem,
+int launch_as(bool early, int cluster, const char* name, void (*kernel)(Params...), int blocks, int threads, size_t smem,
               cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    if (early) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)cluster;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs++].val.clusterDim.z = 1;
+    }
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
     if (e != cudaSuccess) {
         note_cuda_error(e, name);
@@ -63,7 +70,7 @@ int launch_as(bool early, const char* name, void (*kernel)(Params...), int block
 template <typename... Params, typename... Args>
 int launch(const char* name, void (*kernel)(Params...), int blocks, int threads, size_t smem, cudaStream_t s,
            Args... args) {
-    return launch_as(true, name, kernel, blocks, threads, smem, s, args...);
+    return launch_as(true, 1, name, kernel, blocks, threads, smem, s, args...);
 }
 #define SR_LAUNCH(...)                                      \
     do {                                                    \

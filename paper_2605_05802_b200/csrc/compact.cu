@@ -3,11 +3,14 @@
 // zero-variance filter of the dynamic-sampling baseline (a group whose advantages are all
 // zero adds nothing to the gradient, Section 2.1).
 //
-// Stream compaction in three launches, no waiting between blocks: every CTA counts the
+// Up to eight tiles: one cluster (see kept_scatter_kernel).  Otherwise stream compaction in three
+// launches, no waiting between blocks: every CTA counts the
 // kept groups of its tile of 4096 groups; one CTA turns the tile counts into tile offsets;
 // every CTA recomputes its tile's flags (they come from L2 the second time), scans them,
 // collects its indices in shared memory and writes them out as one contiguous run.  The
 // order is ascending by construction, whatever the scheduling.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 
 namespace sr {
@@ -112,14 +115,17 @@ kept_offsets_kernel(int32_t* __restrict__ tile_count, int n_tiles, int32_t* __re
     if (threadIdx.x == 0) *count = s_carry;
 }
 
-template <bool kVec>
+// kCluster: the grid is one cluster; a tile learns the counts of the tiles before it from their shared
+// memory, and the list takes one launch instead of three (4096 groups: 7.2 -> 3.9 us).
+template <bool kVec, bool kCluster>
 __global__ void __launch_bounds__(kTileThreads)
 kept_scatter_kernel(const uint8_t* __restrict__ stop, const uint8_t* __restrict__ zero_var,
                     int n_groups, const int32_t* __restrict__ tile_offset,
-                    int32_t* __restrict__ index) {
+                    int32_t* __restrict__ index, int32_t* __restrict__ count) {
     grid_begin();
     __shared__ int s_warp[kTileThreads / 32];
     __shared__ int32_t s_idx[kTile];
+    __shared__ int s_total, s_offset;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int base = (blockIdx.x * kTileThreads + threadIdx.x) * kPerThread;
     uint32_t keep = base < n_groups ? kept_bits<kVec>(stop, zero_var, base, n_groups) : 0u;
@@ -144,8 +150,22 @@ kept_scatter_kernel(const uint8_t* __restrict__ stop, const uint8_t* __restrict_
         keep &= keep - 1u;
         s_idx[before++] = base + k;
     }
-    __syncthreads();
-    int32_t* out = index + tile_offset[blockIdx.x];
+    if (kCluster) {
+        const auto cluster = cooperative_groups::this_cluster();
+        if (threadIdx.x == 0) s_total = total;
+        cluster.sync();
+        if (threadIdx.x == 0) {
+            int sum = 0;
+            for (unsigned b = 0; b < blockIdx.x; ++b) sum += *cluster.map_shared_rank(&s_total, b);
+            s_offset = sum;
+            if (blockIdx.x == gridDim.x - 1) *count = sum + total;
+        }
+        cluster.sync();                        // nobody leaves while its count is read
+    } else {
+        if (threadIdx.x == 0) s_offset = tile_offset[blockIdx.x];
+        __syncthreads();
+    }
+    int32_t* out = index + s_offset;
     for (int e = threadIdx.x; e < total; e += kTileThreads) out[e] = s_idx[e];
 }
 
@@ -165,11 +185,13 @@ int launch_kept_groups(const uint8_t* stop, const uint8_t* zero_var, int32_t n_g
     int32_t* tiles = static_cast<int32_t*>(ws);
     const int n_tiles = (n_groups + kTile - 1) / kTile;
     const bool vec = ((reinterpret_cast<uintptr_t>(stop) | reinterpret_cast<uintptr_t>(zero_var)) & 15) == 0;
-    if (vec) SR_LAUNCH("kept_count_kernel", kept_count_kernel<true>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles);
-    else SR_LAUNCH("kept_count_kernel", kept_count_kernel<false>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles);
+    if (n_tiles <= 8) {                            // the portable cluster size
+        return launch_as(true, n_tiles, "kept_scatter_kernel", vec ? kept_scatter_kernel<true, true> : kept_scatter_kernel<false, true>,
+                         n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles, index, count);
+    }
+    SR_LAUNCH("kept_count_kernel", vec ? kept_count_kernel<true> : kept_count_kernel<false>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles);
     SR_LAUNCH("kept_offsets_kernel", kept_offsets_kernel, 1, 1024, 0, s, tiles, n_tiles, count);
-    if (vec) SR_LAUNCH("kept_scatter_kernel", kept_scatter_kernel<true>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles, index);
-    else SR_LAUNCH("kept_scatter_kernel", kept_scatter_kernel<false>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles, index);
+    SR_LAUNCH("kept_scatter_kernel", vec ? kept_scatter_kernel<true, false> : kept_scatter_kernel<false, false>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles, index, count);
     return SR_OK;
 }
 

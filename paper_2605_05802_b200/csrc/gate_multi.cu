@@ -1213,7 +1213,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const int blocks = (int)(want < 3LL * sms ? want : 3LL * sms);
     // (an ordinary launch: CTAs made resident while the tail of prep still fills some SMs would
     // crowd onto the others, 478 us instead of 434 for the token-level batch of 1024 groups)
-    const int rc = launch_as(false, "multi_dp_kernel", multi_dp_kernel, blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u);
+    const int rc = launch_as(false, 1, "multi_dp_kernel", multi_dp_kernel, blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u);
     if (rc != SR_OK) return rc;
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[3], s));
     SR_LAUNCH("multi_finish_kernel", multi_finish_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, dist, flag, exact, gpb);
