@@ -40,6 +40,8 @@
 //
 // Which rollout of a pair is the pattern is fixed by a round-robin tournament on the
 // indices, so that every pattern CTA of `prep` serves the same number of texts.
+#include <atomic>
+
 #include "common.cuh"
 
 namespace sr {
@@ -52,7 +54,6 @@ constexpr int kNumBins = 2048;      // kTimeBuckets * kNumClasses of them used
 constexpr int kOrderThreads = 1024;
 constexpr int kAlonePairs = 1024;   // batches of up to this many pairs are ordered by one CTA
 constexpr uint32_t kLocNone = 0x7FFFu;    // bit 15 clear, far above any row: shifts to 0
-constexpr uint32_t kLocOpen = 0xFFFFFFFFu;   // look-up not finished
 constexpr uint32_t kLocRow = 0x8000u;     // | index of the symbol's mask row
 constexpr uint32_t kLocChain = 0xC000u;   // | first position of the symbol's occurrence chain
 constexpr uint32_t kChainEnd = 0xFFFFu;
@@ -89,7 +90,7 @@ struct Ctl {               // control block in the workspace
 };
 
 struct MultiWs {
-    size_t off_dist, off_desc, off_loc, off_next, off_order, off_ctl, off_flag, off_rows, total;
+    size_t off_dist, off_desc, off_loc, off_next, off_order, off_ctl, off_flag, off_rows, off_names, total;
     int pitch;             // uint16 elements per loc / chain row
     int row_words;         // 32-bit words of a mask row: one per 32 pattern positions
     int row_cap;           // mask rows a pattern may have
@@ -116,6 +117,8 @@ MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K) {
     w.row_cap = (K + 7) >> 3;
     w.off_rows = off;
     off = align_up(off + (size_t)n_groups * N * w.row_cap * w.row_words * 4 + 256, 256);
+    w.off_names = off;
+    off = align_up(off + (size_t)n_groups * N * w.pitch * 2, 256);
     w.total = off;
     return w;
 }
@@ -221,94 +224,115 @@ __device__ __forceinline__ int clamp_len(const int32_t* lens, size_t idx, int K,
     return min(len, K);
 }
 
-// ------------------------------------------------------------------------ prep
-// Hash table of a pattern's symbols in shared memory.  A symbol times an odd constant is a
-// one-to-one map of the 32-bit words, so the upper bits of the product (the home bucket) and the lower
-// ones (the tag) name the symbol, and a slot of 32 bits can say all there is to know:
-//     tag | how many buckets from its home (0..2; 3: empty) | position of the symbol's first claimant
-// With four buckets of two slots per position these fields fill a word exactly.  A bucket is one
-// 8-byte load, and in 97 look-ups of a hundred the only one.  (Single slots, eight per position, sent
-// 8 % of the look-ups to a second slot, and so nearly every warp through a loop of three or four probes:
-// 370 instructions for four columns of a warp; slots of 64 bits with the whole symbol, four per
-// position, took the same space and collided as often.)
-// A symbol that finds no slot in its three buckets is left out and its positions are listed: a
-// look-up that runs into six foreign symbols searches the list, or the pattern itself where the
-// list was too short.
-constexpr int kMaxTexts = SR_MAX_N / 2;        // texts a pattern is paired with
+// ----------------------------------------------------------------------- names
+// Names for the symbols of a group: all holders of a symbol agree on one of their positions (rollout x
+// pitch + place).  Every position writes itself to the slot of a table that its symbol hashes to
+// (whichever write lands last stays), and if the position found there afterwards holds the same symbol,
+// that is the name; the symbols that lost their slot to another one go on with another hash, and every
+// round names at least one symbol of each slot.  One CTA per group.  With the names, 16 bits
+// each, a pattern's look-up table is an array: no hashing, no probing, no comparing in prep, which serves
+// every text (N - 1) / 2 times.  (The table of hashed 32-bit slots that prep had instead took 280 warp
+// instructions for four columns of a warp's lanes.)
 constexpr uint32_t kHashMul = 0x9E3779B1u;
-constexpr uint32_t kSlotEmpty = 0xFFFFFFFFu;
-constexpr uint32_t kMaxProbe = 2u;
-constexpr int kMaxListed = 8;
+constexpr int kMaxTexts = SR_MAX_N / 2;        // texts a pattern is paired with
 
-struct PatternTable {
-    uint32_t* slot;                    // [4 << pos_bits and kMaxProbe more][2]
-    int pos_bits, log_buckets;         // log_buckets = 2 + pos_bits
-    uint32_t pos_mask;
-    __device__ __forceinline__ uint32_t home(uint32_t x) const { return x >> (32 - log_buckets); }
-    __device__ __forceinline__ uint32_t tag(uint32_t x, uint32_t d) const { return (x << log_buckets) | (d << pos_bits); }
-    __device__ __forceinline__ bool holds(uint32_t e, uint32_t want) const { return ((e ^ want) & ~pos_mask) == 0u; }
-    __device__ __forceinline__ uint32_t position(uint32_t e) const { return e & pos_mask; }
-    // what a bucket says about a symbol: its position, not here nor further on, or neither
-    __device__ __forceinline__ uint32_t look(uint2 b, uint32_t want) const {
-        const bool first = holds(b.x, want);
-        uint32_t r = b.y == kSlotEmpty ? kLocNone : kLocOpen;
-        if (first || holds(b.y, want)) r = position(first ? b.x : b.y);
-        return r;
+__global__ void __launch_bounds__(1024)
+multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int table_log, int g_base) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_len[SR_MAX_N];
+    const int N = a.N, K = a.K, tid = threadIdx.x, nthr = blockDim.x;
+    const int row_quads = pitch >> 2, items = N * row_quads;
+    int32_t* s_sym = reinterpret_cast<int32_t*>(smem);                             // [N][pitch]
+    uint16_t* s_table = reinterpret_cast<uint16_t*>(s_sym + N * pitch);            // [1 << table_log]
+    grid_begin();
+    const int g = g_base + blockIdx.x;
+    const int32_t* seqs = a.seqs + (size_t)g * N * a.stride;
+    uint2* out = reinterpret_cast<uint2*>(names + (size_t)g * N * pitch);
+    if (tid < N) {
+        bool neg = false;
+        s_len[tid] = clamp_len(a.lens, (size_t)g * N + tid, K, neg);
+        if (neg && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
     }
-};
-
-// Position of the first `sym` among those left out of the table, m if there is none.
-__device__ __noinline__ uint32_t first_left_out(const int32_t* __restrict__ pat, int32_t sym, int m,
-                                                const uint16_t* s_list, int n_list) {
-    uint32_t first = (uint32_t)m;
-    if (n_list <= kMaxListed) {
-        for (int k = 0; k < n_list; ++k)
-            if (__ldg(pat + s_list[k]) == sym) first = min(first, (uint32_t)s_list[k]);
-    } else {
-        for (first = 0u; first < (uint32_t)m && __ldg(pat + first) != sym; ) ++first;
+    __syncthreads();
+    const int shift = 32 - table_log;
+#pragma unroll 4
+    for (int e = tid; e < items; e += nthr) {
+        const int i = (int)__umulhi((uint32_t)e, inv_row), q = e - i * row_quads, live = s_len[i] - 4 * q;
+        if (live <= 0) continue;
+        const int4 v = __ldg(reinterpret_cast<const int4*>(seqs + (size_t)(uint32_t)i * (uint32_t)a.stride) + q);
+        reinterpret_cast<int4*>(s_sym)[e] = v;
+        s_table[((uint32_t)v.x * kHashMul) >> shift] = (uint16_t)(4 * e);
+        if (live > 1) s_table[((uint32_t)v.y * kHashMul) >> shift] = (uint16_t)(4 * e + 1);
+        if (live > 2) s_table[((uint32_t)v.z * kHashMul) >> shift] = (uint16_t)(4 * e + 2);
+        if (live > 3) s_table[((uint32_t)v.w * kHashMul) >> shift] = (uint16_t)(4 * e + 3);
     }
-    return first;
+    __syncthreads();
+    uint32_t open = 0u;                            // the thread's positions without a name, four bits an item
+    int b = 0;
+#pragma unroll 2
+    for (int e = tid; e < items; e += nthr, b += 4) {
+        const int i = (int)__umulhi((uint32_t)e, inv_row), q = e - i * row_quads, live = s_len[i] - 4 * q;
+        if (live <= 0) continue;
+        const int4 v = reinterpret_cast<const int4*>(s_sym)[e];
+        const int32_t sym[4] = {v.x, v.y, v.z, v.w};
+        uint32_t name[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) name[k] = s_table[((uint32_t)sym[k] * kHashMul) >> shift];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (k >= live) name[k] = 0u;           // any name will do
+            else if (s_sym[name[k]] != sym[k]) open |= 1u << (b + k);
+        }
+        out[e] = make_uint2(name[0] | (name[1] << 16), name[2] | (name[3] << 16));
+    }
+    uint32_t mul = kHashMul;
+    for (int round = 0; round < SR_MAX_N * SR_MAX_K; ++round) {
+        if (!__syncthreads_or(open != 0u)) break;
+        mul = mul * 0x2C1B3C6Du + 0x297A2D3Au;     // stays odd
+        for (uint32_t o = open; o; o &= o - 1u) {
+            const int c = __ffs(o) - 1, pos = 4 * (tid + (c >> 2) * nthr) + (c & 3);
+            s_table[((uint32_t)s_sym[pos] * mul) >> shift] = (uint16_t)pos;
+        }
+        __syncthreads();
+        for (uint32_t o = open; o; o &= o - 1u) {
+            const int c = __ffs(o) - 1, pos = 4 * (tid + (c >> 2) * nthr) + (c & 3);
+            const uint32_t name = s_table[((uint32_t)s_sym[pos] * mul) >> shift];
+            if (s_sym[name] != s_sym[pos]) continue;
+            reinterpret_cast<uint16_t*>(out)[pos] = (uint16_t)name;
+            open &= ~(1u << c);
+        }
+    }
 }
 
+// ------------------------------------------------------------------------ prep
 // One CTA per pattern.  Per text it also counts the columns whose symbol does not occur in the
 // pattern at all and the positions at which text and pattern differ: bounds of the pair's distance that
 // cost next to nothing here.  Where they meet the pair is done.
 template <bool kDecide>
 __global__ void __launch_bounds__(kPrepThreads, 6)
 multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base) {
-    grid_begin();
     extern __shared__ __align__(16) unsigned char smem[];
-    uint32_t* s_info = reinterpret_cast<uint32_t*>(smem);         // [pitch] see below
-    uint32_t* s_slot = s_info + W.pitch;                          // [slots]
-    // (At K = 1024 the 36 KB of dynamic plus the static shared memory sit just under the size
-    // at which six CTAs share an SM.)
-    __shared__ int64_t s_text[kMaxTexts], s_stream[kMaxTexts];    // where a text's symbols and stream begin
-    __shared__ int s_txt[kMaxTexts], s_len[kMaxTexts], s_qstart[kMaxTexts + 1], s_cp[kMaxTexts];
+    uint32_t* s_info = reinterpret_cast<uint32_t*>(smem);             // [pitch] see below
+    uint16_t* s_map = reinterpret_cast<uint16_t*>(s_info + W.pitch);  // [N * pitch] stream entry of every name
+    __shared__ int64_t s_stream[kMaxTexts];                           // where a text's stream begins
+    __shared__ int s_txt[kMaxTexts], s_len[kMaxTexts], s_cstart[kMaxTexts + 1], s_cp[kMaxTexts];
     __shared__ uint32_t s_count[kMaxTexts];  // differing positions | absent columns << 16
     __shared__ uint32_t s_flag[kMaxTexts];   // the stream holds row or chain entries
     __shared__ int s_repeats[4];     // symbols with >= 2, 3, 4 occurrences; mask rows handed out
-    __shared__ int s_over;           // positions left out of the table, and the first of them
-    __shared__ uint16_t s_list[kMaxListed];
 
     const int N = a.N, K = a.K, P = pairs_of(N);
     const int tid = threadIdx.x, lane = tid & 31;
     const int M = (N & 1) ? N : N - 1;                // the last rollout of an even group is never a pattern
     const int g = g_base + blockIdx.x / M, i = blockIdx.x % M;
+    if (tid < 4) s_repeats[tid] = 0;
+    for (int e = tid; 8 * e < N * W.pitch; e += kPrepThreads)
+        reinterpret_cast<uint4*>(s_map)[e] = make_uint4(kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u);
+    for (int e = tid; 4 * e < W.pitch; e += kPrepThreads) reinterpret_cast<uint4*>(s_info)[e] = make_uint4(0u, 0u, 0u, 0u);
+    grid_begin();
     bool neg = false;
     const int m = clamp_len(a.lens, (size_t)g * N + i, K, neg);
-    const int pos_bits = max(6, 32 - __clz(max(m, 1) - 1));       // of positions 0 .. m - 1
-    const PatternTable table{s_slot, pos_bits, 2 + pos_bits, (1u << pos_bits) - 1u};
-    const int slots = (8 << pos_bits) + 8;
-    if (tid < 4) s_repeats[tid] = 0;
-    if (tid == 4) s_over = 0;
-    // The texts this pattern is paired with, one warp per text.  The warp also measures the
-    // common prefix of pattern and text (128 positions per trip, stopping at the first
-    // mismatch): rollouts of one group start from the same state and often agree on their
-    // first symbols, and the edit distance of two sequences equals that of what is left
-    // after a common prefix is removed, so those rows and columns are never looked up nor
-    // run through the recurrence.
-    const int32_t* pat = a.seqs + ((size_t)g * N + i) * a.stride;
-    const int4* pat4 = reinterpret_cast<const int4*>(pat);
+    const uint16_t* names = reinterpret_cast<const uint16_t*>(ws + W.off_names) + (size_t)g * N * W.pitch;
+    const uint16_t* pat = names + i * W.pitch;
     // Which rollout of a pair is the pattern follows a round-robin tournament: with M = N
     // for odd N and N - 1 otherwise, rollout i < M is the pattern against the `half` rollouts
     // after it (cyclically among the first M) and, for even N, against the last rollout,
@@ -318,101 +342,74 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     const int half = (M - 1) / 2;
     const int n_before = max(0, i - half), n_after = min(i + half, M - 1) - i;
     const int ntxt = n_before + n_after + ((N & 1) ? 0 : 1);
-    // the clears fall to the warps without a text, or to all if each has one
-    const int clearing = ntxt < kPrepThreads / 32 ? kPrepThreads - 32 * ntxt : kPrepThreads;
-    if (const int q = kPrepThreads - 1 - tid; q < clearing) {
-        for (int e = q; 4 * e < m; e += clearing) reinterpret_cast<uint4*>(s_info)[e] = make_uint4(0u, 0u, 0u, 0u);
-        for (int e = q; 4 * e < slots; e += clearing)
-            reinterpret_cast<uint4*>(s_slot)[e] = make_uint4(kSlotEmpty, kSlotEmpty, kSlotEmpty, kSlotEmpty);
-    }
+    // The texts, one warp per text.  The warp measures the common prefix of pattern and text (256
+    // positions per trip, stopping at the first mismatch): rollouts of one group start from
+    // the same state and often agree on their first symbols, and the edit distance of two
+    // sequences equals that of what is left after a common prefix is removed, so those rows
+    // and columns are never looked up nor run through the recurrence.
     for (int t = tid >> 5; t < ntxt; t += kPrepThreads / 32) {
         const int j = t < n_before ? t : (t < n_before + n_after ? i + 1 + (t - n_before) : N - 1);
-        bool neg_t = false;
-        const int n = clamp_len(a.lens, (size_t)g * N + j, K, neg_t);
-        const int64_t row = ((int64_t)g * N + j) * a.stride;
-        const int4* txt4 = reinterpret_cast<const int4*>(a.seqs + row);
+        const int n = clamp_len(a.lens, (size_t)g * N + j, K, neg);
         const int lo = min(m, n);
         int cp = lo;                                  // first mismatch; min(m, n) = none found
-        for (int base = 0; base < lo && cp == lo; base += 128) {
-            const int at = base + 4 * lane;
-            int eq = 4;                               // symbols of the lane's quad that agree
+        for (int base = 0; base < lo && cp == lo; base += 256) {
+            const int at = base + 8 * lane;
+            int eq = 8;                               // names of the lane's eight that agree
             if (at < lo) {
-                const int4 u = __ldg(pat4 + (at >> 2)), v = __ldg(txt4 + (at >> 2));
-                eq = u.x != v.x ? 0 : (u.y != v.y ? 1 : (u.z != v.z ? 2 : (u.w != v.w ? 3 : 4)));
+                const uint4 u = *reinterpret_cast<const uint4*>(pat + at);
+                const uint4 v = *reinterpret_cast<const uint4*>(names + j * W.pitch + at);
+                const uint32_t x[4] = {u.x ^ v.x, u.y ^ v.y, u.z ^ v.z, u.w ^ v.w};
+#pragma unroll
+                for (int w = 3; w >= 0; --w)
+                    if (x[w]) eq = 2 * w + ((x[w] & 0xFFFFu) ? 0 : 1);
             }
-            const unsigned b = __ballot_sync(0xFFFFFFFFu, eq < 4);
+            const unsigned b = __ballot_sync(0xFFFFFFFFu, eq < 8);
             if (b) {
                 const int first = __ffs(b) - 1;
-                cp = min(base + 4 * first + __shfl_sync(0xFFFFFFFFu, eq, first), lo);
+                cp = min(base + 8 * first + __shfl_sync(0xFFFFFFFFu, eq, first), lo);
             }
         }
         if (lane == 0) {
             s_txt[t] = j;
             s_len[t] = n;
-            s_text[t] = row;
             s_stream[t] = ((int64_t)g * P + pair_index(min(i, j), max(i, j), N)) * W.pitch;
             s_count[t] = 0u;
             s_flag[t] = 0u;
             s_cp[t] = cp >= lo ? -1 : cp;             // -1: one prefix is the start of the other, nothing is left to do
-            if (neg_t && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
         }
     }
     __syncthreads();
-    if (tid == 0) {
-        int quads = 0;
+    if (tid == 0) {                                   // chunks of 32 quads of columns, a warp's trip each
+        int chunks = 0;
         for (int t = 0; t < ntxt; ++t) {
-            s_qstart[t] = quads;
-            quads += s_cp[t] < 0 ? 0 : (s_len[t] - (s_cp[t] & ~31) + 3) >> 2;
+            s_cstart[t] = chunks;
+            chunks += s_cp[t] < 0 ? 0 : (s_len[t] - (s_cp[t] & ~31) + 127) >> 7;
         }
-        s_qstart[ntxt] = quads;
+        s_cstart[ntxt] = chunks;
     }
-    // Every position claims the slot of its symbol or counts itself as a further occurrence
-    // with the position that did (s_info[claimant]).
-    uint32_t my_first[kPosPerThread];
-    bool repeated = false;           // or left out
+    // Every position claims its name's entry; those that find another one there count as further
+    // occurrences with the position that stayed (s_info[claimant]).
+    uint32_t my_name[kPosPerThread], my_first[kPosPerThread];
+#pragma unroll
+    for (int k = 0; k < kPosPerThread; ++k) {
+        const int p = tid + k * kPrepThreads;
+        my_name[k] = p < m ? pat[p] : 0u;
+        if (p < m) s_map[my_name[k]] = (uint16_t)p;
+    }
+    __syncthreads();
+    bool repeated = false;
 #pragma unroll
     for (int k = 0; k < kPosPerThread; ++k) {
         const uint32_t p = tid + k * kPrepThreads;
         my_first[k] = p;
         if (p >= (uint32_t)m) continue;
-        const uint32_t x = (uint32_t)__ldg(pat + p) * kHashMul, h = table.home(x);
-        bool placed = false;
-        for (uint32_t d = 0; !placed && d <= kMaxProbe; ++d) {
-            const uint32_t want = table.tag(x, d);
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                uint32_t* at = &s_slot[2u * (h + d) + half];
-                uint32_t e = *at;
-                if (e == kSlotEmpty) e = atomicCAS(at, kSlotEmpty, want | p);
-                if (e == kSlotEmpty) { placed = true; break; }
-                if (table.holds(e, want)) {
-                    my_first[k] = table.position(e);
-                    placed = true;
-                    break;
-                }
-            }
-        }
-        if (!placed) {
-            const int at = atomicAdd(&s_over, 1);
-            if (at < kMaxListed) s_list[at] = (uint16_t)p;
-            my_first[k] = kLocOpen;
-            repeated = true;
-        } else if (my_first[k] != p) {
+        my_first[k] = s_map[my_name[k]];
+        if (my_first[k] != p) {
             atomicAdd(&s_info[my_first[k]], 1u);
             repeated = true;
         }
     }
     if (__syncthreads_or(repeated)) {
-        if (s_over) {
-#pragma unroll
-            for (int k = 0; k < kPosPerThread; ++k) {
-                const uint32_t p = tid + k * kPrepThreads;
-                if (my_first[k] != kLocOpen) continue;
-                my_first[k] = first_left_out(pat, __ldg(pat + p), m, s_list, s_over);
-                if (my_first[k] != p) atomicAdd(&s_info[my_first[k]], 1u);
-            }
-            __syncthreads();
-        }
         // Symbols with several occurrences.  In written language a few tokens make up much of
         // every rollout (a third of the columns of such a text meet a symbol that occurs more
         // than once, the most common one dozens of times), so these get a row of match words,
@@ -437,7 +434,12 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             const int p = tid + k * kPrepThreads;
             if (p >= m || my_first[k] != (uint32_t)p) continue;
             const uint32_t more = s_info[p];
-            s_info[p] = more == 0u ? (uint32_t)p : (more >= need ? kLocRow | (uint32_t)atomicAdd(&s_repeats[3], 1) : (kChainEnd << 16) | kLocChain | (uint32_t)p);
+            uint32_t code = (uint32_t)p;
+            if (more != 0u) {
+                code = more >= need ? kLocRow | (uint32_t)atomicAdd(&s_repeats[3], 1) : (kChainEnd << 16) | kLocChain | (uint32_t)p;
+                s_map[my_name[k]] = (uint16_t)code;             // what the streams of the texts say
+            }
+            s_info[p] = code;
         }
         __syncthreads();
         uint32_t* rows = reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * N + i) * W.row_cap * W.row_words;
@@ -461,88 +463,49 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         }
     }
     const bool named = s_repeats[0] > 0;
-    const int left_out = s_over;
+    if (named) __syncthreads();                       // the map's entries are final
 
-    // Match streams of all texts, four columns per thread and trip: one 16-byte load of
-    // symbols, four independent look-ups, one 8-byte store.
+    // Match streams of all texts, four columns per lane and trip: one 8-byte load of names, four
+    // look-ups, one 8-byte store.
     uint16_t* locs = reinterpret_cast<uint16_t*>(ws + W.off_loc);
-    const int total_quads = s_qstart[ntxt];
-    for (int base = tid - lane; base < total_quads; base += kPrepThreads) {
-        const int item = min(base + lane, total_quads - 1);        // lanes past the end run along
-        const bool live = base + lane < total_quads;
-        int t = 0;
-        while (item >= s_qstart[t + 1]) ++t;
-        const int q = ((s_cp[t] & ~31) >> 2) + item - s_qstart[t];      // quad index within the text
-        const int4 sym4 = __ldg(reinterpret_cast<const int4*>(a.seqs + s_text[t]) + q);
-        const int32_t sym[4] = {sym4.x, sym4.y, sym4.z, sym4.w};
-        uint32_t home[4], want[4], l[4];
-        uint2 e[4];
-        bool more = false;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const uint32_t x = (uint32_t)sym[u] * kHashMul;
-            home[u] = table.home(x);
-            want[u] = table.tag(x, 0u);
-            e[u] = reinterpret_cast<const uint2*>(s_slot)[home[u]];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            l[u] = table.look(e[u], want[u]);
-            more |= l[u] == kLocOpen;
-        }
-        for (uint32_t d = 1; more && d <= kMaxProbe; ++d) {        // the home bucket holds two foreign symbols
-            more = false;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (l[u] != kLocOpen) continue;
-                l[u] = table.look(reinterpret_cast<const uint2*>(s_slot)[home[u] + d], want[u] | (d << pos_bits));
-                more |= l[u] == kLocOpen;
-            }
-        }
-        if (more) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (l[u] != kLocOpen) continue;
-                l[u] = kLocNone;
-                if (left_out) {
-                    const uint32_t p = first_left_out(pat, sym[u], m, s_list, left_out);
-                    if (p < (uint32_t)m) l[u] = p;
-                }
-            }
-        }
-        if (named) {                                   // positions to stream entries
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (l[u] != kLocNone) l[u] = reinterpret_cast<const uint16_t*>(s_info)[2u * l[u]];
-        }
-        // The last quad of a text is filled up with symbols of their own that the pattern is
-        // extended by as well: a common suffix leaves the distance as it is, and the recurrence
-        // always runs whole quads, whose four columns the compiler can then interleave.
-        const int left = s_len[t] - 4 * q;             // columns of this quad that exist (>= 1)
-#pragma unroll
-        for (int u = 1; u < 4; ++u)
-            if (u >= left) l[u] = (uint32_t)(m + u - left);
-        if (live) reinterpret_cast<uint2*>(locs + s_stream[t])[q] = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
-        if (named && ((l[0] | l[1] | l[2] | l[3]) & kLocRow)) s_flag[t] = 1u;
-        // positions below both lengths whose symbol is not the pattern's symbol at the same place,
-        // and columns without any match
+    const int chunks = s_cstart[ntxt];
+    int t = 0;
+    for (int c = tid >> 5; c < chunks; c += kPrepThreads / 32) {
+        while (c >= s_cstart[t + 1]) ++t;
+        const int n = s_len[t], q = ((s_cp[t] & ~31) >> 2) + 32 * (c - s_cstart[t]) + lane;   // quad within the text
+        const int left = n - 4 * q;                    // columns of this quad that exist
         uint32_t count = 0u;
-        const int both = min(m, s_len[t]) - 4 * q;     // columns of this quad below both lengths
-        if (both > 0) {
-            const int4 own = __ldg(pat4 + q);
-            count = (sym[0] != own.x) + (both > 1 && sym[1] != own.y) + (both > 2 && sym[2] != own.z) +
-                    (both > 3 && sym[3] != own.w);
-        }
+        bool row = false;
+        if (left > 0) {
+            const uint2 v = *reinterpret_cast<const uint2*>(names + s_txt[t] * W.pitch + 4 * q);
+            uint32_t l[4] = {s_map[v.x & 0xFFFFu], s_map[v.x >> 16], s_map[v.y & 0xFFFFu], s_map[v.y >> 16]};
+            // The last quad of a text is filled up with symbols of their own that the pattern is
+            // extended by as well: a common suffix leaves the distance as it is, and the recurrence
+            // always runs whole quads, whose four columns the compiler can then interleave.
+            if (left < 4) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) count += l[u] == kLocNone ? 0x10000u : 0u;
-        if (!live) count = 0u;
-        // quads of a warp follow one another, so most warps work on one text
-        const int t_first = __shfl_sync(0xFFFFFFFFu, t, 0);
-        if (t_first == __shfl_sync(0xFFFFFFFFu, t, 31)) {
-            count = __reduce_add_sync(0xFFFFFFFFu, count);
-            if (lane == 0) atomicAdd(&s_count[t], count);
-        } else if (count) {
-            atomicAdd(&s_count[t], count);
+                for (int u = 1; u < 4; ++u)
+                    if (u >= left) l[u] = (uint32_t)(m + u - left);
+            }
+            reinterpret_cast<uint2*>(locs + s_stream[t])[q] = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
+            row = (l[0] | l[1] | l[2] | l[3]) & kLocRow;
+            // positions below both lengths whose symbol is not the pattern's symbol at the same place,
+            // and columns without any match
+            const int both = min(m - 4 * q, left);     // columns of this quad below both lengths
+            if (both > 0) {
+                const uint2 own = *reinterpret_cast<const uint2*>(pat + 4 * q);
+                const uint32_t x = v.x ^ own.x, y = v.y ^ own.y;
+                count = ((x & 0xFFFFu) != 0u) + (both > 1 && (x >> 16) != 0u) + (both > 2 && (y & 0xFFFFu) != 0u) +
+                        (both > 3 && (y >> 16) != 0u);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) count += l[u] == kLocNone ? 0x10000u : 0u;
+        }
+        count = __reduce_add_sync(0xFFFFFFFFu, count);
+        row = __any_sync(0xFFFFFFFFu, row);
+        if (lane == 0) {
+            if (count) atomicAdd(&s_count[t], count);
+            if (row) s_flag[t] = 1u;
         }
     }
     __syncthreads();
@@ -582,7 +545,6 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             atomicAdd(&ctl->open, open);
         }
     }
-    if (neg && tid == 0 && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
 }
 
 // ----------------------------------------------------------------------- order
@@ -1145,6 +1107,22 @@ multi_finish_kernel(GateArgs a, int32_t* dist, const uint8_t* flag, uint8_t* exa
     if (capped && exact) exact[g] = 0;                       // some distances are lower bounds
 }
 
+// More than 48 KB of shared memory has to be asked for: the most that any call takes, once per device (noted,
+// because asking is host time).
+constexpr int kMostNamesSmem = 200 * 1024;
+int allow_smem() {
+    static std::atomic<bool> allowed[64];
+    int dev = 0;
+    SR_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev >= 0 && dev < 64 && allowed[dev].load(std::memory_order_relaxed)) return SR_OK;
+    const int prep = SR_MAX_K * 4 + SR_MAX_N * SR_MAX_K * 2;
+    SR_CUDA_TRY(cudaFuncSetAttribute(multi_names_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostNamesSmem));
+    SR_CUDA_TRY(cudaFuncSetAttribute(multi_prep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, prep));
+    SR_CUDA_TRY(cudaFuncSetAttribute(multi_prep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, prep));
+    if (dev >= 0 && dev < 64) allowed[dev].store(true, std::memory_order_relaxed);
+    return SR_OK;
+}
+
 }  // namespace
 
 size_t gate_multi_workspace_bytes(int32_t n_groups, int32_t N, int32_t stride, int32_t K) {
@@ -1173,9 +1151,19 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     int32_t* dist = a.pair_dist ? a.pair_dist : reinterpret_cast<int32_t*>(ws + W.off_dist);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
 
-    int pos_bits = 6;
-    while ((1 << pos_bits) < a.K) ++pos_bits;
-    const int prep_smem = (W.pitch + (8 << pos_bits) + 8) * 4, patterns = (a.N & 1) ? a.N : a.N - 1;
+    const int patterns = (a.N & 1) ? a.N : a.N - 1;
+    const int prep_smem = W.pitch * 4 + a.N * W.pitch * 2;
+    // names: at least two slots to a symbol while symbols and table fit
+    const int sym_bytes = a.N * W.pitch * 4, names_threads = a.N * W.pitch > 4 * 8 * 512 ? 1024 : 512;
+    int table_log = 8;
+    while ((1 << table_log) < 2 * a.N * a.K && sym_bytes + (4 << table_log) <= kMostNamesSmem) ++table_log;
+    const int names_smem = sym_bytes + (2 << table_log);
+    const uint32_t inv_row = (uint32_t)(((1ull << 32) + (W.pitch >> 2) - 1) / (W.pitch >> 2));
+    uint16_t* names = reinterpret_cast<uint16_t*>(ws + W.off_names);
+    if (names_smem > 48 * 1024 || prep_smem > 48 * 1024) {
+        const int rc = allow_smem();
+        if (rc != SR_OK) return rc;
+    }
 
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[0], s));
     // what the kernels add up starts at zero (one CTA that orders the batch alone needs nothing)
@@ -1193,6 +1181,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
             const int rc = feed->before(feed->ctx, g0, g1, s);
             if (rc != SR_OK) return rc;
         }
+        SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0);
         if (decide)
             SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<true>, (g1 - g0) * patterns, kPrepThreads, prep_smem, s, a, ws, W, dist, g0);
         else
