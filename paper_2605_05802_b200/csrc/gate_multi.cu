@@ -57,7 +57,6 @@ constexpr uint32_t kLocNone = 0x7FFFu;    // bit 15 clear, far above any row: sh
 constexpr uint32_t kLocRow = 0x8000u;     // | index of the symbol's mask row
 constexpr uint32_t kLocChain = 0xC000u;   // | first position of the symbol's occurrence chain
 constexpr uint32_t kChainEnd = 0xFFFFu;
-constexpr int kPosPerThread = SR_MAX_K / kPrepThreads;
 constexpr int kDpWarpsPerCta = 4;
 constexpr uint32_t kBinMask = 0x7FFu;
 constexpr uint32_t kHasChains = 0x40000000u;
@@ -232,7 +231,8 @@ __device__ __forceinline__ int clamp_len(const int32_t* lens, size_t idx, int K,
 // round names at least one symbol of each slot.  One CTA per group.  With the names, 16 bits
 // each, a pattern's look-up table is an array: no hashing, no probing, no comparing in prep, which serves
 // every text (N - 1) / 2 times.  (The table of hashed 32-bit slots that prep had instead took 280 warp
-// instructions for four columns of a warp's lanes.)
+// instructions for four columns of a warp's lanes; with the names, on 1024 groups of 8 token prefixes, both kernels
+// together take 81 us where it took 104, and 107 against 150 at full length.)
 constexpr uint32_t kHashMul = 0x9E3779B1u;
 constexpr int kMaxTexts = SR_MAX_N / 2;        // texts a pattern is paired with
 
@@ -305,6 +305,11 @@ multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int
 }
 
 // ------------------------------------------------------------------------ prep
+// Top bit of each half of x that is not zero.
+__device__ __forceinline__ uint32_t set_halves(uint32_t x) {
+    return (((x & 0x7FFF7FFFu) + 0x7FFF7FFFu) | x) & 0x80008000u;
+}
+
 // One CTA per pattern.  Per text it also counts the columns whose symbol does not occur in the
 // pattern at all and the positions at which text and pattern differ: bounds of the pair's distance that
 // cost next to nothing here.  Where they meet the pair is done.
@@ -315,7 +320,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     uint32_t* s_info = reinterpret_cast<uint32_t*>(smem);             // [pitch] see below
     uint16_t* s_map = reinterpret_cast<uint16_t*>(s_info + W.pitch);  // [N * pitch] stream entry of every name
     __shared__ int64_t s_stream[kMaxTexts];                           // where a text's stream begins
-    __shared__ int s_txt[kMaxTexts], s_len[kMaxTexts], s_cstart[kMaxTexts + 1], s_cp[kMaxTexts];
+    __shared__ int s_txt[kMaxTexts], s_len[kMaxTexts], s_cp[kMaxTexts];
     __shared__ uint32_t s_count[kMaxTexts];  // differing positions | absent columns << 16
     __shared__ uint32_t s_flag[kMaxTexts];   // the stream holds row or chain entries
     __shared__ int s_repeats[4];     // symbols with >= 2, 3, 4 occurrences; mask rows handed out
@@ -379,32 +384,26 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         }
     }
     __syncthreads();
-    if (tid == 0) {                                   // chunks of 32 quads of columns, a warp's trip each
-        int chunks = 0;
-        for (int t = 0; t < ntxt; ++t) {
-            s_cstart[t] = chunks;
-            chunks += s_cp[t] < 0 ? 0 : (s_len[t] - (s_cp[t] & ~31) + 127) >> 7;
-        }
-        s_cstart[ntxt] = chunks;
-    }
     // Every position claims its name's entry; those that find another one there count as further
-    // occurrences with the position that stayed (s_info[claimant]).
-    uint32_t my_name[kPosPerThread], my_first[kPosPerThread];
-#pragma unroll
-    for (int k = 0; k < kPosPerThread; ++k) {
-        const int p = tid + k * kPrepThreads;
-        my_name[k] = p < m ? pat[p] : 0u;
-        if (p < m) s_map[my_name[k]] = (uint16_t)p;
+    // occurrences with the position that stayed (s_info[claimant]).  Four positions per thread.
+    static_assert(4 * kPrepThreads >= SR_MAX_K, "a position for every thread");
+    const int p0 = 4 * tid, mine = min(max(m - p0, 0), 4);
+    uint32_t my_name[4] = {0u, 0u, 0u, 0u}, my_first[4];
+    if (mine > 0) {
+        const uint2 v = *reinterpret_cast<const uint2*>(pat + p0);
+        my_name[0] = v.x & 0xFFFFu; my_name[1] = v.x >> 16; my_name[2] = v.y & 0xFFFFu; my_name[3] = v.y >> 16;
     }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (k < mine) s_map[my_name[k]] = (uint16_t)(p0 + k);
     __syncthreads();
     bool repeated = false;
 #pragma unroll
-    for (int k = 0; k < kPosPerThread; ++k) {
-        const uint32_t p = tid + k * kPrepThreads;
-        my_first[k] = p;
-        if (p >= (uint32_t)m) continue;
+    for (int k = 0; k < 4; ++k) {
+        my_first[k] = p0 + k;
+        if (k >= mine) continue;
         my_first[k] = s_map[my_name[k]];
-        if (my_first[k] != p) {
+        if (my_first[k] != (uint32_t)(p0 + k)) {
             atomicAdd(&s_info[my_first[k]], 1u);
             repeated = true;
         }
@@ -420,40 +419,44 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         // (the rarest of the repeated ones) is left as a chain of at most seven positions.
         // From here on the lower half of s_info[claimant] is the symbol's stream entry, the upper half
         // the head of the chain of its further positions.
+        // (only claimants of repeated symbols have a count)
+        uint32_t more[4] = {0u, 0u, 0u, 0u};
+        if (mine > 0) {
+            const uint4 v = *reinterpret_cast<const uint4*>(s_info + p0);
+            more[0] = v.x; more[1] = v.y; more[2] = v.z; more[3] = v.w;
+        }
+        const bool claims = (more[0] | more[1] | more[2] | more[3]) != 0u;
+        if (claims) {
 #pragma unroll
-        for (int k = 0; k < kPosPerThread; ++k) {
-            const int p = tid + k * kPrepThreads;
-            if (p >= m || my_first[k] != (uint32_t)p) continue;
-            const uint32_t more = s_info[p];
-            for (uint32_t c = 0; c < 3u && c < more; ++c) atomicAdd(&s_repeats[c], 1);
+            for (int k = 0; k < 4; ++k)
+                for (uint32_t c = 0; c < 3u && c < more[k]; ++c) atomicAdd(&s_repeats[c], 1);
         }
         __syncthreads();
         const uint32_t need = s_repeats[0] <= W.row_cap ? 1u : (s_repeats[1] <= W.row_cap ? 2u : (s_repeats[2] <= W.row_cap ? 3u : 7u));
+        if (claims) {
 #pragma unroll
-        for (int k = 0; k < kPosPerThread; ++k) {
-            const int p = tid + k * kPrepThreads;
-            if (p >= m || my_first[k] != (uint32_t)p) continue;
-            const uint32_t more = s_info[p];
-            uint32_t code = (uint32_t)p;
-            if (more != 0u) {
-                code = more >= need ? kLocRow | (uint32_t)atomicAdd(&s_repeats[3], 1) : (kChainEnd << 16) | kLocChain | (uint32_t)p;
+            for (int k = 0; k < 4; ++k) {
+                if (more[k] == 0u) continue;
+                const uint32_t code = more[k] >= need ? kLocRow | (uint32_t)atomicAdd(&s_repeats[3], 1)
+                                                      : (kChainEnd << 16) | kLocChain | (uint32_t)(p0 + k);
                 s_map[my_name[k]] = (uint16_t)code;             // what the streams of the texts say
+                s_info[p0 + k] = code;
             }
-            s_info[p] = code;
         }
         __syncthreads();
         uint32_t* rows = reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * N + i) * W.row_cap * W.row_words;
         for (int e = tid; e < s_repeats[3] * W.row_words; e += kPrepThreads) rows[e] = 0u;
         __syncthreads();
+        if (claims || repeated) {
 #pragma unroll
-        for (int k = 0; k < kPosPerThread; ++k) {
-            const int p = tid + k * kPrepThreads;
-            if (p >= m) continue;
-            const uint32_t f = my_first[k], info = s_info[f];
-            if ((info & kLocChain) == kLocChain) {
-                if (f != (uint32_t)p) s_info[p] = atomicExch(&s_info[f], ((uint32_t)p << 16) | kLocChain | f);
-            } else if (info & kLocRow) {
-                atomicOr(&rows[(info & 0x3FFFu) * W.row_words + (p >> 5)], 1u << (p & 31));
+            for (int k = 0; k < 4; ++k) {
+                if (more[k] == 0u && my_first[k] == (uint32_t)(p0 + k)) continue;
+                const uint32_t p = p0 + k, f = my_first[k], info = s_info[f];
+                if ((info & kLocChain) == kLocChain) {
+                    if (f != p) s_info[p] = atomicExch(&s_info[f], (p << 16) | kLocChain | f);
+                } else {
+                    atomicOr(&rows[(info & 0x3FFFu) * W.row_words + (p >> 5)], 1u << (p & 31));
+                }
             }
         }
         if (s_repeats[0] > s_repeats[3]) {             // some chains: leave them for the recurrence
@@ -466,43 +469,46 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     if (named) __syncthreads();                       // the map's entries are final
 
     // Match streams of all texts, four columns per lane and trip: one 8-byte load of names, four
-    // look-ups, one 8-byte store.
+    // look-ups, one 8-byte store.  As many warps to a text as there are for each (chunks dealt to all
+    // warps in turn would be even, but then every warp sets up every text).
     uint16_t* locs = reinterpret_cast<uint16_t*>(ws + W.off_loc);
-    const int chunks = s_cstart[ntxt];
-    int t = 0;
-    for (int c = tid >> 5; c < chunks; c += kPrepThreads / 32) {
-        while (c >= s_cstart[t + 1]) ++t;
-        const int n = s_len[t], q = ((s_cp[t] & ~31) >> 2) + 32 * (c - s_cstart[t]) + lane;   // quad within the text
-        const int left = n - 4 * q;                    // columns of this quad that exist
-        uint32_t count = 0u;
-        bool row = false;
-        if (left > 0) {
-            const uint2 v = *reinterpret_cast<const uint2*>(names + s_txt[t] * W.pitch + 4 * q);
-            uint32_t l[4] = {s_map[v.x & 0xFFFFu], s_map[v.x >> 16], s_map[v.y & 0xFFFFu], s_map[v.y >> 16]};
-            // The last quad of a text is filled up with symbols of their own that the pattern is
-            // extended by as well: a common suffix leaves the distance as it is, and the recurrence
-            // always runs whole quads, whose four columns the compiler can then interleave.
-            if (left < 4) {
-#pragma unroll
-                for (int u = 1; u < 4; ++u)
-                    if (u >= left) l[u] = (uint32_t)(m + u - left);
+    const int per_text = max(1, kPrepThreads / 32 / ntxt), warp = tid >> 5, part = warp % per_text;
+    for (int t = warp / per_text; t < ntxt; t += kPrepThreads / 32 / per_text) {
+        if (s_cp[t] < 0) continue;
+        const int n = s_len[t];
+        const uint2* in = reinterpret_cast<const uint2*>(names + s_txt[t] * W.pitch);
+        const uint2* own = reinterpret_cast<const uint2*>(pat);
+        uint2* out = reinterpret_cast<uint2*>(locs + s_stream[t]);
+        uint32_t differ = 0u, present = 0u, seen = 0u, columns = 0u;
+        for (int q = ((s_cp[t] & ~31) >> 2) + 32 * part + lane; 4 * q < n; q += 32 * per_text) {
+            const int left = n - 4 * q;                // columns of this quad that exist
+            const uint2 v = in[q], o = own[q];         // past the pattern's end: still in the group's names or the rows after them
+            uint32_t w0 = s_map[v.x & 0xFFFFu] | ((uint32_t)s_map[v.x >> 16] << 16);
+            uint32_t w1 = s_map[v.y & 0xFFFFu] | ((uint32_t)s_map[v.y >> 16] << 16);
+            // positions below both lengths whose symbol is not the pattern's symbol at the same place
+            uint32_t d0 = set_halves(v.x ^ o.x), d1 = set_halves(v.y ^ o.y);
+            const int both = m - 4 * q;                // columns of this quad below the pattern's length
+            if (left < 4 || both < 4) {
+                const int k = min(left, both);
+                d0 = k > 1 ? d0 : (k == 1 ? d0 & 0xFFFFu : 0u);
+                d1 = k > 3 ? d1 : (k == 3 ? d1 & 0xFFFFu : 0u);
+                // The last quad of a text is filled up with symbols of their own that the pattern is
+                // extended by as well: a common suffix leaves the distance as it is, and the recurrence
+                // always runs whole quads, whose four columns the compiler can then interleave.
+                if (left == 1) w0 = (w0 & 0xFFFFu) | ((uint32_t)m << 16);
+                if (left == 1) w1 = (uint32_t)(m + 1) | ((uint32_t)(m + 2) << 16);
+                if (left == 2) w1 = (uint32_t)m | ((uint32_t)(m + 1) << 16);
+                if (left == 3) w1 = (w1 & 0xFFFFu) | ((uint32_t)m << 16);
             }
-            reinterpret_cast<uint2*>(locs + s_stream[t])[q] = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
-            row = (l[0] | l[1] | l[2] | l[3]) & kLocRow;
-            // positions below both lengths whose symbol is not the pattern's symbol at the same place,
-            // and columns without any match
-            const int both = min(m - 4 * q, left);     // columns of this quad below both lengths
-            if (both > 0) {
-                const uint2 own = *reinterpret_cast<const uint2*>(pat + 4 * q);
-                const uint32_t x = v.x ^ own.x, y = v.y ^ own.y;
-                count = ((x & 0xFFFFu) != 0u) + (both > 1 && (x >> 16) != 0u) + (both > 2 && (y & 0xFFFFu) != 0u) +
-                        (both > 3 && (y >> 16) != 0u);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) count += l[u] == kLocNone ? 0x10000u : 0u;
+            out[q] = make_uint2(w0, w1);
+            seen |= w0 | w1;
+            differ += __popc(d0) + __popc(d1);
+            // columns without any match: 0x7FFF
+            present += __popc(set_halves(w0 ^ (kLocNone * 0x10001u))) + __popc(set_halves(w1 ^ (kLocNone * 0x10001u)));
+            columns += 4u;
         }
-        count = __reduce_add_sync(0xFFFFFFFFu, count);
-        row = __any_sync(0xFFFFFFFFu, row);
+        const uint32_t count = __reduce_add_sync(0xFFFFFFFFu, differ + ((columns - present) << 16));
+        const bool row = __any_sync(0xFFFFFFFFu, (seen & (kLocRow * 0x10001u)) != 0u);
         if (lane == 0) {
             if (count) atomicAdd(&s_count[t], count);
             if (row) s_flag[t] = 1u;
