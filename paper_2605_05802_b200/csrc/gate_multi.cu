@@ -61,7 +61,7 @@ constexpr int kDpWarpsPerCta = 4;
 constexpr uint32_t kBinMask = 0x7FFu;
 constexpr uint32_t kHasChains = 0x40000000u;
 constexpr int32_t kCappedFlag = 0x40000000;   // decide mode: the pair's distance exceeds its cap
-constexpr int kStripShift = 12;
+constexpr int kStripShift = 12, kRowsShift = 22;
 constexpr uint32_t kNeedsDp = 0x80000000u;
 static_assert(kNumBins <= (int)kBinMask + 1 && kTimeBuckets * kNumClasses <= kNumBins, "bin index must fit its field");
 
@@ -69,8 +69,8 @@ struct PairDesc {          // 16 bytes
     uint32_t mn;           // m | n << 16
     uint32_t pat_row;      // g * N + pattern rollout
     uint32_t bin;          // bits 0..10 bin index; bits 12..21 stripped common prefix (symbols,
-                           // a multiple of 4); bit 30 = the pattern has chains; bit 31 = pair
-                           // needs the dp kernel
+                           // a multiple of 4); bits 22..29 mask rows of the pattern; bit 30 = the
+                           // pattern has chains; bit 31 = pair needs the dp kernel
     uint32_t lower;        // bits 0..15 a lower bound of the pair's distance (decide mode),
                            // bits 16..31 an upper bound (mismatching positions + length
                            // difference; in decide mode also capped by what the threshold
@@ -536,7 +536,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         }
         PairDesc d{(uint32_t)m | ((uint32_t)n << 16), (uint32_t)(g * N + i), 0u, (uint32_t)lower | ((uint32_t)upper << 16)};
         if (lower < upper) {                          // otherwise that is the distance
-            d.bin = ((uint32_t)strip << kStripShift) | kNeedsDp | (s_repeats[0] > s_repeats[3] ? kHasChains : 0u);
+            d.bin = ((uint32_t)strip << kStripShift) | ((uint32_t)min(s_repeats[3], 255) << kRowsShift) | kNeedsDp | (s_repeats[0] > s_repeats[3] ? kHasChains : 0u);
             const PairSize z = size_of_desc(d);
             work = work_of_pair(z.m, z.n, z.lb, z.ub);
         }
@@ -712,6 +712,15 @@ __device__ __forceinline__ uint32_t shl_clamp(uint32_t v, uint32_t s) {
     return r;
 }
 
+// Brings `bytes` bytes to L1, 32 a time, `lanes` lanes together.  (Not inlined: it is run once a task.)
+__device__ __noinline__ void touch(const void* from, int bytes, int lane, int lanes) {
+    for (int o = 32 * lane; o < bytes; o += 32 * lanes) {
+        uint32_t x;
+        asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(x) : "l"(static_cast<const char*>(from) + o));
+        (void)x;
+    }
+}
+
 // Loads a lane's R words of a mask row where `p` is set, without a branch: the recurrence around
 // it stays one block of straight-line code.
 template <int R>
@@ -821,6 +830,7 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
     // m, n: rows and columns left after the common prefix of `strip` symbols, which neither
     // side runs through
     bool chains = false;
+    int n_rows = 0;
     int idx = 0, m = 0, n = 0, strip = 0, lb = 0, ub = 0;
     const uint2* loc4 = reinterpret_cast<const uint2*>(locs);
     const uint16_t* nxt = nexts;
@@ -830,6 +840,7 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
         const PairDesc d = descs[idx];
         strip = (int)((d.bin >> kStripShift) & 0x3FFu);
         chains = d.bin & kHasChains;
+        n_rows = (int)((d.bin >> kRowsShift) & 0xFFu);
         n = (int)(d.mn >> 16) - strip;
         m = (int)(d.mn & 0xFFFFu) - strip + (-n & 3);  // both extended to whole quads of columns
         n = (n + 3) & ~3;
@@ -839,6 +850,12 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
         loc4 = reinterpret_cast<const uint2*>(locs + (size_t)idx * W.pitch + strip);
         nxt = nexts + (size_t)d.pat_row * W.pitch;
         rows = masks + (size_t)d.pat_row * (W.row_cap * W.row_words) + (strip >> 5);
+    }
+    if (T >= 16 && valid) {
+        // Few pairs: nothing else hides the latencies of this one, so all that it will read goes to L1 first,
+        // the stream and the pattern's mask rows (16 groups of 8 texts: 78 -> 74 us).
+        touch(loc4, 2 * n, lt, T);
+        touch(rows, 4 * n_rows * W.row_words, lt, T);
     }
     constexpr int H = 32 * R;                          // rows of a stripe
     const int nq = n >> 2;                             // quads of text columns
@@ -1206,9 +1223,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[2], s));
     const long long want = (n_pairs_ll + kDpWarpsPerCta - 1) / kDpWarpsPerCta;
     const int blocks = (int)(want < 3LL * sms ? want : 3LL * sms);
-    // (an ordinary launch: CTAs made resident while the tail of prep still fills some SMs would
+    // (an ordinary launch unless every CTA has an SM: CTAs made resident while the tail of prep still fills some SMs would
     // crowd onto the others, 478 us instead of 434 for the token-level batch of 1024 groups)
-    const int rc = launch_as(false, 1, "multi_dp_kernel", multi_dp_kernel, blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u);
+    const int rc = launch_as(alone && blocks < sms, 1, "multi_dp_kernel", multi_dp_kernel, blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u);
     if (rc != SR_OK) return rc;
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[3], s));
     SR_LAUNCH("multi_finish_kernel", multi_finish_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, dist, flag, exact, gpb);
