@@ -220,7 +220,8 @@ def main():
     P = N * (N - 1) // 2
     cells = W.dp_cells(w.lens, K)
     wcols_full = W.word_columns(w.lens, K)
-    wcols = W.word_columns(w.lens, K, w.seqs)          # what is left after the pairs' common prefixes
+    # what the method runs: without the pairs' common prefixes, inside the bands of their bounds
+    wcols = W.word_columns(w.lens, K, w.seqs, band=True)
     seqs = torch.from_numpy(w.seqs).to(dev)
     lens = torch.from_numpy(w.lens).to(dev)
     rewards = torch.from_numpy(w.rewards).to(dev)
@@ -347,15 +348,15 @@ def main():
                 "ms_per_step": e2e_ms / args.steps,
                 "input": "packed prefixes + int64 row offsets in pinned host memory (sr_gate_host_packed), "
                          "sent in four pieces on a copy stream under the per-group pass; one recurrence launch"},
-        "gpu_launches": 5 * args.steps,
+        "gpu_launches": 7 * args.steps,       # names, prep, bin, order, dp, finish; advantages
         "clocks": clocks,
         "stage_ms": {"prep": stage_ms[0], "order": stage_ms[1], "dp": stage_ms[2], "finish": stage_ms[3]},
         "roofline": {"kernel": "multi_dp_kernel", "bound": "alu", "achieved": achieved, "peak": alu_peak,
-                     "unit": "Gop/s (int32 lane-ops, 10 per 32-row block per column, common prefixes of a pair not counted)",
+                     "unit": "Gop/s (int32 lane-ops, 10 per 32-row block per column, counted inside the bands of the pairs' bounds, common prefixes left out)",
                      "frac": achieved / alu_peak,
                      "peak_basis": f"{sms} SMs x {SM_INT32_LANES} int32 lanes/clk x {peaks['sm_max_mhz']:.0f} MHz (derived)",
                      "traffic": traffic_from_profiles("multi_dp_kernel", os.path.join(ROOT, "paper_2605_05802_b200", "csrc", "gate_multi.cu")),
-                     "word_columns": wcols, "word_columns_before_prefix_removal": wcols_full,
+                     "word_columns": wcols, "word_columns_whole_matrices": wcols_full,
                      "ms_per_launch": dp_ms},
         "verified_against_oracle": verify,
     }
@@ -515,7 +516,7 @@ def main():
         torch.cuda.synchronize()
         dp0 = statistics.median(e5[2].elapsed_time(e5[3]) for e5 in ev0)
         all0 = statistics.median(e5[0].elapsed_time(e5[4]) for e5 in ev0)
-        wc0 = W.word_columns(w0.lens, K, w0.seqs)
+        wc0 = W.word_columns(w0.lens, K, w0.seqs, band=True)
         extras["C4_no_shared_head"] = {"groups": w0.n_groups, "us_gate": all0 * 1e3, "us_dp": dp0 * 1e3,
                                        "gcups": W.dp_cells(w0.lens, K) / (all0 * 1e-3) / 1e9,
                                        "word_columns": wc0, "dp_alu_gops": 10.0 * wc0 / (dp0 * 1e-3) / 1e9,

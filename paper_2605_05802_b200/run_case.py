@@ -2,7 +2,7 @@
 device time.  Handy for profiling a single kernel:
 
     python -m paper_2605_05802_b200.run_case --case c3 --reps 3
-    ncu --set full --clock-control none -k regex:gate_single -c 1 \\
+    ncu --set full --clock-control none -k regex:gate_named -c 1 \\
         python -m paper_2605_05802_b200.run_case --case c3 --reps 3
 
 Cases: c1, c2, c2x128 (65536 groups x N=8, K=15), c3 (4096 groups x N=16), c3x16

@@ -268,12 +268,13 @@ def dp_cells(lens: np.ndarray, K: int) -> int:
     return int(((s1 * s1 - s2) // 2).sum())
 
 
-def _band_units(rows: np.ndarray, cols: np.ndarray, ub: np.ndarray) -> np.ndarray:
+def _band_units(rows: np.ndarray, cols: np.ndarray, lb: np.ndarray, ub: np.ndarray) -> np.ndarray:
     """(column, 32-row block) units inside the band of a rows x cols matrix whose
-    distance is at most ub: diagonals d = row - column with |d| + |(rows - cols) - d| <= ub
-    (at least two diagonals).  Vectorised over pairs; loops over the columns."""
+    distance lies in lb..ub: the diagonals between the corners and the e = min((ub - |rows -
+    cols|) / 2, ub - lb) beyond them on either side (at least two diagonals); none where the
+    bounds meet.  Vectorised over pairs; loops over the columns."""
     D = rows - cols
-    e = np.maximum((ub - np.abs(D)) // 2, 0)
+    e = np.maximum(np.minimum((ub - np.abs(D)) // 2, ub - lb), 0)
     dlo = np.minimum(D, 0) - e
     dhi = np.maximum(D, 0) + e
     dhi = np.where(dhi == dlo, dhi + 1, dhi)
@@ -283,7 +284,12 @@ def _band_units(rows: np.ndarray, cols: np.ndarray, ub: np.ndarray) -> np.ndarra
         hi = np.minimum(c + dhi, rows - 1)
         ok = (c < cols) & (hi >= lo)
         total += np.where(ok, hi // 32 - lo // 32 + 1, 0)
-    return total
+    return np.where(lb < ub, total, 0)
+
+
+def _absent(pattern: np.ndarray, m: np.ndarray, text: np.ndarray, n: np.ndarray, cut: np.ndarray) -> np.ndarray:
+    """Per group: the text's columns from ``cut`` (rounded down to 32) on whose symbol the pattern lacks."""
+    return np.array([int((~np.isin(t[c // 32 * 32:k], p[:r])).sum()) for p, r, t, k, c in zip(pattern, m, text, n, cut)])
 
 
 def word_columns(lens: np.ndarray, K: int, seqs: np.ndarray = None, band: bool = False) -> int:
@@ -293,10 +299,10 @@ def word_columns(lens: np.ndarray, K: int, seqs: np.ndarray = None, band: bool =
     With ``seqs`` the common prefix of every pair, rounded down to a multiple of
     four symbols, is left out (nothing at all if one prefix contains the other):
     the multi-word kernels never run those rows and columns.  With ``band`` a pair
-    also counts no more than the units inside the band that its mismatch count
-    implies (differing positions after the common prefix + length difference is an
-    upper bound of the distance; an optimal alignment stays within the diagonals
-    that bound allows), again in the cheaper orientation."""
+    also counts no more than the units inside the band that its bounds imply, again in the
+    cheaper orientation: differing positions + length difference from above; from below the
+    text columns whose symbol the pattern lacks, plus the length difference where the pattern
+    is the longer one.  A pair whose bounds meet counts nothing."""
     m = np.minimum(np.maximum(lens.astype(np.int64), 0), K)
     total = 0
     N = lens.shape[1]
@@ -318,8 +324,12 @@ def word_columns(lens: np.ndarray, K: int, seqs: np.ndarray = None, band: bool =
                 mism = ((seqs[:, i, :] != seqs[:, j, :]) & (pos < lo.reshape(-1, 1))).sum(axis=1)
                 ub = mism + np.abs(a - b)
                 live = (ra > 0) & (rb > 0)
-                banded = np.minimum(_band_units(np.where(live, ra, 0), np.where(live, rb, 0), ub),
-                                    _band_units(np.where(live, rb, 0), np.where(live, ra, 0), ub))
+                za, zb, gap = np.where(live, ra, 0), np.where(live, rb, 0), np.abs(a - b)
+                at = np.where(live, first, 0)
+                ab = _absent(seqs[:, i], a, seqs[:, j], b, at)
+                ba = _absent(seqs[:, j], b, seqs[:, i], a, at)
+                banded = np.minimum(_band_units(za, zb, np.where(a >= b, a - b + ab, np.maximum(gap, ab)), ub),
+                                    _band_units(zb, za, np.where(b >= a, b - a + ba, np.maximum(gap, ba)), ub))
                 units = np.where(live, np.minimum(units, banded), units)
             total += int(units.sum())
     return total
