@@ -65,6 +65,23 @@ class ClockSampler:
         except OSError:
             self.proc = None
 
+    def samples(self):
+        """Lines written so far (0 when there is no nvidia-smi)."""
+        try:
+            with open(self.path) as f:
+                return sum(1 for _ in f)
+        except (OSError, TypeError):
+            return 0
+
+    def hold(self, fn, upto, seconds=3.0):
+        """Keeps the GPU under fn's load until there are `upto` samples: the timed steps last a few
+        milliseconds, nvidia-smi takes longer to start."""
+        end = time.monotonic() + seconds
+        while self.proc is not None and self.samples() < upto and time.monotonic() < end:
+            for _ in range(20):
+                fn()
+            torch_synchronize()
+
     def stop(self):
         out = {"sm_mhz": None, "sm_max_mhz": None, "reasons": [], "samples": 0}
         if self.proc is None:
@@ -94,6 +111,11 @@ class ClockSampler:
             out.update(sm_mhz=statistics.median(sm), sm_max_mhz=max(mx), reasons=sorted(reasons),
                        samples=len(sm))
         return out
+
+
+def torch_synchronize():
+    import torch
+    torch.cuda.synchronize()
 
 
 def traffic_from_profiles(kernel: str, source_file: str):
@@ -259,6 +281,7 @@ def main():
     sampler = ClockSampler(local)
     if rank == 0:
         sampler.start()
+        sampler.hold(step, 1)
     for _ in range(max(args.warmup, 3)):
         step()
     barrier()
@@ -289,7 +312,10 @@ def main():
         sr.sr_gate_stages(seqs, lens, K, w.threshold, w.norm_mode, pair_sum=ps, mean=mean, stop=stop,
                           workspace=ws, events=e5)
     torch.cuda.synchronize()
-    clocks = sampler.stop() if rank == 0 else None
+    clocks = None
+    if rank == 0:
+        sampler.hold(step, 4, 1.0)
+        clocks = sampler.stop()
     stage_ms = [statistics.median(e5[k].elapsed_time(e5[k + 1]) for e5 in stage_evs) for k in range(4)]
     dp_ms = stage_ms[2]
 
