@@ -34,7 +34,6 @@ namespace {
 constexpr uint32_t kMagic = 0x53524731u;   // "SRG1"
 constexpr int kHistPitch = 32;
 constexpr int kRollThreads = 128;
-constexpr int kAhead = 4;          // pair states in flight per thread
 
 struct IncrLayout {
     size_t off_lens, off_hist, off_pairs, total;
@@ -279,22 +278,36 @@ incr_step_kernel(IncrArgs a) {
     }
 }
 
+// Rollouts of pair e of a CTA, numbered within it, and how many places apart they are in their group.
+__device__ __forceinline__ void pair_at(int e, int N, int P, int kN, uint32_t inv_P, int& gi, int& gj, int& apart) {
+    const int g = kN ? e / P : div20(e, inv_P), pr = kPairs.v[N][e - g * P];
+    gi = g * N + (pr & 0xFF);
+    gj = g * N + (pr >> 8);
+    apart = gj - gi;
+}
+
 // Large batches: one thread per rollout for the match masks, then one per pair for the steps, in a loop.
 // A rollout's stored actions are read once, by one thread, and compared with the new actions
 // of the group's other rollouts (kMasks at a time); the masks go to the pairs through shared memory.  A
 // thread per pair that does its own comparing reads every stored action N - 1 times: the
 // return path of L1 (16 bytes a lane and load) and the indices of its loads were half of that kernel.
-// 30 steps: 65536 groups of 8 792 -> 706 us, 16384 groups of 16 1033 -> 738 us.
-template <int kMasks>
-__global__ void __launch_bounds__(kRollThreads)
+// 30 steps: 65536 groups of 8 792 -> 612 us, 16384 groups of 16 1033 -> 721 us.  (Registers decide: with
+// four pair states in flight the kernel takes 706 us at 60 registers and 884 at 48, where it spills;
+// with one, 656 us at 56, 612 at 48 and 665 at 40.)
+// kN: as above.
+template <int kN, int kMasks>
+__global__ void __launch_bounds__(kRollThreads, kN ? 9 : 8)
 incr_rollout_kernel(IncrArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int N = a.N, P = pairs_of(N), tid = threadIdx.x;
+    const int N = kN ? kN : a.N, P = pairs_of(N), tid = threadIdx.x;
     double* s_term = reinterpret_cast<double*>(smem + a.off_term);      // [gpb][P]
     int32_t* s_dist = reinterpret_cast<int32_t*>(smem + a.off_dist);    // [gpb][P]
     int2* s_roll = reinterpret_cast<int2*>(smem + a.off_roll);          // [gpb * N] length before, action or none
     uint32_t* s_eq = reinterpret_cast<uint32_t*>(smem + a.off_eq);      // [gpb * N][N - 1]
-    const int g = div20(tid, a.inv_N), i = tid - g * N;
+    const int g = kN ? tid / N : div20(tid, a.inv_N), i = tid - g * N;
+    // the thread's first pair: indices and a table, no need to wait for them
+    int gi, gj, ahead;
+    pair_at(tid, N, P, kN, a.inv_P, gi, gj, ahead);
     grid_begin();
     const int g0 = blockIdx.x * a.gpb;
     const int ng = min(a.gpb, a.n_groups - g0);
@@ -309,11 +322,9 @@ incr_rollout_kernel(IncrArgs a) {
     int my_len = 0;
     int32_t my_act = SR_NO_ACTION;
     if (is_roll) { my_len = g_len[tid]; my_act = __ldg(g_new + tid); }
-    // the first pairs' states are on their way while the masks are made
-    uint4 st[kAhead];
-#pragma unroll
-    for (int k = 0; k < kAhead; ++k)
-        if (tid + k * kRollThreads < ng * P) st[k] = g_pairs[tid + k * kRollThreads];
+    // the first pair's state is on its way while the masks are made
+    uint4 st = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < ng * P) st = g_pairs[tid];
     const bool bad = hdr.x != kMagic || hdr.y != (uint32_t)a.n_groups || hdr.z != (uint32_t)N;
     if (bad) {                                     // uniform over the grid: nothing is touched
         if (tid == 0 && a.status) atomicOr(a.status, SR_STATUS_BAD_STATE);
@@ -339,7 +350,7 @@ incr_rollout_kernel(IncrArgs a) {
             uint32_t eq[kMasks];
 #pragma unroll
             for (int k = 0; k < kMasks; ++k) {
-                int j = i + 1 + min(d0 + k, N - 2);
+                int j = i + 1 + (kN ? k : min(d0 + k, N - 2));
                 if (j >= N) j -= N;
                 y[k] = __ldg(g_new + g * N + j);
                 eq[k] = 0u;
@@ -363,7 +374,7 @@ incr_rollout_kernel(IncrArgs a) {
             }
 #pragma unroll
             for (int k = 0; k < kMasks; ++k)
-                if (d0 + k < N - 1) eq_out[d0 + k] = eq[k];
+                if (kN || d0 + k < N - 1) eq_out[d0 + k] = eq[k];
         }
         // nobody else reads this rollout's stored actions or length
         if (my_act != SR_NO_ACTION) {
@@ -372,21 +383,22 @@ incr_rollout_kernel(IncrArgs a) {
         }
     }
     __syncthreads();
-    auto pair = [&](int e, const uint4& state) {
-        const int pg = div20(e, a.inv_P), pr = kPairs.v[N][e - pg * P];
-        const int ri = pr & 0xFF, rj = pr >> 8, gi = pg * N + ri, gj = pg * N + rj;
+    auto pair = [&](int e, uint4 state) {
         const int2 A = s_roll[gi], B = s_roll[gj];
         int m = A.x, n = B.x;
-        const uint32_t eq_y = s_eq[gi * (N - 1) + (rj - ri - 1)], eq_x = s_eq[gj * (N - 1) + (ri - rj + N - 1)];
+        const uint32_t eq_y = s_eq[gi * (N - 1) + ahead - 1], eq_x = s_eq[gj * (N - 1) + N - 1 - ahead];
         const int d = step_pair(state, A.y != SR_NO_ACTION, B.y != SR_NO_ACTION, A.y, B.y, eq_x, eq_y, m, n, g_pairs + e);
         if (a.pair_sum) s_dist[e] = d;
         s_term[e] = a.norm_mode == SR_NORM_NONE ? (double)d : kQuot.v[d * 33 + max(m, n)];
         if (a.pair_dist) a.pair_dist[(size_t)g0 * P + e] = d;
     };
-#pragma unroll
-    for (int k = 0; k < kAhead; ++k)
-        if (tid + k * kRollThreads < ng * P) pair(tid + k * kRollThreads, st[k]);
-    for (int e = tid + kAhead * kRollThreads; e < ng * P; e += kRollThreads) pair(e, g_pairs[e]);
+    if (tid < ng * P) pair(tid, st);
+#pragma unroll 2
+    for (int e = tid + kRollThreads; e < ng * P; e += kRollThreads) {
+        st = g_pairs[e];
+        pair_at(e, N, P, kN, a.inv_P, gi, gj, ahead);
+        pair(e, st);
+    }
     __syncthreads();
     if (tid < ng) {
         GateArgs out{};
@@ -435,14 +447,15 @@ int launch_incr_step(void* state, size_t bytes, const int32_t* new_actions, int3
     int off = 0;
     auto take = [&](int b) { int o = off; off = (off + b + 15) & ~15; return o; };
     // the thread-per-rollout form has the longer chain per thread and pays off once several CTAs of it
-    // share every SM (N = 8: even at 25000 groups; N = 16: at 6000)
-    if ((long long)n_groups * P >= 700000) {
+    // share every SM (N = 8: from 20000 groups on; N = 16: from about 5000)
+    if ((long long)n_groups * P >= 550000) {
         a.gpb = kRollThreads / N;
         a.off_dist = take(pair_sum ? a.gpb * P * 4 : 0);
         a.off_term = take(a.gpb * P * 8);
         a.off_roll = take(a.gpb * N * 8);
         a.off_eq = take(a.gpb * N * (N - 1) * 4);
-        auto kernel = N <= 5 ? incr_rollout_kernel<4> : (N <= 8 ? incr_rollout_kernel<7> : incr_rollout_kernel<8>);
+        auto kernel = N == 8 ? incr_rollout_kernel<8, 7> : (N <= 5 ? incr_rollout_kernel<0, 4>
+                                  : (N <= 8 ? incr_rollout_kernel<0, 7> : incr_rollout_kernel<0, 8>));
         SR_LAUNCH("incr_rollout_kernel", kernel, (n_groups + a.gpb - 1) / a.gpb, kRollThreads, off, s, a);
         return SR_OK;
     }

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("N,max_steps", [(4, 9), (5, 6), (8, 32), (9, 5), (17, 5), (32, 4)])
 def test_large_batches(N, max_steps):
     P = N * (N - 1) // 2
-    G = 700000 // P + 5
+    G = 550000 // P + 5
     rng = np.random.default_rng(N)
     steps = max_steps + 1                                    # the last action finds full rollouts
     vocab = rng.choice([3, 40, 4096], size=(G, 1))
