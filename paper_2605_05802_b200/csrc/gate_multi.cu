@@ -5,10 +5,12 @@
 // block keeps its +1 / -1 vertical deltas in two 32-bit words and is advanced one
 // text column at a time by the bit-vector recurrence, with the horizontal delta
 // leaving a block entering the block below.  The work is organised as a pipeline
-// of four launches on the caller's stream, sharing a caller-provided workspace:
+// of launches on the caller's stream, sharing a caller-provided workspace:
 //
-//   prep     one CTA per (group, pattern rollout): hashes the pattern's symbols
-//            in shared memory, then translates every text paired with it into a
+//   names    one CTA per group: gives every symbol a 16-bit name, the position of one of its
+//            holders.
+//   prep     one CTA per (group, pattern rollout): an array over the names holds the
+//            pattern's positions, and every text paired with it is translated into a
 //            "loc" stream: for text column c the position of the column's symbol in
 //            the pattern (0x7FFF: absent).  A block's match word is then just
 //            1 << (loc - first_row_of_block), no table lookup.  A symbol with several
@@ -715,9 +717,7 @@ __device__ __forceinline__ uint32_t shl_clamp(uint32_t v, uint32_t s) {
 // Brings `bytes` bytes to L1, 32 a time, `lanes` lanes together.  (Not inlined: it is run once a task.)
 __device__ __noinline__ void touch(const void* from, int bytes, int lane, int lanes) {
     for (int o = 32 * lane; o < bytes; o += 32 * lanes) {
-        uint32_t x;
-        asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(x) : "l"(static_cast<const char*>(from) + o));
-        (void)x;
+        asm volatile("{ .reg .u32 x; ld.global.nc.u32 x, [%0]; }" ::"l"(static_cast<const char*>(from) + o));
     }
 }
 
