@@ -215,10 +215,17 @@ size_t sr_gate_host_packed_arena_bytes(int32_t n_groups, int32_t N, int32_t stri
  * the CUDA runtime reserves the array when it loads the image on a device, which with
  * its default lazy loading happens inside the first call there.
  *
- *   - Limit: sr_gate_workspace_bytes(n_groups, N, stride, K) must not exceed
- *     SR_NOALLOC_SCRATCH_BYTES (also returned by sr_gate_noalloc_limit_bytes());
- *     otherwise SR_ERR_SCRATCH_LIMIT, nothing enqueued.  As a guide, 64 groups of
- *     N = 8 at K = 1024, or 1000 groups at K = 64, fit.  K <= 32 has no limit.
+ *   - Limit: with P = N(N-1)/2 and K' = K rounded up to a multiple of 8,
+ *         16640 + n_groups * (1 + 24 P + 2 K' (N + P))
+ *     bytes (the group flags, distances, order, descriptors, K' N and K' P terms each
+ *     rounded up to 256) must not exceed SR_NOALLOC_SCRATCH_BYTES (also returned by
+ *     sr_gate_noalloc_limit_bytes()); otherwise SR_ERR_SCRATCH_LIMIT, nothing enqueued.
+ *     At K = 1024 that is 225 groups of N = 8, 812 of N = 4 or 2716 of N = 2; at K = 64, 3173
+ *     groups of N = 8.  K <= 32 has no limit.
+ *   - The workspace of sr_gate is larger than that (up to about four times), most of it
+ *     match words of symbols that occur several times.  A batch that does not fit with a
+ *     quarter of them (more than 141 groups of N = 8 at K = 1024) runs as two or three parts,
+ *     one after the other on the stream.
  *   - The first call on each device (with K > 32) looks up the array's device address
  *     (a cudaGetSymbolAddress with that device current), which is also when the 16 MiB
  *     are reserved.  Make that first call during set-up, before any stream capture is

@@ -73,7 +73,7 @@ const char* sr_last_cuda_error(void) { return g_cuda_error; }
 size_t sr_gate_workspace_bytes(int32_t n_groups, int32_t N, int32_t stride, int32_t K) {
     if (n_groups < 0 || N < 2 || N > SR_MAX_N || K < 0 || K > stride || K > SR_MAX_K) return 0;
     if (K <= 32) return 0;
-    return gate_multi_workspace_bytes(n_groups, N, stride, K);
+    return gate_multi_workspace_bytes(n_groups, N, K);
 }
 
 int sr_gate(const int32_t* seqs, const int32_t* lens, int32_t n_groups, int32_t N, int32_t stride,
@@ -87,7 +87,7 @@ int sr_gate(const int32_t* seqs, const int32_t* lens, int32_t n_groups, int32_t 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (K <= 32) return launch_gate_single(a, s);
     if (n_groups > 0) {
-        const size_t need = gate_multi_workspace_bytes(n_groups, N, stride, K);
+        const size_t need = gate_multi_workspace_bytes(n_groups, N, K);
         if (workspace == nullptr || workspace_bytes < need ||
             (reinterpret_cast<uintptr_t>(workspace) & 255) != 0)
             return SR_ERR_WORKSPACE;
@@ -109,7 +109,7 @@ int sr_gate_decide(const int32_t* seqs, const int32_t* lens, int32_t n_groups, i
         if (exact && n_groups > 0) SR_CUDA_TRY(cudaMemsetAsync(exact, 1, (size_t)n_groups, s));
         return K <= 32 ? launch_gate_single(a, s) : SR_OK;
     }
-    const size_t need = gate_multi_workspace_bytes(n_groups, N, stride, K);
+    const size_t need = gate_multi_workspace_bytes(n_groups, N, K);
     if (workspace == nullptr || workspace_bytes < need ||
         (reinterpret_cast<uintptr_t>(workspace) & 255) != 0)
         return SR_ERR_WORKSPACE;
@@ -138,7 +138,7 @@ int sr_gate_stages(const int32_t* seqs, const int32_t* lens, int32_t n_groups, i
         for (int k = 1; k < 5; ++k) SR_CUDA_TRY(cudaEventRecord(ev[k], s));
         return SR_OK;
     }
-    const size_t need = gate_multi_workspace_bytes(n_groups, N, stride, K);
+    const size_t need = gate_multi_workspace_bytes(n_groups, N, K);
     if (workspace == nullptr || workspace_bytes < need ||
         (reinterpret_cast<uintptr_t>(workspace) & 255) != 0)
         return SR_ERR_WORKSPACE;

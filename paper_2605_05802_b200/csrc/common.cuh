@@ -205,7 +205,8 @@ HostArena host_arena(int32_t n_groups, int32_t N, int32_t stride, int32_t K);
 // gate_single.cu: prefixes of at most 32 symbols, one 32-bit word per pair.
 int launch_gate_single(const GateArgs& a, cudaStream_t s);
 // gate_multi.cu: prefixes of up to SR_MAX_K symbols, blocked multi-word.
-size_t gate_multi_workspace_bytes(int32_t n_groups, int32_t N, int32_t stride, int32_t K);
+// `row_cap`: mask rows per pattern, at least 1 and at most (K + 7) / 8, which 0 stands for.
+size_t gate_multi_workspace_bytes(int32_t n_groups, int32_t N, int32_t K, int row_cap = 0);
 // `ev`: NULL, or 5 events recorded before prep / after prep / after scan+scatter /
 // after dp / after finish.
 // `decide`: finish groups whose lower-bounded d_K already reaches the threshold without
@@ -220,7 +221,7 @@ struct GroupFeed {
 };
 int launch_gate_multi(const GateArgs& a, void* ws, size_t ws_bytes, cudaStream_t s,
                       const cudaEvent_t* ev = nullptr, bool decide = false, uint8_t* exact = nullptr,
-                      const GroupFeed* feed = nullptr);
+                      const GroupFeed* feed = nullptr, int row_cap = 0);
 // incremental.cu
 size_t incr_state_bytes(int32_t n_groups, int32_t N, int32_t max_steps);
 int launch_incr_init(void* state, size_t bytes, int32_t n_groups, int32_t N, int32_t max_steps,

@@ -69,7 +69,7 @@ static_assert(kNumBins <= (int)kBinMask + 1 && kTimeBuckets * kNumClasses <= kNu
 
 struct PairDesc {          // 16 bytes
     uint32_t mn;           // m | n << 16
-    uint32_t pat_row;      // g * N + pattern rollout
+    uint32_t pat_row;      // g * patterns + pattern rollout
     uint32_t bin;          // bits 0..10 bin index; bits 12..21 stripped common prefix (symbols,
                            // a multiple of 4); bits 22..29 mask rows of the pattern; bit 30 = the
                            // pattern has chains; bit 31 = pair needs the dp kernel
@@ -94,14 +94,20 @@ struct MultiWs {
     size_t off_dist, off_desc, off_loc, off_next, off_order, off_ctl, off_flag, off_rows, off_names, total;
     int pitch;             // uint16 elements per loc / chain row
     int row_words;         // 32-bit words of a mask row: one per 32 pattern positions
+    int patterns;          // rollouts of a group that serve as patterns
     int row_cap;           // mask rows a pattern may have
     int warps;             // warps the dp kernel keeps resident
 };
 
-MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K) {
+// Mask rows for an eighth of the positions: symbols with at least eight occurrences always
+// fit, and 1/rank token frequencies put no more than about K / 10 symbols above one.
+int full_row_cap(int32_t K) { return (K + 7) >> 3; }
+
+MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K, int row_cap) {
     MultiWs w;
     const size_t P = pairs_of(N);
     w.pitch = (K + 7) & ~7;
+    w.patterns = N & 1 ? N : N - 1;       // the last rollout of an even group is never a pattern
     w.warps = 1;
     size_t off = 0;
     w.off_ctl = off;   off = align_up(off + sizeof(Ctl), 256);
@@ -109,15 +115,13 @@ MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K) {
     w.off_dist = off;  off = align_up(off + (size_t)n_groups * P * 4, 256);
     w.off_desc = off;  off = align_up(off + (size_t)n_groups * P * sizeof(PairDesc), 256);
     w.off_order = off; off = align_up(off + (size_t)n_groups * P * 4, 256);
-    w.off_next = off;  off = align_up(off + (size_t)n_groups * N * w.pitch * 2, 256);
+    w.off_next = off;  off = align_up(off + (size_t)n_groups * w.patterns * w.pitch * 2, 256);
     w.off_loc = off;   off = align_up(off + (size_t)n_groups * P * w.pitch * 2, 256);
-    // Mask rows for an eighth of the positions: symbols with at least eight occurrences always
-    // fit, and 1/rank token frequencies put no more than about K / 10 symbols above one.  A team's
-    // lanes cover up to fifteen words more than the pattern has: slack after the last row.
+    // a team's lanes cover up to 31 words more than the pattern has: slack after the last row
     w.row_words = (K + 3 + 31) >> 5;      // the pattern and what pads its texts to whole quads
-    w.row_cap = (K + 7) >> 3;
+    w.row_cap = row_cap;
     w.off_rows = off;
-    off = align_up(off + (size_t)n_groups * N * w.row_cap * w.row_words * 4 + 256, 256);
+    off = align_up(off + (size_t)n_groups * w.patterns * w.row_cap * w.row_words * 4 + 256, 256);
     w.off_names = off;
     off = align_up(off + (size_t)n_groups * N * w.pitch * 2, 256);
     w.total = off;
@@ -329,7 +333,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
 
     const int N = a.N, K = a.K, P = pairs_of(N);
     const int tid = threadIdx.x, lane = tid & 31;
-    const int M = (N & 1) ? N : N - 1;                // the last rollout of an even group is never a pattern
+    const int M = W.patterns;
     const int g = g_base + blockIdx.x / M, i = blockIdx.x % M;
     if (tid < 4) s_repeats[tid] = 0;
     for (int e = tid; 8 * e < N * W.pitch; e += kPrepThreads)
@@ -417,8 +421,9 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         // one per 32 positions, which the recurrence reads in place of its one-hot word.  (Walking
         // a chain of occurrences per column made the recurrence wait for the longest chain of the
         // warp: 16 groups of 8 such texts of up to 1024 tokens took 2.2 ms, with the rows 0.16 ms.)
-        // The pool has room for every symbol with at least eight occurrences; what does not fit
-        // (the rarest of the repeated ones) is left as a chain of at most seven positions.
+        // The full pool has room for every symbol with at least eight occurrences; what does not fit
+        // (the rarest of the repeated ones) is left as a chain of at most seven positions.  In a
+        // smaller pool (see launch_gate_multi) the last symbols to ask get a chain of any length.
         // From here on the lower half of s_info[claimant] is the symbol's stream entry, the upper half
         // the head of the chain of its further positions.
         // (only claimants of repeated symbols have a count)
@@ -439,15 +444,19 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if (more[k] == 0u) continue;
-                const uint32_t code = more[k] >= need ? kLocRow | (uint32_t)atomicAdd(&s_repeats[3], 1)
-                                                      : (kChainEnd << 16) | kLocChain | (uint32_t)(p0 + k);
+                uint32_t code = (kChainEnd << 16) | kLocChain | (uint32_t)(p0 + k);
+                if (more[k] >= need) {
+                    const int row = atomicAdd(&s_repeats[3], 1);
+                    if (row < W.row_cap) code = kLocRow | (uint32_t)row;
+                }
                 s_map[my_name[k]] = (uint16_t)code;             // what the streams of the texts say
                 s_info[p0 + k] = code;
             }
         }
         __syncthreads();
-        uint32_t* rows = reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * N + i) * W.row_cap * W.row_words;
-        for (int e = tid; e < s_repeats[3] * W.row_words; e += kPrepThreads) rows[e] = 0u;
+        uint32_t* rows = reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * M + i) * W.row_cap * W.row_words;
+        const int n_rows = min(s_repeats[3], W.row_cap);
+        for (int e = tid; e < n_rows * W.row_words; e += kPrepThreads) rows[e] = 0u;
         __syncthreads();
         if (claims || repeated) {
 #pragma unroll
@@ -461,9 +470,9 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                 }
             }
         }
-        if (s_repeats[0] > s_repeats[3]) {             // some chains: leave them for the recurrence
+        if (s_repeats[0] > n_rows) {                   // some chains: leave them for the recurrence
             __syncthreads();
-            uint16_t* g_next = reinterpret_cast<uint16_t*>(ws + W.off_next) + ((size_t)g * N + i) * W.pitch;
+            uint16_t* g_next = reinterpret_cast<uint16_t*>(ws + W.off_next) + ((size_t)g * M + i) * W.pitch;
             for (int p = tid; p < m; p += kPrepThreads) g_next[p] = (uint16_t)(s_info[p] >> 16);
         }
     }
@@ -536,9 +545,10 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             lower = m >= n ? m - n + absent : max(n - m, absent);
             upper += (int)(s_count[tid] & 0xFFFFu);
         }
-        PairDesc d{(uint32_t)m | ((uint32_t)n << 16), (uint32_t)(g * N + i), 0u, (uint32_t)lower | ((uint32_t)upper << 16)};
+        PairDesc d{(uint32_t)m | ((uint32_t)n << 16), (uint32_t)(g * M + i), 0u, (uint32_t)lower | ((uint32_t)upper << 16)};
         if (lower < upper) {                          // otherwise that is the distance
-            d.bin = ((uint32_t)strip << kStripShift) | ((uint32_t)min(s_repeats[3], 255) << kRowsShift) | kNeedsDp | (s_repeats[0] > s_repeats[3] ? kHasChains : 0u);
+            const int n_rows = min(s_repeats[3], W.row_cap);
+            d.bin = ((uint32_t)strip << kStripShift) | ((uint32_t)n_rows << kRowsShift) | kNeedsDp | (s_repeats[0] > n_rows ? kHasChains : 0u);
             const PairSize z = size_of_desc(d);
             work = work_of_pair(z.m, z.n, z.lb, z.ub);
         }
@@ -1148,15 +1158,14 @@ int allow_smem() {
 
 }  // namespace
 
-size_t gate_multi_workspace_bytes(int32_t n_groups, int32_t N, int32_t stride, int32_t K) {
-    (void)stride;
-    return multi_layout(n_groups, N, K).total;
+size_t gate_multi_workspace_bytes(int32_t n_groups, int32_t N, int32_t K, int row_cap) {
+    return multi_layout(n_groups, N, K, row_cap > 0 ? row_cap : full_row_cap(K)).total;
 }
 
 int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_t s,
-                      const cudaEvent_t* ev, bool decide, uint8_t* exact, const GroupFeed* feed) {
+                      const cudaEvent_t* ev, bool decide, uint8_t* exact, const GroupFeed* feed, int row_cap) {
     if (a.n_groups == 0) return SR_OK;
-    MultiWs W = multi_layout(a.n_groups, a.N, a.K);
+    MultiWs W = multi_layout(a.n_groups, a.N, a.K, row_cap > 0 ? row_cap : full_row_cap(a.K));
     if (ws_ == nullptr || ws_bytes < W.total || (reinterpret_cast<uintptr_t>(ws_) & 255) != 0)
         return SR_ERR_WORKSPACE;
     unsigned char* ws = static_cast<unsigned char*>(ws_);
@@ -1174,7 +1183,6 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     int32_t* dist = a.pair_dist ? a.pair_dist : reinterpret_cast<int32_t*>(ws + W.off_dist);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
 
-    const int patterns = (a.N & 1) ? a.N : a.N - 1;
     const int prep_smem = W.pitch * 4 + a.N * W.pitch * 2;
     // names: at least two slots to a symbol while symbols and table fit
     const int sym_bytes = a.N * W.pitch * 4, names_threads = a.N * W.pitch > 4 * 8 * 512 ? 1024 : 512;
@@ -1206,9 +1214,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
         }
         SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0);
         if (decide)
-            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<true>, (g1 - g0) * patterns, kPrepThreads, prep_smem, s, a, ws, W, dist, g0);
+            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<true>, (g1 - g0) * W.patterns, kPrepThreads, prep_smem, s, a, ws, W, dist, g0);
         else
-            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<false>, (g1 - g0) * patterns, kPrepThreads, prep_smem, s, a, ws, W, dist, g0);
+            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<false>, (g1 - g0) * W.patterns, kPrepThreads, prep_smem, s, a, ws, W, dist, g0);
     }
     const int gpb = P <= kGroupThreads ? kGroupThreads / P : 1;
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);

@@ -45,6 +45,34 @@ int scratch_address(void** out) {
     return SR_OK;
 }
 
+// The limit (see sr_gate.h): what a batch keeps per pair and per match stream, one array after
+// the other.  It stays as it is whatever the pipeline itself lays out.
+size_t scratch_demand(int32_t n_groups, int32_t N, int32_t K) {
+    const size_t G = n_groups, P = pairs_of(N), row = 2 * (size_t)((K + 7) & ~7);
+    return 16640 + align_up(G, 256) + 2 * align_up(4 * G * P, 256) + align_up(16 * G * P, 256) +
+           align_up(G * N * row, 256) + align_up(G * P * row, 256);
+}
+
+// A batch whose workspace exceeds the array runs in parts, one after the other.  Before it is cut once
+// more its patterns make do with fewer mask rows, down to a quarter of the full number: at K = 1024
+// 32 rows, which hold the symbols that occur four times or more in text with 1/rank frequencies.
+struct Parts {
+    int32_t groups, row_cap;
+};
+Parts parts_of(int32_t n_groups, int32_t N, int32_t K) {
+    const int full = (K + 7) >> 3, least = (full + 3) >> 2;
+    int parts = 1;
+    Parts p;
+    do {
+        p.groups = (int32_t)(((long long)n_groups + parts - 1) / parts);
+        ++parts;
+    } while (p.groups > 1 && gate_multi_workspace_bytes(p.groups, N, K, least) > SR_NOALLOC_SCRATCH_BYTES);
+    p.row_cap = full;
+    while (p.row_cap > least && gate_multi_workspace_bytes(p.groups, N, K, p.row_cap) > SR_NOALLOC_SCRATCH_BYTES)
+        --p.row_cap;
+    return p;
+}
+
 }  // namespace
 }  // namespace sr
 
@@ -59,15 +87,23 @@ extern "C" int sr_gate_noalloc(const int32_t* seqs, const int32_t* lens, int32_t
     if (K <= 32 || n_groups == 0)      // the single-word path needs no scratch at all
         return sr_gate(seqs, lens, n_groups, N, stride, K, threshold, norm_mode, pair_dist, pair_sum,
                        mean, stop, status, nullptr, 0, stream);
-    const size_t need = sr_gate_workspace_bytes(n_groups, N, stride, K);
-    if (need > (size_t)SR_NOALLOC_SCRATCH_BYTES) return SR_ERR_SCRATCH_LIMIT;
+    if (scratch_demand(n_groups, N, K) > SR_NOALLOC_SCRATCH_BYTES) return SR_ERR_SCRATCH_LIMIT;
+    const Parts parts = parts_of(n_groups, N, K);
     void* scratch = nullptr;
-    const int rc = scratch_address(&scratch);
-    if (rc != SR_OK) return rc;
-    // the pipeline clears the part of the scratch that must start at zero (its bin
-    // counters) at the head of every call; everything else is written before it is read
-    return sr_gate(seqs, lens, n_groups, N, stride, K, threshold, norm_mode, pair_dist, pair_sum,
-                   mean, stop, status, scratch, SR_NOALLOC_SCRATCH_BYTES, stream);
+    int rc = scratch_address(&scratch);
+    const size_t P = pairs_of(N);
+    for (int32_t g0 = 0; rc == SR_OK && g0 < n_groups; g0 += parts.groups) {
+        const int32_t ng = n_groups - g0 < parts.groups ? n_groups - g0 : parts.groups;
+        const size_t row0 = (size_t)g0 * N;
+        const GateArgs a{seqs + row0 * stride, lens ? lens + row0 : nullptr, ng, N, stride, K, threshold, norm_mode,
+                         pair_dist ? pair_dist + g0 * P : nullptr, pair_sum ? pair_sum + g0 : nullptr,
+                         mean ? mean + g0 : nullptr, stop + g0, status};
+        // the pipeline clears the part of the scratch that must start at zero (its bin counters)
+        // at the head of every call; everything else is written before it is read
+        rc = launch_gate_multi(a, scratch, SR_NOALLOC_SCRATCH_BYTES, static_cast<cudaStream_t>(stream), nullptr, false,
+                               nullptr, nullptr, parts.row_cap);
+    }
+    return rc;
 }
 
 extern "C" size_t sr_gate_noalloc_limit_bytes(void) { return (size_t)SR_NOALLOC_SCRATCH_BYTES; }

@@ -78,6 +78,73 @@ def test_noalloc_matches_sr_gate_on_consecutive_calls():
         assert np.array_equal(a.view(np.uint8), b.view(np.uint8))
 
 
+_LIMITS = """
+import sys
+sys.path.insert(0, {root!r})
+from paper_2605_05802_b200 import binding
+lib = binding.load()
+up = lambda x: -(-x // 256) * 256
+def demand(G, N, K):                       # as sr_gate.h states it
+    P, k = N * (N - 1) // 2, -(-K // 8) * 8
+    return 16640 + up(G) + 2 * up(4 * G * P) + up(16 * G * P) + up(2 * k * G * N) + up(2 * k * G * P)
+largest = dict()
+for N in (2, 3, 4, 8, 16, 31, 32):
+    for K in (33, 64, 500, 1024):
+        G = 1
+        while demand(2 * G, N, K) <= 16 << 20: G *= 2
+        step = G
+        while step:
+            if demand(G + step, N, K) <= 16 << 20: G += step
+            step //= 2
+        largest[N, K] = G
+        call = lambda G: lib.sr_gate_noalloc(1 << 20, None, G, N, 1024, K, 0.12, 0, None, None, None, 1 << 20, None, None)
+        # no device here: a batch that passes the checks fails at its first CUDA call
+        assert call(G) == binding.SR_ERR_CUDA, (G, N, K)
+        assert call(G + 1) == binding.SR_ERR_SCRATCH_LIMIT, (G, N, K)
+assert (largest[8, 1024], largest[4, 1024], largest[2, 1024], largest[8, 64]) == (225, 812, 2716, 3173), largest
+print("limits ok")
+"""
+
+
+def test_noalloc_takes_every_batch_up_to_its_limit():
+    """The limit is a formula of its own: it does not move with the gate's workspace."""
+    build.build()
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", _LIMITS.format(root=root)], capture_output=True, text=True, timeout=600,
+                         env={**os.environ, "CUDA_VISIBLE_DEVICES": ""})
+    assert out.returncode == 0 and "limits ok" in out.stdout, out.stdout + out.stderr
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("G,N,K", [(142, 8, 1024), (225, 8, 1024), (81, 8, 1023), (2716, 2, 1024), (812, 4, 1024), (877, 8, 256)])
+@pytest.mark.parametrize("tokens", ["uniform", "text", "many repeats"])
+def test_noalloc_in_parts_and_with_fewer_mask_rows(G, N, K, tokens):
+    """Batches near the limit: more than one part, patterns with fewer mask rows than symbols
+    that ask for one ("many repeats": 60 symbols, a dozen or more occurrences each)."""
+    rng = np.random.default_rng(G + len(tokens))
+    stride = (K + 3) // 4 * 4
+    if tokens == "uniform":
+        draw = lambda *shape: rng.integers(0, 150000, size=shape)
+    elif tokens == "text":
+        draw = lambda *shape: np.exp(rng.random(shape) * np.log(150000)) - 1
+    else:
+        draw = lambda *shape: rng.integers(0, 60, size=shape)
+    seqs = draw(G, N, stride).astype(np.int32)
+    alike = rng.random((G, 1, 1)) < 0.5
+    seqs = np.where(alike & (rng.random((G, N, stride)) < 0.9), seqs[:, :1], seqs)
+    lens = rng.integers(K // 2, K + 1, size=(G, N)).astype(np.int32)
+    lens[::5] = K
+    w = W.token_gate(seed=1, n_groups=2, min_len=40, max_len=64)       # for the fields `_run` reads
+    w.seqs, w.lens, w.K = np.ascontiguousarray(seqs), lens, K
+    ws = torch.empty(sr.sr_gate_workspace_bytes(G, N, stride, K), dtype=torch.uint8, device="cuda:0")
+    got, want = _run(sr.sr_gate_noalloc, w, 0.3), _run(sr.sr_gate, w, 0.3, workspace=ws)
+    for a, b in zip(got, want):
+        assert np.array_equal(a.view(np.uint8), b.view(np.uint8))
+    some = np.unique(np.concatenate([rng.integers(0, G, 6), [0, G // 2, G - 1]]))
+    for a, b in zip(got, oracle.gate(seqs[some], lens[some], K, 0.3, w.norm_mode, threads=8)):
+        assert np.array_equal(a[some].view(np.uint8), b.view(np.uint8))
+
+
 _FIRST_CALL = """
 import sys
 sys.path.insert(0, {root!r})
