@@ -24,6 +24,8 @@
 // in the recurrence.  Measured against one-look-up-more tables (64-bit compare-and-swap slots, a
 // byte map per rollout and slot) for K > 16 and direct comparison for K <= 16: 4096 groups of 16, K = 30:
 // 33.7 -> 23 us; 16384 groups of 8, K = 30: 51 -> 31 us; 65536 groups of 8, K = 15, ragged: 64 -> 44 us.
+#include <atomic>
+
 #include "common.cuh"
 
 namespace sr {
@@ -363,6 +365,23 @@ gate_named_kernel(GateArgs a, NamedLayout L, uint32_t two) {
     }
 }
 
+// Only a CTA's group takes more than 48 KB of shared memory, at most 80000 bytes (32 rollouts, K = 32).
+// It has to be asked for: the most that any call takes, for all widths of the kernel, once per
+// device (noted, because asking is host time).  Never less than that, or a thread with a smaller
+// call would take back what another one has just been granted.
+constexpr int kMostSmem = 80000;
+int allow_smem() {
+    static std::atomic<bool> allowed[64];
+    int dev = 0;
+    SR_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev >= 0 && dev < 64 && allowed[dev].load(std::memory_order_relaxed)) return SR_OK;
+    SR_CUDA_TRY(cudaFuncSetAttribute(gate_named_kernel<false, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem));
+    SR_CUDA_TRY(cudaFuncSetAttribute(gate_named_kernel<false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem));
+    SR_CUDA_TRY(cudaFuncSetAttribute(gate_named_kernel<false, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem));
+    if (dev >= 0 && dev < 64) allowed[dev].store(true, std::memory_order_relaxed);
+    return SR_OK;
+}
+
 template <bool kPacked, bool kWarp>
 int launch_gate_named(const GateArgs& a, cudaStream_t s) {
     constexpr bool kAlloc = !kWarp;
@@ -413,16 +432,8 @@ int launch_gate_named(const GateArgs& a, cudaStream_t s) {
                 : items_per_thread == 2 ? gate_named_kernel<kPacked, kWarp, 2>
                                         : gate_named_kernel<kPacked, kWarp, 4>;
     if (smem > 48 * 1024) {
-        // per-device note of what each kernel was already allowed: the opt-in call is host
-        // time on a path whose small calls are launch-bound
-        static int granted[3][64] = {};
-        int* most = granted[items_per_thread <= 1 ? 0 : (items_per_thread == 2 ? 1 : 2)];
-        int dev = 0;
-        SR_CUDA_TRY(cudaGetDevice(&dev));
-        if (dev < 0 || dev >= 64 || most[dev] < smem) {
-            SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            if (dev >= 0 && dev < 64) most[dev] = smem;
-        }
+        const int rc = allow_smem();
+        if (rc != SR_OK) return rc;
     }
     return launch("gate_named_kernel", kernel, blocks, threads, smem, s, a, L, 2u);
 }

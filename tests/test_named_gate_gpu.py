@@ -1,6 +1,10 @@
 """Single-word gate through the kernel that names symbols: batches large enough to leave the direct
 comparison, two patterns per word up to K = 15, a warp or a CTA per group above, odd group sizes,
 lengths around quads, symbols that occur once, everywhere, or fight for one slot of the table."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -36,3 +40,34 @@ def test_named_gate(N, K, symbols):
     seqs = seqs.astype(np.int32)
     want = oracle.gate(seqs, np.maximum(lens, 0), K, 0.3, threads=8)
     assert_gate_matches(gate_gpu(seqs, lens, K, 0.3), want, f"N={N} K={K} {symbols}")
+
+
+_THREADS = """
+import sys, threading
+sys.path[:0] = [{root!r}, {root!r} + "/tests"]
+import numpy as np
+import oracle
+from helpers import assert_gate_matches, gate_gpu
+rng = np.random.default_rng(5)
+gate_gpu(rng.integers(0, 9, size=(2, 4, 8)).astype(np.int32), None, 8, 0.3)      # set-up, one thread
+shapes = [(32, 32), (27, 28), (29, 32), (25, 32), (32, 25), (30, 30), (28, 32), (26, 32)]
+inputs = [rng.integers(0, 40, size=(5, N, 32)).astype(np.int32) for N, K in shapes]
+outs, gate = [None] * len(shapes), threading.Barrier(len(shapes))
+def work(k):
+    gate.wait()
+    for _ in range(3): outs[k] = gate_gpu(inputs[k], None, shapes[k][1], 0.3)
+threads = [threading.Thread(target=work, args=(k,)) for k in range(len(shapes))]
+[t.start() for t in threads]; [t.join() for t in threads]
+for (N, K), seqs, got in zip(shapes, inputs, outs):
+    assert got is not None, (N, K)
+    assert_gate_matches(got, oracle.gate(seqs, None, K, 0.3), (N, K))
+print("threads ok")
+"""
+
+
+def test_first_large_calls_of_several_threads():
+    """Shapes that need more than 48 KB of shared memory, called for the first time in a process by
+    several threads at once: none may be refused for what another one has asked for."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", _THREADS.format(root=root)], capture_output=True, text=True, timeout=600)
+    assert out.returncode == 0 and "threads ok" in out.stdout, out.stdout + out.stderr
