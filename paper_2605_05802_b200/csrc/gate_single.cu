@@ -100,10 +100,9 @@ gate_named_kernel(GateArgs a, NamedLayout L, uint32_t two) {
     uint16_t* s_name = reinterpret_cast<uint16_t*>(base + L.off_name);    // [items][4]
     uint16_t* s_row = reinterpret_cast<uint16_t*>(base + L.off_row);      // [items][4]
     uint32_t* s_peq = reinterpret_cast<uint32_t*>(base + L.off_peq);      // [rows][row_words]
-    int32_t* s_len = reinterpret_cast<int32_t*>(base + L.off_len);        // [rollouts], then row counter, ragged
+    int32_t* s_len = reinterpret_cast<int32_t*>(base + L.off_len);        // [rollouts], then the row counter
     uint8_t* s_order = base + L.off_order;                                // [N]
     int& s_rows = s_len[L.groups * N];
-    int& s_ragged = s_len[L.groups * N + 1];
 
     // before the wait: nothing global in here
     if (ng > 0) {
@@ -117,7 +116,7 @@ gate_named_kernel(GateArgs a, NamedLayout L, uint32_t two) {
         } else {
             for (int w = t; w < L.items * L.row_words; w += nthr) reinterpret_cast<uint4*>(s_peq)[w] = make_uint4(0u, 0u, 0u, 0u);
         }
-        if (!kWarp && t == 0) { s_rows = 0; s_ragged = 0; }
+        if (!kWarp && t == 0) s_rows = 0;
     }
     grid_begin();
     if (ng > 0) {
@@ -141,7 +140,6 @@ gate_named_kernel(GateArgs a, NamedLayout L, uint32_t two) {
                 if (q == 0) {
                     if (len < 0 && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
                     s_len[roll[u]] = min(max(len, 0), K);
-                    if (!kWarp && len < K) s_ragged = 1;
                 }
                 live[u] = min(max(min(len, K) - 4 * q, 0), 4);
             }
@@ -248,16 +246,16 @@ gate_named_kernel(GateArgs a, NamedLayout L, uint32_t two) {
             }
         }
         }
-        if (!kWarp && t < N) {
+        if (!kWarp && t < 32) {
             // rollouts by falling length (ties by index), so that the pairs of a warp have texts
             // of similar lengths
+            const int mine = t < N ? s_len[t] : K;
             int rank = t;
-            if (s_ragged) {
-                const int mine = s_len[t];
+            if (__any_sync(0xFFFFFFFFu, mine < K)) {
                 rank = 0;
                 for (int r = 0; r < N; ++r) rank += s_len[r] > mine || (s_len[r] == mine && r < t);
             }
-            s_order[rank] = (uint8_t)t;
+            if (t < N) s_order[rank] = (uint8_t)t;
         }
         unit_sync<kWarp>();
         // ---- every position sets its bit in its rollout's mask and notes the row's place
@@ -411,7 +409,7 @@ int launch_gate_named(const GateArgs& a, cudaStream_t s) {
     L.off_row = take(kAlloc ? L.items * 8 : 0);
     // allocated rows have at least two holders
     L.off_peq = take((kAlloc ? L.groups * (N * a.K / 2) + 1 : 4 * L.items) * L.row_words * 4);
-    L.off_len = take((L.groups * N + 2) * 4);
+    L.off_len = take((L.groups * N + 1) * 4);
     L.off_order = take(N);
     L.unit_bytes = off;
     int threads, units = 1, items_per_thread;
