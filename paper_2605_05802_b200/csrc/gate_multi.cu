@@ -97,6 +97,7 @@ struct MultiWs {
     int patterns;          // rollouts of a group that serve as patterns
     int row_cap;           // mask rows a pattern may have
     int warps;             // warps the dp kernel keeps resident
+    bool alone;            // one CTA orders the batch, and adds up its work itself
 };
 
 // Mask rows for an eighth of the positions: symbols with at least eight occurrences always
@@ -109,6 +110,7 @@ MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K, int row_cap) {
     w.pitch = (K + 7) & ~7;
     w.patterns = N & 1 ? N : N - 1;       // the last rollout of an even group is never a pattern
     w.warps = 1;
+    w.alone = false;
     size_t off = 0;
     w.off_ctl = off;   off = align_up(off + sizeof(Ctl), 256);
     w.off_flag = off;  off = align_up(off + (size_t)n_groups, 256);
@@ -555,7 +557,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         descs[idx] = d;
         if (kDecide || lower == upper) dist_out[idx] = lower;
     }
-    if (!kDecide) {                                   // decide mode counts the pairs it keeps later
+    if (!kDecide && !W.alone) {                       // decide mode counts the pairs it keeps later
         const int open = __popc(__ballot_sync(0xFFFFFFFFu, work > 0));
         work = __reduce_add_sync(0xFFFFFFFFu, work);
         if (tid == 0 && open) {
@@ -1033,7 +1035,7 @@ constexpr int kGroupThreads = 256;
 constexpr int kMaxPairs = SR_MAX_N * (SR_MAX_N - 1) / 2;       // pairs of a CTA: 256, or one group's
 
 __global__ void __launch_bounds__(kGroupThreads)
-multi_bound_kernel(GateArgs a, PairDesc* descs, Ctl* ctl, uint8_t* flag, uint8_t* exact, int gpb) {
+multi_bound_kernel(GateArgs a, PairDesc* descs, Ctl* ctl, uint8_t* flag, uint8_t* exact, int gpb, bool alone) {
     grid_begin();
     __shared__ double s_term[kMaxPairs], s_sum[kGroupThreads];
     __shared__ int s_lower[kMaxPairs], s_work, s_open;
@@ -1093,7 +1095,7 @@ multi_bound_kernel(GateArgs a, PairDesc* descs, Ctl* ctl, uint8_t* flag, uint8_t
         atomicAdd(&s_open, open);
     }
     __syncthreads();
-    if (tid == 0 && s_open) {
+    if (tid == 0 && s_open && !alone) {
         atomicAdd(&ctl->work, (unsigned long long)s_work);
         atomicAdd(&ctl->open, s_open);
     }
@@ -1198,8 +1200,8 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
 
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[0], s));
     // what the kernels add up starts at zero (one CTA that orders the batch alone needs nothing)
-    const bool alone = n_pairs <= kAlonePairs;
-    if (!alone || decide) SR_CUDA_TRY(cudaMemsetAsync(ctl, 0, offsetof(Ctl, start), s));
+    const bool alone = W.alone = n_pairs <= kAlonePairs;
+    if (!alone) SR_CUDA_TRY(cudaMemsetAsync(ctl, 0, offsetof(Ctl, start), s));
     uint8_t* flag = decide ? ws + W.off_flag : nullptr;
     // The match-stream pass works group by group, so when the groups arrive in pieces it runs
     // piece by piece: `feed->before` enqueues whatever makes groups [g0, g1) ready on `s`.
@@ -1222,7 +1224,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     int32_t* order = reinterpret_cast<int32_t*>(ws + W.off_order);
     if (decide) {
-        SR_LAUNCH("multi_bound_kernel", multi_bound_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, descs, ctl, flag, exact, gpb);
+        SR_LAUNCH("multi_bound_kernel", multi_bound_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, descs, ctl, flag, exact, gpb, alone);
     }
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[1], s));
     const int order_blocks = alone ? 1 : (n_pairs + kOrderThreads - 1) / kOrderThreads;
