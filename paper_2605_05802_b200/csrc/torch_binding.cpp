@@ -81,9 +81,13 @@ struct Args {
         if (v == (unsigned long long)-1 && PyErr_Occurred()) throw Raised();
         return (int32_t)v;
     }
-    double real() {
-        const double v = PyFloat_AsDouble(*at++);
-        if (v == -1.0 && PyErr_Occurred()) throw Raised();
+    double real() {                      // whatever float() takes
+        PyObject* o = *at++;
+        if (PyFloat_Check(o)) return PyFloat_AS_DOUBLE(o);
+        PyObject* f = PyNumber_Float(o);
+        if (f == nullptr) throw Raised();
+        const double v = PyFloat_AS_DOUBLE(f);
+        Py_DECREF(f);
         return v;
     }
     static void* handle(PyObject* stream) {

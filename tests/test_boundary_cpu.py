@@ -233,3 +233,24 @@ def test_binding_refuses_tensors_on_the_wrong_side(lib):
         sr.sr_grpo_advantage(torch.zeros((2, 8)), None, 1e-6, adv=torch.zeros((2, 8)))
     with pytest.raises(ValueError, match="contiguous"):
         sr.sr_gate(seqs.transpose(0, 1), None, 15, 0.12, stop=stop)
+
+
+def test_binding_takes_every_number_that_float_takes(lib):
+    """Thresholds go through float(): numpy and torch scalars, fractions, text from a config file."""
+    import decimal
+    import fractions
+    import numpy as np
+    import torch
+
+    class Stream:                        # no device here: the current stream cannot be asked for
+        cuda_stream = 0
+
+    def call(threshold):                 # an empty batch: nothing is enqueued
+        sr.sr_gate_host_packed(torch.zeros(0, dtype=torch.int32), torch.zeros(1, dtype=torch.int64), 4, 8, 8, threshold,
+                               stop=torch.zeros(0, dtype=torch.uint8), arena=None, stream=Stream())
+
+    for threshold in (0.12, 1, np.float32(0.5), np.int64(2), torch.tensor(0.3), fractions.Fraction(1, 8), decimal.Decimal("0.12"), "0.12"):
+        call(threshold)
+    for threshold in (None, [], "a fifth", 1j):
+        with pytest.raises((TypeError, ValueError)):
+            call(threshold)
