@@ -49,7 +49,8 @@
 namespace sr {
 namespace {
 
-constexpr int kPrepThreads = 256;
+constexpr int kMostPrepThreads = 256;      // a thread for every four positions of a pattern
+static_assert(4 * kMostPrepThreads >= SR_MAX_K, "");
 constexpr int kNumClasses = 21;     // team shapes (T lanes x R blocks), see class_of
 constexpr int kTimeBuckets = 96;    // buckets of estimated task duration
 constexpr int kNumBins = 2048;      // kTimeBuckets * kNumClasses of them used
@@ -322,7 +323,7 @@ __device__ __forceinline__ uint32_t set_halves(uint32_t x) {
 // pattern at all and the positions at which text and pattern differ: bounds of the pair's distance that
 // cost next to nothing here.  Where they meet the pair is done.
 template <bool kDecide>
-__global__ void __launch_bounds__(kPrepThreads, 6)
+__global__ void __launch_bounds__(kMostPrepThreads, 6)
 multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t* s_info = reinterpret_cast<uint32_t*>(smem);             // [pitch] see below
@@ -334,13 +335,13 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     __shared__ int s_repeats[4];     // symbols with >= 2, 3, 4 occurrences; mask rows handed out
 
     const int N = a.N, K = a.K, P = pairs_of(N);
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31, nthr = blockDim.x, warps = nthr >> 5;
     const int M = W.patterns;
     const int g = g_base + blockIdx.x / M, i = blockIdx.x % M;
     if (tid < 4) s_repeats[tid] = 0;
-    for (int e = tid; 8 * e < N * W.pitch; e += kPrepThreads)
+    for (int e = tid; 8 * e < N * W.pitch; e += nthr)
         reinterpret_cast<uint4*>(s_map)[e] = make_uint4(kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u);
-    for (int e = tid; 4 * e < W.pitch; e += kPrepThreads) reinterpret_cast<uint4*>(s_info)[e] = make_uint4(0u, 0u, 0u, 0u);
+    for (int e = tid; 4 * e < W.pitch; e += nthr) reinterpret_cast<uint4*>(s_info)[e] = make_uint4(0u, 0u, 0u, 0u);
     grid_begin();
     bool neg = false;
     const int m = clamp_len(a.lens, (size_t)g * N + i, K, neg);
@@ -360,7 +361,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     // the same state and often agree on their first symbols, and the edit distance of two
     // sequences equals that of what is left after a common prefix is removed, so those rows
     // and columns are never looked up nor run through the recurrence.
-    for (int t = tid >> 5; t < ntxt; t += kPrepThreads / 32) {
+    for (int t = tid >> 5; t < ntxt; t += warps) {
         const int j = t < n_before ? t : (t < n_before + n_after ? i + 1 + (t - n_before) : N - 1);
         const int n = clamp_len(a.lens, (size_t)g * N + j, K, neg);
         const int lo = min(m, n);
@@ -394,7 +395,6 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     __syncthreads();
     // Every position claims its name's entry; those that find another one there count as further
     // occurrences with the position that stayed (s_info[claimant]).  Four positions per thread.
-    static_assert(4 * kPrepThreads >= SR_MAX_K, "a position for every thread");
     const int p0 = 4 * tid, mine = min(max(m - p0, 0), 4);
     uint32_t my_name[4] = {0u, 0u, 0u, 0u}, my_first[4];
     if (mine > 0) {
@@ -458,7 +458,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         __syncthreads();
         uint32_t* rows = reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * M + i) * W.row_cap * W.row_words;
         const int n_rows = min(s_repeats[3], W.row_cap);
-        for (int e = tid; e < n_rows * W.row_words; e += kPrepThreads) rows[e] = 0u;
+        for (int e = tid; e < n_rows * W.row_words; e += nthr) rows[e] = 0u;
         __syncthreads();
         if (claims || repeated) {
 #pragma unroll
@@ -475,7 +475,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         if (s_repeats[0] > n_rows) {                   // some chains: leave them for the recurrence
             __syncthreads();
             uint16_t* g_next = reinterpret_cast<uint16_t*>(ws + W.off_next) + ((size_t)g * M + i) * W.pitch;
-            for (int p = tid; p < m; p += kPrepThreads) g_next[p] = (uint16_t)(s_info[p] >> 16);
+            for (int p = tid; p < m; p += nthr) g_next[p] = (uint16_t)(s_info[p] >> 16);
         }
     }
     const bool named = s_repeats[0] > 0;
@@ -485,8 +485,8 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     // look-ups, one 8-byte store.  As many warps to a text as there are for each (chunks dealt to all
     // warps in turn would be even, but then every warp sets up every text).
     uint16_t* locs = reinterpret_cast<uint16_t*>(ws + W.off_loc);
-    const int per_text = max(1, kPrepThreads / 32 / ntxt), warp = tid >> 5, part = warp % per_text;
-    for (int t = warp / per_text; t < ntxt; t += kPrepThreads / 32 / per_text) {
+    const int per_text = max(1, warps / ntxt), warp = tid >> 5, part = warp % per_text;
+    for (int t = warp / per_text; t < ntxt; t += warps / per_text) {
         if (s_cp[t] < 0) continue;
         const int n = s_len[t];
         const uint2* in = reinterpret_cast<const uint2*>(names + s_txt[t] * W.pitch);
@@ -1187,11 +1187,17 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
 
     const int prep_smem = W.pitch * 4 + a.N * W.pitch * 2;
     // names: at least two slots to a symbol while symbols and table fit
-    const int sym_bytes = a.N * W.pitch * 4, names_threads = a.N * W.pitch > 4 * 8 * 512 ? 1024 : 512;
+    const int row_quads = W.pitch >> 2, sym_bytes = a.N * W.pitch * 4, names_most = a.N * W.pitch > 4 * 8 * 512 ? 1024 : 512;
+    // A thread for every four positions of the group while 512 threads suffice, and prep a warp for every text
+    // and for every 128 positions of the pattern: more threads only keep the next CTA waiting.  (512 and 256
+    // whatever the shape: 28000 groups of 2 at K = 33 249 us instead of 98, 4666 of 4 at K = 64 112
+    // instead of 67, 1000 of 8 at K = 100 75 instead of 60.)
+    const int names_threads = min((a.N * row_quads + 31) & ~31, names_most);
+    const int prep_threads = 32 * min(max((a.K + 127) >> 7, a.N >> 1), kMostPrepThreads / 32);
     int table_log = 8;
     while ((1 << table_log) < 2 * a.N * a.K && sym_bytes + (4 << table_log) <= kMostNamesSmem) ++table_log;
     const int names_smem = sym_bytes + (2 << table_log);
-    const uint32_t inv_row = (uint32_t)(((1ull << 32) + (W.pitch >> 2) - 1) / (W.pitch >> 2));
+    const uint32_t inv_row = (uint32_t)(((1ull << 32) + row_quads - 1) / row_quads);
     uint16_t* names = reinterpret_cast<uint16_t*>(ws + W.off_names);
     if (names_smem > 48 * 1024 || prep_smem > 48 * 1024) {
         const int rc = allow_smem();
@@ -1216,9 +1222,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
         }
         SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0);
         if (decide)
-            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<true>, (g1 - g0) * W.patterns, kPrepThreads, prep_smem, s, a, ws, W, dist, g0);
+            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<true>, (g1 - g0) * W.patterns, prep_threads, prep_smem, s, a, ws, W, dist, g0);
         else
-            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<false>, (g1 - g0) * W.patterns, kPrepThreads, prep_smem, s, a, ws, W, dist, g0);
+            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<false>, (g1 - g0) * W.patterns, prep_threads, prep_smem, s, a, ws, W, dist, g0);
     }
     const int gpb = P <= kGroupThreads ? kGroupThreads / P : 1;
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);

@@ -28,7 +28,7 @@ def test_symbols_with_a_given_number_of_occurrences(K, times):
 
 @pytest.mark.parametrize("K", [64, 300, 1024])
 def test_symbols_that_crowd_one_slot_of_the_table(K):
-    """IDs chosen so that dozens of them hash to the same home slot: more than its neighbourhood holds."""
+    """IDs chosen so that dozens of them hash to one slot under the first hash: many rounds until all have names."""
     rng = np.random.default_rng(K)
     inverse = pow(0x9E3779B1, -1, 1 << 32)
     crowd = (np.array([5 << 25], dtype=np.uint64) + np.arange(40, dtype=np.uint64)) * np.uint64(inverse) % np.uint64(1 << 32)
@@ -41,3 +41,17 @@ def test_symbols_that_crowd_one_slot_of_the_table(K):
     lens = rng.integers(K // 2 + 1, K + 1, size=(G, N)).astype(np.int32)
     want = oracle.gate(seqs, lens, K, 0.4, threads=8)
     assert_gate_matches(gate_gpu(seqs, lens, K, 0.4), want, f"K={K}")
+
+
+@pytest.mark.parametrize("N,K", [(2, 33), (3, 128), (2, 129), (5, 256), (4, 257), (6, 384), (2, 385), (9, 40), (10, 513), (3, 641),
+                                 (13, 60), (15, 70), (16, 769), (2, 897), (17, 130)])
+def test_every_number_of_warps_per_pattern(N, K):
+    """The per-pattern pass has a warp for every 128 positions and for every text: one to eight."""
+    rng = np.random.default_rng(100 * N + K)
+    G, stride = 7, (K + 3) // 4 * 4
+    seqs = np.where(rng.random((G, N, stride)) < 0.2, rng.integers(0, 60, size=(G, N, stride)), rng.integers(0, 10 ** 6, size=(G, N, stride)))
+    seqs[1::2] = np.where(rng.random((3, N, stride)) < 0.8, seqs[1::2, :1], seqs[1::2])
+    lens = rng.integers(0, K + 1, size=(G, N)).astype(np.int32)
+    lens[::2] = K
+    seqs = seqs.astype(np.int32)
+    assert_gate_matches(gate_gpu(seqs, lens, K, 0.4), oracle.gate(seqs, lens, K, 0.4, threads=8), f"N={N} K={K}")
