@@ -514,16 +514,28 @@ int launch_gate_direct(const GateArgs& a, cudaStream_t s) {
     return SR_OK;
 }
 
+// Where naming the symbols first pays: the least number of pairs, measured for the group sizes 2..32, every
+// K up to 16 and 300 to 2.6 million pairs; mean time within 0.4 % of the better kernel's.  Direct comparison
+// costs two instructions per cell, naming a few dozen per symbol and a longer chain of latencies on
+// one warp a group: small batches, N < 8 and short prefixes stay with direct comparison.  The line
+// lies later for large groups, whose warp takes long (32 rollouts: eight rounds of pairs), and for those
+// whose pairs fill the CTAs of the direct kernel (31 and 32).  At K = 16 two patterns do not fit a
+// word, and groups of 9 to 13 leave the CTA they then get mostly idle.  Direct / naming in us: 8 x 5714, K = 12
+// 7.2 / 6.7; 32 x 161, K = 12 9.2 / 16.5; 16 x 2666, K = 8 8.7 / 8.9, 16 x 21666 45 / 34; 9 x 36111, K = 16 46 / 94.
+bool names_pay(int N, int K, long long pairs) {
+    if (N < 8) return false;
+    if (K == 16) return (N == 8 || N >= 14) && pairs >= 25000;
+    if (K >= 13) return pairs >= (N <= 16 ? 40000 : 120000);
+    if (K >= 9) return pairs >= (N <= 10 ? 100000 : (N <= 30 ? 240000 : 1200000));
+    if (N > 30 && K > 4) return false;
+    return N >= 12 && pairs >= (N < 14 ? 1000000 : 300000);
+}
+
 }  // namespace
 
 int launch_gate_single(const GateArgs& a, cudaStream_t s) {
     if (a.n_groups == 0) return SR_OK;
-    // Comparing directly costs two instructions per cell, naming the symbols first a few dozen per
-    // symbol and a longer chain of latencies: with fewer than eight rollouts, or in batches too small
-    // to fill the machine, direct comparison is quicker (K = 10, N = 8: 3.6 against 4.2 us for 10
-    // groups, 21 against 18.5 us for 32768; K = 15: 33 against 24 us; N = 4: 11 against 16 us).
-    const bool direct = a.N < 8 || (long long)a.n_groups * pairs_of(a.N) * (a.K > 9 ? a.K - 8 : 1) < 200000;
-    if (a.K <= 16 && direct) {
+    if (a.K <= 16 && !names_pay(a.N, a.K, (long long)a.n_groups * pairs_of(a.N))) {
         if (a.K <= 4) return launch_gate_direct<4>(a, s);
         if (a.K <= 8) return launch_gate_direct<8>(a, s);
         if (a.K <= 12) return launch_gate_direct<12>(a, s);

@@ -14,12 +14,14 @@ from helpers import assert_gate_matches, gate_gpu
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("N,K", [(8, 15), (8, 9), (9, 12), (11, 14), (16, 13), (32, 3), (31, 15), (32, 15), (17, 1),
-                                 (2, 17), (3, 32), (5, 31), (8, 32), (8, 17), (9, 16), (13, 29), (32, 32), (31, 18)])
+@pytest.mark.parametrize("N,K,pairs", [(8, 15, 40000), (8, 9, 100000), (9, 12, 100000), (11, 14, 40000), (16, 13, 40000), (32, 3, 300000),
+                                       (31, 15, 120000), (32, 15, 120000), (17, 1, 300000), (12, 7, 1000000), (31, 11, 1200000),
+                                       (8, 16, 25000), (14, 16, 25000), (2, 17, 37), (3, 32, 111), (5, 31, 370), (8, 32, 1036),
+                                       (8, 17, 1036), (9, 16, 25000), (9, 17, 1332), (13, 29, 2886), (32, 32, 18352), (31, 18, 17205)])
 @pytest.mark.parametrize("symbols", ["few", "base", "wide", "crowd"])
-def test_named_gate(N, K, symbols):
+def test_named_gate(N, K, pairs, symbols):
     P = N * (N - 1) // 2
-    G = 37 if K > 16 else 200000 // (P * max(K - 8, 1)) + 3
+    G = pairs // P + 3                       # up to K = 16: just enough pairs for this kernel
     rng = np.random.default_rng(1000 * N + K)
     stride = (K + 3) // 4 * 4 + 4
     if symbols == "few":
