@@ -407,6 +407,25 @@ incr_rollout_kernel(IncrArgs a) {
     }
 }
 
+// Steps follow one another on the stream.  A step whose CTAs become resident while the one before still
+// runs crowds onto the SMs that have room: fine while an SM holds little of either, and again when the grid is
+// more than one wave, but in between some SMs get two CTAs and others none.  An ordinary launch
+// between `some` threads per SM and `wave`, one wave.  30 steps, overlapping / ordinary in us: 30000 groups of 2
+// (405 threads per SM) 202 / 134, 33333 of 3 (676) 208 / 152, 3571 of 8 (687) 128 / 114, 1071 of 8 (206) 91 / 98,
+// 8928 of 8 (1716) 167 / 180; thread per rollout, 2173 of 24 (352) 608 / 351, 16666 of 16 (1802) 735 / 749.
+int launch_step(const char* name, void (*kernel)(IncrArgs), int blocks, int threads, int smem, cudaStream_t s,
+                const IncrArgs& a, int some, int wave) {
+    bool early = true;
+    if (blocks > 64) {
+        int dev = 0, sms = 0;
+        SR_CUDA_TRY(cudaGetDevice(&dev));
+        SR_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const long long all = (long long)blocks * threads;
+        early = all <= (long long)some * sms || all > (long long)wave * sms;
+    }
+    return launch_as(early, 1, name, kernel, blocks, threads, smem, s, a);
+}
+
 }  // namespace
 
 size_t incr_state_bytes(int32_t n_groups, int32_t N, int32_t max_steps) {
@@ -456,8 +475,7 @@ int launch_incr_step(void* state, size_t bytes, const int32_t* new_actions, int3
         a.off_eq = take(a.gpb * N * (N - 1) * 4);
         auto kernel = N == 8 ? incr_rollout_kernel<8, 7> : (N <= 5 ? incr_rollout_kernel<0, 4>
                                   : (N <= 8 ? incr_rollout_kernel<0, 7> : incr_rollout_kernel<0, 8>));
-        SR_LAUNCH("incr_rollout_kernel", kernel, (n_groups + a.gpb - 1) / a.gpb, kRollThreads, off, s, a);
-        return SR_OK;
+        return launch_step("incr_rollout_kernel", kernel, (n_groups + a.gpb - 1) / a.gpb, kRollThreads, off, s, a, 0, 1024);
     }
     int gpb = 256 / P;
     if (gpb < 1) gpb = 1;
@@ -470,9 +488,7 @@ int launch_incr_step(void* state, size_t bytes, const int32_t* new_actions, int3
     if (threads < gpb * N) threads = (gpb * N + 31) & ~31;
     if (threads < 64) threads = 64;
     const int blocks = (n_groups + gpb - 1) / gpb;
-    if (N == 8) SR_LAUNCH("incr_step_kernel", incr_step_kernel<8>, blocks, threads, off, s, a);
-    else SR_LAUNCH("incr_step_kernel", incr_step_kernel<0>, blocks, threads, off, s, a);
-    return SR_OK;
+    return launch_step("incr_step_kernel", N == 8 ? incr_step_kernel<8> : incr_step_kernel<0>, blocks, threads, off, s, a, 384, 1536);
 }
 
 }  // namespace sr

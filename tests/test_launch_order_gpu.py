@@ -60,3 +60,29 @@ def test_back_to_back_calls_see_each_other(n_groups, K, captured):
         assert np.array_equal(s.cpu().numpy(), ostop) and np.array_equal(z.cpu().numpy(), ozv), k
         assert np.allclose(a.cpu().numpy(), oadv, rtol=1e-6, atol=0), k
         assert int(c) == len(oidx) and np.array_equal(i.cpu().numpy()[:int(c)], oidx), k
+
+
+@pytest.mark.parametrize("G,N", [(200, 8), (30000, 2), (3571, 8), (12000, 8), (23000, 8), (2173, 24), (70000, 8)])
+def test_steps_back_to_back_see_each_other(G, N):
+    """Incremental steps without synchronisation between them, at sizes on either side of where a step
+    overlaps the one before it."""
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(G + N)
+    steps = 9
+    actions = np.where(rng.random((steps, G, N)) < 0.6, rng.integers(0, 5, size=(steps, G, 1)), rng.integers(0, 5, size=(steps, G, N))).astype(np.int32)
+    given = torch.from_numpy(actions).to(dev)
+    state = torch.empty(sr.sr_incr_state_bytes(G, N, steps), dtype=torch.uint8, device=dev)
+    mean = torch.empty((steps, G), dtype=torch.float64, device=dev)
+    stop = torch.empty((steps, G), dtype=torch.uint8, device=dev)
+    torch.cuda.synchronize()
+    sr.sr_incr_init(state, G, N, steps)
+    for t in range(steps):
+        sr.sr_gate_step_incremental(state, given[t], 0.3, mean=mean[t], stop=stop[t])
+    mean, stop = mean.cpu().numpy(), stop.cpu().numpy()
+    some = np.unique(np.concatenate([rng.integers(0, G, 200), [0, G - 1]]))
+    seqs = np.zeros((len(some), N, 12), dtype=np.int32)
+    seqs[:, :, :steps] = actions[:, some].transpose(1, 2, 0)
+    for t in range(steps):
+        want = oracle.gate(seqs, np.full((len(some), N), t + 1, dtype=np.int32), steps, 0.3, threads=8)
+        assert np.array_equal(mean[t, some].view(np.uint64), want[2].view(np.uint64)), t
+        assert np.array_equal(stop[t, some], want[3]), t
