@@ -459,11 +459,16 @@ int launch_batch_stats(const float* adv, const uint8_t* stop, int32_t n_groups, 
                        int64_t* counts, double* sumsq, cudaStream_t s) {
     const bool vec4 = (N % 4 == 0) && (reinterpret_cast<uintptr_t>(adv) & 15) == 0;
     unsigned long long* const c = reinterpret_cast<unsigned long long*>(counts);
-    // the cluster's eight SMs take no longer for two groups per thread than two clears do
-    if (n_groups <= kClusterCtas * 1024 * 2) {
-        const int threads = n_groups <= kClusterCtas * 256 ? 256 : 1024;
+    // One cluster while its eight SMs take no longer than clears, grid and atomics do (8 us).  That goes with the
+    // bytes, sooner without 16-byte loads, and sooner where the rows of a warp's lanes fall on the
+    // same lines of L1.  Cluster / grid in us: 16384 x 13 5.8 / 8.1, 16384 x 24 6.7 / 8.4, 12000 x 32 12.3 / 8.4;
+    // rows off 16 bytes, 8192 x 20 5.6 / 8.4, 12000 x 16 12.4 / 8.2, 8192 x 32 20.8 / 10.8.
+    const long long most = N % 16 == 0 ? (vec4 ? 1 << 18 : 1 << 17) : (vec4 ? 3 << 17 : 1 << 18);
+    if (n_groups <= kClusterCtas * 1024 * 2 && (long long)n_groups * N <= most) {
         int ctas = 1;
-        while (ctas < kClusterCtas && ctas * threads < n_groups) ctas *= 2;
+        while (ctas < kClusterCtas && ctas * 256 < n_groups) ctas *= 2;
+        int threads = 256;                           // up to two groups per thread
+        if (n_groups > ctas * 256) threads = n_groups >= ctas * 1024 ? 1024 : ((n_groups + ctas - 1) / ctas + 31) & ~31;
         return launch_as(true, ctas, "batch_stats_kernel", batch_stats_kernel<true>, ctas, threads, 0, s, adv, stop, N, n_groups, vec4, c, sumsq);
     }
     SR_CUDA_TRY(cudaMemsetAsync(counts, 0, 3 * sizeof(int64_t), s));

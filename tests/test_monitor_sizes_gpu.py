@@ -26,6 +26,24 @@ def test_batch_stats(G, N):
     assert np.allclose(sumsq.cpu().numpy(), np.asarray(want[1]), rtol=1e-12, atol=0)
 
 
+@pytest.mark.parametrize("G,N,off", [(3000, 32, 0), (8192, 32, 0), (8193, 32, 0), (4096, 32, 1), (4097, 32, 1), (16384, 24, 0), (8456, 31, 0),
+                                     (8457, 31, 0), (13107, 20, 1), (13108, 20, 1), (2304, 5, 3)])
+def test_batch_stats_where_one_cluster_ends(G, N, off):
+    """Either side of the largest batch one cluster takes, with rows on and off 16 bytes."""
+    rng = np.random.default_rng(G + N)
+    adv = rng.standard_normal((G, N)).astype(np.float32)
+    adv[rng.random((G, N)) < 0.3] = 0.0
+    stop = (rng.random(G) < 0.4).astype(np.uint8)
+    given = torch.empty(G * N + off, device=dev)[off:].view(G, N)
+    given.copy_(torch.from_numpy(adv))
+    counts = torch.full((3,), -7, dtype=torch.int64, device=dev)
+    sumsq = torch.full((2,), -7.0, dtype=torch.float64, device=dev)
+    sr.sr_batch_stats(given, torch.from_numpy(stop).to(dev), counts=counts, sumsq=sumsq)
+    want = oracle.batch_stats(adv, stop)
+    assert np.array_equal(counts.cpu().numpy(), np.asarray(want[0]))
+    assert np.allclose(sumsq.cpu().numpy(), np.asarray(want[1]), rtol=1e-12, atol=0)
+
+
 @pytest.mark.parametrize("n", [8 * 4096, 8 * 4096 + 1, 3 * 4096 - 1])
 def test_kept_groups(n):
     rng = np.random.default_rng(n)
