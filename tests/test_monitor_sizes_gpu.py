@@ -44,14 +44,18 @@ def test_batch_stats_where_one_cluster_ends(G, N, off):
     assert np.allclose(sumsq.cpu().numpy(), np.asarray(want[1]), rtol=1e-12, atol=0)
 
 
-@pytest.mark.parametrize("n", [8 * 4096, 8 * 4096 + 1, 3 * 4096 - 1])
-def test_kept_groups(n):
+@pytest.mark.parametrize("n,off", [(8 * 4096, 0), (8 * 4096 + 1, 0), (3 * 4096 - 1, 0), (8 * 4096 + 1, 1), (3 * 4096 - 1, 3), (1000003, 1)])
+def test_kept_groups(n, off):
     rng = np.random.default_rng(n)
     stop, zv = ((rng.random(n) < 0.3).astype(np.uint8) for _ in range(2))
     index = torch.full((n,), -7, dtype=torch.int32, device=dev)
     count = torch.full((1,), -7, dtype=torch.int32, device=dev)
     ws = torch.empty(sr.sr_kept_groups_workspace_bytes(n), dtype=torch.uint8, device=dev)
-    sr.sr_kept_groups(torch.from_numpy(stop).to(dev), torch.from_numpy(zv).to(dev), index=index, count=count, workspace=ws)
+    given = []
+    for flags in (stop, zv):                                      # `off` bytes past a 16-byte boundary
+        given.append(torch.empty(n + off, dtype=torch.uint8, device=dev)[off:])
+        given[-1].copy_(torch.from_numpy(flags))
+    sr.sr_kept_groups(*given, index=index, count=count, workspace=ws)
     want = oracle.kept_groups(stop, zv)
     assert int(count) == want.size and np.array_equal(index.cpu().numpy()[:want.size], want)
 
