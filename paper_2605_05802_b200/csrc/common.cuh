@@ -78,6 +78,15 @@ int launch(const char* name, void (*kernel)(Params...), int blocks, int threads,
         if (rc__ != SR_OK) return rc__;                     \
     } while (0)
 
+// Whether the call is being captured into a graph.  A replayed graph starts a kernel about a microsecond after
+// the one before it has finished, a stream three: where an early launch has a price, in CTAs that
+// crowd onto the SMs the kernel before leaves first, it pays off on a stream and not in a graph.
+inline bool captured(cudaStream_t s) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &status) != cudaSuccess) cudaGetLastError();     // the launch will report it
+    return status == cudaStreamCaptureStatusActive;
+}
+
 // Start of every kernel: lets the next kernel of the stream be set up, then waits until the
 // one before has finished and its writes are visible.  Nothing global is touched before it.
 __device__ __forceinline__ void grid_begin() {

@@ -407,23 +407,19 @@ incr_rollout_kernel(IncrArgs a) {
     }
 }
 
-// Steps follow one another on the stream.  A step whose CTAs become resident while the one before still
-// runs crowds onto the SMs that have room: fine while an SM holds little of either, and again when the grid is
-// more than one wave, but in between some SMs get two CTAs and others none.  An ordinary launch
-// between `some` threads per SM and `wave`, one wave.  30 steps, overlapping / ordinary in us: 30000 groups of 2
-// (405 threads per SM) 202 / 134, 33333 of 3 (676) 208 / 152, 3571 of 8 (687) 128 / 114, 1071 of 8 (206) 91 / 98,
-// 8928 of 8 (1716) 167 / 180; thread per rollout, 2173 of 24 (352) 608 / 351, 16666 of 16 (1802) 735 / 749.
-int launch_step(const char* name, void (*kernel)(IncrArgs), int blocks, int threads, int smem, cudaStream_t s,
-                const IncrArgs& a, int some, int wave) {
-    bool early = true;
-    if (blocks > 64) {
-        int dev = 0, sms = 0;
-        SR_CUDA_TRY(cudaGetDevice(&dev));
-        SR_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const long long all = (long long)blocks * threads;
-        early = all <= (long long)some * sms || all > (long long)wave * sms;
-    }
-    return launch_as(early, 1, name, kernel, blocks, threads, smem, s, a);
+// Steps follow one another.  A step whose CTAs become resident while the one before still runs crowds onto the
+// SMs that have room: fine while an SM holds little of either, and again when the grid is more than one
+// wave, but in between some SMs get two CTAs and others none.  The kernel with a thread per pair then overlaps on
+// a stream, where that still pays, and not in a graph; the one with a thread per rollout, whose CTAs last
+// longer, in neither up to 800 threads per SM.  30 steps, overlapping / ordinary in us: graph, 30000 groups of 2 (405
+// threads per SM) 202 / 134, 33333 of 3 (676) 208 / 152, 3571 of 8 (687) 128 / 114, 1071 of 8 (206) 91 / 98, 8928 of 8
+// (1716) 167 / 180; stream, 3571 of 8 136 / 168; thread per rollout, 2173 of 24 (352) 608 / 351 and 615 / 404,
+// 8333 of 16 (900) 457 / 437 and 470 / 491.
+int sm_count(int& sms) {
+    int dev = 0;
+    SR_CUDA_TRY(cudaGetDevice(&dev));
+    SR_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    return SR_OK;
 }
 
 }  // namespace
@@ -475,7 +471,11 @@ int launch_incr_step(void* state, size_t bytes, const int32_t* new_actions, int3
         a.off_eq = take(a.gpb * N * (N - 1) * 4);
         auto kernel = N == 8 ? incr_rollout_kernel<8, 7> : (N <= 5 ? incr_rollout_kernel<0, 4>
                                   : (N <= 8 ? incr_rollout_kernel<0, 7> : incr_rollout_kernel<0, 8>));
-        return launch_step("incr_rollout_kernel", kernel, (n_groups + a.gpb - 1) / a.gpb, kRollThreads, off, s, a, 0, 1024);
+        const int blocks = (n_groups + a.gpb - 1) / a.gpb;
+        int sms = 0;
+        const int rc = sm_count(sms);
+        if (rc != SR_OK) return rc;
+        return launch_as((long long)blocks * kRollThreads > 800LL * sms, 1, "incr_rollout_kernel", kernel, blocks, kRollThreads, off, s, a);
     }
     int gpb = 256 / P;
     if (gpb < 1) gpb = 1;
@@ -488,7 +488,15 @@ int launch_incr_step(void* state, size_t bytes, const int32_t* new_actions, int3
     if (threads < gpb * N) threads = (gpb * N + 31) & ~31;
     if (threads < 64) threads = 64;
     const int blocks = (n_groups + gpb - 1) / gpb;
-    return launch_step("incr_step_kernel", N == 8 ? incr_step_kernel<8> : incr_step_kernel<0>, blocks, threads, off, s, a, 384, 1536);
+    bool early = true;
+    if (blocks > 64) {                           // 64 CTAs leave most SMs empty
+        int sms = 0;
+        const int rc = sm_count(sms);
+        if (rc != SR_OK) return rc;
+        const long long all = (long long)blocks * threads;
+        early = all <= 384LL * sms || all > 1536LL * sms || !captured(s);
+    }
+    return launch_as(early, 1, "incr_step_kernel", N == 8 ? incr_step_kernel<8> : incr_step_kernel<0>, blocks, threads, off, s, a);
 }
 
 }  // namespace sr
