@@ -192,9 +192,9 @@ int launch_kept_groups(const uint8_t* stop, const uint8_t* zero_var, int32_t n_g
     SR_LAUNCH("kept_count_kernel", vec ? kept_count_kernel<true> : kept_count_kernel<false>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles);
     SR_LAUNCH("kept_offsets_kernel", kept_offsets_kernel, 1, 1024, 0, s, tiles, n_tiles, count);
     // Flags off 16 bytes are read one by one, long enough that it matters where the CTAs are: made resident
-    // while the counts are still being taken they crowd onto some SMs (a million groups 13.8 us, ordinarily
+    // while the counts are still being taken they crowd onto some SMs (in a graph a million groups 13.8 us, ordinarily
     // launched 10.2; on 16 bytes 5.6 and 5.9).
-    return launch_as(vec, 1, "kept_scatter_kernel", vec ? kept_scatter_kernel<true, false> : kept_scatter_kernel<false, false>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles, index, count);
+    return launch_as(vec || !captured(s), 1, "kept_scatter_kernel", vec ? kept_scatter_kernel<true, false> : kept_scatter_kernel<false, false>, n_tiles, kTileThreads, 0, s, stop, zero_var, n_groups, tiles, index, count);
 }
 
 }  // namespace sr
