@@ -322,7 +322,9 @@ __device__ __forceinline__ uint32_t set_halves(uint32_t x) {
 // One CTA per pattern.  Per text it also counts the columns whose symbol does not occur in the
 // pattern at all and the positions at which text and pattern differ: bounds of the pair's distance that
 // cost next to nothing here.  Where they meet the pair is done.
-template <bool kDecide>
+// kThreads: the CTA's threads where they are the most there can be (known at compile time 82 us of the token-level
+// batch of 1024 groups, at run time 84.5), 0 for fewer.
+template <bool kDecide, int kThreads>
 __global__ void __launch_bounds__(kMostPrepThreads, 6)
 multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -335,7 +337,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     __shared__ int s_repeats[4];     // symbols with >= 2, 3, 4 occurrences; mask rows handed out
 
     const int N = a.N, K = a.K, P = pairs_of(N);
-    const int tid = threadIdx.x, lane = tid & 31, nthr = blockDim.x, warps = nthr >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, nthr = kThreads ? kThreads : blockDim.x, warps = nthr >> 5;
     const int M = W.patterns;
     const int g = g_base + blockIdx.x / M, i = blockIdx.x % M;
     if (tid < 4) s_repeats[tid] = 0;
@@ -1152,8 +1154,8 @@ int allow_smem() {
     if (dev >= 0 && dev < 64 && allowed[dev].load(std::memory_order_relaxed)) return SR_OK;
     const int prep = SR_MAX_K * 4 + SR_MAX_N * SR_MAX_K * 2;
     SR_CUDA_TRY(cudaFuncSetAttribute(multi_names_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostNamesSmem));
-    SR_CUDA_TRY(cudaFuncSetAttribute(multi_prep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, prep));
-    SR_CUDA_TRY(cudaFuncSetAttribute(multi_prep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, prep));
+    for (auto kernel : {multi_prep_kernel<true, 0>, multi_prep_kernel<true, kMostPrepThreads>, multi_prep_kernel<false, 0>, multi_prep_kernel<false, kMostPrepThreads>})
+        SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, prep));
     if (dev >= 0 && dev < 64) allowed[dev].store(true, std::memory_order_relaxed);
     return SR_OK;
 }
@@ -1188,12 +1190,13 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const int prep_smem = W.pitch * 4 + a.N * W.pitch * 2;
     // names: at least two slots to a symbol while symbols and table fit
     const int row_quads = W.pitch >> 2, sym_bytes = a.N * W.pitch * 4, names_most = a.N * W.pitch > 4 * 8 * 512 ? 1024 : 512;
-    // A thread for every four positions of the group while 512 threads suffice, and prep a warp for every text
-    // and for every 128 positions of the pattern: more threads only keep the next CTA waiting.  (512 and 256
-    // whatever the shape: 28000 groups of 2 at K = 33 249 us instead of 98, 4666 of 4 at K = 64 112
-    // instead of 67, 1000 of 8 at K = 100 75 instead of 60.)
-    const int names_threads = min((a.N * row_quads + 31) & ~31, names_most);
-    const int prep_threads = 32 * min(max((a.K + 127) >> 7, a.N >> 1), kMostPrepThreads / 32);
+    // A thread for every four positions of the group while 512 threads suffice; and for prep a warp for every 128
+    // positions of the pattern and as many warps to every text, unless there are SMs for all patterns: more
+    // threads only keep the next CTA waiting.  (512 and 256 whatever the shape: 28000 groups of 2 at K = 33 249 us
+    // instead of 98, 4666 of 4 at K = 64 112 instead of 67, 1000 of 8 at K = 100 75 instead of 60.)
+    const int names_threads = min((a.N * row_quads + 31) & ~31, names_most), texts = a.N >> 1;
+    const int fewest = (max((a.K + 127) >> 7, texts) + texts - 1) / texts * texts;
+    const int prep_threads = (long long)a.n_groups * W.patterns <= sms ? kMostPrepThreads : min(32 * fewest, kMostPrepThreads);
     int table_log = 8;
     while ((1 << table_log) < 2 * a.N * a.K && sym_bytes + (4 << table_log) <= kMostNamesSmem) ++table_log;
     const int names_smem = sym_bytes + (2 << table_log);
@@ -1221,10 +1224,10 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
             if (rc != SR_OK) return rc;
         }
         SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0);
-        if (decide)
-            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<true>, (g1 - g0) * W.patterns, prep_threads, prep_smem, s, a, ws, W, dist, g0);
-        else
-            SR_LAUNCH("multi_prep_kernel", multi_prep_kernel<false>, (g1 - g0) * W.patterns, prep_threads, prep_smem, s, a, ws, W, dist, g0);
+        const auto prep = prep_threads == kMostPrepThreads
+            ? (decide ? multi_prep_kernel<true, kMostPrepThreads> : multi_prep_kernel<false, kMostPrepThreads>)
+            : (decide ? multi_prep_kernel<true, 0> : multi_prep_kernel<false, 0>);
+        SR_LAUNCH("multi_prep_kernel", prep, (g1 - g0) * W.patterns, prep_threads, prep_smem, s, a, ws, W, dist, g0);
     }
     const int gpb = P <= kGroupThreads ? kGroupThreads / P : 1;
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
