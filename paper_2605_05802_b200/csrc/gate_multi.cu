@@ -239,9 +239,8 @@ __device__ __forceinline__ int clamp_len(const int32_t* lens, size_t idx, int K,
 // that is the name; the symbols that lost their slot to another one go on with another hash, and every
 // round names at least one symbol of each slot.  One CTA per group.  With the names, 16 bits
 // each, a pattern's look-up table is an array: no hashing, no probing, no comparing in prep, which serves
-// every text (N - 1) / 2 times.  (The table of hashed 32-bit slots that prep had instead took 280 warp
-// instructions for four columns of a warp's lanes; with the names, on 1024 groups of 8 token prefixes, both kernels
-// together take 81 us where it took 104, and 107 against 150 at full length.)
+// every text (N - 1) / 2 times.  Names and prep together, 1024 groups of 8 token prefixes: 82 us, 107 us at full
+// length.  Bound: the latency between the barriers here (three CTAs of 64 KB per SM), instruction issue in prep.
 constexpr uint32_t kHashMul = 0x9E3779B1u;
 constexpr int kMaxTexts = SR_MAX_N / 2;        // texts a pattern is paired with
 
@@ -423,8 +422,8 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         // every rollout (a third of the columns of such a text meet a symbol that occurs more
         // than once, the most common one dozens of times), so these get a row of match words,
         // one per 32 positions, which the recurrence reads in place of its one-hot word.  (Walking
-        // a chain of occurrences per column made the recurrence wait for the longest chain of the
-        // warp: 16 groups of 8 such texts of up to 1024 tokens took 2.2 ms, with the rows 0.16 ms.)
+        // a chain of occurrences makes the recurrence wait for the longest chain of the warp: 141 groups
+        // of 8 such texts of 1024 tokens take 165 us, with a quarter of the rows and chains besides 426.)
         // The full pool has room for every symbol with at least eight occurrences; what does not fit
         // (the rarest of the repeated ones) is left as a chain of at most seven positions.  In a
         // smaller pool (see launch_gate_multi) the last symbols to ask get a chain of any length.
@@ -867,7 +866,7 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
     }
     if (T >= 16 && valid) {
         // Few pairs: nothing else hides the latencies of this one, so all that it will read goes to L1 first,
-        // the stream and the pattern's mask rows (16 groups of 8 texts: 78 -> 74 us).
+        // the stream and the pattern's mask rows (the recurrence of 16 groups of 8 texts: 74 us, 78 without).
         touch(loc4, 2 * n, lt, T);
         touch(rows, 4 * n_rows * W.row_words, lt, T);
     }
@@ -1243,7 +1242,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const long long want = (n_pairs_ll + kDpWarpsPerCta - 1) / kDpWarpsPerCta;
     const int blocks = (int)(want < 3LL * sms ? want : 3LL * sms);
     // (an ordinary launch unless every CTA has an SM: CTAs made resident while the tail of prep still fills some SMs would
-    // crowd onto the others, 478 us instead of 434 for the token-level batch of 1024 groups)
+    // crowd onto the others, 310 us instead of 269 for the token-level batch of 1024 groups)
     const int rc = launch_as(alone && blocks < sms, 1, "multi_dp_kernel", multi_dp_kernel, blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u);
     if (rc != SR_OK) return rc;
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[3], s));

@@ -20,10 +20,9 @@
 //      masks of two patterns share a word, and one recurrence serves two pairs;
 //   4. one thread per group adds the normalised terms in fp64 in pair order, thresholds
 //      (Eq. 2) and writes out, for all groups of a CTA side by side.
-// Bound: instruction issue (0.6 to 0.7 per scheduler and clock, as all integer code here), a third of it
-// in the recurrence.  Measured against one-look-up-more tables (64-bit compare-and-swap slots, a
-// byte map per rollout and slot) for K > 16 and direct comparison for K <= 16: 4096 groups of 16, K = 30:
-// 33.7 -> 23 us; 16384 groups of 8, K = 30: 51 -> 31 us; 65536 groups of 8, K = 15, ragged: 64 -> 44 us.
+// Bound: instruction issue.  65536 groups of 16 at K = 30, a CTA each, issue in 75 % of the scheduler's clocks, 55 % of it
+// the recurrence; 65536 groups of 8 at K = 15, two to a warp, in 63 %, with 42 % of the warp slots filled.
+// 4096 groups of 16, K = 30: 23 us; 16384 groups of 8, K = 30: 31 us; 65536 groups of 8, K = 15, ragged: 44 us.
 #include <atomic>
 
 #include "common.cuh"

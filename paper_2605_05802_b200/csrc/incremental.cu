@@ -108,7 +108,7 @@ struct IncrArgs {
     uint8_t* stop;
     int32_t* status;
     int gpb;                                               // groups per CTA
-    uint32_t inv_P, inv_N;                                 // ceil(2^20 / P), ceil(2^20 / N): thread -> group by multiply-shift (exact below 512)
+    uint32_t inv_P, inv_N;                                 // ceil(2^20 / P), ceil(2^20 / N): x / P by multiply-shift, exact while x (P - 1) < 2^20 (x: pairs of a CTA, at most 1984)
     int off_dist, off_term, off_roll, off_eq;              // shared-memory offsets
     uint32_t one;                                          // 1, as a run-time value
 };
@@ -291,9 +291,9 @@ __device__ __forceinline__ void pair_at(int e, int N, int P, int kN, uint32_t in
 // of the group's other rollouts (kMasks at a time); the masks go to the pairs through shared memory.  A
 // thread per pair that does its own comparing reads every stored action N - 1 times: the
 // return path of L1 (16 bytes a lane and load) and the indices of its loads were half of that kernel.
-// 30 steps: 65536 groups of 8 792 -> 612 us, 16384 groups of 16 1033 -> 721 us.  (Registers decide: with
-// four pair states in flight the kernel takes 706 us at 60 registers and 884 at 48, where it spills;
-// with one, 656 us at 56, 612 at 48 and 665 at 40.)
+// 30 steps, a thread per pair / per rollout: 65536 groups of 8 792 / 612 us, 16384 groups of 16 1033 / 721 us.
+// (Registers decide: with one pair state in flight 656 us at 56 registers, 612 at 48, 665 at 40; with four
+// 706 at 60, and 884 at 48, where it spills.)
 // kN: as above.
 template <int kN, int kMasks>
 __global__ void __launch_bounds__(kRollThreads, kN ? 9 : 8)

@@ -69,8 +69,8 @@ struct EntropyTable {                           // host side
 // into a bit set per rollout by votes (32 names a step), and a pair's Jaccard term is a few popcounts.
 // Two warps match the prefixes (by hash, then symbol by symbol) and the step-K actions; everything is added
 // up in a fixed order.
-// Bound: instruction issue and the latency between its barriers.  Compare-and-swap slots and bit sets over
-// all bigrams took 26 us for 4096 groups of 16 at K = 30, this form 17 us (331 -> 205 us for 65536).
+// Bound: instruction issue (81 % of the scheduler's clocks for 65536 groups of 16 at K = 30, 205 us) and, in small
+// batches, the latency between its barriers (4096 groups 17 us).
 struct SignalLayout {
     int Q, items;                               // quads per rollout, items of the group
     uint32_t inv_Q;                             // ceil(2^20 / Q)

@@ -1,5 +1,5 @@
 """Incremental gate on batches large enough for the thread-per-rollout kernel: every width of its mask
-loop, more and fewer pairs than the states it prefetches, pauses, early ends and full rollouts."""
+loop, more and fewer pairs than threads in a CTA, pauses, early ends and full rollouts."""
 import numpy as np
 import pytest
 

@@ -62,8 +62,9 @@ def test_back_to_back_calls_see_each_other(n_groups, K, captured):
         assert int(c) == len(oidx) and np.array_equal(i.cpu().numpy()[:int(c)], oidx), k
 
 
+@pytest.mark.parametrize("captured", [False, True])
 @pytest.mark.parametrize("G,N", [(200, 8), (30000, 2), (3571, 8), (12000, 8), (23000, 8), (2173, 24), (70000, 8)])
-def test_steps_back_to_back_see_each_other(G, N):
+def test_steps_back_to_back_see_each_other(G, N, captured):
     """Incremental steps without synchronisation between them, at sizes on either side of where a step
     overlaps the one before it."""
     dev = torch.device("cuda:0")
@@ -74,10 +75,23 @@ def test_steps_back_to_back_see_each_other(G, N):
     state = torch.empty(sr.sr_incr_state_bytes(G, N, steps), dtype=torch.uint8, device=dev)
     mean = torch.empty((steps, G), dtype=torch.float64, device=dev)
     stop = torch.empty((steps, G), dtype=torch.uint8, device=dev)
+
+    def episode():
+        sr.sr_incr_init(state, G, N, steps)
+        for t in range(steps):
+            sr.sr_gate_step_incremental(state, given[t], 0.3, mean=mean[t], stop=stop[t])
+
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                episode()
+            graph.replay()
+        else:
+            episode()
     torch.cuda.synchronize()
-    sr.sr_incr_init(state, G, N, steps)
-    for t in range(steps):
-        sr.sr_gate_step_incremental(state, given[t], 0.3, mean=mean[t], stop=stop[t])
     mean, stop = mean.cpu().numpy(), stop.cpu().numpy()
     some = np.unique(np.concatenate([rng.integers(0, G, 200), [0, G - 1]]))
     seqs = np.zeros((len(some), N, 12), dtype=np.int32)
