@@ -17,6 +17,7 @@
 //            occurrences gets a row of match words instead, and the stream names the row.
 //            Bounds of the pair's distance fall out of the look-ups: the columns without any
 //            match in the pattern from below, the differing positions from above.
+//   matches  pairs with few matches get their distance from these alone, a warp each.
 //   bin      team shape of every pair (what the band of its bounds costs at least, see
 //            shape_of_pair) and bin counts.
 //   order    counting sort of the pairs by bin: longest warp tasks first, one team
@@ -83,6 +84,7 @@ struct PairDesc {          // 16 bytes
 struct Ctl {               // control block in the workspace
     unsigned long long work;                   // lane-time of all pairs, about
     int32_t open;                              // and how many they are
+    int32_t few;                               // pairs for multi_matches_kernel, listed where the order goes later
     int32_t hist[kNumBins];
     int32_t fill[kNumBins];                    // what comes before here starts at zero
     int32_t start[kNumBins];
@@ -318,6 +320,11 @@ __device__ __forceinline__ uint32_t set_halves(uint32_t x) {
     return (((x & 0x7FFF7FFFu) + 0x7FFF7FFFu) | x) & 0x80008000u;
 }
 
+constexpr int kMostMatches = 32;           // matches off the main diagonal that multi_matches_kernel has lanes for
+// Whether a pattern of m positions has so few repeated symbols that its pairs may have few matches: 1024 uniform
+// tokens have three or four (of a vocabulary of 32 000 sixteen), as long a text more than a hundred, one of 48 words four.
+__device__ __forceinline__ bool few_repeats(int repeats, int m) { return 32 * repeats <= m + 64; }
+
 // One CTA per pattern.  Per text it also counts the columns whose symbol does not occur in the
 // pattern at all and the positions at which text and pattern differ: bounds of the pair's distance that
 // cost next to nothing here.  Where they meet the pair is done.
@@ -532,7 +539,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     if (tid >= 32) return;                             // descriptors: the texts' threads are in the first warp
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
-    int work = 0;
+    int work = 0, few = -1;
     if (tid < ntxt) {
         const int j = s_txt[tid], n = s_len[tid];
         // the removed prefix is a multiple of four symbols (the match stream is read in 8-byte
@@ -552,19 +559,249 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         if (lower < upper) {                          // otherwise that is the distance
             const int n_rows = min(s_repeats[3], W.row_cap);
             d.bin = ((uint32_t)strip << kStripShift) | ((uint32_t)n_rows << kRowsShift) | kNeedsDp | (s_repeats[0] > n_rows ? kHasChains : 0u);
-            const PairSize z = size_of_desc(d);
-            work = work_of_pair(z.m, z.n, z.lb, z.ub);
         }
         descs[idx] = d;
         if (kDecide || lower == upper) dist_out[idx] = lower;
+        if (lower < upper && upper - lower <= kMostMatches && few_repeats(s_repeats[0], m)) {
+            few = (int)idx;
+        } else if (lower < upper) {
+            const PairSize z = size_of_desc(d);
+            work = work_of_pair(z.m, z.n, z.lb, z.ub);
+        }
     }
-    if (!kDecide && !W.alone) {                       // decide mode counts the pairs it keeps later
+    if (W.alone) return;                              // the CTA that orders the batch counts for itself
+    const unsigned listed = __ballot_sync(0xFFFFFFFFu, few >= 0);
+    if (listed) {
+        int at = 0;
+        if (tid == 0) at = atomicAdd(&ctl->few, __popc(listed));
+        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(listed & ((1u << tid) - 1u));
+        if (few >= 0) reinterpret_cast<int32_t*>(ws + W.off_order)[at] = few;
+    }
+    if (!kDecide) {                                   // decide mode counts the pairs it keeps later
         const int open = __popc(__ballot_sync(0xFFFFFFFFu, work > 0));
         work = __reduce_add_sync(0xFFFFFFFFu, work);
         if (tid == 0 && open) {
             atomicAdd(&ctl->work, (unsigned long long)work);
             atomicAdd(&ctl->open, open);
         }
+    }
+}
+
+// --------------------------------------------------------------------- matches
+// Pairs with few matches.  Besides the main diagonal, on which the two prefixes are compared place by
+// place, two rollouts over a large vocabulary have hardly a symbol in common: a pair of 1024 uniform
+// tokens out of 150 000 has seven matches where a matrix of a million cells says the same.  Between two
+// matches (c, p) that it uses, a path either goes straight, max(columns, rows) edits, or by way of
+// the main diagonal, where it pays for the places that differ; so the distance is a shortest path over the
+// matches off the diagonal (sparse dynamic programming: Eppstein, Galil, Giancarlo and Italiano 1992), one
+// lane each.  A pair whose bounds are further apart than there are lanes has more such columns than that, and the
+// recurrence has it; the others are listed by prep, a warp each.
+// 1024 groups of 8 prefixes of 256..1024 uniform tokens: the recurrence took 174 us for them, this 37 us cold (20 M warp
+// instructions, 1100 a pair: a third to look through the stream, a third for the rows of repeated symbols), and the
+// whole gate went from 270 to 125 us.
+constexpr int kSpan = 128;                               // columns a warp looks through a trip
+constexpr int kSpans = SR_MAX_K / kSpan + 1;             // and one that begins where the longest text ends
+constexpr int kMatchWarps = 8;
+
+// The columns of a pair's stream with matches off the main diagonal, with the column's stream entry (upper half), in
+// `entries`, and in `differ` a bit for every column from `strip` on that differs from the pattern: column
+// strip + 128 s + 4 l + k in bit l of word k of differ[s].  Returns the number of those columns, or more than
+// there are lanes for.
+__device__ __forceinline__ int find_matches(const uint2* stream, const uint2* text, const uint2* pat, int m, int n, int strip,
+                                            uint4* differ, uint32_t* entries) {
+    const int lane = threadIdx.x & 31;
+    int found = 0;
+    auto fetch = [&](int s) {
+        const int q = (strip >> 2) + 32 * s + lane;
+        return 4 * q < n ? __ldg(stream + q) : make_uint2(kLocNone * 0x10001u, kLocNone * 0x10001u);
+    };
+    uint2 ahead[2] = {fetch(0), fetch(1)};
+    for (int s = 0; strip + kSpan * s < n; ++s) {
+        const int q = (strip >> 2) + 32 * s + lane;
+        const int left = min(max(n - 4 * q, 0), 4), both = min(left, max(m - 4 * q, 0));   // columns that exist, and of those with a row
+        const uint2 v = ahead[0];
+        ahead[0] = ahead[1];
+        ahead[1] = fetch(s + 2);
+        const uint32_t at0 = (uint32_t)(4 * q * 0x10001 + 0x10000), at1 = at0 + 0x20002u;   // the places on the main diagonal
+        uint32_t off0 = set_halves(v.x ^ at0), off1 = set_halves(v.y ^ at1);
+        uint32_t d0 = off0, d1 = off1;
+        if ((v.x | v.y) & (kLocRow * 0x10001u)) {      // a symbol that occurs more than once: the names tell
+            const uint2 x = __ldg(text + q), o = __ldg(pat + q);
+            d0 = set_halves(x.x ^ o.x);
+            d1 = set_halves(x.y ^ o.y);
+        }
+        off0 &= set_halves(v.x ^ (kLocNone * 0x10001u));
+        off1 &= set_halves(v.y ^ (kLocNone * 0x10001u));
+        if (left < 4) {
+            off0 = left > 1 ? off0 : (left == 1 ? off0 & 0xFFFFu : 0u);
+            off1 = left == 3 ? off1 & 0xFFFFu : 0u;
+        }
+        if (both < 4) {
+            d0 = both > 1 ? d0 : (both == 1 ? d0 & 0xFFFFu : 0u);
+            d1 = both == 3 ? d1 & 0xFFFFu : 0u;
+        }
+        const unsigned b0 = __ballot_sync(0xFFFFFFFFu, (d0 & 0x8000u) != 0u), b1 = __ballot_sync(0xFFFFFFFFu, (d0 >> 31) != 0u);
+        const unsigned b2 = __ballot_sync(0xFFFFFFFFu, (d1 & 0x8000u) != 0u), b3 = __ballot_sync(0xFFFFFFFFu, (d1 >> 31) != 0u);
+        if (lane == 0) differ[s] = make_uint4(b0, b1, b2, b3);
+        if (!__any_sync(0xFFFFFFFFu, (off0 | off1) != 0u)) continue;
+        const unsigned o0 = __ballot_sync(0xFFFFFFFFu, (off0 & 0x8000u) != 0u), o1 = __ballot_sync(0xFFFFFFFFu, (off0 >> 31) != 0u);
+        const unsigned o2 = __ballot_sync(0xFFFFFFFFu, (off1 & 0x8000u) != 0u), o3 = __ballot_sync(0xFFFFFFFFu, (off1 >> 31) != 0u);
+        const unsigned under = (1u << lane) - 1u;
+        int at = found + __popc(o0 & under) + __popc(o1 & under) + __popc(o2 & under) + __popc(o3 & under);
+        found += __popc(o0) + __popc(o1) + __popc(o2) + __popc(o3);
+        if (found > kMostMatches) return found;
+        if (off0 & 0x8000u) entries[at++] = (uint32_t)(4 * q) | (v.x << 16);      // by column
+        if (off0 >> 31) entries[at++] = (uint32_t)(4 * q + 1) | (v.x & 0xFFFF0000u);
+        if (off1 & 0x8000u) entries[at++] = (uint32_t)(4 * q + 2) | (v.y << 16);
+        if (off1 >> 31) entries[at++] = (uint32_t)(4 * q + 3) | (v.y & 0xFFFF0000u);
+    }
+    __syncwarp();
+    return found;
+}
+
+// The distance of a pair from what find_matches found.  upper: the distance along the main diagonal.  Negative: more
+// matches than there are lanes for.
+__device__ __forceinline__ int distance_by_matches(uint32_t* entries, int count, const uint4* differ, const uint32_t* rows, int row_words,
+                                                   int m, int n, int strip, int upper) {
+    const int lane = threadIdx.x & 31;
+    const int lo = min(m, n);
+    // every entry's matches: one position, or those of a mask row
+    uint32_t node = lane < count ? entries[lane] : 0u;
+    const bool row = lane < count && (node >> 16) >= kLocRow;
+    if (__any_sync(0xFFFFFFFFu, lane < count && (node >> 16) >= kLocChain)) return -1;
+    int total = count;
+    unsigned todo = __ballot_sync(0xFFFFFFFFu, row);
+    if (todo) {
+        const bool single = lane < count && !row;
+        const unsigned singles = __ballot_sync(0xFFFFFFFFu, single);
+        total = __popc(singles);
+        if (single) entries[__popc(singles & ((1u << lane) - 1u))] = node;
+        while (todo) {                                 // eight rows on their way before the first is looked at
+            uint32_t bits[8], column[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                bits[k] = column[k] = 0u;
+                if (todo == 0u) continue;
+                const uint32_t e = __shfl_sync(0xFFFFFFFFu, node, __ffs(todo) - 1);
+                todo &= todo - 1u;
+                column[k] = e & 0xFFFFu;
+                if (lane < row_words) bits[k] = __ldg(rows + ((e >> 16) & 0x3FFFu) * row_words + lane);
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                while (__any_sync(0xFFFFFFFFu, bits[k] != 0u)) {
+                    const int p = bits[k] ? 32 * lane + __ffs(bits[k]) - 1 : -1;
+                    bits[k] &= bits[k] - 1u;
+                    const bool use = p >= strip && p != (int)column[k];
+                    const unsigned b = __ballot_sync(0xFFFFFFFFu, use);
+                    const int at = total + __popc(b & ((1u << lane) - 1u));
+                    total += __popc(b);
+                    if (use && at < kMostMatches) entries[at] = column[k] | ((uint32_t)p << 16);
+                }
+            }
+            if (total > kMostMatches) return -1;
+        }
+        if (total == 0) return upper;
+        __syncwarp();
+        // by column again
+        const uint32_t own = lane < total ? entries[lane] : 0xFFFFFFFFu;
+        int rank = 0;
+        for (int l = 0; l < total; ++l) {
+            const uint32_t other = __shfl_sync(0xFFFFFFFFu, own, l);
+            rank += (other & 0xFFFFu) < (own & 0xFFFFu) || ((other & 0xFFFFu) == (own & 0xFFFFu) && l < lane);
+        }
+        if (lane < total) entries[rank] = own;
+        __syncwarp();
+    }
+    __syncwarp();
+    node = lane < total ? entries[lane] : (uint32_t)strip * 0x10001u;
+    const int c = (int)(node & 0xFFFFu), p = (int)(node >> 16);
+    // places that differ before x
+    int before = 0;
+    if (lane < kSpans && strip + kSpan * lane < n) {
+        const uint4 d = differ[lane];
+        before = __popc(d.x) + __popc(d.y) + __popc(d.z) + __popc(d.w);
+    }
+#pragma unroll
+    for (int d = 1; d < 16; d <<= 1) {
+        const int up = __shfl_up_sync(0xFFFFFFFFu, before, d);
+        if (lane >= d) before += up;
+    }
+    auto differing = [&](int x) {
+        const int rel = x - strip, s = rel / kSpan, l = (rel % kSpan) >> 2, k = rel & 3;
+        const uint4 d = differ[s];
+        const uint32_t under = (1u << l) - 1u, with = under | (1u << l);
+        const int sum = __shfl_sync(0xFFFFFFFFu, before, max(s - 1, 0));
+        return (s > 0 ? sum : 0) + __popc(d.x & (k > 0 ? with : under)) + __popc(d.y & (k > 1 ? with : under)) +
+               __popc(d.z & (k > 2 ? with : under)) + __popc(d.w & under);
+    };
+    const int off = abs(c - p);
+    const int enter = min(c, p), leave = max(c, p) + 1;  // the last place of the diagonal before the match, the first after it
+    const int at_enter = differing(enter), at_leave = differing(min(leave, lo)), at_end = differing(lo);
+    int cost = off + at_enter;                            // up to the match and through it
+    for (int l = 0; l + 1 < total; ++l) {
+        const uint32_t from = __shfl_sync(0xFFFFFFFFu, node, l);
+        const uint32_t paid = __shfl_sync(0xFFFFFFFFu, (uint32_t)cost | ((uint32_t)at_leave << 16), l);
+        const int fc = (int)(from & 0xFFFFu), fp = (int)(from >> 16);
+        int step = max(c - fc, p - fp) - 1;
+        if (max(fc, fp) < enter) step = min(step, abs(fc - fp) + at_enter - (int)(paid >> 16) + off);
+        if (c > fc && p > fp) cost = min(cost, (int)(paid & 0xFFFFu) + step);
+    }
+    int last = max(n - c, m - p) - 1;
+    if (leave <= lo) last = min(last, off + at_end - at_leave + abs(n - m));
+    const int d = lane < total ? cost + last : upper;
+    return min(__reduce_min_sync(0xFFFFFFFFu, d), upper);
+}
+
+// A warp goes through listed pairs as many places apart as there are warps.  decide: the bounds that this leaves are the
+// bound kernel's to add up.
+__global__ void __launch_bounds__(32 * kMatchWarps)
+multi_matches_kernel(unsigned char* ws, MultiWs W, int N, bool decide, int32_t* dist_out) {
+    grid_begin();
+    __shared__ uint4 s_differ[kMatchWarps][kSpans];
+    __shared__ uint32_t s_entries[kMatchWarps][kMostMatches];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, P = pairs_of(N);
+    PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
+    Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
+    const int32_t* list = reinterpret_cast<const int32_t*>(ws + W.off_order);
+    unsigned long long work = 0ull;
+    int still_open = 0;
+    const int few = ctl->few;
+    for (int e = blockIdx.x * kMatchWarps + warp; e < few; e += gridDim.x * kMatchWarps) {
+        const int idx = list[e];
+        const PairDesc d = descs[idx];
+        const int upper = (int)(d.lower >> 16);
+        int dist = -1;
+        const int m = (int)(d.mn & 0xFFFFu), n = (int)(d.mn >> 16), strip = (int)((d.bin >> kStripShift) & 0x3FFu);
+        const int g = (int)(d.pat_row / (uint32_t)W.patterns), i = (int)d.pat_row - g * W.patterns;
+        const int pr = kPairs.v[N][idx - g * P], j = (pr & 0xFF) + (pr >> 8) - i;
+        const uint16_t* names = reinterpret_cast<const uint16_t*>(ws + W.off_names) + (size_t)g * N * W.pitch;
+        __syncwarp();                              // the pair before has been read
+        const int count = find_matches(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(ws + W.off_loc) + (size_t)idx * W.pitch),
+                                       reinterpret_cast<const uint2*>(names + j * W.pitch), reinterpret_cast<const uint2*>(names + i * W.pitch),
+                                       m, n, strip, s_differ[warp], s_entries[warp]);
+        if (count == 0)
+            dist = upper;
+        else if (count <= kMostMatches)
+            dist = distance_by_matches(s_entries[warp], count, s_differ[warp],
+                                       reinterpret_cast<const uint32_t*>(ws + W.off_rows) + (size_t)d.pat_row * (W.row_cap * W.row_words),
+                                       W.row_words, m, n, strip, upper);
+        if (dist >= 0) {
+            if (lane == 0) {
+                descs[idx].bin = 0u;
+                descs[idx].lower = (uint32_t)dist * 0x10001u;
+                dist_out[idx] = dist;
+            }
+        } else {
+            const PairSize z = size_of_desc(d);
+            work += (unsigned long long)work_of_pair(z.m, z.n, z.lb, z.ub);
+            ++still_open;
+        }
+    }
+    if (decide) return;                               // counted later, with what the threshold still allows
+    if (still_open && lane == 0) {
+        atomicAdd(&ctl->work, work);
+        atomicAdd(&ctl->open, still_open);
     }
 }
 
@@ -610,6 +847,7 @@ multi_bin_kernel(PairDesc* descs, Ctl* ctl, int n_pairs, int warps) {
     grid_begin();
     __shared__ int32_t s_hist[kNumBins];
     for (int b = threadIdx.x; b < kNumBins; b += kOrderThreads) s_hist[b] = 0;
+    if (ctl->open == 0) return;                        // bounds and matches have settled the whole batch
     const ShapeGoal goal = shape_goal(ctl->work, ctl->open, warps);
     __syncthreads();
     const int idx = blockIdx.x * kOrderThreads + threadIdx.x;
@@ -680,6 +918,10 @@ multi_order_kernel(PairDesc* descs, int32_t* order, Ctl* ctl, int n_pairs, int w
         }
         __syncthreads();
     } else {
+        if (ctl->open == 0) {
+            if (blockIdx.x == 0 && t == 0) ctl->task_counter = ctl->total_tasks = 0;
+            return;
+        }
         s_hist[2 * t] = ctl->hist[2 * t];
         s_hist[2 * t + 1] = ctl->hist[2 * t + 1];
         const int idx = blockIdx.x * kOrderThreads + t;
@@ -1231,6 +1473,8 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const int gpb = P <= kGroupThreads ? kGroupThreads / P : 1;
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     int32_t* order = reinterpret_cast<int32_t*>(ws + W.off_order);
+    if (!alone)
+        SR_LAUNCH("multi_matches_kernel", multi_matches_kernel, min((n_pairs + kMatchWarps - 1) / kMatchWarps, 16 * sms), 32 * kMatchWarps, 0, s, ws, W, a.N, decide, dist);
     if (decide) {
         SR_LAUNCH("multi_bound_kernel", multi_bound_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, descs, ctl, flag, exact, gpb, alone);
     }
