@@ -32,6 +32,10 @@
 //   finish   one thread per pair for the terms, one per group: ordered fp64 sum of the normalised
 //            terms, threshold, outputs.
 //
+// A batch that leaves most of the GPU idle (runs_in_pairs) takes the names and one launch: prep keeps streams and rows in
+// shared memory, the distances are computed right there, both ways from the ends of the text, and the
+// last CTA of a group evaluates it.
+//
 // Band.  With bounds lb <= d <= ub of a pair's distance an optimal alignment stays on a band of
 // diagonals (band_of), and where the bounds meet nothing is left to compute.  Rollouts that have
 // converged differ in few positions: their bands are narrow, and the T lanes of a team form a ring that
@@ -245,9 +249,10 @@ __device__ __forceinline__ int clamp_len(const int32_t* lens, size_t idx, int K,
 // length.  Bound: the latency between the barriers here (three CTAs of 64 KB per SM), instruction issue in prep.
 constexpr uint32_t kHashMul = 0x9E3779B1u;
 constexpr int kMaxTexts = SR_MAX_N / 2;        // texts a pattern is paired with
+constexpr int kMaxPairs = SR_MAX_N * (SR_MAX_N - 1) / 2;
 
 __global__ void __launch_bounds__(1024)
-multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int table_log, int g_base) {
+multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int table_log, int g_base, int32_t* arrived) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_len[SR_MAX_N];
     const int N = a.N, K = a.K, tid = threadIdx.x, nthr = blockDim.x;
@@ -263,6 +268,7 @@ multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int
         s_len[tid] = clamp_len(a.lens, (size_t)g * N + tid, K, neg);
         if (neg && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
     }
+    if (arrived && tid == 0) arrived[g] = 0;           // see finish_last
     __syncthreads();
     const int shift = 32 - table_log;
 #pragma unroll 4
@@ -320,22 +326,456 @@ __device__ __forceinline__ uint32_t set_halves(uint32_t x) {
     return (((x & 0x7FFF7FFFu) + 0x7FFF7FFFu) | x) & 0x80008000u;
 }
 
-constexpr int kMostMatches = 32;           // matches off the main diagonal that multi_matches_kernel has lanes for
+// ------------------------------------------------------------------ recurrence
+__device__ __forceinline__ uint32_t shl_clamp(uint32_t v, uint32_t s) {
+    uint32_t r;   // PTX shl clamps shift amounts above 31: the result is 0
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));
+    return r;
+}
+
+// One bit-vector column step over the R blocks a lane owns.  `Eq` are the column's match
+// words, (inP, inM) the pre-shift horizontal delta words of the
+// block above (only their top bits matter); returns this lane's last block's words in
+// (inP, inM).
+template <int R>
+__device__ __forceinline__ void column_step(const uint32_t (&Eq)[R],
+                                            uint32_t (&Pv)[R], uint32_t (&Mv)[R],
+                                            uint32_t& inP, uint32_t& inM, uint32_t two) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const uint32_t pv = Pv[r], mv = Mv[r];
+        const uint32_t hm = inM >> 31;
+        // D0: the cells whose value equals that of their upper left neighbour
+        const uint32_t D0 = ((((Eq[r] | hm) & pv) + pv) ^ pv) | (Eq[r] | mv | hm);
+        const uint32_t Ph = mv | ~(D0 | pv);
+        const uint32_t Mh = pv & D0;
+        const uint32_t Phs = __funnelshift_l(inP, Ph, 1);
+        // `two` holds 2 but is a run-time value, so this shift-and-insert is a multiply-add:
+        // it issues on the FMA pipe and leaves the integer ALU, the bottleneck, one
+        // instruction lighter per block (measured: 8 % faster than a second funnel shift)
+        const uint32_t Mhs = Mh * two + hm;              // (Mh << 1) | hm
+        Pv[r] = Mhs | ~(D0 | Phs);
+        Mv[r] = Phs & D0;
+        inP = Ph;
+        inM = Mh;
+    }
+}
+
+// --------------------------------------------------------------------- matches
+// Pairs with few matches.  Besides the main diagonal, on which the two prefixes are compared place by
+// place, two rollouts over a large vocabulary have hardly a symbol in common: a pair of 1024 uniform
+// tokens out of 150 000 has seven matches where a matrix of a million cells says the same.  Between two
+// matches (c, p) that it uses, a path either goes straight, max(columns, rows) edits, or by way of
+// the main diagonal, where it pays for the places that differ; so the distance is a shortest path over the
+// matches off the diagonal (sparse dynamic programming: Eppstein, Galil, Giancarlo and Italiano 1992), one
+// lane each.  A pair whose bounds are further apart than there are lanes has more such columns than that, and the
+// recurrence has it; the others are listed by prep, a warp each.
+// 1024 groups of 8 prefixes of 256..1024 uniform tokens: the recurrence took 174 us for them, this 37 us cold (20 M warp
+// instructions, 1100 a pair: a third to look through the stream, a third for the rows of repeated symbols), and the
+// whole gate went from 270 to 125 us.
+constexpr int kMostMatches = 32;                         // a lane each
 // Whether a pattern of m positions has so few repeated symbols that its pairs may have few matches: 1024 uniform
 // tokens have three or four (of a vocabulary of 32 000 sixteen), as long a text more than a hundred, one of 48 words four.
 __device__ __forceinline__ bool few_repeats(int repeats, int m) { return 32 * repeats <= m + 64; }
+constexpr int kSpan = 128;                               // columns a warp looks through a trip
+constexpr int kSpans = SR_MAX_K / kSpan + 1;             // and one that begins where the longest text ends
+constexpr int kMatchWarps = 8;
+
+// The columns of a pair's stream with matches off the main diagonal, with the column's stream entry (upper half), in
+// `entries`, and in `differ` a bit for every column from `strip` on that differs from the pattern: column
+// strip + 128 s + 4 l + k in bit l of word k of differ[s].  Returns the number of those columns, or more than
+// there are lanes for.
+// (kShared: the stream and, below, the rows are in shared memory.)
+template <bool kShared>
+__device__ __forceinline__ int find_matches(const uint2* stream, const uint2* text, const uint2* pat, int m, int n, int strip,
+                                            uint4* differ, uint32_t* entries) {
+    const int lane = threadIdx.x & 31;
+    int found = 0;
+    auto fetch = [&](int s) {
+        const int q = (strip >> 2) + 32 * s + lane;
+        return 4 * q < n ? (kShared ? stream[q] : __ldg(stream + q)) : make_uint2(kLocNone * 0x10001u, kLocNone * 0x10001u);
+    };
+    uint2 ahead[2] = {fetch(0), fetch(1)};
+    for (int s = 0; strip + kSpan * s < n; ++s) {
+        const int q = (strip >> 2) + 32 * s + lane;
+        const int left = min(max(n - 4 * q, 0), 4), both = min(left, max(m - 4 * q, 0));   // columns that exist, and of those with a row
+        const uint2 v = ahead[0];
+        ahead[0] = ahead[1];
+        ahead[1] = fetch(s + 2);
+        const uint32_t at0 = (uint32_t)(4 * q * 0x10001 + 0x10000), at1 = at0 + 0x20002u;   // the places on the main diagonal
+        uint32_t off0 = set_halves(v.x ^ at0), off1 = set_halves(v.y ^ at1);
+        uint32_t d0 = off0, d1 = off1;
+        if ((v.x | v.y) & (kLocRow * 0x10001u)) {      // a symbol that occurs more than once: the names tell
+            const uint2 x = __ldg(text + q), o = __ldg(pat + q);
+            d0 = set_halves(x.x ^ o.x);
+            d1 = set_halves(x.y ^ o.y);
+        }
+        off0 &= set_halves(v.x ^ (kLocNone * 0x10001u));
+        off1 &= set_halves(v.y ^ (kLocNone * 0x10001u));
+        if (left < 4) {
+            off0 = left > 1 ? off0 : (left == 1 ? off0 & 0xFFFFu : 0u);
+            off1 = left == 3 ? off1 & 0xFFFFu : 0u;
+        }
+        if (both < 4) {
+            d0 = both > 1 ? d0 : (both == 1 ? d0 & 0xFFFFu : 0u);
+            d1 = both == 3 ? d1 & 0xFFFFu : 0u;
+        }
+        const unsigned b0 = __ballot_sync(0xFFFFFFFFu, (d0 & 0x8000u) != 0u), b1 = __ballot_sync(0xFFFFFFFFu, (d0 >> 31) != 0u);
+        const unsigned b2 = __ballot_sync(0xFFFFFFFFu, (d1 & 0x8000u) != 0u), b3 = __ballot_sync(0xFFFFFFFFu, (d1 >> 31) != 0u);
+        if (lane == 0) differ[s] = make_uint4(b0, b1, b2, b3);
+        if (!__any_sync(0xFFFFFFFFu, (off0 | off1) != 0u)) continue;
+        const unsigned o0 = __ballot_sync(0xFFFFFFFFu, (off0 & 0x8000u) != 0u), o1 = __ballot_sync(0xFFFFFFFFu, (off0 >> 31) != 0u);
+        const unsigned o2 = __ballot_sync(0xFFFFFFFFu, (off1 & 0x8000u) != 0u), o3 = __ballot_sync(0xFFFFFFFFu, (off1 >> 31) != 0u);
+        const unsigned under = (1u << lane) - 1u;
+        int at = found + __popc(o0 & under) + __popc(o1 & under) + __popc(o2 & under) + __popc(o3 & under);
+        found += __popc(o0) + __popc(o1) + __popc(o2) + __popc(o3);
+        if (found > kMostMatches) return found;
+        if (off0 & 0x8000u) entries[at++] = (uint32_t)(4 * q) | (v.x << 16);      // by column
+        if (off0 >> 31) entries[at++] = (uint32_t)(4 * q + 1) | (v.x & 0xFFFF0000u);
+        if (off1 & 0x8000u) entries[at++] = (uint32_t)(4 * q + 2) | (v.y << 16);
+        if (off1 >> 31) entries[at++] = (uint32_t)(4 * q + 3) | (v.y & 0xFFFF0000u);
+    }
+    __syncwarp();
+    return found;
+}
+
+// The distance of a pair from what find_matches found.  upper: the distance along the main diagonal.  Negative: more
+// matches than there are lanes for.
+template <bool kShared>
+__device__ __forceinline__ int distance_by_matches(uint32_t* entries, int count, const uint4* differ, const uint32_t* rows, int row_words,
+                                                   int m, int n, int strip, int upper) {
+    const int lane = threadIdx.x & 31;
+    const int lo = min(m, n);
+    // every entry's matches: one position, or those of a mask row
+    uint32_t node = lane < count ? entries[lane] : 0u;
+    const bool row = lane < count && (node >> 16) >= kLocRow;
+    if (__any_sync(0xFFFFFFFFu, lane < count && (node >> 16) >= kLocChain)) return -1;
+    int total = count;
+    unsigned todo = __ballot_sync(0xFFFFFFFFu, row);
+    if (todo) {
+        const bool single = lane < count && !row;
+        const unsigned singles = __ballot_sync(0xFFFFFFFFu, single);
+        total = __popc(singles);
+        if (single) entries[__popc(singles & ((1u << lane) - 1u))] = node;
+        while (todo) {                                 // eight rows on their way before the first is looked at
+            uint32_t bits[8], column[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                bits[k] = column[k] = 0u;
+                if (todo == 0u) continue;
+                const uint32_t e = __shfl_sync(0xFFFFFFFFu, node, __ffs(todo) - 1);
+                todo &= todo - 1u;
+                column[k] = e & 0xFFFFu;
+                const uint32_t* row = rows + ((e >> 16) & 0x3FFFu) * row_words + lane;
+                if (lane < row_words) bits[k] = kShared ? *row : __ldg(row);
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                while (__any_sync(0xFFFFFFFFu, bits[k] != 0u)) {
+                    const int p = bits[k] ? 32 * lane + __ffs(bits[k]) - 1 : -1;
+                    bits[k] &= bits[k] - 1u;
+                    const bool use = p >= strip && p != (int)column[k];
+                    const unsigned b = __ballot_sync(0xFFFFFFFFu, use);
+                    const int at = total + __popc(b & ((1u << lane) - 1u));
+                    total += __popc(b);
+                    if (use && at < kMostMatches) entries[at] = column[k] | ((uint32_t)p << 16);
+                }
+            }
+            if (total > kMostMatches) return -1;
+        }
+        if (total == 0) return upper;
+        __syncwarp();
+        // by column again
+        const uint32_t own = lane < total ? entries[lane] : 0xFFFFFFFFu;
+        int rank = 0;
+        for (int l = 0; l < total; ++l) {
+            const uint32_t other = __shfl_sync(0xFFFFFFFFu, own, l);
+            rank += (other & 0xFFFFu) < (own & 0xFFFFu) || ((other & 0xFFFFu) == (own & 0xFFFFu) && l < lane);
+        }
+        if (lane < total) entries[rank] = own;
+        __syncwarp();
+    }
+    __syncwarp();
+    node = lane < total ? entries[lane] : (uint32_t)strip * 0x10001u;
+    const int c = (int)(node & 0xFFFFu), p = (int)(node >> 16);
+    // places that differ before x
+    int before = 0;
+    if (lane < kSpans && strip + kSpan * lane < n) {
+        const uint4 d = differ[lane];
+        before = __popc(d.x) + __popc(d.y) + __popc(d.z) + __popc(d.w);
+    }
+#pragma unroll
+    for (int d = 1; d < 16; d <<= 1) {
+        const int up = __shfl_up_sync(0xFFFFFFFFu, before, d);
+        if (lane >= d) before += up;
+    }
+    auto differing = [&](int x) {
+        const int rel = x - strip, s = rel / kSpan, l = (rel % kSpan) >> 2, k = rel & 3;
+        const uint4 d = differ[s];
+        const uint32_t under = (1u << l) - 1u, with = under | (1u << l);
+        const int sum = __shfl_sync(0xFFFFFFFFu, before, max(s - 1, 0));
+        return (s > 0 ? sum : 0) + __popc(d.x & (k > 0 ? with : under)) + __popc(d.y & (k > 1 ? with : under)) +
+               __popc(d.z & (k > 2 ? with : under)) + __popc(d.w & under);
+    };
+    const int off = abs(c - p);
+    const int enter = min(c, p), leave = max(c, p) + 1;  // the last place of the diagonal before the match, the first after it
+    const int at_enter = differing(enter), at_leave = differing(min(leave, lo)), at_end = differing(lo);
+    int cost = off + at_enter;                            // up to the match and through it
+    for (int l = 0; l + 1 < total; ++l) {
+        const uint32_t from = __shfl_sync(0xFFFFFFFFu, node, l);
+        const uint32_t paid = __shfl_sync(0xFFFFFFFFu, (uint32_t)cost | ((uint32_t)at_leave << 16), l);
+        const int fc = (int)(from & 0xFFFFu), fp = (int)(from >> 16);
+        int step = max(c - fc, p - fp) - 1;
+        if (max(fc, fp) < enter) step = min(step, abs(fc - fp) + at_enter - (int)(paid >> 16) + off);
+        if (c > fc && p > fp) cost = min(cost, (int)(paid & 0xFFFFu) + step);
+    }
+    int last = max(n - c, m - p) - 1;
+    if (leave <= lo) last = min(last, off + at_end - at_leave + abs(n - m));
+    const int d = lane < total ? cost + last : upper;
+    return min(__reduce_min_sync(0xFFFFFFFFu, d), upper);
+}
+
+// ------------------------------------------------------------------- both ends
+// Pairs by the latency of their columns, for batches that leave most of the GPU idle: one team of lanes runs the
+// recurrence over the first half of the text's columns, another one next to it over the rest from the end
+// backwards (both sequences reversed), so that the chain of columns is half as long; where they meet, the distance is
+// the least sum over the rows of what the two paid (Hirschberg 1975).  A team has T <= 16 lanes of R blocks each, a
+// lane for every stripe; a warp has 16 / T pairs.  Stream and mask rows are in shared memory, where no first use of
+// a row costs a trip to L2, and what a column needs is as good as computed in the stream's entry.
+// Bound: the latency of the columns' chain of operations, then the integer pipe.
+
+// Rows and columns from which looking for few matches costs less than they do here.
+constexpr int kWorthMatches = 512;
+
+// What a stream entry is here: a position, kLocNone, kWideRow | first word of a mask row, or kWideChain | position.
+constexpr uint32_t kWideRow = 0x80000000u, kWideChain = 0xC0000000u;
+__device__ __forceinline__ uint32_t wide_entry(uint32_t e, int row_words) {
+    if (e < kLocRow) return e;
+    return e < kLocChain ? kWideRow | ((e & 0x3FFFu) * (uint32_t)row_words) : kWideChain | (e & 0x3FFFu);
+}
+
+// Loads a lane's R words of a mask row where the entry names one, without a branch.
+template <int R>
+__device__ __forceinline__ void load_wide_row(uint32_t entry, uint32_t row, uint32_t (&Eq)[R]) {
+    static_assert(R >= 1 && R <= 3, "");
+    if constexpr (R == 1)
+        asm volatile("{ .reg .pred p; setp.lt.s32 p, %1, 0xC0000000; @p ld.shared.u32 %0, [%2]; }" : "+r"(Eq[0]) : "r"(entry), "r"(row));
+    else if constexpr (R == 2)
+        asm volatile("{ .reg .pred p; setp.lt.s32 p, %2, 0xC0000000; @p ld.shared.u32 %0, [%3]; @p ld.shared.u32 %1, [%3 + 4]; }"
+            : "+r"(Eq[0]), "+r"(Eq[1]) : "r"(entry), "r"(row));
+    else
+        asm volatile("{ .reg .pred p; setp.lt.s32 p, %3, 0xC0000000; @p ld.shared.u32 %0, [%4]; @p ld.shared.u32 %1, [%4 + 4]; "
+            "@p ld.shared.u32 %2, [%4 + 8]; }"
+            : "+r"(Eq[0]), "+r"(Eq[1]), "+r"(Eq[2]) : "r"(entry), "r"(row));
+}
+
+// The signs of four words, one a byte, the first word's on top.
+__device__ __forceinline__ uint32_t signs(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+    uint32_t a, b, r;
+    asm("prmt.b32 %0, %1, %2, 0xFB00;" : "=r"(a) : "r"(w1), "r"(w0));
+    asm("prmt.b32 %0, %1, %2, 0x00FB;" : "=r"(b) : "r"(w3), "r"(w2));
+    asm("prmt.b32 %0, %1, %2, 0x7610;" : "=r"(r) : "r"(b), "r"(a));
+    return r;
+}
+
+// The distances of a warp's pairs, each in the first lane of its 2 T lanes.  Per pair: loc, its stream (16-bit entries),
+// and wide, room for the wide one, of which it makes use afterwards; m, n: lengths; strip: common prefix to leave out (a
+// multiple of 4, of 32 where the stream names rows); live: false for lanes without a pair.  rows: the pattern's mask
+// rows, turned: the same with the order of a row's bits reversed; info: upper halves lead along the chains.
+template <int R>
+__device__ __forceinline__ int distance_from_both_ends(const uint16_t* loc, uint4* wide, const uint32_t* rows, const uint32_t* turned, int row_words,
+                                                       const uint32_t* info, bool chains, bool live, int m, int n, int strip, int tlog,
+                                                       uint32_t two) {
+    const int lane = threadIdx.x & 31, T = 1 << tlog, gl = lane & (2 * T - 1), lt = lane & (T - 1);
+    const int pad = -n & 3;                            // both are extended to whole quads of columns
+    m = live ? m + pad - strip : 0;
+    n = live ? n + pad - strip : 0;
+    const int W = (m + 31) >> 5, G = (W + R - 1) / R;  // blocks, stripes
+    const int nq = n >> 2, ahead = (nq + 1) >> 1;      // quads, and those of the half that runs forwards
+    const bool back = gl >= T, held = lt < G;
+    const int quads = back ? nq - ahead : ahead;
+    // the wide stream: quads from `ahead` on in the order in which the other half meets their columns; one without
+    // matches at either end
+    const uint2* quad = reinterpret_cast<const uint2*>(loc + strip);
+    for (int k = gl; k < nq; k += 2 * T) {
+        const uint2 q = quad[k];
+        uint32_t e[4] = {q.x & 0xFFFFu, q.x >> 16, q.y & 0xFFFFu, q.y >> 16};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) e[u] = wide_entry(e[u], row_words);
+        wide[1 + k] = k < ahead ? make_uint4(e[0], e[1], e[2], e[3]) : make_uint4(e[3], e[2], e[1], e[0]);
+    }
+    if (gl == 0) wide[0] = make_uint4(kLocNone, kLocNone, kLocNone, kLocNone);
+    if (gl == 1) wide[1 + nq] = make_uint4(kLocNone, kLocNone, kLocNone, kLocNone);
+    __syncwarp();
+    // Backwards, position strip + p is row 32 W - 1 - p: the rows beyond the pattern's end come first, and
+    // with vertical deltas of zero they hand on the +1 of row 0 as it is.
+    const uint32_t sign = back ? ~0u : 1u, four = two * two, next_column = two * 128u;
+    const uint32_t origin = back ? (uint32_t)(32 * W - 1 + strip - 32 * R * lt) : (uint32_t)-(strip + 32 * R * lt);
+    const uint32_t words = (uint32_t)__cvta_generic_to_shared(back ? turned + (row_words - (strip >> 5) - W + R * lt) : rows + ((strip >> 5) + R * lt));
+    const uint4* from = back ? wide + nq : wide + 1;   // the half's first quad
+    const int step = back ? -1 : 1, most = held ? quads : -1;
+    uint32_t Pv[R], Mv[R], endP[R], endM[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) { Pv[r] = 0xFFFFFFFFu; Mv[r] = 0u; }
+    if (back && lt == 0) Pv[0] = 0xFFFFFFFFu << (32 * W - m);
+#pragma unroll
+    for (int r = 0; r < R; ++r) { endP[r] = Pv[r]; endM[r] = Mv[r]; }
+    // the quad for iteration j: none before the lane's first; after its last any will do
+    auto fetch = [&](int j) { return from[step * min(max(j - lt, -1), most)]; };
+    auto match = [&](const uint4& q, uint32_t (&Eq)[4][R]) {
+        const uint32_t e[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t d0 = e[u] * sign + origin;
+#pragma unroll
+            for (int r = 0; r < R; ++r) Eq[u][r] = shl_clamp(1u, d0 - 32u * r);    // 0 for rows and chains
+            load_wide_row<R>(e[u], e[u] * four + words, Eq[u]);
+        }
+        if (!chains) return;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (e[u] < kWideChain) continue;
+            uint32_t p = e[u] & 0x3FFFu;
+            for (int hop = 0; hop < SR_MAX_K && p < (uint32_t)SR_MAX_K; ++hop) {   // a chain ends at 0xFFFF
+                const uint32_t d0 = p * sign + origin;
+#pragma unroll
+                for (int r = 0; r < R; ++r) Eq[u][r] |= shl_clamp(1u, d0 - 32u * r);
+                p = info[p] >> 16;
+            }
+        }
+    };
+    uint32_t Eq[4][R];
+    match(fetch(0), Eq);
+    uint4 q1 = fetch(1);
+    uint32_t outP = 0u, outM = 0u;                     // signs of the deltas that leave the stripe
+    const int last = held ? lt + quads - 1 : -1;       // the iteration after which the words are kept
+    const int iters = __reduce_max_sync(0xFFFFFFFFu, ahead + G - 1);
+    for (int j = 0; j < iters; ++j) {
+        const uint4 q = q1;                            // the quad after this one
+        q1 = fetch(j + 2);
+        // Deltas from the stripe above, which worked on this quad last iteration.  A lane whose first quad is still to come gets
+        // zeros, has no matches, and so leaves its words alone.
+        uint32_t wP = __shfl_up_sync(0xFFFFFFFFu, outP, 1), wM = __shfl_up_sync(0xFFFFFFFFu, outM, 1);
+        if (lt == 0) { wP = 0xFFFFFFFFu; wM = 0u; }    // row 0: +1 everywhere
+        uint32_t next[4][R], cP[4], cM[4];
+        match(q, next);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            cP[u] = wP;
+            cM[u] = wM;
+            column_step<R>(Eq[u], Pv, Mv, cP[u], cM[u], two);
+            wP *= next_column;
+            wM *= next_column;
+        }
+        outP = signs(cP[0], cP[1], cP[2], cP[3]);
+        outM = signs(cM[0], cM[1], cM[2], cM[3]);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            endP[r] = j == last ? Pv[r] : endP[r];
+            endM[r] = j == last ? Mv[r] : endM[r];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) Eq[u][r] = next[u][r];
+        }
+    }
+    // The vertical deltas of the column where the halves meet: forwards along rows 1..m, backwards turned round.
+    uint2* met = reinterpret_cast<uint2*>(wide);
+    __syncwarp();
+    if (held && back) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int w = W - 1 - (R * lt + r);
+            if (w >= 0) met[w] = make_uint2(__brev(endP[r]), __brev(endM[r]));
+        }
+    }
+    __syncwarp();
+    int sum = 0, least = 0, whole = 0;
+    if (held && !back) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int w = R * lt + r;
+            if (w >= W) continue;
+            const uint32_t rows_here = low_mask(min(m - 32 * w, 32));
+            const uint2 b = met[w];
+            const uint32_t bp = b.x & rows_here, bm = b.y & rows_here, fp = endP[r] & rows_here, fm = endM[r] & rows_here;
+            whole += __popc(bp) - __popc(bm);
+            // one row further: the front pays for it, the back does not any more
+#pragma unroll 8
+            for (int k = 0; k < 32; ++k) {
+                sum += (int)((fp >> k) & 1u) + (int)((bm >> k) & 1u) - (int)((fm >> k) & 1u) - (int)((bp >> k) & 1u);
+                least = min(least, sum);
+            }
+        }
+    }
+    int incl = sum;
+#pragma unroll
+    for (int d = 1; d < 16; d <<= 1) {
+        const int up = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (gl >= d) incl += up;
+    }
+    least += incl - sum;
+    if (back) least = 0;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        if (d >= 2 * T) break;
+        whole += __shfl_xor_sync(0xFFFFFFFFu, whole, d);
+        least = min(least, __shfl_xor_sync(0xFFFFFFFFu, least, d));
+    }
+    return n + whole + least;                          // row 0: nothing of the pattern at the front, all of it at the back
+}
+
+// Evaluates group g once the last of its `parts` CTAs is here.  All threads of a CTA call it after writing their distances.
+__device__ __forceinline__ void finish_last(const GateArgs& a, int g, int parts, const int32_t* dist, int32_t* arrived, uint8_t* exact) {
+    __shared__ double s_term[kMaxPairs];
+    __shared__ int32_t s_d[kMaxPairs];
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(arrived, 1) == parts - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    const int N = a.N, P = pairs_of(N);
+    for (int e = threadIdx.x; e < P; e += blockDim.x) {
+        const int pr = kPairs.v[N][e];
+        bool neg = false;
+        const int mi = clamp_len(a.lens, (size_t)g * N + (pr & 0xFF), a.K, neg), mj = clamp_len(a.lens, (size_t)g * N + (pr >> 8), a.K, neg);
+        s_d[e] = __ldcg(dist + (size_t)g * P + e);
+        s_term[e] = pair_term(s_d[e], mi, mj, a.norm_mode);
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double s = 0.0;
+    int isum = 0;
+#pragma unroll 4
+    for (int p = 0; p < P; ++p) {
+        s = __dadd_rn(s, s_term[p]);
+        isum += s_d[p];
+    }
+    const double dk = __ddiv_rn(s, (double)P);
+    if (a.pair_sum) a.pair_sum[g] = isum;
+    if (a.mean) a.mean[g] = dk;
+    a.stop[g] = dk < a.threshold ? 1 : 0;
+    if (exact) exact[g] = 1;
+}
 
 // One CTA per pattern.  Per text it also counts the columns whose symbol does not occur in the
 // pattern at all and the positions at which text and pattern differ: bounds of the pair's distance that
 // cost next to nothing here.  Where they meet the pair is done.
 // kThreads: the CTA's threads where they are the most there can be (known at compile time 82 us of the token-level
 // batch of 1024 groups, at run time 84.5), 0 for fewer.
-template <bool kDecide, int kThreads>
-__global__ void __launch_bounds__(kMostPrepThreads, 6)
-multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base) {
+// kPairs: the whole gate after the names.  Streams and mask rows stay in shared memory, the distances are computed right
+// there, and the last CTA of a group evaluates it.
+template <bool kDecide, int kThreads, bool kPairs>
+__global__ void __launch_bounds__(kMostPrepThreads, kPairs ? 3 : 6)
+multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base, uint8_t* exact, uint32_t two) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t* s_info = reinterpret_cast<uint32_t*>(smem);             // [pitch] see below
     uint16_t* s_map = reinterpret_cast<uint16_t*>(s_info + W.pitch);  // [N * pitch] stream entry of every name
+    // kPairs: [N / 2][pitch] streams, [2][row_cap * row_words] mask rows, and turned round
+    uint16_t* s_loc = s_map + a.N * (W.pitch + 8) + 16;
+    uint32_t* s_rows = reinterpret_cast<uint32_t*>(s_loc + (a.N >> 1) * W.pitch);
     __shared__ int64_t s_stream[kMaxTexts];                           // where a text's stream begins
     __shared__ int s_txt[kMaxTexts], s_len[kMaxTexts], s_cp[kMaxTexts];
     __shared__ uint32_t s_count[kMaxTexts];  // differing positions | absent columns << 16
@@ -464,9 +904,12 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             }
         }
         __syncthreads();
-        uint32_t* rows = reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * M + i) * W.row_cap * W.row_words;
+        uint32_t* rows = kPairs ? s_rows : reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * M + i) * W.row_cap * W.row_words;
         const int n_rows = min(s_repeats[3], W.row_cap);
-        for (int e = tid; e < n_rows * W.row_words; e += nthr) rows[e] = 0u;
+        for (int e = tid; e < n_rows * W.row_words; e += nthr) {
+            rows[e] = 0u;
+            if (kPairs) rows[W.row_cap * W.row_words + e] = 0u;
+        }
         __syncthreads();
         if (claims || repeated) {
 #pragma unroll
@@ -476,11 +919,13 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                 if ((info & kLocChain) == kLocChain) {
                     if (f != p) s_info[p] = atomicExch(&s_info[f], (p << 16) | kLocChain | f);
                 } else {
-                    atomicOr(&rows[(info & 0x3FFFu) * W.row_words + (p >> 5)], 1u << (p & 31));
+                    uint32_t* row = rows + (info & 0x3FFFu) * W.row_words;
+                    atomicOr(row + (p >> 5), 1u << (p & 31));
+                    if (kPairs) atomicOr(row + (W.row_cap + 1) * W.row_words - 1 - (p >> 5), 0x80000000u >> (p & 31));
                 }
             }
         }
-        if (s_repeats[0] > n_rows) {                   // some chains: leave them for the recurrence
+        if (!kPairs && s_repeats[0] > n_rows) {        // some chains: leave them for the recurrence
             __syncthreads();
             uint16_t* g_next = reinterpret_cast<uint16_t*>(ws + W.off_next) + ((size_t)g * M + i) * W.pitch;
             for (int p = tid; p < m; p += nthr) g_next[p] = (uint16_t)(s_info[p] >> 16);
@@ -499,7 +944,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         const int n = s_len[t];
         const uint2* in = reinterpret_cast<const uint2*>(names + s_txt[t] * W.pitch);
         const uint2* own = reinterpret_cast<const uint2*>(pat);
-        uint2* out = reinterpret_cast<uint2*>(locs + s_stream[t]);
+        uint2* out = reinterpret_cast<uint2*>(kPairs ? s_loc + t * W.pitch : locs + s_stream[t]);
         uint32_t differ = 0u, present = 0u, seen = 0u, columns = 0u;
         for (int q = ((s_cp[t] & ~31) >> 2) + 32 * part + lane; 4 * q < n; q += 32 * per_text) {
             const int left = n - 4 * q;                // columns of this quad that exist
@@ -536,25 +981,77 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         }
     }
     __syncthreads();
+    // Bounds of a pair's distance.  Upper: substitute the differing positions, insert or delete the rest.  Lower:
+    // every text column without a match costs an edit, and if the pattern is at least as long as the text,
+    // m - n rows are deleted besides.
+    auto bounds = [&](int t, int strip, int& lower, int& upper) {
+        const int n = s_len[t];
+        lower = upper = abs(m - n);                   // one prefix starts the other (or is empty)
+        if (strip < 0) return;
+        const int absent = (int)(s_count[t] >> 16);
+        lower = m >= n ? m - n + absent : max(n - m, absent);
+        upper += (int)(s_count[t] & 0xFFFFu);
+    };
+    // The removed prefix is a multiple of four symbols (the match stream is read in 8-byte
+    // quads), and of 32 where the stream refers to mask rows (whose words start there).
+    auto removed = [&](int t) { return s_cp[t] < 0 ? -1 : (s_cp[t] & (s_flag[t] ? ~31 : ~3)); };
+    if constexpr (kPairs) {
+        __shared__ uint4 s_differ[kMostPrepThreads / 32][kSpans];
+        __shared__ uint32_t s_entries[kMostPrepThreads / 32][kMostMatches];
+        __shared__ int s_dist[kMaxTexts];              // the distance, or -1: to be computed
+        // first what the bounds and few matches settle
+        for (int t = warp; t < ntxt; t += warps) {
+            const int n = s_len[t], strip = removed(t);
+            int lower, upper;
+            bounds(t, strip, lower, upper);
+            int d = lower < upper ? -1 : lower;
+            if (d < 0 && upper - lower <= kMostMatches && few_repeats(s_repeats[0], m) && n + m - 2 * strip > kWorthMatches) {
+                __syncwarp();
+                const int count = find_matches<true>(reinterpret_cast<const uint2*>(s_loc + t * W.pitch), reinterpret_cast<const uint2*>(names + s_txt[t] * W.pitch),
+                                                     reinterpret_cast<const uint2*>(pat), m, n, strip, s_differ[warp], s_entries[warp]);
+                if (count == 0) d = upper;
+                else if (count <= kMostMatches)
+                    d = distance_by_matches<true>(s_entries[warp], count, s_differ[warp], s_rows, W.row_words, m, n, strip, upper);
+            }
+            if (lane == 0) {
+                s_dist[t] = d;
+                if (d >= 0) dist_out[(size_t)g * P + pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N)] = d;
+            }
+        }
+        __syncthreads();
+        // Teams of as many lanes as the pattern has blocks, 16 at the most, and as many pairs to a warp as have room.
+        const bool chains = s_repeats[0] > min(s_repeats[3], W.row_cap);
+        const uint32_t* turned = s_rows + W.row_cap * W.row_words;
+        uint4* s_wide = reinterpret_cast<uint4*>(s_map);              // the map is not needed any more
+        const int blocks = (m + 3 + 31) >> 5, tlog = min(32 - __clz(max(blocks, 1) - 1), 4), share = 16 >> tlog;
+        for (int t0 = warp * share; t0 < ntxt; t0 += warps * share) {
+            const int t = min(t0 + (lane >> (tlog + 1)), ntxt - 1);
+            const bool live = t0 + (lane >> (tlog + 1)) < ntxt && s_dist[t] < 0;
+            if (!__any_sync(0xFFFFFFFFu, live)) continue;
+            const int n = s_len[t], strip = live ? removed(t) : 0;
+            const uint16_t* loc = s_loc + t * W.pitch;
+            // (lanes without a text share two quads of their own)
+            uint4* wide = s_wide + (t0 + (lane >> (tlog + 1)) < ntxt ? t * ((W.pitch + 8) >> 2) : (N * (W.pitch + 8)) >> 3);
+            const int high = __reduce_max_sync(0xFFFFFFFFu, live ? (m + (-n & 3) - strip + 31) >> 5 : 0);
+            int d;
+            if (high <= 16) d = distance_from_both_ends<1>(loc, wide, s_rows, turned, W.row_words, s_info, chains, live, m, n, strip, tlog, two);
+            else if (high <= 32) d = distance_from_both_ends<2>(loc, wide, s_rows, turned, W.row_words, s_info, chains, live, m, n, strip, tlog, two);
+            else d = distance_from_both_ends<3>(loc, wide, s_rows, turned, W.row_words, s_info, chains, live, m, n, strip, tlog, two);
+            if (live && (lane & ((2 << tlog) - 1)) == 0) dist_out[(size_t)g * P + pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N)] = d;
+        }
+        finish_last(a, g, M, dist_out, reinterpret_cast<int32_t*>(ws + W.off_order) + g, exact);
+        return;
+    }
     if (tid >= 32) return;                             // descriptors: the texts' threads are in the first warp
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
     int work = 0, few = -1;
     if (tid < ntxt) {
         const int j = s_txt[tid], n = s_len[tid];
-        // the removed prefix is a multiple of four symbols (the match stream is read in 8-byte
-        // quads), and of 32 where the stream refers to mask rows (whose words start there)
-        const int strip = s_cp[tid] < 0 ? -1 : (s_cp[tid] & (s_flag[tid] ? ~31 : ~3));
+        const int strip = removed(tid);
         const size_t idx = (size_t)g * P + pair_index(min(i, j), max(i, j), N);
-        // Upper bound of the distance: substitute the differing positions, insert or delete the
-        // rest.  Lower bound: every text column without a match costs an edit, and if the pattern
-        // is at least as long as the text, m - n rows are deleted besides.
-        int lower = abs(m - n), upper = lower;        // one prefix starts the other (or is empty)
-        if (strip >= 0) {
-            const int absent = (int)(s_count[tid] >> 16);
-            lower = m >= n ? m - n + absent : max(n - m, absent);
-            upper += (int)(s_count[tid] & 0xFFFFu);
-        }
+        int lower, upper;
+        bounds(tid, strip, lower, upper);
         PairDesc d{(uint32_t)m | ((uint32_t)n << 16), (uint32_t)(g * M + i), 0u, (uint32_t)lower | ((uint32_t)upper << 16)};
         if (lower < upper) {                          // otherwise that is the distance
             const int n_rows = min(s_repeats[3], W.row_cap);
@@ -587,172 +1084,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     }
 }
 
-// --------------------------------------------------------------------- matches
-// Pairs with few matches.  Besides the main diagonal, on which the two prefixes are compared place by
-// place, two rollouts over a large vocabulary have hardly a symbol in common: a pair of 1024 uniform
-// tokens out of 150 000 has seven matches where a matrix of a million cells says the same.  Between two
-// matches (c, p) that it uses, a path either goes straight, max(columns, rows) edits, or by way of
-// the main diagonal, where it pays for the places that differ; so the distance is a shortest path over the
-// matches off the diagonal (sparse dynamic programming: Eppstein, Galil, Giancarlo and Italiano 1992), one
-// lane each.  A pair whose bounds are further apart than there are lanes has more such columns than that, and the
-// recurrence has it; the others are listed by prep, a warp each.
-// 1024 groups of 8 prefixes of 256..1024 uniform tokens: the recurrence took 174 us for them, this 37 us cold (20 M warp
-// instructions, 1100 a pair: a third to look through the stream, a third for the rows of repeated symbols), and the
-// whole gate went from 270 to 125 us.
-constexpr int kSpan = 128;                               // columns a warp looks through a trip
-constexpr int kSpans = SR_MAX_K / kSpan + 1;             // and one that begins where the longest text ends
-constexpr int kMatchWarps = 8;
-
-// The columns of a pair's stream with matches off the main diagonal, with the column's stream entry (upper half), in
-// `entries`, and in `differ` a bit for every column from `strip` on that differs from the pattern: column
-// strip + 128 s + 4 l + k in bit l of word k of differ[s].  Returns the number of those columns, or more than
-// there are lanes for.
-__device__ __forceinline__ int find_matches(const uint2* stream, const uint2* text, const uint2* pat, int m, int n, int strip,
-                                            uint4* differ, uint32_t* entries) {
-    const int lane = threadIdx.x & 31;
-    int found = 0;
-    auto fetch = [&](int s) {
-        const int q = (strip >> 2) + 32 * s + lane;
-        return 4 * q < n ? __ldg(stream + q) : make_uint2(kLocNone * 0x10001u, kLocNone * 0x10001u);
-    };
-    uint2 ahead[2] = {fetch(0), fetch(1)};
-    for (int s = 0; strip + kSpan * s < n; ++s) {
-        const int q = (strip >> 2) + 32 * s + lane;
-        const int left = min(max(n - 4 * q, 0), 4), both = min(left, max(m - 4 * q, 0));   // columns that exist, and of those with a row
-        const uint2 v = ahead[0];
-        ahead[0] = ahead[1];
-        ahead[1] = fetch(s + 2);
-        const uint32_t at0 = (uint32_t)(4 * q * 0x10001 + 0x10000), at1 = at0 + 0x20002u;   // the places on the main diagonal
-        uint32_t off0 = set_halves(v.x ^ at0), off1 = set_halves(v.y ^ at1);
-        uint32_t d0 = off0, d1 = off1;
-        if ((v.x | v.y) & (kLocRow * 0x10001u)) {      // a symbol that occurs more than once: the names tell
-            const uint2 x = __ldg(text + q), o = __ldg(pat + q);
-            d0 = set_halves(x.x ^ o.x);
-            d1 = set_halves(x.y ^ o.y);
-        }
-        off0 &= set_halves(v.x ^ (kLocNone * 0x10001u));
-        off1 &= set_halves(v.y ^ (kLocNone * 0x10001u));
-        if (left < 4) {
-            off0 = left > 1 ? off0 : (left == 1 ? off0 & 0xFFFFu : 0u);
-            off1 = left == 3 ? off1 & 0xFFFFu : 0u;
-        }
-        if (both < 4) {
-            d0 = both > 1 ? d0 : (both == 1 ? d0 & 0xFFFFu : 0u);
-            d1 = both == 3 ? d1 & 0xFFFFu : 0u;
-        }
-        const unsigned b0 = __ballot_sync(0xFFFFFFFFu, (d0 & 0x8000u) != 0u), b1 = __ballot_sync(0xFFFFFFFFu, (d0 >> 31) != 0u);
-        const unsigned b2 = __ballot_sync(0xFFFFFFFFu, (d1 & 0x8000u) != 0u), b3 = __ballot_sync(0xFFFFFFFFu, (d1 >> 31) != 0u);
-        if (lane == 0) differ[s] = make_uint4(b0, b1, b2, b3);
-        if (!__any_sync(0xFFFFFFFFu, (off0 | off1) != 0u)) continue;
-        const unsigned o0 = __ballot_sync(0xFFFFFFFFu, (off0 & 0x8000u) != 0u), o1 = __ballot_sync(0xFFFFFFFFu, (off0 >> 31) != 0u);
-        const unsigned o2 = __ballot_sync(0xFFFFFFFFu, (off1 & 0x8000u) != 0u), o3 = __ballot_sync(0xFFFFFFFFu, (off1 >> 31) != 0u);
-        const unsigned under = (1u << lane) - 1u;
-        int at = found + __popc(o0 & under) + __popc(o1 & under) + __popc(o2 & under) + __popc(o3 & under);
-        found += __popc(o0) + __popc(o1) + __popc(o2) + __popc(o3);
-        if (found > kMostMatches) return found;
-        if (off0 & 0x8000u) entries[at++] = (uint32_t)(4 * q) | (v.x << 16);      // by column
-        if (off0 >> 31) entries[at++] = (uint32_t)(4 * q + 1) | (v.x & 0xFFFF0000u);
-        if (off1 & 0x8000u) entries[at++] = (uint32_t)(4 * q + 2) | (v.y << 16);
-        if (off1 >> 31) entries[at++] = (uint32_t)(4 * q + 3) | (v.y & 0xFFFF0000u);
-    }
-    __syncwarp();
-    return found;
-}
-
-// The distance of a pair from what find_matches found.  upper: the distance along the main diagonal.  Negative: more
-// matches than there are lanes for.
-__device__ __forceinline__ int distance_by_matches(uint32_t* entries, int count, const uint4* differ, const uint32_t* rows, int row_words,
-                                                   int m, int n, int strip, int upper) {
-    const int lane = threadIdx.x & 31;
-    const int lo = min(m, n);
-    // every entry's matches: one position, or those of a mask row
-    uint32_t node = lane < count ? entries[lane] : 0u;
-    const bool row = lane < count && (node >> 16) >= kLocRow;
-    if (__any_sync(0xFFFFFFFFu, lane < count && (node >> 16) >= kLocChain)) return -1;
-    int total = count;
-    unsigned todo = __ballot_sync(0xFFFFFFFFu, row);
-    if (todo) {
-        const bool single = lane < count && !row;
-        const unsigned singles = __ballot_sync(0xFFFFFFFFu, single);
-        total = __popc(singles);
-        if (single) entries[__popc(singles & ((1u << lane) - 1u))] = node;
-        while (todo) {                                 // eight rows on their way before the first is looked at
-            uint32_t bits[8], column[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                bits[k] = column[k] = 0u;
-                if (todo == 0u) continue;
-                const uint32_t e = __shfl_sync(0xFFFFFFFFu, node, __ffs(todo) - 1);
-                todo &= todo - 1u;
-                column[k] = e & 0xFFFFu;
-                if (lane < row_words) bits[k] = __ldg(rows + ((e >> 16) & 0x3FFFu) * row_words + lane);
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                while (__any_sync(0xFFFFFFFFu, bits[k] != 0u)) {
-                    const int p = bits[k] ? 32 * lane + __ffs(bits[k]) - 1 : -1;
-                    bits[k] &= bits[k] - 1u;
-                    const bool use = p >= strip && p != (int)column[k];
-                    const unsigned b = __ballot_sync(0xFFFFFFFFu, use);
-                    const int at = total + __popc(b & ((1u << lane) - 1u));
-                    total += __popc(b);
-                    if (use && at < kMostMatches) entries[at] = column[k] | ((uint32_t)p << 16);
-                }
-            }
-            if (total > kMostMatches) return -1;
-        }
-        if (total == 0) return upper;
-        __syncwarp();
-        // by column again
-        const uint32_t own = lane < total ? entries[lane] : 0xFFFFFFFFu;
-        int rank = 0;
-        for (int l = 0; l < total; ++l) {
-            const uint32_t other = __shfl_sync(0xFFFFFFFFu, own, l);
-            rank += (other & 0xFFFFu) < (own & 0xFFFFu) || ((other & 0xFFFFu) == (own & 0xFFFFu) && l < lane);
-        }
-        if (lane < total) entries[rank] = own;
-        __syncwarp();
-    }
-    __syncwarp();
-    node = lane < total ? entries[lane] : (uint32_t)strip * 0x10001u;
-    const int c = (int)(node & 0xFFFFu), p = (int)(node >> 16);
-    // places that differ before x
-    int before = 0;
-    if (lane < kSpans && strip + kSpan * lane < n) {
-        const uint4 d = differ[lane];
-        before = __popc(d.x) + __popc(d.y) + __popc(d.z) + __popc(d.w);
-    }
-#pragma unroll
-    for (int d = 1; d < 16; d <<= 1) {
-        const int up = __shfl_up_sync(0xFFFFFFFFu, before, d);
-        if (lane >= d) before += up;
-    }
-    auto differing = [&](int x) {
-        const int rel = x - strip, s = rel / kSpan, l = (rel % kSpan) >> 2, k = rel & 3;
-        const uint4 d = differ[s];
-        const uint32_t under = (1u << l) - 1u, with = under | (1u << l);
-        const int sum = __shfl_sync(0xFFFFFFFFu, before, max(s - 1, 0));
-        return (s > 0 ? sum : 0) + __popc(d.x & (k > 0 ? with : under)) + __popc(d.y & (k > 1 ? with : under)) +
-               __popc(d.z & (k > 2 ? with : under)) + __popc(d.w & under);
-    };
-    const int off = abs(c - p);
-    const int enter = min(c, p), leave = max(c, p) + 1;  // the last place of the diagonal before the match, the first after it
-    const int at_enter = differing(enter), at_leave = differing(min(leave, lo)), at_end = differing(lo);
-    int cost = off + at_enter;                            // up to the match and through it
-    for (int l = 0; l + 1 < total; ++l) {
-        const uint32_t from = __shfl_sync(0xFFFFFFFFu, node, l);
-        const uint32_t paid = __shfl_sync(0xFFFFFFFFu, (uint32_t)cost | ((uint32_t)at_leave << 16), l);
-        const int fc = (int)(from & 0xFFFFu), fp = (int)(from >> 16);
-        int step = max(c - fc, p - fp) - 1;
-        if (max(fc, fp) < enter) step = min(step, abs(fc - fp) + at_enter - (int)(paid >> 16) + off);
-        if (c > fc && p > fp) cost = min(cost, (int)(paid & 0xFFFFu) + step);
-    }
-    int last = max(n - c, m - p) - 1;
-    if (leave <= lo) last = min(last, off + at_end - at_leave + abs(n - m));
-    const int d = lane < total ? cost + last : upper;
-    return min(__reduce_min_sync(0xFFFFFFFFu, d), upper);
-}
-
+// --------------------------------------------------------------- matches kernel
 // A warp goes through listed pairs as many places apart as there are warps.  decide: the bounds that this leaves are the
 // bound kernel's to add up.
 __global__ void __launch_bounds__(32 * kMatchWarps)
@@ -777,13 +1109,13 @@ multi_matches_kernel(unsigned char* ws, MultiWs W, int N, bool decide, int32_t* 
         const int pr = kPairs.v[N][idx - g * P], j = (pr & 0xFF) + (pr >> 8) - i;
         const uint16_t* names = reinterpret_cast<const uint16_t*>(ws + W.off_names) + (size_t)g * N * W.pitch;
         __syncwarp();                              // the pair before has been read
-        const int count = find_matches(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(ws + W.off_loc) + (size_t)idx * W.pitch),
+        const int count = find_matches<false>(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(ws + W.off_loc) + (size_t)idx * W.pitch),
                                        reinterpret_cast<const uint2*>(names + j * W.pitch), reinterpret_cast<const uint2*>(names + i * W.pitch),
                                        m, n, strip, s_differ[warp], s_entries[warp]);
         if (count == 0)
             dist = upper;
         else if (count <= kMostMatches)
-            dist = distance_by_matches(s_entries[warp], count, s_differ[warp],
+            dist = distance_by_matches<false>(s_entries[warp], count, s_differ[warp],
                                        reinterpret_cast<const uint32_t*>(ws + W.off_rows) + (size_t)d.pat_row * (W.row_cap * W.row_words),
                                        W.row_words, m, n, strip, upper);
         if (dist >= 0) {
@@ -963,12 +1295,6 @@ multi_order_kernel(PairDesc* descs, int32_t* order, Ctl* ctl, int n_pairs, int w
 }
 
 // -------------------------------------------------------------------------- dp
-__device__ __forceinline__ uint32_t shl_clamp(uint32_t v, uint32_t s) {
-    uint32_t r;   // PTX shl clamps shift amounts above 31: the result is 0
-    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));
-    return r;
-}
-
 // Brings `bytes` bytes to L1, 32 a time, `lanes` lanes together.  (Not inlined: it is run once a task.)
 __device__ __noinline__ void touch(const void* from, int bytes, int lane, int lanes) {
     for (int o = 32 * lane; o < bytes; o += 32 * lanes) {
@@ -1022,34 +1348,6 @@ __device__ __forceinline__ void add_chains(uint2 q, uint32_t rowbase, const uint
             for (int r = 0; r < R; ++r) Eq[u][r] |= shl_clamp(1u, dd - 32u * r);
             p = __ldg(nxt + p);
         }
-    }
-}
-
-// One bit-vector column step over the R blocks a lane owns.  `Eq` are the column's match
-// words, (inP, inM) the pre-shift horizontal delta words of the
-// block above (only their top bits matter); returns this lane's last block's words in
-// (inP, inM).
-template <int R>
-__device__ __forceinline__ void column_step(const uint32_t (&Eq)[R],
-                                            uint32_t (&Pv)[R], uint32_t (&Mv)[R],
-                                            uint32_t& inP, uint32_t& inM, uint32_t two) {
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const uint32_t pv = Pv[r], mv = Mv[r];
-        const uint32_t hm = inM >> 31;
-        // D0: the cells whose value equals that of their upper left neighbour
-        const uint32_t D0 = ((((Eq[r] | hm) & pv) + pv) ^ pv) | (Eq[r] | mv | hm);
-        const uint32_t Ph = mv | ~(D0 | pv);
-        const uint32_t Mh = pv & D0;
-        const uint32_t Phs = __funnelshift_l(inP, Ph, 1);
-        // `two` holds 2 but is a run-time value, so this shift-and-insert is a multiply-add:
-        // it issues on the FMA pipe and leaves the integer ALU, the bottleneck, one
-        // instruction lighter per block (measured: 8 % faster than a second funnel shift)
-        const uint32_t Mhs = Mh * two + hm;              // (Mh << 1) | hm
-        Pv[r] = Mhs | ~(D0 | Phs);
-        Mv[r] = Phs & D0;
-        inP = Ph;
-        inM = Mh;
     }
 }
 
@@ -1275,7 +1573,6 @@ multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
 // One thread per pair, gpb groups per CTA (more pairs than threads: several per thread); one
 // thread per group for the ordered sums.
 constexpr int kGroupThreads = 256;
-constexpr int kMaxPairs = SR_MAX_N * (SR_MAX_N - 1) / 2;       // pairs of a CTA: 256, or one group's
 
 __global__ void __launch_bounds__(kGroupThreads)
 multi_bound_kernel(GateArgs a, PairDesc* descs, Ctl* ctl, uint8_t* flag, uint8_t* exact, int gpb, bool alone) {
@@ -1385,6 +1682,13 @@ multi_finish_kernel(GateArgs a, int32_t* dist, const uint8_t* flag, uint8_t* exa
     if (capped && exact) exact[g] = 0;                       // some distances are lower bounds
 }
 
+// Which batches take every pair from both ends instead of sorting the pairs into warp tasks: those whose
+// work leaves the SMs idle anyway.  Both sides at the line for texts, us: 600 groups of 8 at K = 48 49 and 46, 250 at 256 45 and
+// 58, at 512 83 and 92; 150 at 1024 about 140 both; four groups of 8 at 1024 41 and 84.  With more texts to a pattern than a CTA
+// has warps the line lies lower (16 groups of 24 at 1024: 174 and 149).  The decide mode has less to do the
+// other way, where bounds settle most groups: 40 groups of 8 at 256 24 and 27 to 50, but at 512 47 and 29.
+bool runs_in_pairs(int n_pairs, int N, int K, bool decide) { return decide ? K <= 256 && n_pairs <= 2800 : (long long)n_pairs * (K + 384) <= (N <= 17 ? 6400000LL : 4200000LL); }
+
 // More than 48 KB of shared memory has to be asked for: the most that any call takes, once per device (noted,
 // because asking is host time).
 constexpr int kMostNamesSmem = 200 * 1024;
@@ -1395,8 +1699,10 @@ int allow_smem() {
     if (dev >= 0 && dev < 64 && allowed[dev].load(std::memory_order_relaxed)) return SR_OK;
     const int prep = SR_MAX_K * 4 + SR_MAX_N * SR_MAX_K * 2;
     SR_CUDA_TRY(cudaFuncSetAttribute(multi_names_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostNamesSmem));
-    for (auto kernel : {multi_prep_kernel<true, 0>, multi_prep_kernel<true, kMostPrepThreads>, multi_prep_kernel<false, 0>, multi_prep_kernel<false, kMostPrepThreads>})
+    for (auto kernel : {multi_prep_kernel<true, 0, false>, multi_prep_kernel<true, kMostPrepThreads, false>, multi_prep_kernel<false, 0, false>, multi_prep_kernel<false, kMostPrepThreads, false>})
         SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, prep));
+    for (auto kernel : {multi_prep_kernel<false, 0, true>, multi_prep_kernel<false, kMostPrepThreads, true>})
+        SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostNamesSmem));
     if (dev >= 0 && dev < 64) allowed[dev].store(true, std::memory_order_relaxed);
     return SR_OK;
 }
@@ -1428,7 +1734,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     int32_t* dist = a.pair_dist ? a.pair_dist : reinterpret_cast<int32_t*>(ws + W.off_dist);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
 
-    const int prep_smem = W.pitch * 4 + a.N * W.pitch * 2;
+    const bool in_pairs = !feed && runs_in_pairs(n_pairs, a.N, a.K, decide);
+    const int prep_smem = in_pairs ? W.pitch * 4 + a.N * (W.pitch + 8) * 2 + 32 + (a.N >> 1) * W.pitch * 2 + (2 * W.row_cap * W.row_words + 8) * 4
+                                   : W.pitch * 4 + a.N * W.pitch * 2;
     // names: at least two slots to a symbol while symbols and table fit
     const int row_quads = W.pitch >> 2, sym_bytes = a.N * W.pitch * 4, names_most = a.N * W.pitch > 4 * 8 * 512 ? 1024 : 512;
     // A thread for every four positions of the group while 512 threads suffice; and for prep a warp for every 128
@@ -1443,7 +1751,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const int names_smem = sym_bytes + (2 << table_log);
     const uint32_t inv_row = (uint32_t)(((1ull << 32) + row_quads - 1) / row_quads);
     uint16_t* names = reinterpret_cast<uint16_t*>(ws + W.off_names);
-    if (names_smem > 48 * 1024 || prep_smem > 48 * 1024) {
+    if (names_smem > 47 * 1024 || prep_smem > 36 * 1024) {    // with what the kernels declare
         const int rc = allow_smem();
         if (rc != SR_OK) return rc;
     }
@@ -1451,7 +1759,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[0], s));
     // what the kernels add up starts at zero (one CTA that orders the batch alone needs nothing)
     const bool alone = W.alone = n_pairs <= kAlonePairs;
-    if (!alone) SR_CUDA_TRY(cudaMemsetAsync(ctl, 0, offsetof(Ctl, start), s));
+    if (!alone && !in_pairs) SR_CUDA_TRY(cudaMemsetAsync(ctl, 0, offsetof(Ctl, start), s));
     uint8_t* flag = decide ? ws + W.off_flag : nullptr;
     // The match-stream pass works group by group, so when the groups arrive in pieces it runs
     // piece by piece: `feed->before` enqueues whatever makes groups [g0, g1) ready on `s`.
@@ -1464,11 +1772,17 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
             const int rc = feed->before(feed->ctx, g0, g1, s);
             if (rc != SR_OK) return rc;
         }
-        SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0);
+        SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0,
+                  in_pairs ? reinterpret_cast<int32_t*>(ws + W.off_order) : nullptr);
         const auto prep = prep_threads == kMostPrepThreads
-            ? (decide ? multi_prep_kernel<true, kMostPrepThreads> : multi_prep_kernel<false, kMostPrepThreads>)
-            : (decide ? multi_prep_kernel<true, 0> : multi_prep_kernel<false, 0>);
-        SR_LAUNCH("multi_prep_kernel", prep, (g1 - g0) * W.patterns, prep_threads, prep_smem, s, a, ws, W, dist, g0);
+            ? (in_pairs ? multi_prep_kernel<false, kMostPrepThreads, true>
+                        : decide ? multi_prep_kernel<true, kMostPrepThreads, false> : multi_prep_kernel<false, kMostPrepThreads, false>)
+            : (in_pairs ? multi_prep_kernel<false, 0, true> : decide ? multi_prep_kernel<true, 0, false> : multi_prep_kernel<false, 0, false>);
+        SR_LAUNCH("multi_prep_kernel", prep, (g1 - g0) * W.patterns, prep_threads, prep_smem, s, a, ws, W, dist, g0, exact, 2u);
+    }
+    if (in_pairs) {
+        if (ev) for (int k = 1; k <= 4; ++k) SR_CUDA_TRY(cudaEventRecord(ev[k], s));
+        return SR_OK;
     }
     const int gpb = P <= kGroupThreads ? kGroupThreads / P : 1;
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
