@@ -34,7 +34,7 @@
 //
 // A batch that leaves most of the GPU idle (runs_in_pairs) takes the names and one launch: prep keeps streams and rows in
 // shared memory, the distances are computed right there, both ways from the ends of the text, and the
-// last CTA of a group evaluates it.
+// last CTA of a group evaluates it (where there are even fewer, it names the symbols too, and the gate is one launch).
 //
 // Band.  With bounds lb <= d <= ub of a pair's distance an optimal alignment stays on a band of
 // diagonals (band_of), and where the bounds meet nothing is left to compute.  Rollouts that have
@@ -48,6 +48,8 @@
 // Which rollout of a pair is the pattern is fixed by a round-robin tournament on the
 // indices, so that every pattern CTA of `prep` serves the same number of texts.
 #include <atomic>
+
+#include <cooperative_groups.h>
 
 #include "common.cuh"
 
@@ -251,26 +253,12 @@ constexpr uint32_t kHashMul = 0x9E3779B1u;
 constexpr int kMaxTexts = SR_MAX_N / 2;        // texts a pattern is paired with
 constexpr int kMaxPairs = SR_MAX_N * (SR_MAX_N - 1) / 2;
 
-__global__ void __launch_bounds__(1024)
-multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int table_log, int g_base, int32_t* arrived) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_len[SR_MAX_N];
-    const int N = a.N, K = a.K, tid = threadIdx.x, nthr = blockDim.x;
-    const int row_quads = pitch >> 2, items = N * row_quads;
-    int32_t* s_sym = reinterpret_cast<int32_t*>(smem);                             // [N][pitch]
-    uint16_t* s_table = reinterpret_cast<uint16_t*>(s_sym + N * pitch);            // [1 << table_log]
-    grid_begin();
-    const int g = g_base + blockIdx.x;
+// s_sym: [N][pitch], s_table: [1 << table_log], s_len: the prefixes' lengths, out: [N][pitch].  All threads of a CTA, after a barrier.
+__device__ __forceinline__ void name_symbols(const GateArgs& a, int g, const int* s_len, int32_t* s_sym, uint16_t* s_table, int table_log,
+                                             int pitch, uint32_t inv_row, uint2* out) {
+    const int N = a.N, tid = threadIdx.x, nthr = blockDim.x;
+    const int row_quads = pitch >> 2, items = N * row_quads, shift = 32 - table_log;
     const int32_t* seqs = a.seqs + (size_t)g * N * a.stride;
-    uint2* out = reinterpret_cast<uint2*>(names + (size_t)g * N * pitch);
-    if (tid < N) {
-        bool neg = false;
-        s_len[tid] = clamp_len(a.lens, (size_t)g * N + tid, K, neg);
-        if (neg && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
-    }
-    if (arrived && tid == 0) arrived[g] = 0;           // see finish_last
-    __syncthreads();
-    const int shift = 32 - table_log;
 #pragma unroll 4
     for (int e = tid; e < items; e += nthr) {
         const int i = (int)__umulhi((uint32_t)e, inv_row), q = e - i * row_quads, live = s_len[i] - 4 * q;
@@ -318,6 +306,25 @@ multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int
             open &= ~(1u << c);
         }
     }
+}
+
+__global__ void __launch_bounds__(1024)
+multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int table_log, int g_base, int32_t* arrived) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_len[SR_MAX_N];
+    const int N = a.N, tid = threadIdx.x;
+    int32_t* s_sym = reinterpret_cast<int32_t*>(smem);
+    grid_begin();
+    const int g = g_base + blockIdx.x;
+    if (tid < N) {
+        bool neg = false;
+        s_len[tid] = clamp_len(a.lens, (size_t)g * N + tid, a.K, neg);
+        if (neg && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
+    }
+    if (arrived && tid == 0) arrived[g] = 0;           // see finish_last
+    __syncthreads();
+    name_symbols(a, g, s_len, s_sym, reinterpret_cast<uint16_t*>(s_sym + N * pitch), table_log, pitch, inv_row,
+                 reinterpret_cast<uint2*>(names + (size_t)g * N * pitch));
 }
 
 // ------------------------------------------------------------------------ prep
@@ -406,7 +413,7 @@ __device__ __forceinline__ int find_matches(const uint2* stream, const uint2* te
         uint32_t off0 = set_halves(v.x ^ at0), off1 = set_halves(v.y ^ at1);
         uint32_t d0 = off0, d1 = off1;
         if ((v.x | v.y) & (kLocRow * 0x10001u)) {      // a symbol that occurs more than once: the names tell
-            const uint2 x = __ldg(text + q), o = __ldg(pat + q);
+            const uint2 x = kShared ? text[q] : __ldg(text + q), o = kShared ? pat[q] : __ldg(pat + q);
             d0 = set_halves(x.x ^ o.x);
             d1 = set_halves(x.y ^ o.y);
         }
@@ -723,19 +730,26 @@ __device__ __forceinline__ int distance_from_both_ends(const uint16_t* loc, uint
     return n + whole + least;                          // row 0: nothing of the pattern at the front, all of it at the back
 }
 
-// Evaluates group g once the last of its `parts` CTAs is here.  All threads of a CTA call it after writing their distances.
+// Evaluates group g once all of its `parts` CTAs are here: the first of a cluster's, or the last to count itself in
+// `arrived`.  All threads of a CTA call it after writing their distances.
+template <bool kCluster>
 __device__ __forceinline__ void finish_last(const GateArgs& a, int g, int parts, const int32_t* dist, int32_t* arrived, uint8_t* exact) {
     __shared__ double s_term[kMaxPairs];
     __shared__ int32_t s_d[kMaxPairs];
-    __shared__ bool s_last;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(arrived, 1) == parts - 1;
-        __threadfence();
+    if constexpr (kCluster) {
+        cooperative_groups::this_cluster().sync();
+        if (blockIdx.x % parts != 0) return;
+    } else {
+        __shared__ bool s_last;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            s_last = atomicAdd(arrived, 1) == parts - 1;
+            __threadfence();
+        }
+        __syncthreads();
+        if (!s_last) return;
     }
-    __syncthreads();
-    if (!s_last) return;
     const int N = a.N, P = pairs_of(N);
     for (int e = threadIdx.x; e < P; e += blockDim.x) {
         const int pr = kPairs.v[N][e];
@@ -767,15 +781,19 @@ __device__ __forceinline__ void finish_last(const GateArgs& a, int g, int parts,
 // batch of 1024 groups, at run time 84.5), 0 for fewer.
 // kPairs: the whole gate after the names.  Streams and mask rows stay in shared memory, the distances are computed right
 // there, and the last CTA of a group evaluates it.
-template <bool kDecide, int kThreads, bool kPairs>
+// kOwnNames: the whole gate.  A group's CTAs are a cluster, and each of them names all of the group's symbols for itself.
+template <bool kDecide, int kThreads, bool kPairs, bool kOwnNames>
 __global__ void __launch_bounds__(kMostPrepThreads, kPairs ? 3 : 6)
-multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base, uint8_t* exact, uint32_t two) {
+multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base, uint8_t* exact, uint32_t inv_row, int table_log,
+                  uint32_t two) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t* s_info = reinterpret_cast<uint32_t*>(smem);             // [pitch] see below
     uint16_t* s_map = reinterpret_cast<uint16_t*>(s_info + W.pitch);  // [N * pitch] stream entry of every name
     // kPairs: [N / 2][pitch] streams, [2][row_cap * row_words] mask rows, and turned round
     uint16_t* s_loc = s_map + a.N * (W.pitch + 8) + 16;
     uint32_t* s_rows = reinterpret_cast<uint32_t*>(s_loc + (a.N >> 1) * W.pitch);
+    // kOwnNames: [N][pitch] names, [N][pitch] symbols and their table
+    uint16_t* s_names = reinterpret_cast<uint16_t*>(s_rows + ((2 * W.row_cap * W.row_words + 11) & ~3));
     __shared__ int64_t s_stream[kMaxTexts];                           // where a text's stream begins
     __shared__ int s_txt[kMaxTexts], s_len[kMaxTexts], s_cp[kMaxTexts];
     __shared__ uint32_t s_count[kMaxTexts];  // differing positions | absent columns << 16
@@ -793,8 +811,19 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     grid_begin();
     bool neg = false;
     const int m = clamp_len(a.lens, (size_t)g * N + i, K, neg);
-    const uint16_t* names = reinterpret_cast<const uint16_t*>(ws + W.off_names) + (size_t)g * N * W.pitch;
+    const uint16_t* names = kOwnNames ? s_names : reinterpret_cast<const uint16_t*>(ws + W.off_names) + (size_t)g * N * W.pitch;
     const uint16_t* pat = names + i * W.pitch;
+    if constexpr (kOwnNames) {
+        __shared__ int s_all_len[SR_MAX_N];
+        if (tid < N) {
+            bool negative = false;
+            s_all_len[tid] = clamp_len(a.lens, (size_t)g * N + tid, K, negative);
+            if (negative && i == 0 && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
+        }
+        __syncthreads();
+        int32_t* s_sym = reinterpret_cast<int32_t*>(s_names + N * W.pitch);
+        name_symbols(a, g, s_all_len, s_sym, reinterpret_cast<uint16_t*>(s_sym + N * W.pitch), table_log, W.pitch, inv_row, reinterpret_cast<uint2*>(s_names));
+    }
     // Which rollout of a pair is the pattern follows a round-robin tournament: with M = N
     // for odd N and N - 1 otherwise, rollout i < M is the pattern against the `half` rollouts
     // after it (cyclically among the first M) and, for even N, against the last rollout,
@@ -1039,7 +1068,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             else d = distance_from_both_ends<3>(loc, wide, s_rows, turned, W.row_words, s_info, chains, live, m, n, strip, tlog, two);
             if (live && (lane & ((2 << tlog) - 1)) == 0) dist_out[(size_t)g * P + pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N)] = d;
         }
-        finish_last(a, g, M, dist_out, reinterpret_cast<int32_t*>(ws + W.off_order) + g, exact);
+        finish_last<kOwnNames>(a, g, M, dist_out, reinterpret_cast<int32_t*>(ws + W.off_order) + g, exact);
         return;
     }
     if (tid >= 32) return;                             // descriptors: the texts' threads are in the first warp
@@ -1689,6 +1718,14 @@ multi_finish_kernel(GateArgs a, int32_t* dist, const uint8_t* flag, uint8_t* exa
 // other way, where bounds settle most groups: 40 groups of 8 at 256 24 and 27 to 50, but at 512 47 and 29.
 bool runs_in_pairs(int n_pairs, int N, int K, bool decide) { return decide ? K <= 256 && n_pairs <= 2800 : (long long)n_pairs * (K + 384) <= (N <= 17 ? 6400000LL : 4200000LL); }
 
+// And which of them name a group's symbols in each of its CTAs, a cluster of them, and do without the launch and the latency
+// of the names kernel: while the SMs have room for the work that is done several times (all 4 groups of 8 at K = 48
+// 13.3 -> 11.6 us, 40 of them at 512 40.4 -> 33.7, but 80 at 512 48.5 -> 56.3, and 400 at 100 44.2 -> 48.6).
+bool names_for_itself(int n_groups, int patterns, int symbols, int sms) {
+    const long long ctas = (long long)n_groups * patterns;
+    return patterns <= 8 && symbols <= 4096 && ctas <= 4 * sms && ctas * symbols <= 1200000LL;
+}
+
 // More than 48 KB of shared memory has to be asked for: the most that any call takes, once per device (noted,
 // because asking is host time).
 constexpr int kMostNamesSmem = 200 * 1024;
@@ -1699,9 +1736,10 @@ int allow_smem() {
     if (dev >= 0 && dev < 64 && allowed[dev].load(std::memory_order_relaxed)) return SR_OK;
     const int prep = SR_MAX_K * 4 + SR_MAX_N * SR_MAX_K * 2;
     SR_CUDA_TRY(cudaFuncSetAttribute(multi_names_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostNamesSmem));
-    for (auto kernel : {multi_prep_kernel<true, 0, false>, multi_prep_kernel<true, kMostPrepThreads, false>, multi_prep_kernel<false, 0, false>, multi_prep_kernel<false, kMostPrepThreads, false>})
+    for (auto kernel : {multi_prep_kernel<true, 0, false, false>, multi_prep_kernel<true, kMostPrepThreads, false, false>, multi_prep_kernel<false, 0, false, false>, multi_prep_kernel<false, kMostPrepThreads, false, false>})
         SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, prep));
-    for (auto kernel : {multi_prep_kernel<false, 0, true>, multi_prep_kernel<false, kMostPrepThreads, true>})
+    for (auto kernel : {multi_prep_kernel<false, 0, true, false>, multi_prep_kernel<false, kMostPrepThreads, true, false>,
+                        multi_prep_kernel<false, 0, true, true>, multi_prep_kernel<false, kMostPrepThreads, true, true>})
         SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostNamesSmem));
     if (dev >= 0 && dev < 64) allowed[dev].store(true, std::memory_order_relaxed);
     return SR_OK;
@@ -1735,8 +1773,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
 
     const bool in_pairs = !feed && runs_in_pairs(n_pairs, a.N, a.K, decide);
-    const int prep_smem = in_pairs ? W.pitch * 4 + a.N * (W.pitch + 8) * 2 + 32 + (a.N >> 1) * W.pitch * 2 + (2 * W.row_cap * W.row_words + 8) * 4
-                                   : W.pitch * 4 + a.N * W.pitch * 2;
+    const bool own_names = in_pairs && names_for_itself(a.n_groups, W.patterns, a.N * W.pitch, sms);
     // names: at least two slots to a symbol while symbols and table fit
     const int row_quads = W.pitch >> 2, sym_bytes = a.N * W.pitch * 4, names_most = a.N * W.pitch > 4 * 8 * 512 ? 1024 : 512;
     // A thread for every four positions of the group while 512 threads suffice; and for prep a warp for every 128
@@ -1751,6 +1788,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const int names_smem = sym_bytes + (2 << table_log);
     const uint32_t inv_row = (uint32_t)(((1ull << 32) + row_quads - 1) / row_quads);
     uint16_t* names = reinterpret_cast<uint16_t*>(ws + W.off_names);
+    int prep_smem = W.pitch * 4 + a.N * W.pitch * 2;
+    if (in_pairs) prep_smem += a.N * 16 + 32 + (a.N >> 1) * W.pitch * 2 + ((2 * W.row_cap * W.row_words + 11) & ~3) * 4;
+    if (own_names) prep_smem += a.N * W.pitch * 2 + names_smem;
     if (names_smem > 47 * 1024 || prep_smem > 36 * 1024) {    // with what the kernels declare
         const int rc = allow_smem();
         if (rc != SR_OK) return rc;
@@ -1772,13 +1812,19 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
             const int rc = feed->before(feed->ctx, g0, g1, s);
             if (rc != SR_OK) return rc;
         }
-        SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0,
+        if (!own_names)
+            SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0,
                   in_pairs ? reinterpret_cast<int32_t*>(ws + W.off_order) : nullptr);
         const auto prep = prep_threads == kMostPrepThreads
-            ? (in_pairs ? multi_prep_kernel<false, kMostPrepThreads, true>
-                        : decide ? multi_prep_kernel<true, kMostPrepThreads, false> : multi_prep_kernel<false, kMostPrepThreads, false>)
-            : (in_pairs ? multi_prep_kernel<false, 0, true> : decide ? multi_prep_kernel<true, 0, false> : multi_prep_kernel<false, 0, false>);
-        SR_LAUNCH("multi_prep_kernel", prep, (g1 - g0) * W.patterns, prep_threads, prep_smem, s, a, ws, W, dist, g0, exact, 2u);
+            ? (own_names ? multi_prep_kernel<false, kMostPrepThreads, true, true>
+               : in_pairs ? multi_prep_kernel<false, kMostPrepThreads, true, false>
+               : decide ? multi_prep_kernel<true, kMostPrepThreads, false, false> : multi_prep_kernel<false, kMostPrepThreads, false, false>)
+            : (own_names ? multi_prep_kernel<false, 0, true, true>
+               : in_pairs ? multi_prep_kernel<false, 0, true, false>
+               : decide ? multi_prep_kernel<true, 0, false, false> : multi_prep_kernel<false, 0, false, false>);
+        const int rc = launch_as(true, own_names ? W.patterns : 1, "multi_prep_kernel", prep, (g1 - g0) * W.patterns, prep_threads, prep_smem, s,
+                                 a, ws, W, dist, g0, exact, inv_row, table_log, 2u);
+        if (rc != SR_OK) return rc;
     }
     if (in_pairs) {
         if (ev) for (int k = 1; k <= 4; ++k) SR_CUDA_TRY(cudaEventRecord(ev[k], s));
