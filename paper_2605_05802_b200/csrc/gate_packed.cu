@@ -70,6 +70,10 @@ struct EventSet {
     ~EventSet() { for (int k = 0; k < n; ++k) cudaEventDestroy(ev[k]); }
 };
 
+// Symbols from which they are sent in pieces: less is on the link for no longer than the launches of a pass per piece
+// take (80 groups of 8 at K = 48 99 us in pieces, 38 in one; 200 at 256, 1.6 MB, 138 and 97; at 3 to 4 MB both are alike).
+constexpr long long kPieceBytes = 2ll << 20;
+
 struct PackedArena {
     size_t off_packed, off_start, inner, total;     // `inner`: where the padded-input arena begins
 };
@@ -145,7 +149,7 @@ int sr_gate_host_packed(const int32_t* symbols, const int64_t* row_start, int32_
     // whole gate into pieces was measured and lost: the kernels of a quarter of a token-level
     // batch take almost as long as those of the whole batch, because a few long pairs set the
     // time of the recurrence launch.
-    if (cs != nullptr && cs != s && K > 32 && n_groups >= 64) {
+    if (cs != nullptr && cs != s && K > 32 && n_groups >= 64 && total * 4 >= kPieceBytes) {
         constexpr int kPieces = 4;
         EventSet events;                                  // [0] fork, [1 + c] piece c copied
         for (int k = 0; k < 1 + kPieces; ++k) SR_CUDA_TRY(events.add());
