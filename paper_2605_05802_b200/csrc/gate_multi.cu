@@ -105,7 +105,11 @@ struct MultiWs {
     int row_words;         // 32-bit words of a mask row: one per 32 pattern positions
     int patterns;          // rollouts of a group that serve as patterns
     int row_cap;           // mask rows a pattern may have
+    int rows_pitch;        // 32-bit words from one pattern's mask rows to the next's: a multiple of four
     int warps;             // warps the dp kernel keeps resident
+    uint32_t inv_patterns; // 2^32 / patterns, rounded up
+    int text_warps, text_stride;   // prep: warps to a text, texts that the CTA's warps take at a time
+    uint32_t inv_text_warps;       // 2^32 / text_warps, rounded up
     bool alone;            // one CTA orders the batch, and adds up its work itself
 };
 
@@ -119,6 +123,9 @@ MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K, int row_cap) {
     w.pitch = (K + 7) & ~7;
     w.patterns = N & 1 ? N : N - 1;       // the last rollout of an even group is never a pattern
     w.warps = 1;
+    w.text_warps = w.text_stride = 1;
+    w.inv_text_warps = 0u;
+    w.inv_patterns = (uint32_t)(((1ull << 32) + w.patterns - 1) / w.patterns);
     w.alone = false;
     size_t off = 0;
     w.off_ctl = off;   off = align_up(off + sizeof(Ctl), 256);
@@ -131,8 +138,9 @@ MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K, int row_cap) {
     // a team's lanes cover up to 31 words more than the pattern has: slack after the last row
     w.row_words = (K + 3 + 31) >> 5;      // the pattern and what pads its texts to whole quads
     w.row_cap = row_cap;
+    w.rows_pitch = (w.row_cap * w.row_words + 3) & ~3;
     w.off_rows = off;
-    off = align_up(off + (size_t)n_groups * w.patterns * w.row_cap * w.row_words * 4 + 256, 256);
+    off = align_up(off + (size_t)n_groups * w.patterns * w.rows_pitch * 4 + 256, 256);
     w.off_names = off;
     off = align_up(off + (size_t)n_groups * N * w.pitch * 2, 256);
     w.total = off;
@@ -377,9 +385,6 @@ __device__ __forceinline__ void column_step(const uint32_t (&Eq)[R],
 // matches off the diagonal (sparse dynamic programming: Eppstein, Galil, Giancarlo and Italiano 1992), one
 // lane each.  A pair whose bounds are further apart than there are lanes has more such columns than that, and the
 // recurrence has it; the others are listed by prep, a warp each.
-// 1024 groups of 8 prefixes of 256..1024 uniform tokens: the recurrence took 174 us for them, this 37 us cold (20 M warp
-// instructions, 1100 a pair: a third to look through the stream, a third for the rows of repeated symbols), and the
-// whole gate went from 270 to 125 us.
 constexpr int kMostMatches = 32;                         // a lane each
 // Whether a pattern of m positions has so few repeated symbols that its pairs may have few matches: 1024 uniform
 // tokens have three or four (of a vocabulary of 32 000 sixteen), as long a text more than a hundred, one of 48 words four.
@@ -789,11 +794,11 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t* s_info = reinterpret_cast<uint32_t*>(smem);             // [pitch] see below
     uint16_t* s_map = reinterpret_cast<uint16_t*>(s_info + W.pitch);  // [N * pitch] stream entry of every name
-    // kPairs: [N / 2][pitch] streams, [2][row_cap * row_words] mask rows, and turned round
+    // kPairs: [N / 2][pitch] streams, [2][rows_pitch] mask rows, and turned round
     uint16_t* s_loc = s_map + a.N * (W.pitch + 8) + 16;
     uint32_t* s_rows = reinterpret_cast<uint32_t*>(s_loc + (a.N >> 1) * W.pitch);
     // kOwnNames: [N][pitch] names, [N][pitch] symbols and their table
-    uint16_t* s_names = reinterpret_cast<uint16_t*>(s_rows + ((2 * W.row_cap * W.row_words + 11) & ~3));
+    uint16_t* s_names = reinterpret_cast<uint16_t*>(s_rows + (2 * W.rows_pitch + 8));
     __shared__ int64_t s_stream[kMaxTexts];                           // where a text's stream begins
     __shared__ int s_txt[kMaxTexts], s_len[kMaxTexts], s_cp[kMaxTexts];
     __shared__ uint32_t s_count[kMaxTexts];  // differing positions | absent columns << 16
@@ -803,7 +808,10 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     const int N = a.N, K = a.K, P = pairs_of(N);
     const int tid = threadIdx.x, lane = tid & 31, nthr = kThreads ? kThreads : blockDim.x, warps = nthr >> 5;
     const int M = W.patterns;
-    const int g = g_base + blockIdx.x / M, i = blockIdx.x % M;
+    // (divisions by what only the host knows are its to prepare: five of them were a sixth of a warp's instructions)
+    int gl = M > 1 ? (int)__umulhi(blockIdx.x, W.inv_patterns) : (int)blockIdx.x;
+    if (gl * M > (int)blockIdx.x) --gl;
+    const int g = g_base + gl, i = (int)blockIdx.x - gl * M;
     if (tid < 4) s_repeats[tid] = 0;
     for (int e = tid; 8 * e < N * W.pitch; e += nthr)
         reinterpret_cast<uint4*>(s_map)[e] = make_uint4(kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u);
@@ -912,32 +920,47 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             more[0] = v.x; more[1] = v.y; more[2] = v.z; more[3] = v.w;
         }
         const bool claims = (more[0] | more[1] | more[2] | more[3]) != 0u;
-        if (claims) {
+        const bool any_claims = __any_sync(0xFFFFFFFFu, claims);
+        if (any_claims) {                              // symbols with >= 2, 3, 4 occurrences, ten bits each
+            uint32_t occur = 0u;
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                for (uint32_t c = 0; c < 3u && c < more[k]; ++c) atomicAdd(&s_repeats[c], 1);
+            for (int k = 0; k < 4; ++k) occur += (more[k] > 0u ? 1u : 0u) + (more[k] > 1u ? 1u << 10 : 0u) + (more[k] > 2u ? 1u << 20 : 0u);
+            occur = __reduce_add_sync(0xFFFFFFFFu, occur) >> (10 * min(lane, 2)) & 0x3FFu;
+            if (lane < 3 && occur) atomicAdd(&s_repeats[lane], (int)occur);
         }
         __syncthreads();
         const uint32_t need = s_repeats[0] <= W.row_cap ? 1u : (s_repeats[1] <= W.row_cap ? 2u : (s_repeats[2] <= W.row_cap ? 3u : 7u));
-        if (claims) {
+        if (any_claims) {
+            int asks = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) asks += more[k] >= need;
+            int row = asks;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int up = __shfl_up_sync(0xFFFFFFFFu, row, d);
+                if (lane >= d) row += up;
+            }
+            int first_row = 0;
+            if (lane == 31 && row) first_row = atomicAdd(&s_repeats[3], row);
+            row += __shfl_sync(0xFFFFFFFFu, first_row, 31) - asks;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if (more[k] == 0u) continue;
                 uint32_t code = (kChainEnd << 16) | kLocChain | (uint32_t)(p0 + k);
                 if (more[k] >= need) {
-                    const int row = atomicAdd(&s_repeats[3], 1);
                     if (row < W.row_cap) code = kLocRow | (uint32_t)row;
+                    ++row;
                 }
                 s_map[my_name[k]] = (uint16_t)code;             // what the streams of the texts say
                 s_info[p0 + k] = code;
             }
         }
         __syncthreads();
-        uint32_t* rows = kPairs ? s_rows : reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * M + i) * W.row_cap * W.row_words;
+        uint32_t* rows = kPairs ? s_rows : reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * M + i) * W.rows_pitch;
         const int n_rows = min(s_repeats[3], W.row_cap);
-        for (int e = tid; e < n_rows * W.row_words; e += nthr) {
-            rows[e] = 0u;
-            if (kPairs) rows[W.row_cap * W.row_words + e] = 0u;
+        for (int e = tid; 4 * e < n_rows * W.row_words; e += nthr) {
+            reinterpret_cast<uint4*>(rows)[e] = make_uint4(0u, 0u, 0u, 0u);
+            if (kPairs) reinterpret_cast<uint4*>(rows + W.rows_pitch)[e] = make_uint4(0u, 0u, 0u, 0u);
         }
         __syncthreads();
         if (claims || repeated) {
@@ -950,7 +973,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                 } else {
                     uint32_t* row = rows + (info & 0x3FFFu) * W.row_words;
                     atomicOr(row + (p >> 5), 1u << (p & 31));
-                    if (kPairs) atomicOr(row + (W.row_cap + 1) * W.row_words - 1 - (p >> 5), 0x80000000u >> (p & 31));
+                    if (kPairs) atomicOr(row + W.rows_pitch + W.row_words - 1 - (p >> 5), 0x80000000u >> (p & 31));
                 }
             }
         }
@@ -967,21 +990,23 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     // look-ups, one 8-byte store.  As many warps to a text as there are for each (chunks dealt to all
     // warps in turn would be even, but then every warp sets up every text).
     uint16_t* locs = reinterpret_cast<uint16_t*>(ws + W.off_loc);
-    const int per_text = max(1, warps / ntxt), warp = tid >> 5, part = warp % per_text;
-    for (int t = warp / per_text; t < ntxt; t += warps / per_text) {
+    const int per_text = W.text_warps, warp = tid >> 5, first_text = per_text > 1 ? (int)__umulhi((uint32_t)warp, W.inv_text_warps) : warp;
+    const int part = warp - first_text * per_text;
+    for (int t = first_text; t < ntxt; t += W.text_stride) {
         if (s_cp[t] < 0) continue;
         const int n = s_len[t];
         const uint2* in = reinterpret_cast<const uint2*>(names + s_txt[t] * W.pitch);
         const uint2* own = reinterpret_cast<const uint2*>(pat);
         uint2* out = reinterpret_cast<uint2*>(kPairs ? s_loc + t * W.pitch : locs + s_stream[t]);
-        uint32_t differ = 0u, present = 0u, seen = 0u, columns = 0u;
+        uint32_t differ = 0u, absent = 0u, seen = 0u;
         for (int q = ((s_cp[t] & ~31) >> 2) + 32 * part + lane; 4 * q < n; q += 32 * per_text) {
             const int left = n - 4 * q;                // columns of this quad that exist
             const uint2 v = in[q], o = own[q];         // past the pattern's end: still in the group's names or the rows after them
             uint32_t w0 = s_map[v.x & 0xFFFFu] | ((uint32_t)s_map[v.x >> 16] << 16);
             uint32_t w1 = s_map[v.y & 0xFFFFu] | ((uint32_t)s_map[v.y >> 16] << 16);
             // positions below both lengths whose symbol is not the pattern's symbol at the same place
-            uint32_t d0 = set_halves(v.x ^ o.x), d1 = set_halves(v.y ^ o.y);
+            // (names have 15 bits: the sum of a half does not reach the other)
+            uint32_t d0 = ((v.x ^ o.x) + 0x7FFF7FFFu) & 0x80008000u, d1 = ((v.y ^ o.y) + 0x7FFF7FFFu) & 0x80008000u;
             const int both = m - 4 * q;                // columns of this quad below the pattern's length
             if (left < 4 || both < 4) {
                 const int k = min(left, both);
@@ -998,11 +1023,10 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             out[q] = make_uint2(w0, w1);
             seen |= w0 | w1;
             differ += __popc(d0) + __popc(d1);
-            // columns without any match: 0x7FFF
-            present += __popc(set_halves(w0 ^ (kLocNone * 0x10001u))) + __popc(set_halves(w1 ^ (kLocNone * 0x10001u)));
-            columns += 4u;
+            // columns without any match, 0x7FFF: the only entries with bit 14 and without bit 15
+            absent += __popc(w0 & ~(w0 >> 1) & 0x40004000u) + __popc(w1 & ~(w1 >> 1) & 0x40004000u);
         }
-        const uint32_t count = __reduce_add_sync(0xFFFFFFFFu, differ + ((columns - present) << 16));
+        const uint32_t count = __reduce_add_sync(0xFFFFFFFFu, differ + (absent << 16));
         const bool row = __any_sync(0xFFFFFFFFu, (seen & (kLocRow * 0x10001u)) != 0u);
         if (lane == 0) {
             if (count) atomicAdd(&s_count[t], count);
@@ -1050,7 +1074,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         __syncthreads();
         // Teams of as many lanes as the pattern has blocks, 16 at the most, and as many pairs to a warp as have room.
         const bool chains = s_repeats[0] > min(s_repeats[3], W.row_cap);
-        const uint32_t* turned = s_rows + W.row_cap * W.row_words;
+        const uint32_t* turned = s_rows + W.rows_pitch;
         uint4* s_wide = reinterpret_cast<uint4*>(s_map);              // the map is not needed any more
         const int blocks = (m + 3 + 31) >> 5, tlog = min(32 - __clz(max(blocks, 1) - 1), 4), share = 16 >> tlog;
         for (int t0 = warp * share; t0 < ntxt; t0 += warps * share) {
@@ -1134,7 +1158,9 @@ multi_matches_kernel(unsigned char* ws, MultiWs W, int N, bool decide, int32_t* 
         const int upper = (int)(d.lower >> 16);
         int dist = -1;
         const int m = (int)(d.mn & 0xFFFFu), n = (int)(d.mn >> 16), strip = (int)((d.bin >> kStripShift) & 0x3FFu);
-        const int g = (int)(d.pat_row / (uint32_t)W.patterns), i = (int)d.pat_row - g * W.patterns;
+        int g = W.patterns > 1 ? (int)__umulhi(d.pat_row, W.inv_patterns) : (int)d.pat_row;
+        if (g * W.patterns > (int)d.pat_row) --g;
+        const int i = (int)d.pat_row - g * W.patterns;
         const int pr = kPairs.v[N][idx - g * P], j = (pr & 0xFF) + (pr >> 8) - i;
         const uint16_t* names = reinterpret_cast<const uint16_t*>(ws + W.off_names) + (size_t)g * N * W.pitch;
         __syncwarp();                              // the pair before has been read
@@ -1145,7 +1171,7 @@ multi_matches_kernel(unsigned char* ws, MultiWs W, int N, bool decide, int32_t* 
             dist = upper;
         else if (count <= kMostMatches)
             dist = distance_by_matches<false>(s_entries[warp], count, s_differ[warp],
-                                       reinterpret_cast<const uint32_t*>(ws + W.off_rows) + (size_t)d.pat_row * (W.row_cap * W.row_words),
+                                       reinterpret_cast<const uint32_t*>(ws + W.off_rows) + (size_t)d.pat_row * W.rows_pitch,
                                        W.row_words, m, n, strip, upper);
         if (dist >= 0) {
             if (lane == 0) {
@@ -1431,7 +1457,7 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
         // rows are 16-byte aligned and strip is a multiple of 4 entries: 8-byte loads
         loc4 = reinterpret_cast<const uint2*>(locs + (size_t)idx * W.pitch + strip);
         nxt = nexts + (size_t)d.pat_row * W.pitch;
-        rows = masks + (size_t)d.pat_row * (W.row_cap * W.row_words) + (strip >> 5);
+        rows = masks + (size_t)d.pat_row * W.rows_pitch + (strip >> 5);
     }
     if (T >= 16 && valid) {
         // Few pairs: nothing else hides the latencies of this one, so all that it will read goes to L1 first,
@@ -1783,13 +1809,16 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const int names_threads = min((a.N * row_quads + 31) & ~31, names_most), texts = a.N >> 1;
     const int fewest = (max((a.K + 127) >> 7, texts) + texts - 1) / texts * texts;
     const int prep_threads = (long long)a.n_groups * W.patterns <= sms ? kMostPrepThreads : min(32 * fewest, kMostPrepThreads);
+    W.text_warps = max(1, (prep_threads >> 5) / texts);
+    W.text_stride = (prep_threads >> 5) / W.text_warps;
+    W.inv_text_warps = (uint32_t)(((1ull << 32) + W.text_warps - 1) / W.text_warps);
     int table_log = 8;
     while ((1 << table_log) < 2 * a.N * a.K && sym_bytes + (4 << table_log) <= kMostNamesSmem) ++table_log;
     const int names_smem = sym_bytes + (2 << table_log);
     const uint32_t inv_row = (uint32_t)(((1ull << 32) + row_quads - 1) / row_quads);
     uint16_t* names = reinterpret_cast<uint16_t*>(ws + W.off_names);
     int prep_smem = W.pitch * 4 + a.N * W.pitch * 2;
-    if (in_pairs) prep_smem += a.N * 16 + 32 + (a.N >> 1) * W.pitch * 2 + ((2 * W.row_cap * W.row_words + 11) & ~3) * 4;
+    if (in_pairs) prep_smem += a.N * 16 + 32 + (a.N >> 1) * W.pitch * 2 + (2 * W.rows_pitch + 8) * 4;
     if (own_names) prep_smem += a.N * W.pitch * 2 + names_smem;
     if (names_smem > 47 * 1024 || prep_smem > 36 * 1024) {    // with what the kernels declare
         const int rc = allow_smem();
