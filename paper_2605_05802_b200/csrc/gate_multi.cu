@@ -1759,6 +1759,16 @@ bool names_for_itself(int n_groups, int patterns, int symbols, int sms) {
     return patterns <= 8 && symbols <= 4096 && ctas <= 4 * sms && ctas * symbols <= 1200000LL;
 }
 
+// Shared memory that keeps more CTAs than its share off every SM.  They start early, on the SMs that the names kernel leaves
+// first, and three of them there take longer than two on every SM (40 groups of 8 texts of 1024: 68 us, 60 with this; an
+// ordinary launch spreads them as well, but costs small batches 2 us).  Not for clusters, which then wait for
+// seven SMs of one GPC with that much to spare (40 groups at 512: 33 us, 43 with this).
+int even_smem(long long ctas, int sms) {
+    constexpr int kSm = 227 * 1024, kDeclared = 10 * 1024;       // what an SM has; what the kernel declares and the driver adds
+    const long long share = (ctas + sms - 1) / sms;
+    return share < 2 || share > 6 ? 0 : kSm / (int)(share + 1) + 1024 - kDeclared;
+}
+
 // More than 48 KB of shared memory has to be asked for: the most that any call takes, once per device (noted,
 // because asking is host time).
 constexpr int kMostNamesSmem = 200 * 1024;
@@ -1827,6 +1837,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     int prep_smem = W.pitch * 4 + a.N * W.pitch * 2;
     if (in_pairs) prep_smem += a.N * 16 + 32 + (a.N >> 1) * W.pitch * 2 + (2 * W.rows_pitch + 8) * 4;
     if (own_names) prep_smem += a.N * W.pitch * 2 + names_smem;
+    else if (in_pairs) prep_smem = max(prep_smem, even_smem((long long)a.n_groups * W.patterns, sms));
     if (names_smem > 47 * 1024 || prep_smem > 36 * 1024) {    // with what the kernels declare
         const int rc = allow_smem();
         if (rc != SR_OK) return rc;
