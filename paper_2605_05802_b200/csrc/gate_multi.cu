@@ -594,11 +594,17 @@ __device__ __forceinline__ uint32_t signs(uint32_t w0, uint32_t w1, uint32_t w2,
 // and wide, room for the wide one, of which it makes use afterwards; m, n: lengths; strip: common prefix to leave out (a
 // multiple of 4, of 32 where the stream names rows); live: false for lanes without a pair.  rows: the pattern's mask
 // rows, turned: the same with the order of a row's bits reversed; info: upper halves lead along the chains.
-template <int R>
+// kTwo: a team is a whole warp, the pair's other one the next warp (of an even one), and `tlog` the number of a barrier for
+// the two; the distance is then in the even warp's first lane.  With 32 lanes a half of 1024 columns takes 159
+// iterations of one block instead of 143 of two.
+template <int R, bool kTwo = false>
 __device__ __forceinline__ int distance_from_both_ends(const uint16_t* loc, uint4* wide, const uint32_t* rows, const uint32_t* turned, int row_words,
                                                        const uint32_t* info, bool chains, bool live, int m, int n, int strip, int tlog,
                                                        uint32_t two) {
-    const int lane = threadIdx.x & 31, T = 1 << tlog, gl = lane & (2 * T - 1), lt = lane & (T - 1);
+    const int lane = threadIdx.x & 31, T = kTwo ? 32 : 1 << tlog, gl = (int)threadIdx.x & (2 * T - 1), lt = lane & (T - 1);
+    auto meet = [&]() {
+        if (kTwo) asm volatile("bar.sync %0, 64;" ::"r"(tlog) : "memory"); else __syncwarp();
+    };
     const int pad = -n & 3;                            // both are extended to whole quads of columns
     m = live ? m + pad - strip : 0;
     n = live ? n + pad - strip : 0;
@@ -618,7 +624,7 @@ __device__ __forceinline__ int distance_from_both_ends(const uint16_t* loc, uint
     }
     if (gl == 0) wide[0] = make_uint4(kLocNone, kLocNone, kLocNone, kLocNone);
     if (gl == 1) wide[1 + nq] = make_uint4(kLocNone, kLocNone, kLocNone, kLocNone);
-    __syncwarp();
+    meet();
     // Backwards, position strip + p is row 32 W - 1 - p: the rows beyond the pattern's end come first, and
     // with vertical deltas of zero they hand on the +1 of row 0 as it is.
     const uint32_t sign = back ? ~0u : 1u, four = two * two, next_column = two * 128u;
@@ -691,7 +697,7 @@ __device__ __forceinline__ int distance_from_both_ends(const uint16_t* loc, uint
     }
     // The vertical deltas of the column where the halves meet: forwards along rows 1..m, backwards turned round.
     uint2* met = reinterpret_cast<uint2*>(wide);
-    __syncwarp();
+    meet();
     if (held && back) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -699,7 +705,7 @@ __device__ __forceinline__ int distance_from_both_ends(const uint16_t* loc, uint
             if (w >= 0) met[w] = make_uint2(__brev(endP[r]), __brev(endM[r]));
         }
     }
-    __syncwarp();
+    meet();
     int sum = 0, least = 0, whole = 0;
     if (held && !back) {
 #pragma unroll
@@ -720,7 +726,7 @@ __device__ __forceinline__ int distance_from_both_ends(const uint16_t* loc, uint
     }
     int incl = sum;
 #pragma unroll
-    for (int d = 1; d < 16; d <<= 1) {
+    for (int d = 1; d < (kTwo ? 32 : 16); d <<= 1) {
         const int up = __shfl_up_sync(0xFFFFFFFFu, incl, d);
         if (gl >= d) incl += up;
     }
@@ -728,7 +734,7 @@ __device__ __forceinline__ int distance_from_both_ends(const uint16_t* loc, uint
     if (back) least = 0;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        if (d >= 2 * T) break;
+        if (!kTwo && d >= 2 * T) break;
         whole += __shfl_xor_sync(0xFFFFFFFFu, whole, d);
         least = min(least, __shfl_xor_sync(0xFFFFFFFFu, least, d));
     }
@@ -787,7 +793,9 @@ __device__ __forceinline__ void finish_last(const GateArgs& a, int g, int parts,
 // kPairs: the whole gate after the names.  Streams and mask rows stay in shared memory, the distances are computed right
 // there, and the last CTA of a group evaluates it.
 // kOwnNames: the whole gate.  A group's CTAs are a cluster, and each of them names all of the group's symbols for itself.
-template <bool kDecide, int kThreads, bool kPairs, bool kOwnNames>
+// kTwoWarps: patterns of more than 512 positions and no more than two texts, a CTA to an SM: a pair has two warps (40
+// groups of 4 texts of 1024: 48 -> 37 us; with four texts the integer pipe is busy already, 16 groups of 8: 46 -> 48).
+template <bool kDecide, int kThreads, bool kPairs, bool kOwnNames, bool kTwoWarps = false>
 __global__ void __launch_bounds__(kMostPrepThreads, kPairs ? 3 : 6)
 multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base, uint8_t* exact, uint32_t inv_row, int table_log,
                   uint32_t two) {
@@ -1076,6 +1084,19 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         const bool chains = s_repeats[0] > min(s_repeats[3], W.row_cap);
         const uint32_t* turned = s_rows + W.rows_pitch;
         uint4* s_wide = reinterpret_cast<uint4*>(s_map);              // the map is not needed any more
+        if constexpr (kTwoWarps) {
+            const int t = warp >> 1;
+            if (t < ntxt && s_dist[t] < 0) {
+                const int n = s_len[t], strip = removed(t), high = (m + (-n & 3) - strip + 31) >> 5;
+                const uint16_t* loc = s_loc + t * W.pitch;
+                uint4* wide = s_wide + t * ((W.pitch + 8) >> 2);
+                const int d = high <= 32 ? distance_from_both_ends<1, true>(loc, wide, s_rows, turned, W.row_words, s_info, chains, true, m, n, strip, 1 + t, two)
+                                         : distance_from_both_ends<2, true>(loc, wide, s_rows, turned, W.row_words, s_info, chains, true, m, n, strip, 1 + t, two);
+                if ((tid & 63) == 0) dist_out[(size_t)g * P + pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N)] = d;
+            }
+            finish_last<kOwnNames>(a, g, M, dist_out, reinterpret_cast<int32_t*>(ws + W.off_order) + g, exact);
+            return;
+        }
         const int blocks = (m + 3 + 31) >> 5, tlog = min(32 - __clz(max(blocks, 1) - 1), 4), share = 16 >> tlog;
         for (int t0 = warp * share; t0 < ntxt; t0 += warps * share) {
             const int t = min(t0 + (lane >> (tlog + 1)), ntxt - 1);
@@ -1782,7 +1803,8 @@ int allow_smem() {
     for (auto kernel : {multi_prep_kernel<true, 0, false, false>, multi_prep_kernel<true, kMostPrepThreads, false, false>, multi_prep_kernel<false, 0, false, false>, multi_prep_kernel<false, kMostPrepThreads, false, false>})
         SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, prep));
     for (auto kernel : {multi_prep_kernel<false, 0, true, false>, multi_prep_kernel<false, kMostPrepThreads, true, false>,
-                        multi_prep_kernel<false, 0, true, true>, multi_prep_kernel<false, kMostPrepThreads, true, true>})
+                        multi_prep_kernel<false, 0, true, true>, multi_prep_kernel<false, kMostPrepThreads, true, true>,
+                        multi_prep_kernel<false, kMostPrepThreads, true, false, true>, multi_prep_kernel<false, kMostPrepThreads, true, true, true>})
         SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostNamesSmem));
     if (dev >= 0 && dev < 64) allowed[dev].store(true, std::memory_order_relaxed);
     return SR_OK;
@@ -1863,7 +1885,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
             SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0,
                   in_pairs ? reinterpret_cast<int32_t*>(ws + W.off_order) : nullptr);
         const auto prep = prep_threads == kMostPrepThreads
-            ? (own_names ? multi_prep_kernel<false, kMostPrepThreads, true, true>
+            ? (in_pairs && a.K > 512 && texts <= 2 && a.n_groups * W.patterns <= sms
+                   ? (own_names ? multi_prep_kernel<false, kMostPrepThreads, true, true, true> : multi_prep_kernel<false, kMostPrepThreads, true, false, true>)
+               : own_names ? multi_prep_kernel<false, kMostPrepThreads, true, true>
                : in_pairs ? multi_prep_kernel<false, kMostPrepThreads, true, false>
                : decide ? multi_prep_kernel<true, kMostPrepThreads, false, false> : multi_prep_kernel<false, kMostPrepThreads, false, false>)
             : (own_names ? multi_prep_kernel<false, 0, true, true>
