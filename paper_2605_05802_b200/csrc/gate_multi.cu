@@ -260,6 +260,8 @@ __device__ __forceinline__ int clamp_len(const int32_t* lens, size_t idx, int K,
 constexpr uint32_t kHashMul = 0x9E3779B1u;
 constexpr int kMaxTexts = SR_MAX_N / 2;        // texts a pattern is paired with
 constexpr int kMaxPairs = SR_MAX_N * (SR_MAX_N - 1) / 2;
+constexpr int kMostOwnPatterns = 8;            // of groups whose CTAs are a cluster: the portable size
+constexpr int kMaxOwnPairs = kMostOwnPatterns * (kMostOwnPatterns + 1) / 2;
 
 // s_sym: [N][pitch], s_table: [1 << table_log], s_len: the prefixes' lengths, out: [N][pitch].  All threads of a CTA, after a barrier.
 __device__ __forceinline__ void name_symbols(const GateArgs& a, int g, const int* s_len, int32_t* s_sym, uint16_t* s_table, int table_log,
@@ -329,7 +331,7 @@ multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int
         s_len[tid] = clamp_len(a.lens, (size_t)g * N + tid, a.K, neg);
         if (neg && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
     }
-    if (arrived && tid == 0) arrived[g] = 0;           // see finish_last
+    if (arrived && tid == 0) arrived[g] = 0;           // see arrive_last
     __syncthreads();
     name_symbols(a, g, s_len, s_sym, reinterpret_cast<uint16_t*>(s_sym + N * pitch), table_log, pitch, inv_row,
                  reinterpret_cast<uint2*>(names + (size_t)g * N * pitch));
@@ -741,33 +743,16 @@ __device__ __forceinline__ int distance_from_both_ends(const uint16_t* loc, uint
     return n + whole + least;                          // row 0: nothing of the pattern at the front, all of it at the back
 }
 
-// Evaluates group g once all of its `parts` CTAs are here: the first of a cluster's, or the last to count itself in
-// `arrived`.  All threads of a CTA call it after writing their distances.
-template <bool kCluster>
-__device__ __forceinline__ void finish_last(const GateArgs& a, int g, int parts, const int32_t* dist, int32_t* arrived, uint8_t* exact) {
+// Sum, threshold and outputs of group g by one CTA, from what distance(pair) and length(rollout) give.
+template <class Distance, class Length>
+__device__ __forceinline__ void evaluate_group(const GateArgs& a, int g, uint8_t* exact, Distance distance, Length length) {
     __shared__ double s_term[kMaxPairs];
     __shared__ int32_t s_d[kMaxPairs];
-    if constexpr (kCluster) {
-        cooperative_groups::this_cluster().sync();
-        if (blockIdx.x % parts != 0) return;
-    } else {
-        __shared__ bool s_last;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            s_last = atomicAdd(arrived, 1) == parts - 1;
-            __threadfence();
-        }
-        __syncthreads();
-        if (!s_last) return;
-    }
     const int N = a.N, P = pairs_of(N);
     for (int e = threadIdx.x; e < P; e += blockDim.x) {
         const int pr = kPairs.v[N][e];
-        bool neg = false;
-        const int mi = clamp_len(a.lens, (size_t)g * N + (pr & 0xFF), a.K, neg), mj = clamp_len(a.lens, (size_t)g * N + (pr >> 8), a.K, neg);
-        s_d[e] = __ldcg(dist + (size_t)g * P + e);
-        s_term[e] = pair_term(s_d[e], mi, mj, a.norm_mode);
+        s_d[e] = distance(e);
+        s_term[e] = pair_term(s_d[e], length(pr & 0xFF), length(pr >> 8), a.norm_mode);
     }
     __syncthreads();
     if (threadIdx.x != 0) return;
@@ -783,6 +768,19 @@ __device__ __forceinline__ void finish_last(const GateArgs& a, int g, int parts,
     if (a.mean) a.mean[g] = dk;
     a.stop[g] = dk < a.threshold ? 1 : 0;
     if (exact) exact[g] = 1;
+}
+
+// Whether this is the last of the group's `parts` CTAs to come here.  All threads of a CTA call it after writing their distances.
+__device__ __forceinline__ bool arrive_last(int parts, int32_t* arrived) {
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(arrived, 1) == parts - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    return s_last;
 }
 
 // One CTA per pattern.  Per text it also counts the columns whose symbol does not occur in the
@@ -825,12 +823,16 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         reinterpret_cast<uint4*>(s_map)[e] = make_uint4(kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u);
     for (int e = tid; 4 * e < W.pitch; e += nthr) reinterpret_cast<uint4*>(s_info)[e] = make_uint4(0u, 0u, 0u, 0u);
     grid_begin();
+    if (kOwnNames) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");     // the wait: before the first distance
     bool neg = false;
     const int m = clamp_len(a.lens, (size_t)g * N + i, K, neg);
     const uint16_t* names = kOwnNames ? s_names : reinterpret_cast<const uint16_t*>(ws + W.off_names) + (size_t)g * N * W.pitch;
     const uint16_t* pat = names + i * W.pitch;
+    // kOwnNames: the group's lengths, and in the cluster's first CTA its distances.  (The others write there once it has started.)
+    __shared__ int s_all_len[kOwnNames ? SR_MAX_N : 1];
+    __shared__ int32_t s_all_dist[kOwnNames ? kMaxOwnPairs : 1];
+    const auto cluster = cooperative_groups::this_cluster();
     if constexpr (kOwnNames) {
-        __shared__ int s_all_len[SR_MAX_N];
         if (tid < N) {
             bool negative = false;
             s_all_len[tid] = clamp_len(a.lens, (size_t)g * N + tid, K, negative);
@@ -1060,6 +1062,21 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         __shared__ uint4 s_differ[kMostPrepThreads / 32][kSpans];
         __shared__ uint32_t s_entries[kMostPrepThreads / 32][kMostMatches];
         __shared__ int s_dist[kMaxTexts];              // the distance, or -1: to be computed
+        auto settle = [&](int t, int d) {
+            const int pair = pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N);
+            if (kOwnNames) *cluster.map_shared_rank(s_all_dist + pair, 0) = d;
+            if (!kOwnNames || a.pair_dist) dist_out[(size_t)g * P + pair] = d;
+        };
+        auto finish = [&]() {
+            if constexpr (kOwnNames) {
+                cluster.sync();
+                if (i == 0) evaluate_group(a, g, exact, [&](int e) { return s_all_dist[e]; }, [&](int r) { return s_all_len[r]; });
+            } else if (arrive_last(M, reinterpret_cast<int32_t*>(ws + W.off_order) + g)) {
+                evaluate_group(a, g, exact, [&](int e) { return __ldcg(dist_out + (size_t)g * P + e); },
+                               [&](int r) { bool negative = false; return clamp_len(a.lens, (size_t)g * N + r, K, negative); });
+            }
+        };
+        if (kOwnNames) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         // first what the bounds and few matches settle
         for (int t = warp; t < ntxt; t += warps) {
             const int n = s_len[t], strip = removed(t);
@@ -1076,7 +1093,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             }
             if (lane == 0) {
                 s_dist[t] = d;
-                if (d >= 0) dist_out[(size_t)g * P + pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N)] = d;
+                if (d >= 0) settle(t, d);
             }
         }
         __syncthreads();
@@ -1092,9 +1109,9 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                 uint4* wide = s_wide + t * ((W.pitch + 8) >> 2);
                 const int d = high <= 32 ? distance_from_both_ends<1, true>(loc, wide, s_rows, turned, W.row_words, s_info, chains, true, m, n, strip, 1 + t, two)
                                          : distance_from_both_ends<2, true>(loc, wide, s_rows, turned, W.row_words, s_info, chains, true, m, n, strip, 1 + t, two);
-                if ((tid & 63) == 0) dist_out[(size_t)g * P + pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N)] = d;
+                if ((tid & 63) == 0) settle(t, d);
             }
-            finish_last<kOwnNames>(a, g, M, dist_out, reinterpret_cast<int32_t*>(ws + W.off_order) + g, exact);
+            finish();
             return;
         }
         const int blocks = (m + 3 + 31) >> 5, tlog = min(32 - __clz(max(blocks, 1) - 1), 4), share = 16 >> tlog;
@@ -1111,9 +1128,9 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             if (high <= 16) d = distance_from_both_ends<1>(loc, wide, s_rows, turned, W.row_words, s_info, chains, live, m, n, strip, tlog, two);
             else if (high <= 32) d = distance_from_both_ends<2>(loc, wide, s_rows, turned, W.row_words, s_info, chains, live, m, n, strip, tlog, two);
             else d = distance_from_both_ends<3>(loc, wide, s_rows, turned, W.row_words, s_info, chains, live, m, n, strip, tlog, two);
-            if (live && (lane & ((2 << tlog) - 1)) == 0) dist_out[(size_t)g * P + pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N)] = d;
+            if (live && (lane & ((2 << tlog) - 1)) == 0) settle(t, d);
         }
-        finish_last<kOwnNames>(a, g, M, dist_out, reinterpret_cast<int32_t*>(ws + W.off_order) + g, exact);
+        finish();
         return;
     }
     if (tid >= 32) return;                             // descriptors: the texts' threads are in the first warp
@@ -1777,7 +1794,7 @@ bool runs_in_pairs(int n_pairs, int N, int K, bool decide) { return decide ? K <
 // 13.3 -> 11.6 us, 40 of them at 512 40.4 -> 33.7, but 80 at 512 48.5 -> 56.3, and 400 at 100 44.2 -> 48.6).
 bool names_for_itself(int n_groups, int patterns, int symbols, int sms) {
     const long long ctas = (long long)n_groups * patterns;
-    return patterns <= 8 && symbols <= 4096 && ctas <= 4 * sms && ctas * symbols <= 1200000LL;
+    return patterns <= kMostOwnPatterns && symbols <= 4096 && ctas <= 4 * sms && ctas * symbols <= 1200000LL;
 }
 
 // Shared memory that keeps more CTAs than its share off every SM.  They start early, on the SMs that the names kernel leaves
