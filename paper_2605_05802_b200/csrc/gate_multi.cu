@@ -1795,10 +1795,11 @@ bool runs_in_pairs(int n_pairs, int N, int K, bool decide) { return decide ? K <
 
 // And which of them name a group's symbols in each of its CTAs, a cluster of them, and do without the launch and the latency
 // of the names kernel: while the SMs have room for the work that is done several times (all 4 groups of 8 at K = 48
-// 13.3 -> 11.6 us, 40 of them at 512 40.4 -> 33.7, but 80 at 512 48.5 -> 56.3, and 400 at 100 44.2 -> 48.6).
+// 13.3 -> 11.6 us, 40 of them at 512 40.4 -> 33.7, 21 at 600 49.7 -> 40.7, but 80 at 512 48.5 -> 56.3, 16 at 1024 43 -> 57,
+// and 400 at 100 44.2 -> 48.6).
 bool names_for_itself(int n_groups, int patterns, int symbols, int sms) {
     const long long ctas = (long long)n_groups * patterns;
-    return patterns <= kMostOwnPatterns && symbols <= 4096 && ctas <= 4 * sms && ctas * symbols <= 1200000LL;
+    return patterns <= kMostOwnPatterns && symbols <= 5000 && ctas <= 4 * sms && ctas * symbols <= 1200000LL;
 }
 
 // Shared memory that keeps more CTAs than its share off every SM.  They start early, on the SMs that the names kernel leaves
