@@ -774,6 +774,42 @@ __device__ __forceinline__ void evaluate_group(const GateArgs& a, int g, uint8_t
     if (exact) exact[g] = 1;
 }
 
+// Decide mode: d_K of group g on its pairs' lower bounds, and where the mask is all that is wanted on the upper ones (see
+// multi_bound_kernel).  True, in all threads, if that settles the group; its outputs are then written.
+__device__ __forceinline__ int settle_group(const GateArgs& a, int g, uint8_t* exact, const int32_t* lower, const int32_t* upper, const int* len) {
+    __shared__ double s_below[kMaxOwnPairs], s_above[kMaxOwnPairs];
+    __shared__ int s_settled_here;
+    const int N = a.N, P = pairs_of(N);
+    for (int e = threadIdx.x; e < P; e += blockDim.x) {
+        const int pr = kPairs.v[N][e], m = len[pr & 0xFF], n = len[pr >> 8];
+        s_below[e] = pair_term(lower[e], m, n, a.norm_mode);
+        s_above[e] = pair_term(upper[e], m, n, a.norm_mode);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double below = 0.0, above = 0.0;
+        int isum = 0;
+#pragma unroll 4
+        for (int p = 0; p < P; ++p) {
+            below = __dadd_rn(below, s_below[p]);
+            above = __dadd_rn(above, s_above[p]);
+            isum += lower[p];
+        }
+        const double dk = __ddiv_rn(below, (double)P);
+        const bool mask_only = !a.pair_dist && !a.pair_sum && !a.mean && !exact;
+        const bool cut = mask_only && __ddiv_rn(above, (double)P) < a.threshold;
+        s_settled_here = !(dk < a.threshold) || cut;
+        if (s_settled_here) {
+            if (a.pair_sum) a.pair_sum[g] = isum;
+            if (a.mean) a.mean[g] = dk;
+            if (exact) exact[g] = 0;
+            a.stop[g] = cut ? 1 : 0;
+        }
+    }
+    __syncthreads();
+    return s_settled_here;
+}
+
 // Whether this is the last of the group's `parts` CTAs to come here.  All threads of a CTA call it after writing their distances.
 __device__ __forceinline__ bool arrive_last(int parts, int32_t* arrived) {
     __shared__ bool s_last;
@@ -795,12 +831,15 @@ __device__ __forceinline__ bool arrive_last(int parts, int32_t* arrived) {
 // kPairs: the whole gate after the names.  Streams and mask rows stay in shared memory, the distances are computed right
 // there, and the last CTA of a group evaluates it.
 // kOwnNames: the whole gate.  A group's CTAs are a cluster, and each of them names all of the group's symbols for itself.
+// kDecide and kPairs: a group's CTAs are a cluster, whose first one sums up the pairs' bounds, as multi_bound_kernel does; no
+// distance is computed for a group that they settle.
 // kTwoWarps: patterns of more than 512 positions and no more than two texts, a CTA to an SM: a pair has two warps (40
 // groups of 4 texts of 1024: 48 -> 37 us; with four texts the integer pipe is busy already, 16 groups of 8: 46 -> 48).
 template <bool kDecide, int kThreads, bool kPairs, bool kOwnNames, bool kTwoWarps = false>
 __global__ void __launch_bounds__(kMostPrepThreads, kPairs ? 3 : 6)
 multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base, uint8_t* exact, uint32_t inv_row, int table_log,
                   uint32_t two) {
+    constexpr bool kCluster = kOwnNames || (kDecide && kPairs);
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t* s_info = reinterpret_cast<uint32_t*>(smem);             // [pitch] see below
     uint16_t* s_map = reinterpret_cast<uint16_t*>(s_info + W.pitch);  // [N * pitch] stream entry of every name
@@ -827,21 +866,26 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         reinterpret_cast<uint4*>(s_map)[e] = make_uint4(kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u);
     for (int e = tid; 4 * e < W.pitch; e += nthr) reinterpret_cast<uint4*>(s_info)[e] = make_uint4(0u, 0u, 0u, 0u);
     grid_begin();
-    if (kOwnNames) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");     // the wait: before the first distance
+    if (kCluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");     // the wait: before the first distance
     bool neg = false;
     const int m = clamp_len(a.lens, (size_t)g * N + i, K, neg);
     const uint16_t* names = kOwnNames ? s_names : reinterpret_cast<const uint16_t*>(ws + W.off_names) + (size_t)g * N * W.pitch;
     const uint16_t* pat = names + i * W.pitch;
-    // kOwnNames: the group's lengths, and in the cluster's first CTA its distances.  (The others write there once it has started.)
-    __shared__ int s_all_len[kOwnNames ? SR_MAX_N : 1];
-    __shared__ int32_t s_all_dist[kOwnNames ? kMaxOwnPairs : 1];
+    // kCluster: the group's lengths, and in the cluster's first CTA its distances (and upper bounds).  (The others write
+    // there once it has started.)
+    __shared__ int s_all_len[kCluster ? SR_MAX_N : 1];
+    __shared__ int32_t s_all_dist[kCluster ? kMaxOwnPairs : 1];
+    __shared__ int32_t s_all_upper[kCluster && kDecide ? kMaxOwnPairs : 1];
+    __shared__ int s_settled;
     const auto cluster = cooperative_groups::this_cluster();
-    if constexpr (kOwnNames) {
+    if constexpr (kCluster) {
         if (tid < N) {
             bool negative = false;
             s_all_len[tid] = clamp_len(a.lens, (size_t)g * N + tid, K, negative);
-            if (negative && i == 0 && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
+            if (kOwnNames && negative && i == 0 && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
         }
+    }
+    if constexpr (kOwnNames) {
         __syncthreads();
         int32_t* s_sym = reinterpret_cast<int32_t*>(s_names + N * W.pitch);
         name_symbols(a, g, s_all_len, s_sym, reinterpret_cast<uint16_t*>(s_sym + N * W.pitch), table_log, W.pitch, inv_row, reinterpret_cast<uint2*>(s_names));
@@ -1068,11 +1112,11 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         __shared__ int s_dist[kMaxTexts];              // the distance, or -1: to be computed
         auto settle = [&](int t, int d) {
             const int pair = pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N);
-            if (kOwnNames) *cluster.map_shared_rank(s_all_dist + pair, 0) = d;
-            if (!kOwnNames || a.pair_dist) dist_out[(size_t)g * P + pair] = d;
+            if (kCluster) *cluster.map_shared_rank(s_all_dist + pair, 0) = d;
+            if (!kCluster || a.pair_dist) dist_out[(size_t)g * P + pair] = d;
         };
         auto finish = [&]() {
-            if constexpr (kOwnNames) {
+            if constexpr (kCluster) {
                 cluster.sync();
                 if (i == 0) evaluate_group(a, g, exact, [&](int e) { return s_all_dist[e]; }, [&](int r) { return s_all_len[r]; });
             } else if (arrive_last(M, reinterpret_cast<int32_t*>(ws + W.off_order) + g)) {
@@ -1080,14 +1124,20 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                                [&](int r) { bool negative = false; return clamp_len(a.lens, (size_t)g * N + r, K, negative); });
             }
         };
-        if (kOwnNames) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+        if (kCluster) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         // first what the bounds and few matches settle
         for (int t = warp; t < ntxt; t += warps) {
             const int n = s_len[t], strip = removed(t);
             int lower, upper;
             bounds(t, strip, lower, upper);
             int d = lower < upper ? -1 : lower;
-            if (d < 0 && upper - lower <= kMostMatches && few_repeats(s_repeats[0], m) && n + m - 2 * strip > kWorthMatches) {
+            if (kDecide) {                             // bounds first; few matches are no cheaper than what follows
+                if (lane == 0) {
+                    const int pair = pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N);
+                    *cluster.map_shared_rank(s_all_upper + pair, 0) = upper;
+                    if (d < 0) settle(t, lower);
+                }
+            } else if (d < 0 && upper - lower <= kMostMatches && few_repeats(s_repeats[0], m) && n + m - 2 * strip > kWorthMatches) {
                 __syncwarp();
                 const int count = find_matches<true>(reinterpret_cast<const uint2*>(s_loc + t * W.pitch), reinterpret_cast<const uint2*>(names + s_txt[t] * W.pitch),
                                                      reinterpret_cast<const uint2*>(pat), m, n, strip, s_differ[warp], s_entries[warp]);
@@ -1099,6 +1149,15 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                 s_dist[t] = d;
                 if (d >= 0) settle(t, d);
             }
+        }
+        if constexpr (kDecide) {
+            cluster.sync();
+            if (i == 0) {
+                const int settled = settle_group(a, g, exact, s_all_dist, s_all_upper, s_all_len);
+                if (tid < M) *cluster.map_shared_rank(&s_settled, tid) = settled;
+            }
+            cluster.sync();
+            if (s_settled) return;
         }
         __syncthreads();
         // Teams of as many lanes as the pattern has blocks, 16 at the most, and as many pairs to a warp as have room.
@@ -1789,9 +1848,10 @@ multi_finish_kernel(GateArgs a, int32_t* dist, const uint8_t* flag, uint8_t* exa
 // Which batches take every pair from both ends instead of sorting the pairs into warp tasks: those whose
 // work leaves the SMs idle anyway.  Both sides at the line for texts, us: 600 groups of 8 at K = 48 49 and 46, 250 at 256 45 and
 // 58, at 512 83 and 92; 150 at 1024 about 140 both; four groups of 8 at 1024 41 and 84.  With more texts to a pattern than a CTA
-// has warps the line lies lower (16 groups of 24 at 1024: 174 and 149).  The decide mode has less to do the
-// other way, where bounds settle most groups: 40 groups of 8 at 256 24 and 27 to 50, but at 512 47 and 29.
-bool runs_in_pairs(int n_pairs, int N, int K, bool decide) { return decide ? K <= 256 && n_pairs <= 2800 : (long long)n_pairs * (K + 384) <= (N <= 17 ? 6400000LL : 4200000LL); }
+// has warps the line lies lower (16 groups of 24 at 1024: 174 and 149).  The decide mode does so for
+// groups of up to eight, whose CTAs are a cluster that sums up the bounds first (40 groups of 8 texts of 512: 29 -> 15 us ragged, 72 -> 28 at
+// full length; 250 of 256: 31 and 62 without this, about the same with it).
+bool runs_in_pairs(int n_pairs, int N, int K, bool decide) { return decide ? N <= kMostOwnPatterns && n_pairs <= 7000 && (long long)n_pairs * (K + 384) <= 6400000LL : (long long)n_pairs * (K + 384) <= (N <= 17 ? 6400000LL : 4200000LL); }
 
 // And which of them name a group's symbols in each of its CTAs, a cluster of them, and do without the launch and the latency
 // of the names kernel: while the SMs have room for the work that is done several times (all 4 groups of 8 at K = 48
@@ -1826,7 +1886,9 @@ int allow_smem() {
         SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, prep));
     for (auto kernel : {multi_prep_kernel<false, 0, true, false>, multi_prep_kernel<false, kMostPrepThreads, true, false>,
                         multi_prep_kernel<false, 0, true, true>, multi_prep_kernel<false, kMostPrepThreads, true, true>,
-                        multi_prep_kernel<false, kMostPrepThreads, true, false, true>, multi_prep_kernel<false, kMostPrepThreads, true, true, true>})
+                        multi_prep_kernel<false, kMostPrepThreads, true, false, true>, multi_prep_kernel<false, kMostPrepThreads, true, true, true>,
+                        multi_prep_kernel<true, 0, true, false>, multi_prep_kernel<true, kMostPrepThreads, true, false>,
+                        multi_prep_kernel<true, 0, true, true>, multi_prep_kernel<true, kMostPrepThreads, true, true>})
         SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostNamesSmem));
     if (dev >= 0 && dev < 64) allowed[dev].store(true, std::memory_order_relaxed);
     return SR_OK;
@@ -1860,6 +1922,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
 
     const bool in_pairs = !feed && runs_in_pairs(n_pairs, a.N, a.K, decide);
+    const bool clusters = in_pairs && decide;         // whose CTAs sum up their bounds together
     const bool own_names = in_pairs && names_for_itself(a.n_groups, W.patterns, a.N * W.pitch, sms);
     // names: at least two slots to a symbol while symbols and table fit; above 4096 symbols one, and four CTAs to an SM instead
     // of three (1024 groups of 8 of up to 1024: 122.0 -> 120.1 us)
@@ -1882,8 +1945,8 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     int prep_smem = W.pitch * 4 + a.N * W.pitch * 2;
     if (in_pairs) prep_smem += a.N * 16 + 32 + (a.N >> 1) * W.pitch * 2 + (2 * W.rows_pitch + 8) * 4;
     if (own_names) prep_smem += a.N * W.pitch * 2 + names_smem;
-    else if (in_pairs) prep_smem = max(prep_smem, even_smem((long long)a.n_groups * W.patterns, sms));
-    if (names_smem > 47 * 1024 || prep_smem > 36 * 1024) {    // with what the kernels declare
+    else if (in_pairs && !clusters) prep_smem = max(prep_smem, even_smem((long long)a.n_groups * W.patterns, sms));
+    if (names_smem > 47 * 1024 || prep_smem > 35 * 1024) {    // with what the kernels declare
         const int rc = allow_smem();
         if (rc != SR_OK) return rc;
     }
@@ -1907,16 +1970,18 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
         if (!own_names)
             SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0,
                   in_pairs ? reinterpret_cast<int32_t*>(ws + W.off_order) : nullptr);
-        const auto prep = prep_threads == kMostPrepThreads
-            ? (in_pairs && a.K > 512 && texts <= 2 && a.n_groups * W.patterns <= sms
-                   ? (own_names ? multi_prep_kernel<false, kMostPrepThreads, true, true, true> : multi_prep_kernel<false, kMostPrepThreads, true, false, true>)
-               : own_names ? multi_prep_kernel<false, kMostPrepThreads, true, true>
-               : in_pairs ? multi_prep_kernel<false, kMostPrepThreads, true, false>
-               : decide ? multi_prep_kernel<true, kMostPrepThreads, false, false> : multi_prep_kernel<false, kMostPrepThreads, false, false>)
-            : (own_names ? multi_prep_kernel<false, 0, true, true>
-               : in_pairs ? multi_prep_kernel<false, 0, true, false>
-               : decide ? multi_prep_kernel<true, 0, false, false> : multi_prep_kernel<false, 0, false, false>);
-        const int rc = launch_as(true, own_names ? W.patterns : 1, "multi_prep_kernel", prep, (g1 - g0) * W.patterns, prep_threads, prep_smem, s,
+        const int cluster = own_names || clusters ? W.patterns : 1;
+        const bool most = prep_threads == kMostPrepThreads;
+        const auto in_memory = decide ? (most ? multi_prep_kernel<true, kMostPrepThreads, false, false> : multi_prep_kernel<true, 0, false, false>)
+                                      : (most ? multi_prep_kernel<false, kMostPrepThreads, false, false> : multi_prep_kernel<false, 0, false, false>);
+        const auto pairs = decide ? (most ? multi_prep_kernel<true, kMostPrepThreads, true, false> : multi_prep_kernel<true, 0, true, false>)
+                                  : (most ? multi_prep_kernel<false, kMostPrepThreads, true, false> : multi_prep_kernel<false, 0, true, false>);
+        const auto alone_pairs = decide ? (most ? multi_prep_kernel<true, kMostPrepThreads, true, true> : multi_prep_kernel<true, 0, true, true>)
+                                        : (most ? multi_prep_kernel<false, kMostPrepThreads, true, true> : multi_prep_kernel<false, 0, true, true>);
+        const bool in_twos = in_pairs && most && !decide && a.K > 512 && texts <= 2 && a.n_groups * W.patterns <= sms;
+        const auto prep = in_twos ? (own_names ? multi_prep_kernel<false, kMostPrepThreads, true, true, true> : multi_prep_kernel<false, kMostPrepThreads, true, false, true>)
+                        : own_names ? alone_pairs : in_pairs ? pairs : in_memory;
+        const int rc = launch_as(true, cluster, "multi_prep_kernel", prep, (g1 - g0) * W.patterns, prep_threads, prep_smem, s,
                                  a, ws, W, dist, g0, exact, inv_row, table_log, 2u);
         if (rc != SR_OK) return rc;
     }
