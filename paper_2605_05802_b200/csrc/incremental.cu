@@ -109,7 +109,7 @@ struct IncrArgs {
     int32_t* status;
     int gpb;                                               // groups per CTA
     uint32_t inv_P, inv_N;                                 // ceil(2^20 / P), ceil(2^20 / N): x / P by multiply-shift, exact while x (P - 1) < 2^20 (x: pairs of a CTA, at most 1984)
-    int off_dist, off_term, off_roll, off_eq;              // shared-memory offsets
+    int off_dist, off_term, off_roll, off_eq, off_state;              // shared-memory offsets
     uint32_t one;                                          // 1, as a run-time value
 };
 
@@ -295,7 +295,7 @@ __device__ __forceinline__ void pair_at(int e, int N, int P, int kN, uint32_t in
 // (Registers decide: with one pair state in flight 656 us at 56 registers, 612 at 48, 665 at 40; with four
 // 706 at 60, and 884 at 48, where it spills.)
 // kN: as above.
-template <int kN, int kMasks>
+template <int kN, int kMasks, bool kStaged>
 __global__ void __launch_bounds__(kRollThreads, kN ? 9 : 8)
 incr_rollout_kernel(IncrArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -304,6 +304,7 @@ incr_rollout_kernel(IncrArgs a) {
     int32_t* s_dist = reinterpret_cast<int32_t*>(smem + a.off_dist);    // [gpb][P]
     int2* s_roll = reinterpret_cast<int2*>(smem + a.off_roll);          // [gpb * N] length before, action or none
     uint32_t* s_eq = reinterpret_cast<uint32_t*>(smem + a.off_eq);      // [gpb * N][N - 1]
+    uint4* s_state = reinterpret_cast<uint4*>(smem + a.off_state);      // [gpb][P] pair states
     const int g = kN ? tid / N : div20(tid, a.inv_N), i = tid - g * N;
     // the thread's first pair: indices and a table, no need to wait for them
     int gi, gj, ahead;
@@ -322,9 +323,16 @@ incr_rollout_kernel(IncrArgs a) {
     int my_len = 0;
     int32_t my_act = SR_NO_ACTION;
     if (is_roll) { my_len = g_len[tid]; my_act = __ldg(g_new + tid); }
-    // the first pair's state is on its way while the masks are made
+    // the first pair's state is on its way while the masks are made (kStaged: all of the thread's, without registers)
     uint4 st = make_uint4(0u, 0u, 0u, 0u);
-    if (tid < ng * P) st = g_pairs[tid];
+    if constexpr (kStaged) {
+        for (int e = tid; e < ng * P; e += kRollThreads) {
+            const uint32_t to = (uint32_t)__cvta_generic_to_shared(s_state + e);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to), "l"(g_pairs + e) : "memory");
+        }
+    } else if (tid < ng * P) {
+        st = g_pairs[tid];
+    }
     const bool bad = hdr.x != kMagic || hdr.y != (uint32_t)a.n_groups || hdr.z != (uint32_t)N;
     if (bad) {                                     // uniform over the grid: nothing is touched
         if (tid == 0 && a.status) atomicOr(a.status, SR_STATUS_BAD_STATE);
@@ -382,6 +390,7 @@ incr_rollout_kernel(IncrArgs a) {
             g_len[tid] = my_len + 1;
         }
     }
+    if constexpr (kStaged) asm volatile("cp.async.wait_all;" ::: "memory");       // each thread reads what it has copied itself
     __syncthreads();
     auto pair = [&](int e, uint4 state) {
         const int2 A = s_roll[gi], B = s_roll[gj];
@@ -392,10 +401,10 @@ incr_rollout_kernel(IncrArgs a) {
         s_term[e] = a.norm_mode == SR_NORM_NONE ? (double)d : kQuot.v[d * 33 + max(m, n)];
         if (a.pair_dist) a.pair_dist[(size_t)g0 * P + e] = d;
     };
-    if (tid < ng * P) pair(tid, st);
+    if (tid < ng * P) pair(tid, kStaged ? s_state[tid] : st);
 #pragma unroll 2
     for (int e = tid + kRollThreads; e < ng * P; e += kRollThreads) {
-        st = g_pairs[e];
+        st = kStaged ? s_state[e] : g_pairs[e];
         pair_at(e, N, P, kN, a.inv_P, gi, gj, ahead);
         pair(e, st);
     }
@@ -462,15 +471,19 @@ int launch_incr_step(void* state, size_t bytes, const int32_t* new_actions, int3
     int off = 0;
     auto take = [&](int b) { int o = off; off = (off + b + 15) & ~15; return o; };
     // the thread-per-rollout form has the longer chain per thread and pays off once several CTAs of it
-    // share every SM (N = 8: from 20000 groups on; N = 16: from about 5000)
-    if ((long long)n_groups * P >= 550000) {
+    // share every SM (N = 8: from 17000 groups on, 30 steps on 19600 275 and 250 us, on 14000 215 and 241; N = 16: from about 5000)
+    if ((long long)n_groups * P >= (N == 8 ? 470000 : 550000)) {
         a.gpb = kRollThreads / N;
         a.off_dist = take(pair_sum ? a.gpb * P * 4 : 0);
         a.off_term = take(a.gpb * P * 8);
         a.off_roll = take(a.gpb * N * 8);
         a.off_eq = take(a.gpb * N * (N - 1) * 4);
-        auto kernel = N == 8 ? incr_rollout_kernel<8, 7> : (N <= 5 ? incr_rollout_kernel<0, 4>
-                                  : (N <= 8 ? incr_rollout_kernel<0, 7> : incr_rollout_kernel<0, 8>));
+        // Groups of 8 up to a wave and a half: the loads of one CTA's states are what the others of its SM wait for as well
+        // (30 steps on 20000 groups 264 -> 249 us, 46000 449 -> 434, 65536 614 -> 617; 5000 of 16 370 -> 398).
+        const bool staged = N == 8 && (long long)n_groups * P < 1300000;
+        a.off_state = take(staged ? a.gpb * P * 16 : 0);
+        auto kernel = N == 8 ? (staged ? incr_rollout_kernel<8, 7, true> : incr_rollout_kernel<8, 7, false>) : (N <= 5 ? incr_rollout_kernel<0, 4, false>
+                                  : (N <= 8 ? incr_rollout_kernel<0, 7, false> : incr_rollout_kernel<0, 8, false>));
         const int blocks = (n_groups + a.gpb - 1) / a.gpb;
         int sms = 0;
         const int rc = sm_count(sms);
