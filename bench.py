@@ -241,9 +241,6 @@ def main():
     G, N, stride, K = w.n_groups, w.N, w.stride, w.K
     P = N * (N - 1) // 2
     cells = W.dp_cells(w.lens, K)
-    wcols_full = W.word_columns(w.lens, K)
-    # what the method runs: without the pairs' common prefixes, inside the bands of their bounds
-    wcols = W.word_columns(w.lens, K, w.seqs, band=True)
     seqs = torch.from_numpy(w.seqs).to(dev)
     lens = torch.from_numpy(w.lens).to(dev)
     rewards = torch.from_numpy(w.rewards).to(dev)
@@ -317,7 +314,7 @@ def main():
         sampler.hold(step, 4, 1.0)
         clocks = sampler.stop()
     stage_ms = [statistics.median(e5[k].elapsed_time(e5[k + 1]) for e5 in stage_evs) for k in range(4)]
-    dp_ms = stage_ms[2]
+    prep_ms = stage_ms[0]
 
     # ------------------------------------------------------------------ end to end
     # host side: the batch as a rollout buffer holds it, prefixes back to back plus row offsets
@@ -360,7 +357,10 @@ def main():
     value = cells * world * args.steps / (total_ms * 1e-3) / 1e9
     e2e_value = cells * world * args.steps / (e2e_ms * 1e-3) / 1e9
     alu_peak = sms * SM_INT32_LANES * peaks["sm_max_mhz"] * 1e6 / 1e9          # Gop/s
-    achieved = 10.0 * wcols / (dp_ms * 1e-3) / 1e9
+    # Uniform tokens leave the recurrence nothing to do: names, look-ups and the pairs' few matches are the step, and what
+    # they cannot do without is the symbols in and a distance per pair out.
+    gate_bytes = int(np.minimum(w.lens, K).sum()) * 4 + G * N * 4 + G * P * 4
+    achieved = gate_bytes / (prep_ms * 1e-3) / 1e9
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": max(args.warmup, 3), "ms_per_step": total_ms / args.steps, "higher_is_better": True,
@@ -374,16 +374,14 @@ def main():
                 "ms_per_step": e2e_ms / args.steps,
                 "input": "packed prefixes + int64 row offsets in pinned host memory (sr_gate_host_packed), "
                          "sent in four pieces on a copy stream under the per-group pass; one recurrence launch"},
-        "gpu_launches": 7 * args.steps,       # names, prep, bin, order, dp, finish; advantages
+        "gpu_launches": 8 * args.steps,       # names, prep, matches, bin, order, dp, finish; advantages
         "clocks": clocks,
         "stage_ms": {"prep": stage_ms[0], "order": stage_ms[1], "dp": stage_ms[2], "finish": stage_ms[3]},
-        "roofline": {"kernel": "multi_dp_kernel", "bound": "alu", "achieved": achieved, "peak": alu_peak,
-                     "unit": "Gop/s (int32 lane-ops, 10 per 32-row block per column, counted inside the bands of the pairs' bounds, common prefixes left out)",
-                     "frac": achieved / alu_peak,
-                     "peak_basis": f"{sms} SMs x {SM_INT32_LANES} int32 lanes/clk x {peaks['sm_max_mhz']:.0f} MHz (derived)",
-                     "traffic": traffic_from_profiles("multi_dp_kernel", os.path.join(ROOT, "paper_2605_05802_b200", "csrc", "gate_multi.cu")),
-                     "word_columns": wcols, "word_columns_whole_matrices": wcols_full,
-                     "ms_per_launch": dp_ms},
+        "roofline": {"kernel": "multi_names_kernel + multi_prep_kernel + multi_matches_kernel", "bound": "hbm", "achieved": achieved,
+                     "peak": peaks["hbm_gbs"], "unit": "GB/s (symbols and lengths in, distances out) of measured copy", "frac": achieved / peaks["hbm_gbs"],
+                     "limited_by": "instruction issue: naming, 640 look-ups a pair and text, 1100 warp instructions a pair for its matches",
+                     "traffic": traffic_from_profiles("multi_prep_kernel", os.path.join(ROOT, "paper_2605_05802_b200", "csrc", "gate_multi.cu")),
+                     "ms_per_launch": prep_ms},
         "verified_against_oracle": verify,
     }
 
@@ -396,15 +394,6 @@ def main():
             ms = min(timed(lambda: sr.sr_probe_int32(var, 2000, sms * 8, 256, sink), 5, do_flush=False))
             probe[name] = sr.sr_probe_int32_ops(2000, sms * 8, 256) / (ms * 1e-3) / 1e9
         extras["int32_probe_gops"] = probe
-        # the recurrence is 8 logic : 2 add; logic issues on the int32 ALU only, adds can also
-        # issue on the FMA pipe, so the logic-only rate is the pipe's own ceiling
-        line["roofline"]["peak_probe_logic"] = probe["logic"]
-        line["roofline"]["frac_of_probe_logic"] = achieved / probe["logic"]
-        # the recurrence's own mix (8 logic : 2 add) measured register-only on this GPU: the
-        # adds also issue on the FMA pipe, so this ceiling is a little above the logic rate
-        line["roofline"]["peak_probe_mix"] = probe["mix8l2a"]
-        line["roofline"]["frac_of_probe_mix"] = achieved / probe["mix8l2a"]
-
         def gate_case(wl, reps=20):
             g, n, st = wl.seqs.shape
             p = n * (n - 1) // 2
@@ -525,9 +514,9 @@ def main():
         extras["e2e_padded_input"] = {"ms_per_step": statistics.median(ms),
                                       "gcups": cells / (statistics.median(ms) * 1e-3) / 1e9,
                                       "h2d_bytes_per_step": h_seqs.numel() * 4 + h_lens.numel() * 4 + h_rew.numel() * 4 + h_stop.numel()}
-        # the same pipeline on inputs without common prefixes (odd groups diverge from the
-        # first token): nothing is removed, so this line shows the dp kernel on whole matrices
-        w0 = W.token_gate(seed=3, n_groups=args.groups, shared_head=False)
+        # the recurrence: the same batch over 3000 symbols, whose pairs have hundreds of matches.  (8 logic : 2 add; logic
+        # issues on the int32 ALU only, adds can also issue on the FMA pipe, so the logic-only rate is the pipe's own ceiling)
+        w0 = W.token_gate(seed=3, n_groups=args.groups, vocab=3000)
         s0 = torch.from_numpy(w0.seqs).to(dev)
         l0 = torch.from_numpy(w0.lens).to(dev)
         ev0 = []
@@ -543,10 +532,11 @@ def main():
         dp0 = statistics.median(e5[2].elapsed_time(e5[3]) for e5 in ev0)
         all0 = statistics.median(e5[0].elapsed_time(e5[4]) for e5 in ev0)
         wc0 = W.word_columns(w0.lens, K, w0.seqs, band=True)
-        extras["C4_no_shared_head"] = {"groups": w0.n_groups, "us_gate": all0 * 1e3, "us_dp": dp0 * 1e3,
-                                       "gcups": W.dp_cells(w0.lens, K) / (all0 * 1e-3) / 1e9,
-                                       "word_columns": wc0, "dp_alu_gops": 10.0 * wc0 / (dp0 * 1e-3) / 1e9,
-                                       "dp_alu_frac": 10.0 * wc0 / (dp0 * 1e-3) / 1e9 / alu_peak}
+        extras["C4_vocab_3000"] = {"groups": w0.n_groups, "us_gate": all0 * 1e3, "us_dp": dp0 * 1e3,
+                                   "gcups": W.dp_cells(w0.lens, K) / (all0 * 1e-3) / 1e9,
+                                   "word_columns": wc0, "dp_alu_gops": 10.0 * wc0 / (dp0 * 1e-3) / 1e9,
+                                   "dp_alu_frac": 10.0 * wc0 / (dp0 * 1e-3) / 1e9 / alu_peak,
+                                   "dp_alu_frac_of_probe_logic": 10.0 * wc0 / (dp0 * 1e-3) / 1e9 / probe["logic"]}
         # small token-level batches (teams of up to a whole warp per pair)
         for small in (16, 64):
             ws_ = W.token_gate(seed=3, n_groups=small)
