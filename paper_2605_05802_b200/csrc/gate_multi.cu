@@ -52,6 +52,7 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "stream_words.cuh"
 
 namespace sr {
 namespace {
@@ -63,8 +64,6 @@ constexpr int kTimeBuckets = 96;    // buckets of estimated task duration
 constexpr int kNumBins = 2048;      // kTimeBuckets * kNumClasses of them used
 constexpr int kOrderThreads = 1024;
 constexpr int kAlonePairs = 1024;   // batches of up to this many pairs are ordered by one CTA
-constexpr uint32_t kLocNone = 0x7FFFu;    // bit 15 clear, far above any row: shifts to 0
-constexpr uint32_t kLocRow = 0x8000u;     // | index of the symbol's mask row
 constexpr uint32_t kLocChain = 0xC000u;   // | first position of the symbol's occurrence chain
 constexpr uint32_t kChainEnd = 0xFFFFu;
 constexpr int kDpWarpsPerCta = 4;
@@ -337,12 +336,6 @@ multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int
                  reinterpret_cast<uint2*>(names + (size_t)g * N * pitch));
 }
 
-// ------------------------------------------------------------------------ prep
-// Top bit of each half of x that is not zero.
-__device__ __forceinline__ uint32_t set_halves(uint32_t x) {
-    return (((x & 0x7FFF7FFFu) + 0x7FFF7FFFu) | x) & 0x80008000u;
-}
-
 // ------------------------------------------------------------------ recurrence
 __device__ __forceinline__ uint32_t shl_clamp(uint32_t v, uint32_t s) {
     uint32_t r;   // PTX shl clamps shift amounts above 31: the result is 0
@@ -395,8 +388,8 @@ constexpr int kSpan = 128;                               // columns a warp looks
 constexpr int kSpans = SR_MAX_K / kSpan + 1;             // and one that begins where the longest text ends
 constexpr int kMatchWarps = 8;
 
-// The columns of a pair's stream with matches off the main diagonal, with the column's stream entry (upper half), in
-// `entries`, and in `differ` a bit for every column from `strip` on that differs from the pattern: column
+// The columns of a pair's stream with matches off the main diagonal, with the column's stream entry (upper half: a mask
+// row, or a position from `strip` on, so that no place before `strip` is ever asked for), in `entries`, and in `differ` a bit for every column from `strip` on that differs from the pattern: column
 // strip + 128 s + 4 l + k in bit l of word k of differ[s].  Returns the number of those columns, or more than
 // there are lanes for.
 // (kShared: the stream and, below, the rows are in shared memory.)
@@ -421,15 +414,13 @@ __device__ __forceinline__ int find_matches(const uint2* stream, const uint2* te
             continue;
         }
         const uint32_t at0 = (uint32_t)(4 * q * 0x10001 + 0x10000), at1 = at0 + 0x20002u;   // the places on the main diagonal
-        uint32_t off0 = set_halves(v.x ^ at0), off1 = set_halves(v.y ^ at1);
-        uint32_t d0 = off0, d1 = off1;
+        uint32_t d0 = set_halves(v.x ^ at0), d1 = set_halves(v.y ^ at1);
+        uint32_t off0 = matches_beside(v.x, at0, strip), off1 = matches_beside(v.y, at1, strip);
         if ((v.x | v.y) & (kLocRow * 0x10001u)) {      // a symbol that occurs more than once: the names tell
             const uint2 x = kShared ? text[q] : __ldg(text + q), o = kShared ? pat[q] : __ldg(pat + q);
             d0 = set_halves(x.x ^ o.x);
             d1 = set_halves(x.y ^ o.y);
         }
-        off0 &= set_halves(v.x ^ (kLocNone * 0x10001u));
-        off1 &= set_halves(v.y ^ (kLocNone * 0x10001u));
         if (left < 4) {
             off0 = left > 1 ? off0 : (left == 1 ? off0 & 0xFFFFu : 0u);
             off1 = left == 3 ? off1 & 0xFFFFu : 0u;
@@ -516,7 +507,7 @@ __device__ __forceinline__ int distance_by_matches(uint32_t* entries, int count,
     __syncwarp();
     node = lane < total ? entries[lane] : (uint32_t)strip * 0x10001u;
     const int c = (int)(node & 0xFFFFu), p = (int)(node >> 16);
-    // places that differ before x
+    // places that differ before x, strip <= x <= lo: columns begin at strip, and so do the positions of all nodes
     int before = 0;
     if (lane < kSpans && strip + kSpan * lane < n) {
         const uint4 d = differ[lane];

@@ -43,3 +43,31 @@ def test_gate_with_few_matches(G, N, K, vocab):
     seqs, lens = _batch(rng, G, N, K, vocab)
     want = oracle.gate(seqs, lens, K, 0.4, 0, threads=8)
     assert_gate_matches(gate_gpu(seqs, lens, K, 0.4, 0), want, f"G={G} N={N} K={K} vocab={vocab}")
+
+
+def _recurring_heads(rng, G, N, K):
+    """Groups that share a head of 200 symbols and more; the tails of every other rollout take up to thirty symbols of the
+    head again, which so occur once in the patterns of the others, before the place where the pair begins to differ."""
+    stride = (K + 3) // 4 * 4
+    lens = rng.integers(K // 2, K + 1, size=(G, N)).astype(np.int32)
+    lens[:, 0] = K
+    seqs = np.zeros((G, N, stride), dtype=np.int32)
+    for g in range(G):
+        head = min(int(rng.integers(200, 901)), K - 40)
+        symbols = rng.choice(1 << 20, size=stride * (N + 1), replace=False)
+        for i in range(N):
+            row = np.concatenate([symbols[:head], symbols[stride * (i + 1):stride * (i + 2) - head]])
+            if i % 2:
+                again = min(int(rng.integers(1, 31)), stride - head)
+                row[head + rng.choice(stride - head, size=again, replace=False)] = symbols[rng.choice(head, size=again, replace=False)]
+            seqs[g, i, :lens[g, i]] = row[:lens[g, i]]
+    return seqs, lens
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("G,N,K", [(41, 16, 1024), (41, 16, 1001), (6, 8, 1024), (5, 5, 997), (12, 8, 400)])
+def test_symbols_of_the_common_prefix_that_come_again(G, N, K):
+    rng = np.random.default_rng(G * K)
+    seqs, lens = _recurring_heads(rng, G, N, K)
+    want = oracle.gate(seqs, lens, K, 0.4, 0, threads=8)
+    assert_gate_matches(gate_gpu(seqs, lens, K, 0.4, 0), want, f"G={G} N={N} K={K}")
