@@ -90,6 +90,8 @@ struct Ctl {               // control block in the workspace
     unsigned long long work;                   // lane-time of all pairs, about
     int32_t open;                              // and how many they are
     int32_t few;                               // pairs for multi_matches_kernel, listed where the order goes later
+    unsigned long long maybe_work;             // pairs that it may take too, listed there from the end on, and their lane-time
+    int32_t maybe, must;                       // and pairs that it cannot
     int32_t hist[kNumBins];
     int32_t fill[kNumBins];                    // what comes before here starts at zero
     int32_t start[kNumBins];
@@ -384,6 +386,16 @@ constexpr int kMostMatches = 32;                         // a lane each
 // Whether a pattern of m positions has so few repeated symbols that its pairs may have few matches: 1024 uniform
 // tokens have three or four (of a vocabulary of 32 000 sixteen), as long a text more than a hundred, one of 48 words four.
 __device__ __forceinline__ bool few_repeats(int repeats, int m) { return 32 * repeats <= m + 64; }
+// And whether a warp finds them for less than the recurrence's `work` (see work_of_pair) on `length` places of which
+// `differ` differ: there is a match or more to every column between the bounds, and where the two agree, one to every place of
+// a repeated symbol.  The weights are the warp's, in the units of `work`, drawn from nine
+// sets on 13 shapes of K = 48 to 1024 and 16 kinds of batch (all pairs listed: 8000 groups of 8 ragged texts of 48 362 us,
+// 238 with this, 243 without any search; 3000 of 100 172, 122 and 124; 400 of 16 with 256 of 3000 symbols 144, 111 and 111).
+__device__ __forceinline__ bool worth_listing(int columns, int repeats, int differ, int length, int work) {
+    return (2000 + 1000 * columns + 700 * repeats) * length + 1300 * repeats * (length - differ) <= work * length;
+}
+// Columns between the bounds up to which a pair is taken for its matches where it is not worth it by itself (see below).
+constexpr int kFewColumns = 12;
 constexpr int kSpan = 128;                               // columns a warp looks through a trip
 constexpr int kSpans = SR_MAX_K / kSpan + 1;             // and one that begins where the longest text ends
 constexpr int kMatchWarps = 8;
@@ -1190,7 +1202,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     if (tid >= 32) return;                             // descriptors: the texts' threads are in the first warp
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
-    int work = 0, few = -1;
+    int work = 0, few = -1, maybe = -1;
     if (tid < ntxt) {
         const int j = s_txt[tid], n = s_len[tid];
         const int strip = removed(tid);
@@ -1204,34 +1216,50 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         }
         descs[idx] = d;
         if (kDecide || lower == upper) dist_out[idx] = lower;
-        if (!kDecide && lower < upper && upper - lower <= kMostMatches && few_repeats(s_repeats[0], m)) {
-            few = (int)idx;
-        } else if (lower < upper) {
+        if (lower < upper) {
             const PairSize z = size_of_desc(d);
             work = work_of_pair(z.m, z.n, z.lb, z.ub);
+            if (!kDecide && upper - lower <= kMostMatches && few_repeats(s_repeats[0], m)) {
+                if (worth_listing(upper - lower, s_repeats[0], (int)(s_count[tid] & 0xFFFFu), min(m, n) - strip, work)) few = (int)idx;
+                else if (upper - lower <= kFewColumns) maybe = (int)idx;
+            }
         }
     }
     if (kDecide || W.alone) return;                   // counted later: what the bounds leave; by the CTA that orders the batch
-    const unsigned listed = __ballot_sync(0xFFFFFFFFu, few >= 0);
+    int32_t* list = reinterpret_cast<int32_t*>(ws + W.off_order);
+    const unsigned listed = __ballot_sync(0xFFFFFFFFu, few >= 0), maybes = __ballot_sync(0xFFFFFFFFu, maybe >= 0);
+    const unsigned musts = __ballot_sync(0xFFFFFFFFu, work > 0 && few < 0 && maybe < 0);
     if (listed) {
         int at = 0;
         if (tid == 0) at = atomicAdd(&ctl->few, __popc(listed));
         at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(listed & ((1u << tid) - 1u));
-        if (few >= 0) reinterpret_cast<int32_t*>(ws + W.off_order)[at] = few;
+        if (few >= 0) list[at] = few;
     }
-    const int open = __popc(__ballot_sync(0xFFFFFFFFu, work > 0));
-    work = __reduce_add_sync(0xFFFFFFFFu, work);
-    if (tid == 0 && open) {
-        atomicAdd(&ctl->work, (unsigned long long)work);
-        atomicAdd(&ctl->open, open);
+    if (maybes) {
+        int at = 0;
+        if (tid == 0) at = atomicAdd(&ctl->maybe, __popc(maybes));
+        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(maybes & ((1u << tid) - 1u));
+        if (maybe >= 0) list[a.n_groups * P - 1 - at] = maybe;
+        const int sum = __reduce_add_sync(0xFFFFFFFFu, maybe >= 0 ? work : 0);
+        if (tid == 0) atomicAdd(&ctl->maybe_work, (unsigned long long)sum);
+    }
+    if (musts) {
+        work = __reduce_add_sync(0xFFFFFFFFu, few < 0 && maybe < 0 ? work : 0);
+        if (tid == 0) {
+            atomicAdd(&ctl->work, (unsigned long long)work);
+            atomicAdd(&ctl->open, __popc(musts));
+            atomicAdd(&ctl->must, __popc(musts));
+        }
     }
 }
 
 // --------------------------------------------------------------- matches kernel
 // A warp goes through listed pairs as many places apart as there are warps.  (Not in decide mode: most of these
-// pairs' groups are dismissed by their bounds.)
+// pairs' groups are dismissed by their bounds.)  Pairs that are not worth it by themselves are looked at if no pair has to go
+// to the recurrence: the batch is then done here as a rule, and the latency of what comes after it is more than they cost
+// (1024 groups of uniform tokens: 122 us, 142 without these).
 __global__ void __launch_bounds__(32 * kMatchWarps)
-multi_matches_kernel(unsigned char* ws, MultiWs W, int N, int32_t* dist_out) {
+multi_matches_kernel(unsigned char* ws, MultiWs W, int N, int n_pairs, int32_t* dist_out) {
     grid_begin();
     __shared__ uint4 s_differ[kMatchWarps][kSpans];
     __shared__ uint32_t s_entries[kMatchWarps][kMostMatches];
@@ -1241,9 +1269,13 @@ multi_matches_kernel(unsigned char* ws, MultiWs W, int N, int32_t* dist_out) {
     const int32_t* list = reinterpret_cast<const int32_t*>(ws + W.off_order);
     unsigned long long work = 0ull;
     int still_open = 0;
-    const int few = ctl->few;
-    for (int e = blockIdx.x * kMatchWarps + warp; e < few; e += gridDim.x * kMatchWarps) {
-        const int idx = list[e];
+    const int few = ctl->few, all = few + (ctl->must == 0 ? ctl->maybe : 0);
+    if (blockIdx.x == 0 && threadIdx.x == 0 && ctl->must != 0 && ctl->maybe != 0) {
+        atomicAdd(&ctl->work, ctl->maybe_work);
+        atomicAdd(&ctl->open, ctl->maybe);
+    }
+    for (int e = blockIdx.x * kMatchWarps + warp; e < all; e += gridDim.x * kMatchWarps) {
+        const int idx = list[e < few ? e : n_pairs - 1 - (e - few)];
         const PairDesc d = descs[idx];
         const int upper = (int)(d.lower >> 16);
         int dist = -1;
@@ -1984,7 +2016,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     int32_t* order = reinterpret_cast<int32_t*>(ws + W.off_order);
     if (!alone && !decide)
-        SR_LAUNCH("multi_matches_kernel", multi_matches_kernel, min((n_pairs + kMatchWarps - 1) / kMatchWarps, 16 * sms), 32 * kMatchWarps, 0, s, ws, W, a.N, dist);
+        SR_LAUNCH("multi_matches_kernel", multi_matches_kernel, min((n_pairs + kMatchWarps - 1) / kMatchWarps, 16 * sms), 32 * kMatchWarps, 0, s, ws, W, a.N, n_pairs, dist);
     if (decide) {
         SR_LAUNCH("multi_bound_kernel", multi_bound_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, descs, ctl, flag, exact, gpb, alone,
                   !a.pair_dist && !a.pair_sum && !a.mean && !exact);

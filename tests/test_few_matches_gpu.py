@@ -71,3 +71,13 @@ def test_symbols_of_the_common_prefix_that_come_again(G, N, K):
     seqs, lens = _recurring_heads(rng, G, N, K)
     want = oracle.gate(seqs, lens, K, 0.4, 0, threads=8)
     assert_gate_matches(gate_gpu(seqs, lens, K, 0.4, 0), want, f"G={G} N={N} K={K}")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("G,N,K,vocab", [(2200, 8, 48, 3000), (1500, 8, 100, 400), (1500, 8, 100, 100000), (5000, 2, 256, 3000), (60, 16, 256, 3000)])
+def test_short_prefixes_with_few_matches(G, N, K, vocab):
+    """Some of a batch's pairs listed and some left to the recurrence: about where one costs as much as the other."""
+    rng = np.random.default_rng(vocab + K)
+    seqs, lens = _batch(rng, G, N, K, vocab)
+    want = oracle.gate(seqs, lens, K, 0.4, 0, threads=8)
+    assert_gate_matches(gate_gpu(seqs, lens, K, 0.4, 0), want, f"G={G} N={N} K={K} vocab={vocab}")
