@@ -58,6 +58,7 @@ namespace sr {
 namespace {
 
 constexpr int kMostPrepThreads = 256;      // a thread for every four positions of a pattern
+constexpr int kTextThreads = 16 * SR_MAX_N;  // a warp for every text of a pattern
 static_assert(4 * kMostPrepThreads >= SR_MAX_K, "");
 constexpr int kNumClasses = 21;     // team shapes (T lanes x R blocks), see class_of
 constexpr int kTimeBuckets = 96;    // buckets of estimated task duration
@@ -831,6 +832,10 @@ __device__ __forceinline__ bool arrive_last(int parts, int32_t* arrived) {
 // cost next to nothing here.  Where they meet the pair is done.
 // kThreads: the CTA's threads where they are the most there can be (known at compile time 82 us of the token-level
 // batch of 1024 groups, at run time 84.5), 0 for fewer.
+// kTextThreads: a warp for every text where there are more than eight and a pair takes a warp (kPairs, K > 253), while every CTA
+// has an SM: the ninth text and those after it do not wait for the first eight (6 groups of 20 texts of 850 that differ in 2 % of
+// their places: 120 -> 69 us, 107 sorted; with more CTAs than SMs three of 256 threads to an SM are as good or better, 18 groups of
+// 18 diverging ones 112 and 123).
 // kPairs: the whole gate after the names.  Streams and mask rows stay in shared memory, the distances are computed right
 // there, and the last CTA of a group evaluates it.
 // kOwnNames: the whole gate.  A group's CTAs are a cluster, and each of them names all of the group's symbols for itself.
@@ -839,7 +844,7 @@ __device__ __forceinline__ bool arrive_last(int parts, int32_t* arrived) {
 // kTwoWarps: patterns of more than 512 positions and no more than two texts, a CTA to an SM: a pair has two warps (40
 // groups of 4 texts of 1024: 48 -> 37 us; with four texts the integer pipe is busy already, 16 groups of 8: 46 -> 48).
 template <bool kDecide, int kThreads, bool kPairs, bool kOwnNames, bool kTwoWarps = false>
-__global__ void __launch_bounds__(kMostPrepThreads, kPairs ? 3 : 6)
+__global__ void __launch_bounds__(kThreads > kMostPrepThreads ? kThreads : kMostPrepThreads, kThreads > kMostPrepThreads ? 1 : kPairs ? 3 : 6)
 multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base, uint8_t* exact, uint32_t inv_row, int table_log,
                   uint32_t two) {
     constexpr bool kCluster = kOwnNames || (kDecide && kPairs);
@@ -1110,8 +1115,9 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     // quads), and of 32 where the stream refers to mask rows (whose words start there).
     auto removed = [&](int t) { return s_cp[t] < 0 ? -1 : (s_cp[t] & (s_flag[t] ? ~31 : ~3)); };
     if constexpr (kPairs) {
-        __shared__ uint4 s_differ[kMostPrepThreads / 32][kSpans];
-        __shared__ uint32_t s_entries[kMostPrepThreads / 32][kMostMatches];
+        constexpr int kWarps = (kThreads > kMostPrepThreads ? kThreads : kMostPrepThreads) / 32;
+        __shared__ uint4 s_differ[kWarps][kSpans];
+        __shared__ uint32_t s_entries[kWarps][kMostMatches];
         __shared__ int s_dist[kMaxTexts];              // the distance, or -1: to be computed
         auto settle = [&](int t, int d) {
             const int pair = pair_index(min(i, s_txt[t]), max(i, s_txt[t]), N);
@@ -1885,6 +1891,9 @@ multi_finish_kernel(GateArgs a, int32_t* dist, const uint8_t* flag, uint8_t* exa
     if (capped && exact) exact[g] = 0;                       // some distances are lower bounds
 }
 
+// The longest prefixes for which a team has no more than eight lanes there, and two pairs a warp.
+constexpr int kMostEightLanes = 253;
+
 // Which batches take every pair from both ends instead of sorting the pairs into warp tasks: those whose
 // work leaves the SMs idle anyway.  Both sides at the line for texts, us: 600 groups of 8 at K = 48 49 and 46, 250 at 256 45 and
 // 58, at 512 83 and 92; 150 at 1024 about 140 both; four groups of 8 at 1024 41 and 84.  With more texts to a pattern than a CTA
@@ -1925,6 +1934,7 @@ int allow_smem() {
     for (auto kernel : {multi_prep_kernel<true, 0, false, false>, multi_prep_kernel<true, kMostPrepThreads, false, false>, multi_prep_kernel<false, 0, false, false>, multi_prep_kernel<false, kMostPrepThreads, false, false>})
         SR_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, prep));
     for (auto kernel : {multi_prep_kernel<false, 0, true, false>, multi_prep_kernel<false, kMostPrepThreads, true, false>,
+                        multi_prep_kernel<false, kTextThreads, true, false>,
                         multi_prep_kernel<false, 0, true, true>, multi_prep_kernel<false, kMostPrepThreads, true, true>,
                         multi_prep_kernel<false, kMostPrepThreads, true, false, true>, multi_prep_kernel<false, kMostPrepThreads, true, true, true>,
                         multi_prep_kernel<true, 0, true, false>, multi_prep_kernel<true, kMostPrepThreads, true, false>,
@@ -1973,7 +1983,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     // instead of 98, 4666 of 4 at K = 64 112 instead of 67, 1000 of 8 at K = 100 75 instead of 60.)
     const int names_threads = min((a.N * row_quads + 31) & ~31, names_most), texts = a.N >> 1;
     const int fewest = (max((a.K + 127) >> 7, texts) + texts - 1) / texts * texts;
-    const int prep_threads = (long long)a.n_groups * W.patterns <= sms ? kMostPrepThreads : min(32 * fewest, kMostPrepThreads);
+    const bool an_sm_each = (long long)a.n_groups * W.patterns <= sms;
+    const bool many_texts = in_pairs && !decide && an_sm_each && 32 * texts > kMostPrepThreads && a.K > kMostEightLanes;
+    const int prep_threads = many_texts ? kTextThreads : an_sm_each ? kMostPrepThreads : min(32 * fewest, kMostPrepThreads);
     W.text_warps = max(1, (prep_threads >> 5) / texts);
     W.text_stride = (prep_threads >> 5) / W.text_warps;
     W.inv_text_warps = (uint32_t)(((1ull << 32) + W.text_warps - 1) / W.text_warps);
@@ -2018,8 +2030,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
                                   : (most ? multi_prep_kernel<false, kMostPrepThreads, true, false> : multi_prep_kernel<false, 0, true, false>);
         const auto alone_pairs = decide ? (most ? multi_prep_kernel<true, kMostPrepThreads, true, true> : multi_prep_kernel<true, 0, true, true>)
                                         : (most ? multi_prep_kernel<false, kMostPrepThreads, true, true> : multi_prep_kernel<false, 0, true, true>);
-        const bool in_twos = in_pairs && most && !decide && a.K > 512 && texts <= 2 && a.n_groups * W.patterns <= sms;
+        const bool in_twos = in_pairs && most && !decide && a.K > 512 && texts <= 2 && an_sm_each;
         const auto prep = in_twos ? (own_names ? multi_prep_kernel<false, kMostPrepThreads, true, true, true> : multi_prep_kernel<false, kMostPrepThreads, true, false, true>)
+                        : many_texts ? multi_prep_kernel<false, kTextThreads, true, false>
                         : own_names ? alone_pairs : in_pairs ? pairs : in_memory;
         const int rc = launch_as(true, cluster, "multi_prep_kernel", prep, (g1 - g0) * W.patterns, prep_threads, prep_smem, s,
                                  a, ws, W, dist, g0, exact, inv_row, table_log, 2u);

@@ -44,3 +44,13 @@ def test_negative_lengths_are_reported(N, K):
     got = gate_gpu(seqs, lens, K, 0.5, 0, status=status)
     assert status == [1]
     assert_gate_matches(got, oracle.gate(seqs, np.maximum(lens, 0), K, 0.5, 0, threads=8), f"N={N} K={K}")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("G,N,K,vocab", [(2, 17, 254, 80), (1, 18, 254, 80), (2, 20, 513, 150), (1, 32, 1024, 340), (4, 32, 300, 100), (5, 32, 300, 100), (3, 18, 253, 80)])
+def test_more_texts_than_warps(G, N, K, vocab):
+    """Patterns with up to sixteen texts: a warp for each while every CTA has an SM, eight warps in turns beyond that."""
+    rng = np.random.default_rng(G * K + N)
+    seqs, lens = _batch(rng, G, N, K, vocab)
+    want = oracle.gate(seqs, lens, K, 0.5, 0, threads=8)
+    assert_gate_matches(gate_gpu(seqs, lens, K, 0.5, 0), want, f"G={G} N={N} K={K}")
