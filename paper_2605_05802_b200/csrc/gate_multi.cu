@@ -1894,13 +1894,29 @@ multi_finish_kernel(GateArgs a, int32_t* dist, const uint8_t* flag, uint8_t* exa
 // The longest prefixes for which a team has no more than eight lanes there, and two pairs a warp.
 constexpr int kMostEightLanes = 253;
 
-// Which batches take every pair from both ends instead of sorting the pairs into warp tasks: those whose
-// work leaves the SMs idle anyway.  Both sides at the line for texts, us: 600 groups of 8 at K = 48 49 and 46, 250 at 256 45 and
-// 58, at 512 83 and 92; 150 at 1024 about 140 both; four groups of 8 at 1024 41 and 84.  With more texts to a pattern than a CTA
-// has warps the line lies lower (16 groups of 24 at 1024: 174 and 149).  The decide mode does so for
-// groups of up to eight, whose CTAs are a cluster that sums up the bounds first (40 groups of 8 texts of 512: 29 -> 15 us ragged, 72 -> 28 at
-// full length; 250 of 256: 31 and 62 without this, about the same with it).
-bool runs_in_pairs(int n_pairs, int N, int K, bool decide) { return decide ? N <= kMostOwnPatterns && n_pairs <= 7000 && (long long)n_pairs * (K + 384) <= 6400000LL : (long long)n_pairs * (K + 384) <= (N <= 17 ? 6400000LL : 4200000LL); }
+// Which batches take every pair from both ends instead of sorting the pairs into warp tasks: those whose work leaves the SMs
+// idle anyway.  Whole matrices are run there and bands in the other place, so the line lies where the batches that have the
+// narrowest bands stop to gain (pairs with 2 % of their places substituted, or 5 % edited, of texts, uniform tokens, 3000 and 100
+// symbols, and diverging texts, 2676 shapes of 2 to 32 rollouts and K = 33 to 1024; diverging batches would gain up to twice as
+// many groups).  It falls with the lanes that a pair takes (up to 8, 16, 16 of two blocks), and where a CTA has only one text or
+// two for its warps.  In the last fifth before the line the worst kind of
+// batch takes 0.84 of the time it takes sorted, 1.05 at most, all kinds 0.72.
+// With more than eight texts to a pattern a pair of 16 lanes waits for others of its CTA: then while there are SMs for
+// all CTAs, or half of them (K <= 512).
+// The decide mode does so for groups of up to eight, whose CTAs are a cluster that sums up the bounds first; clusters
+// of three fit an SM's share worst, and the sorted way has fewer pairs to run.
+bool runs_in_pairs(int n_groups, int N, int K, int sms, bool decide) {
+    const long long n_pairs = (long long)n_groups * pairs_of(N), ctas = (long long)n_groups * (N & 1 ? N : N - 1);
+    const int texts = N >> 1, lanes = K <= (texts == 1 ? 128 : kMostEightLanes) ? 0 : K <= 512 ? 1 : 2;
+    if (decide) {
+        constexpr int kMost[kMostOwnPatterns + 1][3] = {{}, {}, {4500, 1000, 1000}, {1000, 1000, 500}, {2400, 2400, 1000}, {2400, 2400, 1000},
+                                                        {3500, 1900, 1700}, {3500, 1900, 1700}, {3500, 3200, 2100}};
+        return N <= kMostOwnPatterns && n_pairs <= 7000 && n_pairs * (K + 384) <= 1000LL * kMost[N][lanes];
+    }
+    if (texts > 8 && lanes > 0) return ctas <= (lanes == 1 ? 2 : 1) * sms;
+    constexpr int kMost[5][3] = {{4500, 1000, 1000}, {4500, 3500, 2500}, {6400, 3500, 2300}, {6400, 4000, 3000}, {4200, 0, 0}};
+    return n_pairs * (K + 384) <= 1000LL * kMost[texts <= 3 ? texts - 1 : texts <= 8 ? 3 : 4][lanes];
+}
 
 // And which of them name a group's symbols in each of its CTAs, a cluster of them, and do without the launch and the latency
 // of the names kernel: while the SMs have room for the work that is done several times (all 4 groups of 8 at K = 48
@@ -1971,7 +1987,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     int32_t* dist = a.pair_dist ? a.pair_dist : reinterpret_cast<int32_t*>(ws + W.off_dist);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
 
-    const bool in_pairs = !feed && runs_in_pairs(n_pairs, a.N, a.K, decide);
+    const bool in_pairs = !feed && runs_in_pairs(a.n_groups, a.N, a.K, sms, decide);
     const bool clusters = in_pairs && decide;         // whose CTAs sum up their bounds together
     const bool own_names = in_pairs && names_for_itself(a.n_groups, W.patterns, a.N * W.pitch, sms);
     // names: at least two slots to a symbol while symbols and table fit; above 4096 symbols one, and four CTAs to an SM instead
