@@ -17,8 +17,8 @@
 //            occurrences gets a row of match words instead, and the stream names the row.
 //            Bounds of the pair's distance fall out of the look-ups: the columns without any
 //            match in the pattern from below, the differing positions from above.
-//   matches  pairs with few matches get their distance from these alone, a warp each.
-//   bin      team shape of every pair (what the band of its bounds costs at least, see
+//   bin      pairs with few matches get their distance from these alone, a warp each; the others
+//            a team shape (what the band of their bounds costs at least, see
 //            shape_of_pair) and bin counts.
 //   order    counting sort of the pairs by bin: longest warp tasks first, one team
 //            shape and similar durations per bin; warp-task table.  (One launch does both for
@@ -69,6 +69,7 @@ constexpr uint32_t kLocChain = 0xC000u;   // | first position of the symbol's oc
 constexpr uint32_t kChainEnd = 0xFFFFu;
 constexpr int kDpWarpsPerCta = 4;
 constexpr uint32_t kBinMask = 0x7FFu;
+constexpr uint32_t kListed = 0x800u;          // see multi_bin_kernel
 constexpr uint32_t kHasChains = 0x40000000u;
 constexpr int32_t kCappedFlag = 0x40000000;   // decide mode: the pair's distance exceeds its cap
 constexpr int kStripShift = 12, kRowsShift = 22;
@@ -78,7 +79,7 @@ static_assert(kNumBins <= (int)kBinMask + 1 && kTimeBuckets * kNumClasses <= kNu
 struct PairDesc {          // 16 bytes
     uint32_t mn;           // m | n << 16
     uint32_t pat_row;      // g * patterns + pattern rollout
-    uint32_t bin;          // bits 0..10 bin index; bits 12..21 stripped common prefix (symbols,
+    uint32_t bin;          // bits 0..10 bin index; bit 11 listed for its few matches; bits 12..21 stripped common prefix (symbols,
                            // a multiple of 4); bits 22..29 mask rows of the pattern; bit 30 = the
                            // pattern has chains; bit 31 = pair needs the dp kernel
     uint32_t lower;        // bits 0..15 a lower bound of the pair's distance (decide mode),
@@ -88,11 +89,12 @@ struct PairDesc {          // 16 bytes
 };
 
 struct Ctl {               // control block in the workspace
-    unsigned long long work;                   // lane-time of all pairs, about
-    int32_t open;                              // and how many they are
-    int32_t few;                               // pairs for multi_matches_kernel, listed where the order goes later
-    unsigned long long maybe_work;             // pairs that it may take too, listed there from the end on, and their lane-time
-    int32_t maybe, must;                       // and pairs that it cannot
+    unsigned long long work;                   // lane-time of the pairs for the recurrence, about
+    unsigned long long maybe_work, few_work;   // of those that are counted next
+    int32_t open;                              // how many they are
+    int32_t maybe;                             // pairs for it or for their few matches, listed from the end of where the order goes
+    int32_t few;                               // pairs for their few matches, listed from there on
+    int32_t failed;                            // and how many of the listed ones had too many
     int32_t hist[kNumBins];
     int32_t fill[kNumBins];                    // what comes before here starts at zero
     int32_t start[kNumBins];
@@ -1225,98 +1227,33 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         if (lower < upper) {
             const PairSize z = size_of_desc(d);
             work = work_of_pair(z.m, z.n, z.lb, z.ub);
-            if (!kDecide && upper - lower <= kMostMatches && few_repeats(s_repeats[0], m)) {
-                if (worth_listing(upper - lower, s_repeats[0], (int)(s_count[tid] & 0xFFFFu), min(m, n) - strip, work)) few = (int)idx;
-                else if (upper - lower <= kFewColumns) maybe = (int)idx;
+            if (!kDecide && !W.alone && upper - lower <= kMostMatches && few_repeats(s_repeats[0], m)) {
+                if (worth_listing(upper - lower, s_repeats[0], (int)(s_count[tid] & 0xFFFFu), min(m, n) - strip, work)) {
+                    few = (int)idx;
+                    descs[idx].bin = d.bin | kListed;
+                } else if (upper - lower <= kFewColumns) {
+                    maybe = (int)idx;
+                }
             }
         }
     }
     if (kDecide || W.alone) return;                   // counted later: what the bounds leave; by the CTA that orders the batch
     int32_t* list = reinterpret_cast<int32_t*>(ws + W.off_order);
-    const unsigned listed = __ballot_sync(0xFFFFFFFFu, few >= 0), maybes = __ballot_sync(0xFFFFFFFFu, maybe >= 0);
-    const unsigned musts = __ballot_sync(0xFFFFFFFFu, work > 0 && few < 0 && maybe < 0);
-    if (listed) {
+    auto note = [&](bool here, int32_t* count, unsigned long long* sum) {     // the place of this thread's pair among those noted
+        const unsigned all = __ballot_sync(0xFFFFFFFFu, here);
+        if (all == 0u) return 0;
+        const int lane_time = __reduce_add_sync(0xFFFFFFFFu, here ? work : 0);
         int at = 0;
-        if (tid == 0) at = atomicAdd(&ctl->few, __popc(listed));
-        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(listed & ((1u << tid) - 1u));
-        if (few >= 0) list[at] = few;
-    }
-    if (maybes) {
-        int at = 0;
-        if (tid == 0) at = atomicAdd(&ctl->maybe, __popc(maybes));
-        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(maybes & ((1u << tid) - 1u));
-        if (maybe >= 0) list[a.n_groups * P - 1 - at] = maybe;
-        const int sum = __reduce_add_sync(0xFFFFFFFFu, maybe >= 0 ? work : 0);
-        if (tid == 0) atomicAdd(&ctl->maybe_work, (unsigned long long)sum);
-    }
-    if (musts) {
-        work = __reduce_add_sync(0xFFFFFFFFu, few < 0 && maybe < 0 ? work : 0);
         if (tid == 0) {
-            atomicAdd(&ctl->work, (unsigned long long)work);
-            atomicAdd(&ctl->open, __popc(musts));
-            atomicAdd(&ctl->must, __popc(musts));
+            at = atomicAdd(count, __popc(all));
+            atomicAdd(sum, (unsigned long long)lane_time);
         }
-    }
-}
-
-// --------------------------------------------------------------- matches kernel
-// A warp goes through listed pairs as many places apart as there are warps.  (Not in decide mode: most of these
-// pairs' groups are dismissed by their bounds.)  Pairs that are not worth it by themselves are looked at if no pair has to go
-// to the recurrence: the batch is then done here as a rule, and the latency of what comes after it is more than they cost
-// (1024 groups of uniform tokens: 122 us, 142 without these).
-__global__ void __launch_bounds__(32 * kMatchWarps)
-multi_matches_kernel(unsigned char* ws, MultiWs W, int N, int n_pairs, int32_t* dist_out) {
-    grid_begin();
-    __shared__ uint4 s_differ[kMatchWarps][kSpans];
-    __shared__ uint32_t s_entries[kMatchWarps][kMostMatches];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, P = pairs_of(N);
-    PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
-    Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
-    const int32_t* list = reinterpret_cast<const int32_t*>(ws + W.off_order);
-    unsigned long long work = 0ull;
-    int still_open = 0;
-    const int few = ctl->few, all = few + (ctl->must == 0 ? ctl->maybe : 0);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && ctl->must != 0 && ctl->maybe != 0) {
-        atomicAdd(&ctl->work, ctl->maybe_work);
-        atomicAdd(&ctl->open, ctl->maybe);
-    }
-    for (int e = blockIdx.x * kMatchWarps + warp; e < all; e += gridDim.x * kMatchWarps) {
-        const int idx = list[e < few ? e : n_pairs - 1 - (e - few)];
-        const PairDesc d = descs[idx];
-        const int upper = (int)(d.lower >> 16);
-        int dist = -1;
-        const int m = (int)(d.mn & 0xFFFFu), n = (int)(d.mn >> 16), strip = (int)((d.bin >> kStripShift) & 0x3FFu);
-        int g = W.patterns > 1 ? (int)__umulhi(d.pat_row, W.inv_patterns) : (int)d.pat_row;
-        if (g * W.patterns > (int)d.pat_row) --g;
-        const int i = (int)d.pat_row - g * W.patterns;
-        const int pr = kPairs.v[N][idx - g * P], j = (pr & 0xFF) + (pr >> 8) - i;
-        const uint16_t* names = reinterpret_cast<const uint16_t*>(ws + W.off_names) + (size_t)g * N * W.pitch;
-        __syncwarp();                              // the pair before has been read
-        const int count = find_matches<false>(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(ws + W.off_loc) + (size_t)idx * W.pitch),
-                                       reinterpret_cast<const uint2*>(names + j * W.pitch), reinterpret_cast<const uint2*>(names + i * W.pitch),
-                                       m, n, strip, s_differ[warp], s_entries[warp]);
-        if (count == 0)
-            dist = upper;
-        else if (count <= kMostMatches)
-            dist = distance_by_matches<false>(s_entries[warp], count, s_differ[warp],
-                                       reinterpret_cast<const uint32_t*>(ws + W.off_rows) + (size_t)d.pat_row * W.rows_pitch,
-                                       W.row_words, m, n, strip, upper);
-        if (dist >= 0) {
-            if (lane == 0) {
-                descs[idx].bin = 0u;
-                descs[idx].lower = (uint32_t)dist * 0x10001u;
-                dist_out[idx] = dist;
-            }
-        } else {
-            const PairSize z = size_of_desc(d);
-            work += (unsigned long long)work_of_pair(z.m, z.n, z.lb, z.ub);
-            ++still_open;
-        }
-    }
-    if (still_open && lane == 0) {
-        atomicAdd(&ctl->work, work);
-        atomicAdd(&ctl->open, still_open);
-    }
+        return __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(all & ((1u << tid) - 1u));
+    };
+    const int at_few = note(few >= 0, &ctl->few, &ctl->few_work), at_maybe = note(maybe >= 0, &ctl->maybe, &ctl->maybe_work);
+    if (few >= 0) list[at_few] = few;
+    if (maybe >= 0) list[a.n_groups * P - 1 - at_maybe] = maybe;
+    note(work > 0 && few < 0 && maybe < 0, &ctl->open, &ctl->work);
 }
 
 // ----------------------------------------------------------------------- order
@@ -1355,28 +1292,84 @@ __device__ __forceinline__ ShapeGoal shape_goal(unsigned long long work, int ope
     return ShapeGoal{1.25f * (float)work / lanes, lanes / (float)max(open, 1)};
 }
 
-// Every pair's shape and bin, and the bin counts.
-__global__ void __launch_bounds__(kOrderThreads)
-multi_bin_kernel(PairDesc* descs, Ctl* ctl, int n_pairs, int warps) {
+// The first `bin_blocks` CTAs: every pair's shape and bin, and the bin counts.  The warps of the others go through the listed
+// pairs, as many places apart as there are of them, and bin those with too many matches themselves.  (In one launch:
+// a text, for which little or nothing is listed, does not wait for another one: 150 groups of 16 texts of 700 that differ in
+// 2 % of their places 138 -> 134 us, 3000 of 8 ragged ones of 100 119 -> 117.  None are listed
+// in decide mode: most pairs' groups are dismissed by their bounds.)
+// Pairs that are not worth it by themselves are looked at if no pair has to go to the recurrence: the batch is then done
+// here as a rule, and the latency of what comes after it is more than they cost (1024 groups of uniform tokens: 122 us, 142
+// without these).  What fails then is shaped as if one in eight did.
+constexpr int kBinPairs = 32 * kMatchWarps;               // pairs that a CTA bins
+__global__ void __launch_bounds__(32 * kMatchWarps)
+multi_bin_kernel(unsigned char* ws, MultiWs W, int N, int n_pairs, int bin_blocks, int32_t* dist_out) {
     grid_begin();
-    __shared__ int32_t s_hist[kNumBins];
-    for (int b = threadIdx.x; b < kNumBins; b += kOrderThreads) s_hist[b] = 0;
-    if (ctl->open == 0) return;                        // bounds and matches have settled the whole batch
-    const ShapeGoal goal = shape_goal(ctl->work, ctl->open, warps);
-    __syncthreads();
-    const int idx = blockIdx.x * kOrderThreads + threadIdx.x;
-    if (idx < n_pairs) {
+    PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
+    Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
+    const bool any = ctl->open != 0;
+    const unsigned long long lane_time = any ? ctl->work + ctl->maybe_work : (ctl->few_work + ctl->maybe_work) / 8;
+    const ShapeGoal goal = shape_goal(lane_time, any ? ctl->open + ctl->maybe : (ctl->few + ctl->maybe) / 8, W.warps);
+    auto bin_of = [&](const PairDesc& d) {
+        const PairSize z = size_of_desc(d);
+        return bin_of_shape(shape_of_pair(z.m, z.n, z.lb, z.ub, goal));
+    };
+    if ((int)blockIdx.x < bin_blocks) {
+        if (!any) return;
+        __shared__ int32_t s_hist[kNumBins];
+        for (int b = threadIdx.x; b < kNumBins; b += 32 * kMatchWarps) s_hist[b] = 0;
+        __syncthreads();
+        const int idx = blockIdx.x * kBinPairs + threadIdx.x;
+        if (idx < n_pairs) {
+            const PairDesc d = descs[idx];
+            if ((d.bin & (kNeedsDp | kListed)) == kNeedsDp) {
+                const int bin = bin_of(d);
+                descs[idx].bin = d.bin | (uint32_t)bin;
+                atomicAdd(&s_hist[bin], 1);
+            }
+        }
+        __syncthreads();
+        for (int b = threadIdx.x; b < kNumBins; b += 32 * kMatchWarps)
+            if (s_hist[b]) atomicAdd(&ctl->hist[b], s_hist[b]);
+        return;
+    }
+    __shared__ uint4 s_differ[kMatchWarps][kSpans];
+    __shared__ uint32_t s_entries[kMatchWarps][kMostMatches];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, P = pairs_of(N);
+    const int32_t* list = reinterpret_cast<const int32_t*>(ws + W.off_order);
+    const int few = ctl->few, all = few + (any ? 0 : ctl->maybe);
+    for (int e = ((int)blockIdx.x - bin_blocks) * kMatchWarps + warp; e < all; e += ((int)gridDim.x - bin_blocks) * kMatchWarps) {
+        const int idx = list[e < few ? e : n_pairs - 1 - (e - few)];
         const PairDesc d = descs[idx];
-        if (d.bin & kNeedsDp) {
-            const PairSize z = size_of_desc(d);
-            const int bin = bin_of_shape(shape_of_pair(z.m, z.n, z.lb, z.ub, goal));
+        const int upper = (int)(d.lower >> 16);
+        int dist = -1;
+        const int m = (int)(d.mn & 0xFFFFu), n = (int)(d.mn >> 16), strip = (int)((d.bin >> kStripShift) & 0x3FFu);
+        int g = W.patterns > 1 ? (int)__umulhi(d.pat_row, W.inv_patterns) : (int)d.pat_row;
+        if (g * W.patterns > (int)d.pat_row) --g;
+        const int i = (int)d.pat_row - g * W.patterns;
+        const int pr = kPairs.v[N][idx - g * P], j = (pr & 0xFF) + (pr >> 8) - i;
+        const uint16_t* names = reinterpret_cast<const uint16_t*>(ws + W.off_names) + (size_t)g * N * W.pitch;
+        __syncwarp();                              // the pair before has been read
+        const int count = find_matches<false>(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(ws + W.off_loc) + (size_t)idx * W.pitch),
+                                       reinterpret_cast<const uint2*>(names + j * W.pitch), reinterpret_cast<const uint2*>(names + i * W.pitch),
+                                       m, n, strip, s_differ[warp], s_entries[warp]);
+        if (count == 0)
+            dist = upper;
+        else if (count <= kMostMatches)
+            dist = distance_by_matches<false>(s_entries[warp], count, s_differ[warp],
+                                       reinterpret_cast<const uint32_t*>(ws + W.off_rows) + (size_t)d.pat_row * W.rows_pitch,
+                                       W.row_words, m, n, strip, upper);
+        if (lane != 0) continue;
+        if (dist >= 0) {
+            descs[idx].bin = 0u;
+            descs[idx].lower = (uint32_t)dist * 0x10001u;
+            dist_out[idx] = dist;
+        } else {
+            const int bin = bin_of(d);
             descs[idx].bin = d.bin | (uint32_t)bin;
-            atomicAdd(&s_hist[bin], 1);
+            atomicAdd(&ctl->hist[bin], 1);
+            atomicAdd(&ctl->failed, 1);
         }
     }
-    __syncthreads();
-    for (int b = threadIdx.x; b < kNumBins; b += kOrderThreads)
-        if (s_hist[b]) atomicAdd(&ctl->hist[b], s_hist[b]);
 }
 
 // Counting sort of the pairs by bin: longest warp tasks first, one team shape and similar
@@ -1432,7 +1425,7 @@ multi_order_kernel(PairDesc* descs, int32_t* order, Ctl* ctl, int n_pairs, int w
         }
         __syncthreads();
     } else {
-        if (ctl->open == 0) {
+        if (ctl->open == 0 && ctl->failed == 0) {      // bounds and matches have settled the whole batch
             if (blockIdx.x == 0 && t == 0) ctl->task_counter = ctl->total_tasks = 0;
             return;
         }
@@ -2061,15 +2054,14 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const int gpb = P <= kGroupThreads ? kGroupThreads / P : 1;
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     int32_t* order = reinterpret_cast<int32_t*>(ws + W.off_order);
-    if (!alone && !decide)
-        SR_LAUNCH("multi_matches_kernel", multi_matches_kernel, min((n_pairs + kMatchWarps - 1) / kMatchWarps, 16 * sms), 32 * kMatchWarps, 0, s, ws, W, a.N, n_pairs, dist);
     if (decide) {
         SR_LAUNCH("multi_bound_kernel", multi_bound_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, descs, ctl, flag, exact, gpb, alone,
                   !a.pair_dist && !a.pair_sum && !a.mean && !exact);
     }
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[1], s));
     const int order_blocks = alone ? 1 : (n_pairs + kOrderThreads - 1) / kOrderThreads;
-    if (!alone) SR_LAUNCH("multi_bin_kernel", multi_bin_kernel, order_blocks, kOrderThreads, 0, s, descs, ctl, n_pairs, W.warps);
+    const int bin_blocks = (n_pairs + kBinPairs - 1) / kBinPairs, match_blocks = decide ? 0 : min((n_pairs + kMatchWarps - 1) / kMatchWarps, 16 * sms);
+    if (!alone) SR_LAUNCH("multi_bin_kernel", multi_bin_kernel, bin_blocks + match_blocks, 32 * kMatchWarps, 0, s, ws, W, a.N, n_pairs, bin_blocks, dist);
     SR_LAUNCH("multi_order_kernel", alone ? multi_order_kernel<true> : multi_order_kernel<false>, order_blocks, kOrderThreads, 0, s, descs, order, ctl, n_pairs, W.warps);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[2], s));
     const long long want = (n_pairs_ll + kDpWarpsPerCta - 1) / kDpWarpsPerCta;
