@@ -314,7 +314,7 @@ def main():
         sampler.hold(step, 4, 1.0)
         clocks = sampler.stop()
     stage_ms = [statistics.median(e5[k].elapsed_time(e5[k + 1]) for e5 in stage_evs) for k in range(4)]
-    prep_ms = stage_ms[0]
+    prep_ms = stage_ms[0] + stage_ms[1]
 
     # ------------------------------------------------------------------ end to end
     # host side: the batch as a rollout buffer holds it, prefixes back to back plus row offsets
@@ -357,7 +357,7 @@ def main():
     value = cells * world * args.steps / (total_ms * 1e-3) / 1e9
     e2e_value = cells * world * args.steps / (e2e_ms * 1e-3) / 1e9
     alu_peak = sms * SM_INT32_LANES * peaks["sm_max_mhz"] * 1e6 / 1e9          # Gop/s
-    # Uniform tokens leave the recurrence nothing to do: names, look-ups and the pairs' few matches are the step, and what
+    # Uniform tokens leave the recurrence nothing to do: names, look-ups and the pairs' few matches (in the binning launch) are the step, and what
     # they cannot do without is the symbols in and a distance per pair out.
     gate_bytes = int(np.minimum(w.lens, K).sum()) * 4 + G * N * 4 + G * P * 4
     achieved = gate_bytes / (prep_ms * 1e-3) / 1e9
@@ -374,14 +374,14 @@ def main():
                 "ms_per_step": e2e_ms / args.steps,
                 "input": "packed prefixes + int64 row offsets in pinned host memory (sr_gate_host_packed), "
                          "sent in four pieces on a copy stream under the per-group pass; one recurrence launch"},
-        "gpu_launches": 8 * args.steps,       # names, prep, matches, bin, order, dp, finish; advantages
+        "gpu_launches": (7 if args.groups >= 512 else 2) * args.steps,       # names, prep, bin, order, dp, finish; advantages (smaller batches: two at the least)
         "clocks": clocks,
         "stage_ms": {"prep": stage_ms[0], "order": stage_ms[1], "dp": stage_ms[2], "finish": stage_ms[3]},
-        "roofline": {"kernel": "multi_names_kernel + multi_prep_kernel + multi_matches_kernel", "bound": "hbm", "achieved": achieved,
+        "roofline": {"kernel": "multi_names_kernel + multi_prep_kernel + multi_bin_kernel + multi_order_kernel", "bound": "hbm", "achieved": achieved,
                      "peak": peaks["hbm_gbs"], "unit": "GB/s (symbols and lengths in, distances out) of measured copy", "frac": achieved / peaks["hbm_gbs"],
                      "limited_by": "instruction issue: naming, 640 look-ups a pair and text, 1100 warp instructions a pair for its matches",
-                     "traffic": traffic_from_profiles("multi_prep_kernel", os.path.join(ROOT, "paper_2605_05802_b200", "csrc", "gate_multi.cu")),
-                     "ms_per_launch": prep_ms},
+                     "traffic": None, "traffic_prep_kernel": traffic_from_profiles("multi_prep_kernel", os.path.join(ROOT, "paper_2605_05802_b200", "csrc", "gate_multi.cu")),
+                     "ms_of_the_four": prep_ms},
         "verified_against_oracle": verify,
     }
 
@@ -497,7 +497,7 @@ def main():
                                       "us_sr_gate_same_threshold": statistics.median(ms_gate) * 1e3,
                                       "groups_computed_exactly": int(ex.sum().item()),
                                       "groups_cut": int(stop_ref.sum().item()),
-                                      "note": "above about 0.35 most groups have to be computed anyway and sr_gate is the faster call"}
+                                      "note": "pairs with few matches are not looked for in this mode, so sr_gate is the faster call on uniform tokens where many groups stay open"}
         # restore the headline outputs for the checks below
         sr.sr_gate(seqs, lens, K, w.threshold, w.norm_mode, pair_sum=ps, mean=mean, stop=stop, workspace=ws)
         torch.cuda.synchronize()

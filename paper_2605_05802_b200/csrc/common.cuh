@@ -216,8 +216,8 @@ int launch_gate_single(const GateArgs& a, cudaStream_t s);
 // gate_multi.cu: prefixes of up to SR_MAX_K symbols, blocked multi-word.
 // `row_cap`: mask rows per pattern, at least 1 and at most (K + 7) / 8, which 0 stands for.
 size_t gate_multi_workspace_bytes(int32_t n_groups, int32_t N, int32_t K, int row_cap = 0);
-// `ev`: NULL, or 5 events recorded before prep / after prep / after scan+scatter /
-// after dp / after finish.
+// `ev`: NULL, or 5 events recorded before names / after prep / after bin (few matches) and order /
+// after dp / after finish; a small batch, whose gate is one launch after the names, records the last four together.
 // `decide`: finish groups whose lower-bounded d_K already reaches the threshold without
 // running their pairs; `exact` (may be NULL) then receives 1 per group computed exactly.
 // `feed`: NULL, or the groups become ready on the stream in `pieces` pieces: before the

@@ -260,7 +260,7 @@ __device__ __forceinline__ int clamp_len(const int32_t* lens, size_t idx, int K,
 // round names at least one symbol of each slot.  One CTA per group.  With the names, 16 bits
 // each, a pattern's look-up table is an array: no hashing, no probing, no comparing in prep, which serves
 // every text (N - 1) / 2 times.  Names and prep together, 1024 groups of 8 token prefixes: 82 us, 107 us at full
-// length.  Bound: the latency between the barriers here (three CTAs of 64 KB per SM), instruction issue in prep.
+// length.  Bound: the latency between the barriers here (four CTAs of 48 KB per SM), instruction issue in prep.
 constexpr uint32_t kHashMul = 0x9E3779B1u;
 constexpr int kMaxTexts = SR_MAX_N / 2;        // texts a pattern is paired with
 constexpr int kMaxPairs = SR_MAX_N * (SR_MAX_N - 1) / 2;
@@ -2067,7 +2067,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const long long want = (n_pairs_ll + kDpWarpsPerCta - 1) / kDpWarpsPerCta;
     const int blocks = (int)(want < 3LL * sms ? want : 3LL * sms);
     // (an ordinary launch unless every CTA has an SM: CTAs made resident while the tail of prep still fills some SMs would
-    // crowd onto the others, 310 us instead of 269 for the token-level batch of 1024 groups)
+    // crowd onto the others, 310 us instead of 269 for 1024 groups of uniform tokens when these still took the recurrence)
     const int rc = launch_as(alone && blocks < sms, 1, "multi_dp_kernel", multi_dp_kernel, blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u);
     if (rc != SR_OK) return rc;
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[3], s));

@@ -478,7 +478,7 @@ int launch_incr_step(void* state, size_t bytes, const int32_t* new_actions, int3
         a.off_term = take(a.gpb * P * 8);
         a.off_roll = take(a.gpb * N * 8);
         a.off_eq = take(a.gpb * N * (N - 1) * 4);
-        // Groups of 8 up to a wave and a half: the loads of one CTA's states are what the others of its SM wait for as well
+        // Groups of 8 up to a little over two waves (nine CTAs an SM): the loads of one CTA's states are what the others of its SM wait for as well
         // (30 steps on 20000 groups 264 -> 249 us, 46000 449 -> 434, 65536 614 -> 617; 5000 of 16 370 -> 398).
         const bool staged = N == 8 && (long long)n_groups * P < 1300000;
         a.off_state = take(staged ? a.gpb * P * 16 : 0);
