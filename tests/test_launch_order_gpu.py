@@ -62,6 +62,50 @@ def test_back_to_back_calls_see_each_other(n_groups, K, captured):
         assert int(c) == len(oidx) and np.array_equal(i.cpu().numpy()[:int(c)], oidx), k
 
 
+@pytest.mark.parametrize("decide", [False, True])
+@pytest.mark.parametrize("n_groups,K", [(16, 1024), (16, 512), (5, 200), (300, 1024)])
+def test_replayed_multi_word_calls(n_groups, K, decide):
+    """The routes of the multi-word gate from one captured graph on changing inputs: the last CTA of a group counts the
+    arrivals, a cluster hands over its distances or settles its group from bounds, a sorted batch counts its bins."""
+    dev = torch.device("cuda:0")
+    batches = [W.token_gate(seed=s, n_groups=n_groups, min_len=40, max_len=K) for s in range(3)]
+    host = [(torch.from_numpy(w.seqs).to(dev), torch.from_numpy(w.lens).to(dev)) for w in batches]
+    seqs, lens = (torch.empty_like(x) for x in host[0])
+    G, N, stride = seqs.shape
+    threshold = float(np.median(oracle.gate(batches[0].seqs, batches[0].lens, K, 0.0, threads=8)[2]))
+    stop = torch.empty(G, dtype=torch.uint8, device=dev)
+    mean = None if decide else torch.empty(G, dtype=torch.float64, device=dev)
+    ws = torch.empty(sr.sr_gate_workspace_bytes(G, N, stride, K), dtype=torch.uint8, device=dev)
+
+    def step():
+        if decide:
+            sr.sr_gate_decide(seqs, lens, K, threshold, stop=stop, workspace=ws)
+        else:
+            sr.sr_gate(seqs, lens, K, threshold, mean=mean, stop=stop, workspace=ws)
+
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        for dst, src in zip((seqs, lens), host[0]):
+            dst.copy_(src)
+        step()
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            step()
+            step()
+        got = []
+        for k in range(9):
+            for dst, src in zip((seqs, lens), host[k % 3]):
+                dst.copy_(src)
+            graph.replay()
+            got.append((stop.clone(), None if decide else mean.clone()))
+    torch.cuda.synchronize()
+    want = [oracle.gate(w.seqs, w.lens, K, threshold, threads=8) for w in batches]
+    for k, (s, m) in enumerate(got):
+        assert np.array_equal(s.cpu().numpy(), want[k % 3][3]), k
+        assert decide or np.array_equal(m.cpu().numpy(), want[k % 3][2]), k
+
+
 @pytest.mark.parametrize("captured", [False, True])
 @pytest.mark.parametrize("G,N", [(200, 8), (30000, 2), (3571, 8), (12000, 8), (23000, 8), (2173, 24), (70000, 8)])
 def test_steps_back_to_back_see_each_other(G, N, captured):

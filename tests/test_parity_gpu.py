@@ -477,6 +477,28 @@ def test_advantage_edges():
             _check_adv(r, None, eps)
 
 
+@pytest.mark.parametrize("N", [2, 4, 7, 8, 9, 12, 15, 16, 17, 20, 24, 25, 32])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_advantages_of_every_group_size(N, offset):
+    """Every bound on the number of places, with 16-byte aligned rows and one float past them."""
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(N)
+    r = rng.random((301, N)).astype(np.float32)
+    r[0], r[1, 0] = 0.3, np.nan
+    drop = (rng.random(301) < 0.2).astype(np.uint8)
+    rewards = torch.empty(301 * N + 4, device=dev)[offset:offset + 301 * N].view(301, N)
+    rewards.copy_(torch.from_numpy(r))
+    whole = torch.full((301 * N + 8,), 77.0, device=dev)
+    adv = whole[offset:offset + 301 * N].view(301, N)
+    zv = torch.full((301,), 9, dtype=torch.uint8, device=dev)
+    sr.sr_grpo_advantage(rewards, torch.from_numpy(drop).to(dev), 1e-6, adv=adv, zero_var=zv)
+    oadv, ozv = oracle.advantage(r, drop, 1e-6)
+    assert np.array_equal(zv.cpu().numpy(), ozv)
+    got = adv.cpu().numpy()
+    assert np.allclose(got, oadv, rtol=1e-6, atol=0, equal_nan=True) and np.array_equal(got == 0, oadv == 0)
+    assert bool((whole[:offset] == 77).all()) and bool((whole[offset + 301 * N:] == 77).all())
+
+
 def test_binding_refuses_short_or_misplaced_buffers():
     """An output that cannot hold what the call writes, or a host tensor where the library
     expects device memory, is refused by the binding before anything is launched."""
