@@ -1893,7 +1893,7 @@ constexpr int kMostEightLanes = 253;
 // symbols, and diverging texts, 2676 shapes of 2 to 32 rollouts and K = 33 to 1024; diverging batches would gain up to twice as
 // many groups).  It falls with the lanes that a pair takes (up to 8, 16, 16 of two blocks), and where a CTA has only one text or
 // two for its warps.  In the last fifth before the line the worst kind of
-// batch takes 0.84 of the time it takes sorted, 1.05 at most, all kinds 0.72.
+// batch takes 0.86 of the time it takes sorted, 1.05 at most, all kinds 0.74.
 // With more than eight texts to a pattern a pair of 16 lanes waits for others of its CTA: then while there are SMs for
 // all CTAs, or half of them (K <= 512).
 // The decide mode does so for groups of up to eight, whose CTAs are a cluster that sums up the bounds first; clusters
@@ -1907,7 +1907,7 @@ bool runs_in_pairs(int n_groups, int N, int K, int sms, bool decide) {
         return N <= kMostOwnPatterns && n_pairs <= 7000 && n_pairs * (K + 384) <= 1000LL * kMost[N][lanes];
     }
     if (texts > 8 && lanes > 0) return ctas <= (lanes == 1 ? 2 : 1) * sms;
-    constexpr int kMost[5][3] = {{4500, 1000, 1000}, {4500, 3500, 2500}, {6400, 3500, 2300}, {6400, 4000, 3000}, {4200, 0, 0}};
+    constexpr int kMost[5][3] = {{4500, 1400, 1000}, {4500, 3900, 2900}, {6400, 3900, 2500}, {6400, 4200, 3400}, {4200, 0, 0}};
     return n_pairs * (K + 384) <= 1000LL * kMost[texts <= 3 ? texts - 1 : texts <= 8 ? 3 : 4][lanes];
 }
 
