@@ -1301,15 +1301,15 @@ __device__ __forceinline__ ShapeGoal shape_goal(unsigned long long work, int ope
 // here as a rule, and the latency of what comes after it is more than they cost (1024 groups of uniform tokens: 122 us, 142
 // without these).  What fails then is shaped as if one in eight did.
 constexpr int kBinPairs = 32 * kMatchWarps;               // pairs that a CTA bins
-__global__ void __launch_bounds__(32 * kMatchWarps)
+__global__ void __launch_bounds__(32 * kMatchWarps, 5)
 multi_bin_kernel(unsigned char* ws, MultiWs W, int N, int n_pairs, int bin_blocks, int32_t* dist_out) {
     grid_begin();
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
     const bool any = ctl->open != 0;
-    const unsigned long long lane_time = any ? ctl->work + ctl->maybe_work : (ctl->few_work + ctl->maybe_work) / 8;
-    const ShapeGoal goal = shape_goal(lane_time, any ? ctl->open + ctl->maybe : (ctl->few + ctl->maybe) / 8, W.warps);
-    auto bin_of = [&](const PairDesc& d) {
+    auto bin_of = [&](const PairDesc& d) {                   // (the goal anew for each: few need it where registers count)
+        const unsigned long long lane_time = any ? ctl->work + ctl->maybe_work : (ctl->few_work + ctl->maybe_work) / 8;
+        const ShapeGoal goal = shape_goal(lane_time, any ? ctl->open + ctl->maybe : (ctl->few + ctl->maybe) / 8, W.warps);
         const PairSize z = size_of_desc(d);
         return bin_of_shape(shape_of_pair(z.m, z.n, z.lb, z.ub, goal));
     };
