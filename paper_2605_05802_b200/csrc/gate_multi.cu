@@ -185,11 +185,14 @@ __host__ __device__ inline int quad_cost(int R, bool ring) { return 26 * R + (ri
 
 struct Shape { int tlog, R, time; };
 
+// Quads of match words that a lane has under way (see dp_task).
+__host__ __device__ constexpr int quads_ahead(int R) { return R <= 2 ? 2 : 1; }
+
 // Team shape of a pair of m rows x n columns (what is left after the common prefix) whose
 // distance lies in lb..ub.  Either the team's lanes hold the whole pattern, or, where the
 // band is narrow enough, they form a ring that follows it: stripe g + T may only enter
-// the band three iterations after stripe g has left it, w + 32 R + 11 < T (32 R + 4) for a band
-// of w + 1 diagonals.  The shape with the least lane-time wins, where one that takes longer than
+// the band 2 quads_ahead(R) + 1 iterations after stripe g has left it, w + 32 R + 3 + 8 quads_ahead(R) < T (32 R + 4) for a
+// band of w + 1 diagonals.  The shape with the least lane-time wins, where one that takes longer than
 // the goal's limit counts for more in the proportion by which it does, and lanes that would be
 // idle otherwise are free.
 struct ShapeGoal { float limit, free_lanes; };
@@ -202,9 +205,10 @@ __device__ inline Shape shape_of_pair(int m, int n, int lb, int ub, ShapeGoal go
     float best_score = 3.0e38f;
 #pragma unroll
     for (int t = 0; t <= 5; ++t) {
-        const int T = 1 << t, room = w + 11 - 4 * T;
+        const int T = 1 << t, room = w + 11 - 4 * T, far = room + 8;
         // all blocks on the team's lanes; a ring of stripes as low as the band allows
-        const int full_R = (W + T - 1) >> t, ring_R = t == 0 ? 99 : (room < 0 ? 1 : room / (32 * (T - 1)) + 1);
+        const int full_R = (W + T - 1) >> t, ring_R = t == 0 ? 99 : far < 64 * (T - 1) ? (far < 0 ? 1 : far / (32 * (T - 1)) + 1) : max(room / (32 * (T - 1)) + 1, 3);
+        static_assert(quads_ahead(2) == 2 && quads_ahead(3) == 1, "");
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const int R = k ? ring_R : full_R;
@@ -1636,24 +1640,30 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
     int acc = 0;
     const uint2 none = make_uint2(kLocNone | (kLocNone << 16), kLocNone | (kLocNone << 16));
     auto fetch = [&](int j) { return (uint32_t)(j - js) <= span ? __ldg(stream + j) : none; };
-    uint32_t Eq[4][R];
-    {
-        const uint2 q = fetch(0);
+    // Match words are asked for kAhead iterations before they are used.  One is not enough for a trip to L2 where lanes hold
+    // little of a pattern and an iteration is short: 1024 groups of 8 texts of 1024 that differ in 1 % of their places
+    // 366 us, 316 with two; with two for R = 3 and 4 as well diverging ones 312, 338.
+    constexpr int kAhead = quads_ahead(R);
+    uint32_t words_of[kAhead][4][R];
+    uint2 quads[kAhead];
+#pragma unroll
+    for (int s = 0; s < kAhead; ++s) {
+        const uint2 q = fetch(s);
         const uint32_t loc[4] = {q.x & 0xFFFFu, q.x >> 16, q.y & 0xFFFFu, q.y >> 16};
 #pragma unroll
-        for (int u = 0; u < 4; ++u) match_words<R>(loc[u], rowbase, words, W.row_words, Eq[u]);
-        if (any_chains) add_chains<R>(q, rowbase, nxt, Eq);
+        for (int u = 0; u < 4; ++u) match_words<R>(loc[u], rowbase, words, W.row_words, words_of[s][u]);
+        if (any_chains) add_chains<R>(q, rowbase, nxt, words_of[s]);
+        quads[s] = fetch(kAhead + s);
     }
-    uint2 q1 = fetch(1);
 
     // The body is one block of straight-line code, so that the compiler can fill the latencies of
     // one column's chain of operations with the others' and with the next quad's match words:
     // a lane outside its stripe's quads runs along.  Before them it leaves its words alone by
     // itself (no matches, nothing coming in from above: all-ones stay all-ones); after them its
     // words are kept.
-    for (int j = 0; j < iters; ++j) {
-        const uint2 q = q1;                            // the quad after this one
-        q1 = fetch(j + 2);
+    auto step = [&](int j, uint32_t (&Eq)[4][R], uint2& next) {
+        const uint2 q = next;                          // the quad kAhead after this one
+        next = fetch(j + 2 * kAhead);
         const bool active = (uint32_t)(j - js) <= span;
         // deltas leaving the stripe above for this quad (it worked on it last iteration)
         uint32_t wP = __shfl_sync(0xFFFFFFFFu, outP, src) << 28, wM = __shfl_sync(0xFFFFFFFFu, outM, src) << 28;
@@ -1691,6 +1701,11 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
                 for (int r = 0; r < R; ++r) { Pv[r] = 0xFFFFFFFFu; Mv[r] = 0u; }
             }
         }
+    };
+    // (two copies of the body, so that what is under way stays in its registers; the last may find no quad left)
+    for (int j = 0; j < iters; j += kAhead) {
+#pragma unroll
+        for (int s = 0; s < kAhead; ++s) step(j + s, words_of[s], quads[s]);
     }
     if (!ring) {
         // D[m][n] = n + (sum of the vertical deltas of the last column over rows 1..m)
