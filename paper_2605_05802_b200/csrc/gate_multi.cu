@@ -67,7 +67,7 @@ constexpr int kOrderThreads = 1024;
 constexpr int kAlonePairs = 1024;   // batches of up to this many pairs are ordered by one CTA
 constexpr uint32_t kLocChain = 0xC000u;   // | first position of the symbol's occurrence chain
 constexpr uint32_t kChainEnd = 0xFFFFu;
-constexpr int kDpWarpsPerCta = 4;
+constexpr int kDpWarps = 12, kMostDpWarps = 16;   // of an SM, see multi_dp_kernel
 constexpr uint32_t kBinMask = 0x7FFu;
 constexpr uint32_t kListed = 0x800u;          // see multi_bin_kernel
 constexpr uint32_t kHasChains = 0x40000000u;
@@ -110,7 +110,7 @@ struct MultiWs {
     int patterns;          // rollouts of a group that serve as patterns
     int row_cap;           // mask rows a pattern may have
     int rows_pitch;        // 32-bit words from one pattern's mask rows to the next's: a multiple of four
-    int warps;             // warps the dp kernel keeps resident
+    int warps;             // warps of the recurrence for which the shapes are chosen
     uint32_t inv_patterns; // 2^32 / patterns, rounded up
     int text_warps, text_stride;   // prep: warps to a text, texts that the CTA's warps take at a time
     uint32_t inv_text_warps;       // 2^32 / text_warps, rounded up
@@ -1729,8 +1729,15 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
     if (valid && lt == 0) dist_out[idx] = ring && acc > ub ? ((ub + 1) | kCappedFlag) : acc;
 }
 
-// Persistent warps pull warp tasks, longest first, from the bins' task list.
-__global__ void __launch_bounds__(kDpWarpsPerCta * 32)
+// One CTA an SM, whose warps take the bins' warp tasks, longest first.  The first tasks are dealt out, four to an SM, then four
+// more, so that every scheduler has the same number to within one, and neighbours, which run the same code on the same rows,
+// are on one SM; the others are pulled.  (All of them pulled, by three CTAs of four warps, up to three ended up on one
+// scheduler and none on others: decide mode at 0.12, 1024 groups of 8 texts of 1024, 1044 tasks, 234 -> 219 us; with
+// twelve warps the 1796 tasks of 1024 groups over 3000 symbols took two rounds, 671 -> 550 us.)  Sixteen warps where they hold all
+// tasks, and where there are more than twice as many; in between, where few rounds end in a tail that is the longer the
+// more warps share a scheduler, twelve (1024 groups of diverging ragged texts, 4148 tasks: 299 us, 331 with sixteen; 6000 of 256 over
+// 100 symbols, 10495 tasks, 806 and 739).
+__global__ void __launch_bounds__(kMostDpWarps * 32, 1)
 multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
     grid_begin();
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
@@ -1741,15 +1748,15 @@ multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
     const uint32_t* masks = reinterpret_cast<const uint32_t*>(ws + W.off_rows);
     const int lane = threadIdx.x & 31;
     const int total = ctl->total_tasks;
-    // As many warps as tasks or more: the tasks are dealt out, four to a CTA, and the CTAs go round the SMs.  Pulled, they end up
-    // three to a scheduler here and none there (1024 groups of 8 texts of 1024 at 0.12 in decide mode, 1044 tasks: 234 us, 220
-    // dealt).  More tasks are pulled from the start: warps that begin together then get neighbours, which run the same
-    // code on the same rows (1024 groups of diverging texts 682 us, 768 with the first tasks dealt).
-    const bool dealt = total <= kDpWarpsPerCta * (int)gridDim.x;
+    const int warp = (int)(threadIdx.x >> 5), most = kMostDpWarps * (int)gridDim.x;
+    const bool at_once = total <= most, fewer = !at_once && total <= 2 * most;
+    if (fewer && warp >= kDpWarps) return;
+    const int dealt = (fewer ? kDpWarps : kMostDpWarps) * (int)gridDim.x;
     for (int round = 0;; ++round) {                   // (with the task kept from round to round the recurrence comes out 10 % slower)
         int task = 0;
-        if (dealt) task = round ? total : kDpWarpsPerCta * (int)blockIdx.x + (int)(threadIdx.x >> 5);
-        else if (lane == 0) task = atomicAdd(&ctl->task_counter, 1);
+        if (round == 0) task = 4 * ((int)blockIdx.x + (int)gridDim.x * (warp >> 2)) + (warp & 3);
+        else if (at_once) task = total;
+        else if (lane == 0) task = dealt + atomicAdd(&ctl->task_counter, 1);
         task = __shfl_sync(0xFFFFFFFFu, task, 0);
         if (task >= total) break;
         int k = 0, hi = kNumBins;                     // last bin whose first task is <= task
@@ -1993,10 +2000,7 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     int dev = 0, sms = 0;
     SR_CUDA_TRY(cudaGetDevice(&dev));
     SR_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // the dp kernel's persistent grid: 3 CTAs of 4 warps per SM (3 warps per scheduler): enough to
-    // keep the integer pipe busy, few enough that most tasks are pulled dynamically, longest
-    // first (measured best among 2..6 warps per scheduler)
-    W.warps = 3 * kDpWarpsPerCta * sms;
+    W.warps = kDpWarps * sms;
     const int n_pairs = (int)n_pairs_ll;
     int32_t* dist = a.pair_dist ? a.pair_dist : reinterpret_cast<int32_t*>(ws + W.off_dist);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
@@ -2085,11 +2089,10 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     if (!alone) SR_LAUNCH("multi_bin_kernel", multi_bin_kernel, bin_blocks + match_blocks, 32 * kMatchWarps, 0, s, ws, W, a.N, n_pairs, bin_blocks, dist);
     SR_LAUNCH("multi_order_kernel", alone ? multi_order_kernel<true> : multi_order_kernel<false>, order_blocks, kOrderThreads, 0, s, descs, order, ctl, n_pairs, W.warps);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[2], s));
-    const long long want = (n_pairs_ll + kDpWarpsPerCta - 1) / kDpWarpsPerCta;
-    const int blocks = (int)(want < 3LL * sms ? want : 3LL * sms);
+    const int blocks = n_pairs < sms ? n_pairs : sms;
     // (an ordinary launch unless every CTA has an SM: CTAs made resident while the tail of prep still fills some SMs would
     // crowd onto the others, 310 us instead of 269 for 1024 groups of uniform tokens when these still took the recurrence)
-    const int rc = launch_as(alone && blocks < sms, 1, "multi_dp_kernel", multi_dp_kernel, blocks, kDpWarpsPerCta * 32, 0, s, ws, W, dist, 2u);
+    const int rc = launch_as(alone && (n_pairs + 3) / 4 < sms, 1, "multi_dp_kernel", multi_dp_kernel, blocks, kMostDpWarps * 32, 0, s, ws, W, dist, 2u);
     if (rc != SR_OK) return rc;
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[3], s));
     SR_LAUNCH("multi_finish_kernel", multi_finish_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, dist, flag, exact, gpb);

@@ -19,7 +19,7 @@ def test_bands_at_the_limits_of_rings(G, N, K):
     stride = (K + 3) // 4 * 4
     seqs = np.zeros((G, N, stride), dtype=np.int32)
     for g in range(G):
-        base = rng.permutation(10 ** 6)[:stride]
+        base = rng.integers(0, 2 ** 31 - 1, size=stride, dtype=np.int32)
         repeats = rng.integers(0, stride, size=stride // 8)              # symbols with mask rows
         base[repeats] = base[rng.integers(0, stride, size=repeats.size)]
         seqs[g] = base
