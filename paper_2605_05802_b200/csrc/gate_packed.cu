@@ -39,7 +39,11 @@ struct FeedCtx {
     int N, stride;
     cudaEvent_t* copied;      // one event per piece, recorded on the copy stream
     int pieces, n_groups;
+    int first;                // the batch's group that is this feed's first
 };
+
+// Groups of a feed before its piece c, as the pipeline cuts them.
+int piece_begin(int n_groups, int pieces, int c) { return (int)((long long)n_groups * c / pieces); }
 
 int unpack_rows(const FeedCtx& f, int g0, int g1, cudaStream_t s) {
     const size_t row0 = (size_t)g0 * f.N;
@@ -52,9 +56,9 @@ int feed_piece(void* ctx, int g0, int g1, cudaStream_t s) {
     const FeedCtx& f = *static_cast<const FeedCtx*>(ctx);
     // the piece index follows from g0 the same way the pipeline cut the groups
     int c = 0;
-    while (c + 1 < f.pieces && (int)((long long)f.n_groups * (c + 1) / f.pieces) <= g0) ++c;
+    while (c + 1 < f.pieces && piece_begin(f.n_groups, f.pieces, c + 1) <= g0) ++c;
     SR_CUDA_TRY(cudaStreamWaitEvent(s, f.copied[c], 0));
-    return unpack_rows(f, g0, g1, s);
+    return unpack_rows(f, f.first + g0, f.first + g1, s);
 }
 
 // Events of one call; destroyed when the call returns, whichever way (an event that is
@@ -73,6 +77,12 @@ struct EventSet {
 // Symbols from which they are sent in pieces: less is on the link for no longer than the launches of a pass per piece
 // take (80 groups of 8 at K = 48 99 us in pieces, 38 in one; 200 at 256, 1.6 MB, 138 and 97; at 3 to 4 MB both are alike).
 constexpr long long kPieceBytes = 2ll << 20;
+
+// Symbols from which the gate itself runs in two parts, the first one under the copy of the second.  It pays once the copy of
+// half the batch takes longer than the tails of a second set of launches: in one part / in two, 21 MB of ragged texts of
+// 1024 743 / 688 us, 34 MB of full ones 1033 / 902, 17 MB of pairs of 700 478 / 472; 13 MB of groups of 4 432 / 455,
+// 9 MB of ragged texts 420 / 453.
+constexpr long long kPartBytes = 14ll << 20;
 
 struct PackedArena {
     size_t off_packed, off_start, inner, total;     // `inner`: where the padded-input arena begins
@@ -140,37 +150,57 @@ int sr_gate_host_packed(const int32_t* symbols, const int64_t* row_start, int32_
                 pair_sum ? reinterpret_cast<int32_t*>(di + h.off_sum) : nullptr,
                 mean ? reinterpret_cast<double*>(di + h.off_mean) : nullptr,
                 di + h.off_stop, status ? reinterpret_cast<int32_t*>(di + h.off_status) : nullptr};
-    FeedCtx f{d_packed, d_start, d_seqs, d_lens, N, stride, nullptr, 1, n_groups};
+    FeedCtx f{d_packed, d_start, d_seqs, d_lens, N, stride, nullptr, 1, n_groups, 0};
     if (status) SR_CUDA_TRY(cudaMemcpyAsync(di + h.off_status, status, 4, cudaMemcpyHostToDevice, s));
     cudaStream_t cs = static_cast<cudaStream_t>(copy_stream);
-    // With a copy stream and long prefixes the symbols go over in four pieces of whole groups
-    // and the per-group pass of the gate (match streams) runs on each piece while the next one
-    // is still on the link; the recurrence then runs ONCE over the whole batch.  Cutting the
-    // whole gate into pieces was measured and lost: the kernels of a quarter of a token-level
-    // batch take almost as long as those of the whole batch, because a few long pairs set the
-    // time of the recurrence launch.
+    // With a copy stream and long prefixes the symbols go over in pieces of whole groups, and the per-group pass of the gate
+    // (match streams) runs on each piece while the next one is still on the link.  The rest of the gate runs once over the whole batch,
+    // or, where there is enough to copy, once over the first half, while the second is on the link, and once over that.  The
+    // two use the same workspace, one after the other.  (More parts lose: the few long pairs of a quarter set the time of its
+    // recurrence.)
     if (cs != nullptr && cs != s && K > 32 && n_groups >= 64 && total * 4 >= kPieceBytes) {
-        constexpr int kPieces = 4;
-        EventSet events;                                  // [0] fork, [1 + c] piece c copied
-        for (int k = 0; k < 1 + kPieces; ++k) SR_CUDA_TRY(events.add());
+        constexpr int kMostPieces = 4;
+        const bool halves = total * 4 >= kPartBytes;
+        const int parts = halves ? 2 : 1, pieces[2] = {halves ? 2 : kMostPieces, 1};
+        const int cut[3] = {0, halves ? n_groups / 2 : n_groups, n_groups};
+        EventSet events;                                  // [0] fork, then one for each piece that has been copied
+        for (int k = 0; k < 1 + kMostPieces; ++k) SR_CUDA_TRY(events.add());
         // the copies must not overtake earlier work on `stream` that uses the arena
         SR_CUDA_TRY(cudaEventRecord(events.ev[0], s));
         SR_CUDA_TRY(cudaStreamWaitEvent(cs, events.ev[0], 0));
         SR_CUDA_TRY(cudaMemcpyAsync(d_start, row_start, (rows + 1) * 8, cudaMemcpyHostToDevice, cs));
-        for (int c = 0; c < kPieces; ++c) {
-            const size_t row0 = (size_t)((long long)n_groups * c / kPieces) * N;
-            const size_t row1 = (size_t)((long long)n_groups * (c + 1) / kPieces) * N;
-            const long long s0 = row_start[row0], s1 = row_start[row1];
-            if (s1 > s0)
-                SR_CUDA_TRY(cudaMemcpyAsync(d_packed + s0, symbols + s0, (size_t)(s1 - s0) * 4,
-                                            cudaMemcpyHostToDevice, cs));
-            SR_CUDA_TRY(cudaEventRecord(events.ev[1 + c], cs));
+        int at = 1;
+        for (int p = 0; p < parts; ++p) {
+            for (int c = 0; c < pieces[p]; ++c) {
+                const size_t row0 = (size_t)(cut[p] + piece_begin(cut[p + 1] - cut[p], pieces[p], c)) * N;
+                const size_t row1 = (size_t)(cut[p] + piece_begin(cut[p + 1] - cut[p], pieces[p], c + 1)) * N;
+                const long long s0 = row_start[row0], s1 = row_start[row1];
+                if (s1 > s0)
+                    SR_CUDA_TRY(cudaMemcpyAsync(d_packed + s0, symbols + s0, (size_t)(s1 - s0) * 4,
+                                                cudaMemcpyHostToDevice, cs));
+                SR_CUDA_TRY(cudaEventRecord(events.ev[at++], cs));
+            }
         }
-        f.copied = events.ev + 1;
-        f.pieces = kPieces;
-        const GroupFeed feed{kPieces, feed_piece, &f};
-        const int rc = launch_gate_multi(ga, di + h.off_ws, h.total - h.off_ws, s, nullptr, false, nullptr, &feed);
-        if (rc != SR_OK) return rc;
+        at = 1;
+        for (int p = 0; p < parts; ++p) {
+            const size_t g0 = cut[p], row0 = g0 * N;
+            f.copied = events.ev + at;
+            f.pieces = pieces[p];
+            f.first = cut[p];
+            f.n_groups = cut[p + 1] - cut[p];
+            at += pieces[p];
+            GateArgs part = ga;
+            part.seqs += row0 * stride;
+            part.lens += row0;
+            part.n_groups = f.n_groups;
+            if (part.pair_dist) part.pair_dist += g0 * P;
+            if (part.pair_sum) part.pair_sum += g0;
+            if (part.mean) part.mean += g0;
+            part.stop += g0;
+            const GroupFeed feed{f.pieces, feed_piece, &f};
+            const int rc = launch_gate_multi(part, di + h.off_ws, h.total - h.off_ws, s, nullptr, false, nullptr, &feed);
+            if (rc != SR_OK) return rc;
+        }
     } else {
         SR_CUDA_TRY(cudaMemcpyAsync(d_start, row_start, (rows + 1) * 8, cudaMemcpyHostToDevice, s));
         if (total > 0)

@@ -1,5 +1,5 @@
 """Packed host input on either side of the size from which it is sent in pieces: equal to the oracle, one call after
-the other on one arena, with rows without symbols and group counts that the pieces do not divide."""
+the other on one arena, with rows without symbols and group counts that the pieces do not divide; the last one is gated in two parts."""
 import numpy as np
 import pytest
 
@@ -9,7 +9,7 @@ from paper_2605_05802_b200 import workloads as W
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("G,N,K", [(64, 8, 1000), (66, 8, 1024), (67, 16, 520), (131, 5, 1001)])
+@pytest.mark.parametrize("G,N,K", [(64, 8, 1000), (66, 8, 1024), (67, 16, 520), (131, 5, 1001), (1901, 2, 1024)])
 def test_packed_input_in_pieces(G, N, K):
     import torch
     import paper_2605_05802_b200 as sr
