@@ -849,8 +849,16 @@ __device__ __forceinline__ bool arrive_last(int parts, int32_t* arrived) {
 // distance is computed for a group that they settle.
 // kTwoWarps: patterns of more than 512 positions and no more than two texts, a CTA to an SM: a pair has two warps (40
 // groups of 4 texts of 1024: 48 -> 37 us; with four texts the integer pipe is busy already, 16 groups of 8: 46 -> 48).
+// Small batches of fewer threads a CTA than that: no more than 72 registers, or seven CTAs of 128 threads do not fit an SM (301 groups of
+// 5 of 501 at 74 registers 65.3 us, at 72 60.5).
+template <bool kDecide, int kThreads, bool kPairs, bool kOwnNames>
+struct PrepBounds {
+    static constexpr bool kFew = kPairs && !kDecide && !kOwnNames && kThreads == 0;
+    static constexpr int kMost = kThreads > kMostPrepThreads ? kThreads : kFew ? kMostPrepThreads - 32 : kMostPrepThreads;
+    static constexpr int kCtas = kThreads > kMostPrepThreads ? 1 : kFew ? 4 : kPairs ? 3 : 6;
+};
 template <bool kDecide, int kThreads, bool kPairs, bool kOwnNames, bool kTwoWarps = false>
-__global__ void __launch_bounds__(kThreads > kMostPrepThreads ? kThreads : kMostPrepThreads, kThreads > kMostPrepThreads ? 1 : kPairs ? 3 : 6)
+__global__ void __launch_bounds__(PrepBounds<kDecide, kThreads, kPairs, kOwnNames>::kMost, PrepBounds<kDecide, kThreads, kPairs, kOwnNames>::kCtas)
 multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, int g_base, uint8_t* exact, uint32_t inv_row, int table_log,
                   uint32_t two) {
     constexpr bool kCluster = kOwnNames || (kDecide && kPairs);
@@ -866,7 +874,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     __shared__ int s_txt[kMaxTexts], s_len[kMaxTexts], s_cp[kMaxTexts];
     __shared__ uint32_t s_count[kMaxTexts];  // differing positions | absent columns << 16
     __shared__ uint32_t s_flag[kMaxTexts];   // the stream holds row or chain entries
-    __shared__ int s_repeats[4];     // symbols with >= 2, 3, 4 occurrences; mask rows handed out
+    __shared__ int s_repeats[5];     // symbols with >= 2, 3, 4 occurrences; mask rows handed out to frequent ones, asked for by others
 
     const int N = a.N, K = a.K, P = pairs_of(N);
     const int tid = threadIdx.x, lane = tid & 31, nthr = kThreads ? kThreads : blockDim.x, warps = nthr >> 5;
@@ -875,7 +883,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
     int gl = M > 1 ? (int)__umulhi(blockIdx.x, W.inv_patterns) : (int)blockIdx.x;
     if (gl * M > (int)blockIdx.x) --gl;
     const int g = g_base + gl, i = (int)blockIdx.x - gl * M;
-    if (tid < 4) s_repeats[tid] = 0;
+    if (tid < 5) s_repeats[tid] = 0;
     for (int e = tid; 8 * e < N * W.pitch; e += nthr)
         reinterpret_cast<uint4*>(s_map)[e] = make_uint4(kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u, kLocNone * 0x10001u);
     for (int e = tid; 4 * e < W.pitch; e += nthr) reinterpret_cast<uint4*>(s_info)[e] = make_uint4(0u, 0u, 0u, 0u);
@@ -982,7 +990,10 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         // of 8 such texts of 1024 tokens take 165 us, with a quarter of the rows and chains besides 426.)
         // The full pool has room for every symbol with at least eight occurrences; what does not fit
         // (the rarest of the repeated ones) is left as a chain of at most seven positions.  In a
-        // smaller pool (see launch_gate_multi) the last symbols to ask get a chain of any length.
+        // smaller pool (see launch_gate_multi) the last symbols to ask get a chain of any length.  The rows that frequent
+        // symbols leave are handed to others, so that the pool is used up before there is a chain (1024 groups of 8 of 1024
+        // symbols out of 3000, 140 of which repeat in a pattern: 554 -> 416 us where they differ in 2 % of their places, 325 -> 284 diverging;
+        // 438 of diverging texts of 200 71 -> 62).
         // From here on the lower half of s_info[claimant] is the symbol's stream entry, the upper half
         // the head of the chain of its further positions.
         // (only claimants of repeated symbols have a count)
@@ -1015,6 +1026,13 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             int first_row = 0;
             if (lane == 31 && row) first_row = atomicAdd(&s_repeats[3], row);
             row += __shfl_sync(0xFFFFFFFFu, first_row, 31) - asks;
+            int rest = W.row_cap;                      // the others' rows: behind theirs, whoever comes first
+            if (need == 2u || need == 3u) {
+                int others = 0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) others += more[k] > 0u && more[k] < need;
+                if (others) rest = s_repeats[need - 1u] + atomicAdd(&s_repeats[4], others);
+            }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if (more[k] == 0u) continue;
@@ -1022,6 +1040,9 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                 if (more[k] >= need) {
                     if (row < W.row_cap) code = kLocRow | (uint32_t)row;
                     ++row;
+                } else {
+                    if (rest < W.row_cap) code = kLocRow | (uint32_t)rest;
+                    ++rest;
                 }
                 s_map[my_name[k]] = (uint16_t)code;             // what the streams of the texts say
                 s_info[p0 + k] = code;
@@ -1029,7 +1050,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         }
         __syncthreads();
         uint32_t* rows = kPairs ? s_rows : reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * M + i) * W.rows_pitch;
-        const int n_rows = min(s_repeats[3], W.row_cap);
+        const int n_rows = min(s_repeats[3] + s_repeats[4], W.row_cap);
         for (int e = tid; 4 * e < n_rows * W.row_words; e += nthr) {
             reinterpret_cast<uint4*>(rows)[e] = make_uint4(0u, 0u, 0u, 0u);
             if (kPairs) reinterpret_cast<uint4*>(rows + W.rows_pitch)[e] = make_uint4(0u, 0u, 0u, 0u);
@@ -1176,7 +1197,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         }
         __syncthreads();
         // Teams of as many lanes as the pattern has blocks, 16 at the most, and as many pairs to a warp as have room.
-        const bool chains = s_repeats[0] > min(s_repeats[3], W.row_cap);
+        const bool chains = s_repeats[0] > min(s_repeats[3] + s_repeats[4], W.row_cap);
         const uint32_t* turned = s_rows + W.rows_pitch;
         uint4* s_wide = reinterpret_cast<uint4*>(s_map);              // the map is not needed any more
         if constexpr (kTwoWarps) {
@@ -1223,7 +1244,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         bounds(tid, strip, lower, upper);
         PairDesc d{(uint32_t)m | ((uint32_t)n << 16), (uint32_t)(g * M + i), 0u, (uint32_t)lower | ((uint32_t)upper << 16)};
         if (lower < upper) {                          // otherwise that is the distance
-            const int n_rows = min(s_repeats[3], W.row_cap);
+            const int n_rows = min(s_repeats[3] + s_repeats[4], W.row_cap);
             d.bin = ((uint32_t)strip << kStripShift) | ((uint32_t)n_rows << kRowsShift) | kNeedsDp | (s_repeats[0] > n_rows ? kHasChains : 0u);
         }
         descs[idx] = d;
@@ -1950,12 +1971,12 @@ bool names_for_itself(int n_groups, int patterns, int symbols, int sms) {
 
 // Shared memory that keeps more CTAs than its share off every SM.  They start early, on the SMs that the names kernel leaves
 // first, and three of them there take longer than two on every SM (40 groups of 8 texts of 1024: 68 us, 60 with this; an
-// ordinary launch spreads them as well, but costs small batches 2 us).  Not for clusters, which then wait for
+// ordinary launch spreads them as well, but costs small batches 2 us; 500 groups of 3 of 200, eleven CTAs an SM: 33.8, 30.0 with this).  Not for clusters, which then wait for
 // seven SMs of one GPC with that much to spare (40 groups at 512: 33 us, 43 with this).
 int even_smem(long long ctas, int sms) {
     constexpr int kSm = 227 * 1024, kDeclared = 10 * 1024;       // what an SM has; what the kernel declares and the driver adds
     const long long share = (ctas + sms - 1) / sms;
-    return share < 2 || share > 6 ? 0 : kSm / (int)(share + 1) + 1024 - kDeclared;
+    return share < 2 || share > 20 ? 0 : kSm / (int)(share + 1) + 1024 - kDeclared;
 }
 
 // More than 48 KB of shared memory has to be asked for: the most that any call takes, once per device (noted,

@@ -55,3 +55,26 @@ def test_every_number_of_warps_per_pattern(N, K):
     lens[::2] = K
     seqs = seqs.astype(np.int32)
     assert_gate_matches(gate_gpu(seqs, lens, K, 0.4), oracle.gate(seqs, lens, K, 0.4, threads=8), f"N={N} K={K}")
+
+
+@pytest.mark.parametrize("N,G", [(4, 6), (2, 2600)])        # computed in the CTAs of the patterns; sorted into warp tasks
+@pytest.mark.parametrize("K", [40, 200, 1024])
+def test_rows_left_by_frequent_symbols_go_to_others(N, G, K):
+    """Patterns whose repeated symbols just fit the pool of mask rows or exceed it by a few or many, with occurrences of two to
+    five mixed: frequent ones have rows, others take what is left, the last ones are chains."""
+    rng = np.random.default_rng(K + G)
+    cap, stride = (K + 7) // 8, (K + 3) // 4 * 4
+    seqs = np.empty((G, N, stride), dtype=np.int32)
+    for g in range(G if G < 100 else 40):
+        often = [0, 1, cap - 1, cap, cap + 1][g % 5]          # symbols of three to five occurrences, and of two
+        times = np.concatenate([rng.integers(3, 6, size=often), np.full(max(cap + [-1, 0, 1, 3, cap][g % 7 % 5] - often, 0), 2)])
+        times = times[np.cumsum(times) <= K]
+        pool = np.concatenate([np.repeat(np.arange(times.size), times), 10 ** 6 + np.arange(stride)])[:stride]
+        for i in range(N):
+            seqs[g, i] = rng.permutation(pool[:stride])
+        seqs[g, 1:, : K // 3] = np.where(rng.random((N - 1, K // 3)) < 0.9, seqs[g, :1, : K // 3], seqs[g, 1:, : K // 3])
+    for g in range(40, G):
+        seqs[g] = seqs[g % 40]
+    lens = np.full((G, N), K, dtype=np.int32)
+    lens[::3] = rng.integers(K - 7, K + 1, size=lens[::3].shape)
+    assert_gate_matches(gate_gpu(seqs, lens, K, 0.4), oracle.gate(seqs, lens, K, 0.4, threads=8), f"G={G} N={N} K={K}")
