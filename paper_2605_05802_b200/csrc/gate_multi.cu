@@ -327,7 +327,7 @@ __device__ __forceinline__ void name_symbols(const GateArgs& a, int g, const int
 }
 
 __global__ void __launch_bounds__(1024)
-multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int table_log, int g_base, int32_t* arrived) {
+multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int table_log, int g_base, int32_t* arrived, uint4* zero, int n_zero) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_len[SR_MAX_N];
     const int N = a.N, tid = threadIdx.x;
@@ -340,6 +340,8 @@ multi_names_kernel(GateArgs a, uint16_t* names, int pitch, uint32_t inv_row, int
         if (neg && a.status) atomicOr(a.status, SR_STATUS_NEG_LEN);
     }
     if (arrived && tid == 0) arrived[g] = 0;           // see arrive_last
+    if (blockIdx.x == 0)                               // what the kernels add up starts at zero
+        for (int e = tid; e < n_zero; e += blockDim.x) zero[e] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     name_symbols(a, g, s_len, s_sym, reinterpret_cast<uint16_t*>(s_sym + N * pitch), table_log, pitch, inv_row,
                  reinterpret_cast<uint2*>(names + (size_t)g * N * pitch));
@@ -2059,9 +2061,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     }
 
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[0], s));
-    // what the kernels add up starts at zero (one CTA that orders the batch alone needs nothing)
-    const bool alone = W.alone = n_pairs <= kAlonePairs;
-    if (!alone && !in_pairs) SR_CUDA_TRY(cudaMemsetAsync(ctl, 0, offsetof(Ctl, start), s));
+    const bool alone = W.alone = n_pairs <= kAlonePairs;      // one CTA orders the batch, and needs nothing to be zero
+    static_assert(offsetof(Ctl, start) <= sizeof(Ctl) - 16, "the last zeros may reach into `start`, which is written later");
+    int n_zero = alone || in_pairs ? 0 : (int)(offsetof(Ctl, start) + 15) / 16;       // (a launch of its own cost every call 2.5 us)
     uint8_t* flag = decide ? ws + W.off_flag : nullptr;
     // The match-stream pass works group by group, so when the groups arrive in pieces it runs
     // piece by piece: `feed->before` enqueues whatever makes groups [g0, g1) ready on `s`.
@@ -2076,7 +2078,8 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
         }
         if (!own_names)
             SR_LAUNCH("multi_names_kernel", multi_names_kernel, g1 - g0, names_threads, names_smem, s, a, names, W.pitch, inv_row, table_log, g0,
-                  in_pairs ? reinterpret_cast<int32_t*>(ws + W.off_order) : nullptr);
+                  in_pairs ? reinterpret_cast<int32_t*>(ws + W.off_order) : nullptr, reinterpret_cast<uint4*>(ctl), n_zero);
+        n_zero = 0;
         const int cluster = own_names || clusters ? W.patterns : 1;
         const bool most = prep_threads == kMostPrepThreads;
         const auto in_memory = decide ? (most ? multi_prep_kernel<true, kMostPrepThreads, false, false> : multi_prep_kernel<true, 0, false, false>)
