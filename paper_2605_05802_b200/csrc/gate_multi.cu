@@ -2114,10 +2114,8 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     SR_LAUNCH("multi_order_kernel", alone ? multi_order_kernel<true> : multi_order_kernel<false>, order_blocks, kOrderThreads, 0, s, descs, order, ctl, n_pairs, W.warps);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[2], s));
     const int blocks = n_pairs < sms ? n_pairs : sms;
-    // (an ordinary launch unless every CTA has an SM: CTAs made resident while the tail of prep still fills some SMs would
-    // crowd onto the others, 310 us instead of 269 for 1024 groups of uniform tokens when these still took the recurrence)
-    const int rc = launch_as(alone && (n_pairs + 3) / 4 < sms, 1, "multi_dp_kernel", multi_dp_kernel, blocks, kMostDpWarps * 32, 0, s, ws, W, dist, 2u);
-    if (rc != SR_OK) return rc;
+    // (launched early like the others: one of its CTAs has the registers of most of an SM, so that no two can end up on one)
+    SR_LAUNCH("multi_dp_kernel", multi_dp_kernel, blocks, kMostDpWarps * 32, 0, s, ws, W, dist, 2u);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[3], s));
     SR_LAUNCH("multi_finish_kernel", multi_finish_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, dist, flag, exact, gpb);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[4], s));
