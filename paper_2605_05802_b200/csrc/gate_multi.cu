@@ -115,6 +115,7 @@ struct MultiWs {
     int text_warps, text_stride;   // prep: warps to a text, texts that the CTA's warps take at a time
     uint32_t inv_text_warps;       // 2^32 / text_warps, rounded up
     bool alone;            // one CTA orders the batch, and adds up its work itself
+    bool rows_later;       // decide mode: prep leaves only the positions' rows, and multi_bin_kernel makes them for open groups
 };
 
 // Mask rows for an eighth of the positions: symbols with at least eight occurrences always
@@ -130,7 +131,7 @@ MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K, int row_cap) {
     w.text_warps = w.text_stride = 1;
     w.inv_text_warps = 0u;
     w.inv_patterns = (uint32_t)(((1ull << 32) + w.patterns - 1) / w.patterns);
-    w.alone = false;
+    w.alone = w.rows_later = false;
     size_t off = 0;
     w.off_ctl = off;   off = align_up(off + sizeof(Ctl), 256);
     w.off_flag = off;  off = align_up(off + (size_t)n_groups, 256);
@@ -1053,11 +1054,13 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         __syncthreads();
         uint32_t* rows = kPairs ? s_rows : reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * M + i) * W.rows_pitch;
         const int n_rows = min(s_repeats[3] + s_repeats[4], W.row_cap);
-        for (int e = tid; 4 * e < n_rows * W.row_words; e += nthr) {
+        const bool later = kDecide && !kPairs && W.rows_later;
+        for (int e = tid; !later && 4 * e < n_rows * W.row_words; e += nthr) {
             reinterpret_cast<uint4*>(rows)[e] = make_uint4(0u, 0u, 0u, 0u);
             if (kPairs) reinterpret_cast<uint4*>(rows + W.rows_pitch)[e] = make_uint4(0u, 0u, 0u, 0u);
         }
-        __syncthreads();
+        if (!later) __syncthreads();
+        uint32_t my_row[4] = {kLocNone, kLocNone, kLocNone, kLocNone};
         if (claims || repeated) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -1065,6 +1068,8 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                 const uint32_t p = p0 + k, f = my_first[k], info = s_info[f];
                 if ((info & kLocChain) == kLocChain) {
                     if (f != p) s_info[p] = atomicExch(&s_info[f], (p << 16) | kLocChain | f);
+                } else if (later) {
+                    my_row[k] = info & 0xFFFFu;
                 } else {
                     uint32_t* row = rows + (info & 0x3FFFu) * W.row_words;
                     atomicOr(row + (p >> 5), 1u << (p & 31));
@@ -1072,6 +1077,7 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                 }
             }
         }
+        if (later && mine > 0) reinterpret_cast<uint2*>(rows + 4)[tid] = make_uint2(my_row[0] | (my_row[1] << 16), my_row[2] | (my_row[3] << 16));
         if (!kPairs && s_repeats[0] > n_rows) {        // some chains: leave them for the recurrence
             __syncthreads();
             uint16_t* g_next = reinterpret_cast<uint16_t*>(ws + W.off_next) + ((size_t)g * M + i) * W.pitch;
@@ -1235,6 +1241,8 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         return;
     }
     if (tid >= 32) return;                             // descriptors: the texts' threads are in the first warp
+    if (kDecide && W.rows_later && tid == 0)
+        reinterpret_cast<uint32_t*>(ws + W.off_rows)[((size_t)g * M + i) * W.rows_pitch] = (uint32_t)min(s_repeats[3] + s_repeats[4], W.row_cap) | ((uint32_t)m << 16);
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
     int work = 0, few = -1, maybe = -1;
@@ -1327,9 +1335,36 @@ __device__ __forceinline__ ShapeGoal shape_goal(unsigned long long work, int ope
 // Pairs that are not worth it by themselves are looked at if no pair has to go to the recurrence: the batch is then done
 // here as a rule, and the latency of what comes after it is more than they cost (1024 groups of uniform tokens: 122 us, 142
 // without these).  What fails then is shaped as if one in eight did.
+// Decide mode: most groups are dismissed by their bounds before anyone reads a mask row, so prep leaves the rows of their positions
+// (16 bits each, behind the number of rows and positions) where the rows will be, and the other CTAs make those of open groups
+// (1024 groups of 8 texts of 1024 at 0.12: 218.6 -> 210.0 us, of which 156 are open; all settled 106 -> 98; all open 165 -> 169; K <= 256
+// no gain).  From K = 257 on the rows' place has room for the list.
 constexpr int kBinPairs = 32 * kMatchWarps;               // pairs that a CTA bins
+
+// A warp: the mask rows of a pattern in place of its positions' rows.
+__device__ __noinline__ void make_rows(uint32_t* rows, int row_words) {
+    const int lane = threadIdx.x & 31, n_rows = (int)(rows[0] & 0xFFFFu), m = (int)(rows[0] >> 16);
+    constexpr int kTrips = SR_MAX_K / 128;
+    uint2 v[kTrips];
+#pragma unroll
+    for (int t = 0; t < kTrips; ++t) {
+        const int q = lane + 32 * t;
+        v[t] = n_rows > 0 && 4 * q < m ? reinterpret_cast<const uint2*>(rows + 4)[q] : make_uint2(kLocNone * 0x10001u, kLocNone * 0x10001u);
+    }
+    __syncwarp();
+    for (int e = lane; 4 * e < n_rows * row_words; e += 32) reinterpret_cast<uint4*>(rows)[e] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < kTrips; ++t) {
+        const uint32_t row[4] = {v[t].x & 0xFFFFu, v[t].x >> 16, v[t].y & 0xFFFFu, v[t].y >> 16};
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (row[k] >= kLocRow) atomicOr(rows + (row[k] & 0x3FFFu) * row_words + ((lane + 32 * t) >> 3), 1u << ((4 * (lane + 32 * t) + k) & 31));
+    }
+}
+
 __global__ void __launch_bounds__(32 * kMatchWarps, 5)
-multi_bin_kernel(unsigned char* ws, MultiWs W, int N, int n_pairs, int bin_blocks, int32_t* dist_out) {
+multi_bin_kernel(unsigned char* ws, MultiWs W, int N, int n_pairs, int bin_blocks, int32_t* dist_out, int row_patterns) {
     grid_begin();
     PairDesc* descs = reinterpret_cast<PairDesc*>(ws + W.off_desc);
     Ctl* ctl = reinterpret_cast<Ctl*>(ws + W.off_ctl);
@@ -1362,6 +1397,15 @@ multi_bin_kernel(unsigned char* ws, MultiWs W, int N, int n_pairs, int bin_block
     __shared__ uint4 s_differ[kMatchWarps][kSpans];
     __shared__ uint32_t s_entries[kMatchWarps][kMostMatches];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, P = pairs_of(N);
+    if (W.rows_later) {
+        if (!any) return;
+        for (int p = ((int)blockIdx.x - bin_blocks) * kMatchWarps + warp; p < row_patterns; p += ((int)gridDim.x - bin_blocks) * kMatchWarps) {
+            int g = W.patterns > 1 ? (int)__umulhi((uint32_t)p, W.inv_patterns) : p;
+            if (g * W.patterns > p) --g;
+            if ((ws + W.off_flag)[g]) make_rows(reinterpret_cast<uint32_t*>(ws + W.off_rows) + (size_t)p * W.rows_pitch, W.row_words);
+        }
+        return;
+    }
     const int32_t* list = reinterpret_cast<const int32_t*>(ws + W.off_order);
     const int few = ctl->few, all = few + (any ? 0 : ctl->maybe);
     for (int e = ((int)blockIdx.x - bin_blocks) * kMatchWarps + warp; e < all; e += ((int)gridDim.x - bin_blocks) * kMatchWarps) {
@@ -2062,6 +2106,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
 
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[0], s));
     const bool alone = W.alone = n_pairs <= kAlonePairs;      // one CTA orders the batch, and needs nothing to be zero
+    const bool mask_only = decide && !a.pair_dist && !a.pair_sum && !a.mean && !exact;
+    // (with d_K wanted the groups that upper bounds would settle stay open too: 256 groups that differ in 1 % of their places 137 us, 143 so)
+    W.rows_later = mask_only && !alone && !in_pairs && a.K > 256;
     static_assert(offsetof(Ctl, start) <= sizeof(Ctl) - 16, "the last zeros may reach into `start`, which is written later");
     int n_zero = alone || in_pairs ? 0 : (int)(offsetof(Ctl, start) + 15) / 16;       // (a launch of its own cost every call 2.5 us)
     uint8_t* flag = decide ? ws + W.off_flag : nullptr;
@@ -2109,8 +2156,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     }
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[1], s));
     const int order_blocks = alone ? 1 : (n_pairs + kOrderThreads - 1) / kOrderThreads;
-    const int bin_blocks = (n_pairs + kBinPairs - 1) / kBinPairs, match_blocks = decide ? 0 : min((n_pairs + kMatchWarps - 1) / kMatchWarps, 16 * sms);
-    if (!alone) SR_LAUNCH("multi_bin_kernel", multi_bin_kernel, bin_blocks + match_blocks, 32 * kMatchWarps, 0, s, ws, W, a.N, n_pairs, bin_blocks, dist);
+    const int bin_blocks = (n_pairs + kBinPairs - 1) / kBinPairs, match_blocks = decide ? (W.rows_later ? min((a.n_groups * W.patterns + kMatchWarps - 1) / kMatchWarps, 8 * sms) : 0)
+                                                                               : min((n_pairs + kMatchWarps - 1) / kMatchWarps, 16 * sms);
+    if (!alone) SR_LAUNCH("multi_bin_kernel", multi_bin_kernel, bin_blocks + match_blocks, 32 * kMatchWarps, 0, s, ws, W, a.N, n_pairs, bin_blocks, dist, a.n_groups * W.patterns);
     SR_LAUNCH("multi_order_kernel", alone ? multi_order_kernel<true> : multi_order_kernel<false>, order_blocks, kOrderThreads, 0, s, descs, order, ctl, n_pairs, W.warps);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[2], s));
     const int blocks = n_pairs < sms ? n_pairs : sms;
