@@ -8,7 +8,7 @@ import oracle
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("G,N,K,vocab", [(40, 8, 300, 40), (25, 5, 520, 2000), (30, 2, 70, 9), (12, 16, 200, 60), (70, 11, 90, 300), (300, 8, 260, 500)])
+@pytest.mark.parametrize("G,N,K,vocab", [(40, 8, 300, 40), (25, 5, 520, 2000), (30, 2, 70, 9), (12, 16, 200, 60), (70, 11, 90, 300), (300, 8, 260, 500), (62, 8, 1000, 3000), (900, 2, 600, 300)])
 def test_mask_alone(G, N, K, vocab):
     import torch
     import paper_2605_05802_b200 as sr
