@@ -854,8 +854,8 @@ __device__ __forceinline__ bool arrive_last(int parts, int32_t* arrived) {
 // groups of 4 texts of 1024: 48 -> 37 us; with four texts the integer pipe is busy already, 16 groups of 8: 46 -> 48).
 // Small batches of fewer threads a CTA than that: no more than 72 registers, or seven CTAs of 128 threads do not fit an SM (301 groups of
 // 5 of 501 at 74 registers 65.3 us, at 72 60.5).
-// Large batches: seven CTAs of 256 threads an SM (36 registers), whose barriers then cost less (1024 groups of uniform tokens of up to
-// 1024 with five 115.2 us, six 109.9, seven 105.0, eight 105.0).
+// Large batches: room for seven CTAs of 256 threads an SM at least (32 registers, which leave room for eight), whose barriers then cost
+// less (1024 groups of uniform tokens of up to 1024 with five 115.2 us, six 109.9, seven 105.0, eight 105.0).
 template <bool kDecide, int kThreads, bool kPairs, bool kOwnNames>
 struct PrepBounds {
     static constexpr bool kFew = kPairs && !kDecide && !kOwnNames && kThreads == 0;
