@@ -836,6 +836,20 @@ __device__ __forceinline__ bool arrive_last(int parts, int32_t* arrived) {
     return s_last;
 }
 
+// Mask rows that frequent symbols leave, for those of a thread's four with fewer occurrences: behind theirs, whoever comes first.
+// (Not inlined: few patterns need it.)
+__device__ __noinline__ void hand_out_rest(uint4 more, uint2 names, uint32_t need, int* repeats, int row_cap, uint16_t* map, uint32_t* info) {
+    const uint32_t m[4] = {more.x, more.y, more.z, more.w}, name[4] = {names.x & 0xFFFFu, names.x >> 16, names.y & 0xFFFFu, names.y >> 16};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (m[k] == 0u || m[k] >= need) continue;
+        const int row = repeats[need - 1u] + atomicAdd(repeats + 4, 1);
+        if (row >= row_cap) continue;
+        map[name[k]] = (uint16_t)(kLocRow | (uint32_t)row);
+        info[k] = kLocRow | (uint32_t)row;
+    }
+}
+
 // One CTA per pattern.  Per text it also counts the columns whose symbol does not occur in the
 // pattern at all and the positions at which text and pattern differ: bounds of the pair's distance that
 // cost next to nothing here.  Where they meet the pair is done.
@@ -1031,13 +1045,6 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
             int first_row = 0;
             if (lane == 31 && row) first_row = atomicAdd(&s_repeats[3], row);
             row += __shfl_sync(0xFFFFFFFFu, first_row, 31) - asks;
-            int rest = W.row_cap;                      // the others' rows: behind theirs, whoever comes first
-            if (need == 2u || need == 3u) {
-                int others = 0;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) others += more[k] > 0u && more[k] < need;
-                if (others) rest = s_repeats[need - 1u] + atomicAdd(&s_repeats[4], others);
-            }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if (more[k] == 0u) continue;
@@ -1045,13 +1052,13 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                 if (more[k] >= need) {
                     if (row < W.row_cap) code = kLocRow | (uint32_t)row;
                     ++row;
-                } else {
-                    if (rest < W.row_cap) code = kLocRow | (uint32_t)rest;
-                    ++rest;
                 }
                 s_map[my_name[k]] = (uint16_t)code;             // what the streams of the texts say
                 s_info[p0 + k] = code;
             }
+            if (need == 2u || need == 3u)
+                hand_out_rest(make_uint4(more[0], more[1], more[2], more[3]), make_uint2(my_name[0] | (my_name[1] << 16), my_name[2] | (my_name[3] << 16)),
+                              need, s_repeats, W.row_cap, s_map, s_info + p0);
         }
         __syncthreads();
         uint32_t* rows = kPairs ? s_rows : reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * M + i) * W.rows_pitch;
