@@ -37,27 +37,38 @@ void note_cuda_error(cudaError_t e, const char* where);
 // which between two dependent kernels of a few microseconds is most of the time (advantages of
 // ten groups, one call after the other: 4.1 -> 2.8 us; an incremental step: 6.1 -> 3.5 us).  Every kernel
 // launched this way calls grid_begin() first, in every thread, so that the completion of a
-// kernel implies that of all before it.  (early = false: an ordinary launch, for a persistent
-// kernel whose CTAs must spread evenly over SMs that the kernel before it no longer occupies.)
+// kernel implies that of all before it.  (early = false: an ordinary launch, for a kernel whose CTAs must spread
+// evenly over SMs that the kernel before it no longer occupies.)
+// most_l1: the kernel needs L1 rather than shared memory.  An SM changes the split of the two only while it is empty, which
+// in a chain of early launches it never is: without this the kernel runs with what those before it left.
+struct LaunchHow {
+    bool early = true;
+    int cluster = 1;
+    bool most_l1 = false;
+};
 template <typename... Params, typename... Args>
-int launch_as(bool early, int cluster, const char* name, void (*kernel)(Params...), int blocks, int threads, size_t smem,
-              cudaStream_t s, Args... args) {
+int launch_how(LaunchHow how, const char* name, void (*kernel)(Params...), int blocks, int threads, size_t smem,
+               cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     cfg.attrs = attr;
-    if (early) {
+    if (how.early) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
     }
-    if (cluster > 1) {
+    if (how.cluster > 1) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
-        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)cluster;
+        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)how.cluster;
         attr[cfg.numAttrs].val.clusterDim.y = 1;
         attr[cfg.numAttrs++].val.clusterDim.z = 1;
+    }
+    if (how.most_l1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[cfg.numAttrs++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxL1;
     }
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
     if (e != cudaSuccess) {
@@ -68,9 +79,14 @@ int launch_as(bool early, int cluster, const char* name, void (*kernel)(Params..
     return SR_OK;
 }
 template <typename... Params, typename... Args>
+int launch_as(bool early, int cluster, const char* name, void (*kernel)(Params...), int blocks, int threads, size_t smem,
+              cudaStream_t s, Args... args) {
+    return launch_how(LaunchHow{early, cluster, false}, name, kernel, blocks, threads, smem, s, args...);
+}
+template <typename... Params, typename... Args>
 int launch(const char* name, void (*kernel)(Params...), int blocks, int threads, size_t smem, cudaStream_t s,
            Args... args) {
-    return launch_as(true, 1, name, kernel, blocks, threads, smem, s, args...);
+    return launch_how(LaunchHow{}, name, kernel, blocks, threads, smem, s, args...);
 }
 #define SR_LAUNCH(...)                                      \
     do {                                                    \

@@ -2171,8 +2171,11 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     SR_LAUNCH("multi_order_kernel", alone ? multi_order_kernel<true> : multi_order_kernel<false>, order_blocks, kOrderThreads, 0, s, descs, order, ctl, n_pairs, W.warps);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[2], s));
     const int blocks = n_pairs < sms ? n_pairs : sms;
-    // (launched early like the others: one of its CTAs has the registers of most of an SM, so that no two can end up on one)
-    SR_LAUNCH("multi_dp_kernel", multi_dp_kernel, blocks, kMostDpWarps * 32, 0, s, ws, W, dist, 2u);
+    // (launched early like the others: one of its CTAs has the registers of most of an SM, so that no two can end up on one.  With the L1
+    // that prep left, 1024 groups of 8 texts of 1024 over 100 symbols that differ in 2 % of their places took 973 us in the decide mode with d_K, 352 with
+    // all of it; a launch that waits for empty SMs costs every sorted call 2.5 us)
+    const int rc = launch_how(LaunchHow{true, 1, true}, "multi_dp_kernel", multi_dp_kernel, blocks, kMostDpWarps * 32, 0, s, ws, W, dist, 2u);
+    if (rc != SR_OK) return rc;
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[3], s));
     SR_LAUNCH("multi_finish_kernel", multi_finish_kernel, (a.n_groups + gpb - 1) / gpb, kGroupThreads, 0, s, a, dist, flag, exact, gpb);
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[4], s));
