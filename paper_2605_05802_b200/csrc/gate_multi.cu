@@ -101,6 +101,7 @@ struct Ctl {               // control block in the workspace
     int32_t task_start[kNumBins + 1];          // first warp task of every bin
     int32_t task_counter;
     int32_t total_tasks;
+    int32_t alike;                             // whether the tasks take about as long each: no less than 0.6 of the longest on average
 };
 
 struct MultiWs {
@@ -242,6 +243,7 @@ __device__ inline int bin_of_shape(const Shape& s) {
     const int bucket = min(max((int)(10.5f * (15.2f - __log2f((float)s.time))), 0), kTimeBuckets - 1);
     return bucket * kNumClasses + class_of(s.tlog, s.R);
 }
+__device__ inline float time_of_bucket(int bucket) { return exp2f(15.2f - (float)bucket / 10.5f); }
 
 // The pair of a descriptor, rows and columns extended to whole quads.
 struct PairSize { int m, n, lb, ub; };
@@ -1452,6 +1454,14 @@ multi_bin_kernel(unsigned char* ws, MultiWs W, int N, int n_pairs, int bin_block
     }
 }
 
+__device__ __forceinline__ void sum_and_max(float& sum, float& most) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
+        most = fmaxf(most, __shfl_xor_sync(0xFFFFFFFFu, most, d));
+    }
+}
+
 // Counting sort of the pairs by bin: longest warp tasks first, one team shape and similar
 // text lengths per bin.  Every CTA turns the bin counts into bin starts by itself (a scan
 // of kNumBins values costs less than a launch) and places kOrderThreads pairs; the first CTA
@@ -1464,6 +1474,7 @@ multi_order_kernel(PairDesc* descs, int32_t* order, Ctl* ctl, int n_pairs, int w
     __shared__ int s_part[32];
     __shared__ int32_t s_start[kNumBins], s_hist[kNumBins];
     __shared__ unsigned long long s_work;
+    __shared__ float s_time[32], s_longest[32];
     __shared__ int s_open;
     const int t = threadIdx.x;
     constexpr int kPer = kAlone ? kAlonePairs / kOrderThreads : 1;
@@ -1521,23 +1532,37 @@ multi_order_kernel(PairDesc* descs, int32_t* order, Ctl* ctl, int n_pairs, int w
     if (kAlone || blockIdx.x == 0) {
         // warp tasks per bin (32 / T pairs per task), exclusive prefix over the bins
         int tasks[2];
+        float time = 0.0f, longest = 0.0f;
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             int tl, rr;
             shape_of_class((2 * t + k) % kNumClasses, tl, rr);
             const int tpw = 32 >> tl;
             tasks[k] = (own[k] + tpw - 1) >> (5 - tl);
+            if (tasks[k] == 0) continue;
+            const float each = time_of_bucket((2 * t + k) / kNumClasses);
+            time += each * (float)tasks[k];
+            longest = fmaxf(longest, each);
         }
+        // (in a fixed order: the same batch is run the same way every time)
+        sum_and_max(time, longest);
+        if ((t & 31) == 0) { s_time[t >> 5] = time; s_longest[t >> 5] = longest; }
         const int task_start = block_exclusive_scan(tasks[0] + tasks[1], s_part);
         ctl->start[2 * t] = start;
         ctl->start[2 * t + 1] = start + own[0];
         ctl->task_start[2 * t] = task_start;
         ctl->task_start[2 * t + 1] = task_start + tasks[0];
         if (kAlone) { ctl->hist[2 * t] = own[0]; ctl->hist[2 * t + 1] = own[1]; }
+        if (t >= kOrderThreads - 32) {
+            time = s_time[t & 31];
+            longest = s_longest[t & 31];
+            sum_and_max(time, longest);
+        }
         if (t == kOrderThreads - 1) {
             ctl->task_start[kNumBins] = task_start + tasks[0] + tasks[1];
             ctl->total_tasks = task_start + tasks[0] + tasks[1];
             ctl->task_counter = 0;
+            ctl->alike = time >= 0.6f * longest * (float)(task_start + tasks[0] + tasks[1]);
         }
     }
     if (!kAlone) {
@@ -1805,14 +1830,29 @@ __device__ __noinline__ void dp_task(int tlog, int pos, bool valid, const PairDe
     if (valid && lt == 0) dist_out[idx] = ring && acc > ub ? ((ub + 1) | kCappedFlag) : acc;
 }
 
+// Time of `total` tasks that all take as long, in tenths of what one takes of a scheduler's pipe, with so many warps a scheduler:
+// full rounds, and what is left, evenly over the schedulers, of which one or two warps do not keep the pipe busy (1024 x 1024
+// places on eight lanes of four blocks: four warps on a scheduler 248 us, three 187, two 131, one 96).
+__device__ __forceinline__ int rounds_cost(int total, int schedulers, int warps) {
+    const int round = schedulers * warps, left = (total % round + schedulers - 1) / schedulers;
+    return 10 * (total / round * warps + left) + (left == 1 ? 6 : left == 2 ? 3 : 0);
+}
+
 // One CTA an SM, whose warps take the bins' warp tasks, longest first.  The first tasks are dealt out, four to an SM, then four
 // more, so that every scheduler has the same number to within one, and neighbours, which run the same code on the same rows,
 // are on one SM; the others are pulled.  (All of them pulled, by three CTAs of four warps, up to three ended up on one
 // scheduler and none on others: decide mode at 0.12, 1024 groups of 8 texts of 1024, 1044 tasks, 234 -> 219 us; with
-// twelve warps the 1796 tasks of 1024 groups over 3000 symbols took two rounds, 671 -> 550 us.)  Sixteen warps where they hold all
-// tasks, and where there are more than twice as many; in between, where few rounds end in a tail that is the longer the
-// more warps share a scheduler, twelve (1024 groups of diverging ragged texts, 4148 tasks: 299 us, 331 with sixteen; 6000 of 256 over
-// 100 symbols, 10495 tasks, 806 and 739).
+// twelve warps the 1796 tasks of 1024 groups over 3000 symbols took two rounds, 671 -> 550 us.)
+// Sixteen warps where they hold all tasks.  Where there are more and they take about as long each, twelve or sixteen by
+// rounds_cost, sixteen in doubt, for more of them hide more of the trips for rows (7000 groups of 256 over 100 symbols 876 us, 974 with twelve;
+// 3000 of uniform tokens with 5 % edits, three rounds of twelve, 240 and 260).  Where they do not, twelve up to twice as many tasks, where few
+// rounds end in a tail that is the longer the more warps share a scheduler (1024 groups of diverging ragged texts, 4148 tasks: 299 us, 331 with
+// sixteen), sixteen above (6000 of 256 over 100 symbols, 10495 tasks, 806 and 739).
+// Tasks that take as long: an SM's warps end a round together, and the first of them to ask took the whole next one, three
+// tasks to one scheduler and none to others.  No scheduler has more than its share of the last round (400 groups of 8 uniform
+// rollouts of 1024 with inserted and deleted tokens, 2802 tasks: 419 -> 370 us; 700 of texts with 2 % edits, 4906 tasks, 714 -> 648).
+// (Over 30 shapes and nine kinds of batch 0.988 of the time without this, at worst 1.03 times it.  The order of
+// tasks dealt out to the end, with no pulling: texts 5 to 8 % slower.)
 __global__ void __launch_bounds__(kMostDpWarps * 32, 1)
 multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
     grid_begin();
@@ -1825,14 +1865,35 @@ multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
     const int lane = threadIdx.x & 31;
     const int total = ctl->total_tasks;
     const int warp = (int)(threadIdx.x >> 5), most = kMostDpWarps * (int)gridDim.x;
-    const bool at_once = total <= most, fewer = !at_once && total <= 2 * most;
+    const bool at_once = total <= most;
+    const bool fewer = !at_once && (ctl->alike ? 23 * rounds_cost(total, 4 * (int)gridDim.x, kDpWarps / 4) < 22 * rounds_cost(total, 4 * (int)gridDim.x, kMostDpWarps / 4)
+                                               : total <= 2 * most);
+    __shared__ int s_last, s_share, s_taken[4];       // first task of the last round, a scheduler's share of it and what each has had
+    if (threadIdx.x == 0) {
+        const int round = (fewer ? kDpWarps : kMostDpWarps) * (int)gridDim.x, left = ctl->alike ? total % round : 0;
+        s_last = total - left;
+        s_share = (left + 4 * (int)gridDim.x - 1) / (4 * (int)gridDim.x);
+        for (int k = 0; k < 4; ++k) s_taken[k] = 0;
+    }
+    __syncthreads();
     if (fewer && warp >= kDpWarps) return;
     const int dealt = (fewer ? kDpWarps : kMostDpWarps) * (int)gridDim.x;
-    for (int round = 0;; ++round) {                   // (with the task kept from round to round the recurrence comes out 10 % slower)
+    // (Written like this on purpose: with the task kept from round to round, without a shuffle in the first one, or with the pulling
+    // in a function of its own the recurrence itself comes out 10 % slower.)
+    for (int round = 0;; ++round) {
         int task = 0;
         if (round == 0) task = 4 * ((int)blockIdx.x + (int)gridDim.x * (warp >> 2)) + (warp & 3);
         else if (at_once) task = total;
-        else if (lane == 0) task = dealt + atomicAdd(&ctl->task_counter, 1);
+        else if (lane == 0) {
+            // A scheduler that has had its share has done with the rest; the shares add up to no less than the round, and whoever has some
+            // left comes back, so that every task is pulled.  (A task of the last round that is met unawares counts as well.)
+            const bool ends = s_last < total && dealt + *reinterpret_cast<volatile int32_t*>(&ctl->task_counter) >= s_last;
+            task = total;
+            if (!ends || atomicAdd(&s_taken[warp & 3], 1) < s_share) {
+                task = dealt + atomicAdd(&ctl->task_counter, 1);
+                if (!ends && task >= s_last) atomicAdd(&s_taken[warp & 3], 1);
+            }
+        }
         task = __shfl_sync(0xFFFFFFFFu, task, 0);
         if (task >= total) break;
         int k = 0, hi = kNumBins;                     // last bin whose first task is <= task
