@@ -62,6 +62,7 @@ constexpr int kTextThreads = 16 * SR_MAX_N;  // a warp for every text of a patte
 static_assert(4 * kMostPrepThreads >= SR_MAX_K, "");
 constexpr int kNumClasses = 21;     // team shapes (T lanes x R blocks), see class_of
 constexpr int kTimeBuckets = 96;    // buckets of estimated task duration
+constexpr float kLongTask = 2000.0f;  // tasks that last longer than it takes to see who is due for one, see multi_dp_kernel
 constexpr int kNumBins = 2048;      // kTimeBuckets * kNumClasses of them used
 constexpr int kOrderThreads = 1024;
 constexpr int kAlonePairs = 1024;   // batches of up to this many pairs are ordered by one CTA
@@ -1562,7 +1563,7 @@ multi_order_kernel(PairDesc* descs, int32_t* order, Ctl* ctl, int n_pairs, int w
             ctl->task_start[kNumBins] = task_start + tasks[0] + tasks[1];
             ctl->total_tasks = task_start + tasks[0] + tasks[1];
             ctl->task_counter = 0;
-            ctl->alike = time >= 0.6f * longest * (float)(task_start + tasks[0] + tasks[1]);
+            ctl->alike = longest >= kLongTask && time >= 0.6f * longest * (float)(task_start + tasks[0] + tasks[1]);
         }
     }
     if (!kAlone) {
