@@ -59,6 +59,7 @@ namespace {
 
 constexpr int kMostPrepThreads = 256;      // a thread for every four positions of a pattern
 constexpr int kTextThreads = 16 * SR_MAX_N;  // a warp for every text of a pattern
+constexpr int kTwoWarpThreads = 64;
 static_assert(4 * kMostPrepThreads >= SR_MAX_K, "");
 constexpr int kNumClasses = 21;     // team shapes (T lanes x R blocks), see class_of
 constexpr int kTimeBuckets = 96;    // buckets of estimated task duration
@@ -123,6 +124,10 @@ struct MultiWs {
 // Mask rows for an eighth of the positions: symbols with at least eight occurrences always
 // fit, and 1/rank token frequencies put no more than about K / 10 symbols above one.
 int full_row_cap(int32_t K) { return (K + 7) >> 3; }
+// Prefixes from which rows that frequent symbols leave are handed to others in groups of four and five, whose rows serve two texts: below, chains cost those
+// few columns no more than the rows cost prep (20000 groups of 4 of 64 over 100 symbols 235 us with them, 222 without, texts alike; 6000 of texts of 256
+// 114 and 120).  In groups of eight they pay from the start (12000 of 48 1 %).
+constexpr int kHandOut = 97;
 
 MultiWs multi_layout(int32_t n_groups, int32_t N, int32_t K, int row_cap) {
     MultiWs w;
@@ -840,8 +845,7 @@ __device__ __forceinline__ bool arrive_last(int parts, int32_t* arrived) {
 }
 
 // Mask rows that frequent symbols leave, for those of a thread's four with fewer occurrences: behind theirs, whoever comes first.
-// (Not inlined: few patterns need it.)
-__device__ __noinline__ void hand_out_rest(uint4 more, uint2 names, uint32_t need, int* repeats, int row_cap, uint16_t* map, uint32_t* info) {
+__device__ __forceinline__ void hand_out_rest(uint4 more, uint2 names, uint32_t need, int* repeats, int row_cap, uint16_t* map, uint32_t* info) {
     const uint32_t m[4] = {more.x, more.y, more.z, more.w}, name[4] = {names.x & 0xFFFFu, names.x >> 16, names.y & 0xFFFFu, names.y >> 16};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -851,6 +855,10 @@ __device__ __noinline__ void hand_out_rest(uint4 more, uint2 names, uint32_t nee
         map[name[k]] = (uint16_t)(kLocRow | (uint32_t)row);
         info[k] = kLocRow | (uint32_t)row;
     }
+}
+// (Where registers are what limits the CTAs of an SM: few patterns need it.  Inlined, decide mode takes 1 % longer; not inlined, the gate up to 3.)
+__device__ __noinline__ void hand_out_rest_apart(uint4 more, uint2 names, uint32_t need, int* repeats, int row_cap, uint16_t* map, uint32_t* info) {
+    hand_out_rest(more, names, need, repeats, row_cap, map, info);
 }
 
 // One CTA per pattern.  Per text it also counts the columns whose symbol does not occur in the
@@ -872,12 +880,14 @@ __device__ __noinline__ void hand_out_rest(uint4 more, uint2 names, uint32_t nee
 // Small batches of fewer threads a CTA than that: no more than 72 registers, or seven CTAs of 128 threads do not fit an SM (301 groups of
 // 5 of 501 at 74 registers 65.3 us, at 72 60.5).
 // Large batches: room for seven CTAs of 256 threads an SM at least (32 registers, which leave room for eight), whose barriers then cost
-// less (1024 groups of uniform tokens of up to 1024 with five 115.2 us, six 109.9, seven 105.0, eight 105.0).
+// less (1024 groups of uniform tokens of up to 1024 with five 115.2 us, six 109.9, seven 105.0, eight 105.0).  CTAs of four warps gain as
+// well (8000 groups of 8 of 64 4 % over six), those of two lose more by 32 registers, spilled, than by fewer of them (20000 groups of 4 of 64
+// over 100 symbols 242 us, 233 with 48).
 template <bool kDecide, int kThreads, bool kPairs, bool kOwnNames>
 struct PrepBounds {
     static constexpr bool kFew = kPairs && !kDecide && !kOwnNames && kThreads == 0;
-    static constexpr int kMost = kThreads > kMostPrepThreads ? kThreads : kFew ? kMostPrepThreads - 32 : kMostPrepThreads;
-    static constexpr int kCtas = kThreads > kMostPrepThreads ? 1 : kFew ? 4 : kPairs ? 3 : 7;
+    static constexpr int kMost = kThreads ? kThreads : kFew ? kMostPrepThreads - 32 : kMostPrepThreads;
+    static constexpr int kCtas = kThreads > kMostPrepThreads ? 1 : kFew ? 4 : kPairs ? 3 : kThreads == kTwoWarpThreads ? 20 : 7;
 };
 template <bool kDecide, int kThreads, bool kPairs, bool kOwnNames, bool kTwoWarps = false>
 __global__ void __launch_bounds__(PrepBounds<kDecide, kThreads, kPairs, kOwnNames>::kMost, PrepBounds<kDecide, kThreads, kPairs, kOwnNames>::kCtas)
@@ -1059,9 +1069,11 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
                 s_map[my_name[k]] = (uint16_t)code;             // what the streams of the texts say
                 s_info[p0 + k] = code;
             }
-            if (need == 2u || need == 3u)
-                hand_out_rest(make_uint4(more[0], more[1], more[2], more[3]), make_uint2(my_name[0] | (my_name[1] << 16), my_name[2] | (my_name[3] << 16)),
-                              need, s_repeats, W.row_cap, s_map, s_info + p0);
+            if ((need == 2u || need == 3u) && (kThreads != kTwoWarpThreads || K >= kHandOut)) {
+                constexpr auto hand_out = kPairs || kDecide ? hand_out_rest_apart : hand_out_rest;
+                hand_out(make_uint4(more[0], more[1], more[2], more[3]), make_uint2(my_name[0] | (my_name[1] << 16), my_name[2] | (my_name[3] << 16)),
+                         need, s_repeats, W.row_cap, s_map, s_info + p0);
+            }
         }
         __syncthreads();
         uint32_t* rows = kPairs ? s_rows : reinterpret_cast<uint32_t*>(ws + W.off_rows) + ((size_t)g * M + i) * W.rows_pitch;
@@ -2200,8 +2212,9 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
         n_zero = 0;
         const int cluster = own_names || clusters ? W.patterns : 1;
         const bool most = prep_threads == kMostPrepThreads;
-        const auto in_memory = decide ? (most ? multi_prep_kernel<true, kMostPrepThreads, false, false> : multi_prep_kernel<true, 0, false, false>)
-                                      : (most ? multi_prep_kernel<false, kMostPrepThreads, false, false> : multi_prep_kernel<false, 0, false, false>);
+        const bool two_warps = prep_threads == kTwoWarpThreads;
+        const auto in_memory = decide ? (two_warps ? multi_prep_kernel<true, kTwoWarpThreads, false, false> : most ? multi_prep_kernel<true, kMostPrepThreads, false, false> : multi_prep_kernel<true, 0, false, false>)
+                                      : (two_warps ? multi_prep_kernel<false, kTwoWarpThreads, false, false> : most ? multi_prep_kernel<false, kMostPrepThreads, false, false> : multi_prep_kernel<false, 0, false, false>);
         const auto pairs = decide ? (most ? multi_prep_kernel<true, kMostPrepThreads, true, false> : multi_prep_kernel<true, 0, true, false>)
                                   : (most ? multi_prep_kernel<false, kMostPrepThreads, true, false> : multi_prep_kernel<false, 0, true, false>);
         const auto alone_pairs = decide ? (most ? multi_prep_kernel<true, kMostPrepThreads, true, true> : multi_prep_kernel<true, 0, true, true>)
