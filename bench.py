@@ -373,7 +373,8 @@ def main():
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "ms_per_step": e2e_ms / args.steps,
                 "input": "packed prefixes + int64 row offsets in pinned host memory (sr_gate_host_packed), "
-                         "sent in pieces on a copy stream under the per-group pass, and gated in two halves"},
+                         "sent in pieces on a copy stream under the per-group pass"
+                         + (", and gated in two halves" if h_sym.numel() * 4 >= 14 << 20 else "")},
         "gpu_launches": (7 if args.groups >= 512 else 2) * args.steps,       # names, prep, bin, order, dp, finish; advantages (smaller batches: two at the least)
         "clocks": clocks,
         "stage_ms": {"prep": stage_ms[0], "order": stage_ms[1], "dp": stage_ms[2], "finish": stage_ms[3]},

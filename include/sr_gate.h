@@ -189,10 +189,12 @@ size_t sr_gate_host_arena_bytes(int32_t n_groups, int32_t N, int32_t stride, int
  *                  all lengths must not exceed n_groups * N * stride
  *   outputs, status, stream: as for sr_gate_host (HOST pointers)
  *   copy_stream    a second cudaStream_t, or NULL.  When given (and different from `stream`,
- *                  K > 32, at least 64 groups and 2 MiB of symbols) they are sent on it in four
+ *                  K > 32, at least 64 groups and 2 MiB of symbols) they are sent on it in
  *                  pieces of whole groups, and the gate's per-group pass runs on each piece while the
- *                  next one is still on the link; the recurrence runs once over the whole
- *                  batch.  Outputs arrive on `stream`, the only stream to synchronise.  This
+ *                  next one is still on the link: four pieces, after which the recurrence runs once
+ *                  over the whole batch, or, from 14 MiB of symbols on, two of the first half and
+ *                  one of the second, each half gated as a batch of its own, one after the other
+ *                  in the same scratch.  Outputs arrive on `stream`, the only stream to synchronise.  This
  *                  path creates and releases a few CUDA events per call (no device memory).
  *   arena          DEVICE scratch of sr_gate_host_packed_arena_bytes(...) bytes, 256-byte
  *                  aligned

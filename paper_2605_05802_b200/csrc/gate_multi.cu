@@ -23,7 +23,7 @@
 //   order    counting sort of the pairs by bin: longest warp tasks first, one team
 //            shape and similar durations per bin; warp-task table.  (One launch does both for
 //            batches of up to a thousand pairs.)
-//   dp       persistent warps pull tasks.  A task is a warp of 32/T teams; a team of
+//   dp       one CTA an SM; its warps are dealt their first tasks and pull the others.  A task is a warp of 32/T teams; a team of
 //            T lanes owns one pair, a lane holding R <= 4 consecutive blocks (32*R rows) in
 //            registers.  Lanes are skewed by four columns; the
 //            delta bits of a lane's last block reach the next lane by warp shuffles.
@@ -1022,10 +1022,11 @@ multi_prep_kernel(GateArgs a, unsigned char* ws, MultiWs W, int32_t* dist_out, i
         // of 8 such texts of 1024 tokens take 165 us, with a quarter of the rows and chains besides 426.)
         // The full pool has room for every symbol with at least eight occurrences; what does not fit
         // (the rarest of the repeated ones) is left as a chain of at most seven positions.  In a
-        // smaller pool (see launch_gate_multi) the last symbols to ask get a chain of any length.  The rows that frequent
-        // symbols leave are handed to others, so that the pool is used up before there is a chain (1024 groups of 8 of 1024
+        // smaller pool (see launch_gate_multi) the last symbols to ask get a chain of any length.  Where the rows suffice for all symbols
+        // of three or of four occurrences, what these leave is handed to others (1024 groups of 8 of 1024
         // symbols out of 3000, 140 of which repeat in a pattern: 554 -> 416 us where they differ in 2 % of their places, 325 -> 284 diverging;
-        // 438 of diverging texts of 200 71 -> 62).
+        // 438 of diverging texts of 200 71 -> 62).  Where they do not, the rows that symbols of eight leave stay empty, and the others are chains
+        // (1024 positions of 150 to 300 equally frequent symbols).
         // From here on the lower half of s_info[claimant] is the symbol's stream entry, the upper half
         // the head of the chain of its further positions.
         // (only claimants of repeated symbols have a count)
@@ -1866,6 +1867,10 @@ __device__ __forceinline__ int rounds_cost(int total, int schedulers, int warps)
 // rollouts of 1024 with inserted and deleted tokens, 2802 tasks: 419 -> 370 us; 700 of texts with 2 % edits, 4906 tasks, 714 -> 648).
 // (Over 30 shapes and nine kinds of batch 0.988 of the time without this, at worst 1.03 times it.  The order of
 // tasks dealt out to the end, with no pulling: texts 5 to 8 % slower.)
+// A CTA starts on an SM that is almost empty, so that tasks dealt to one which waits for another stream's kernel run after the
+// others: 1024 groups of texts that differ in 2 % of their places take 307 us, 323 next to matrix products of 2048 places, 392 while sixteen
+// SMs are held by a kernel that outlasts the call.  (Three CTAs of four warps, launched when the SMs were empty, took 392 alone, 450 next to the products and
+// did not start before the other kernel's end.)
 __global__ void __launch_bounds__(kMostDpWarps * 32, 1)
 multi_dp_kernel(unsigned char* ws, MultiWs W, int32_t* dist_out, uint32_t two) {
     grid_begin();
@@ -2248,7 +2253,10 @@ int launch_gate_multi(const GateArgs& a, void* ws_, size_t ws_bytes, cudaStream_
     const int blocks = n_pairs < sms ? n_pairs : sms;
     // (launched early like the others: one of its CTAs has the registers of most of an SM, so that no two can end up on one.  With the L1
     // that prep left, 1024 groups of 8 texts of 1024 over 100 symbols that differ in 2 % of their places took 973 us in the decide mode with d_K, 352 with
-    // all of it; a launch that waits for empty SMs costs every sorted call 2.5 us)
+    // all of it; a launch that waits for empty SMs costs every sorted call 2.5 us.  The SMs have to be empty once more for the names kernel of the next call: 2 us of 45
+    // for 400 groups in the mask-only mode whose bounds settle the batch, 1 us of 38 for 260, nothing for 1024 or for shorter prefixes.  Half or a quarter
+    // of the shared memory in place of none: no better than without, and the gate 10 % slower.  Bound, bin or order kernel asking in place of this one: the settled batches take as long
+    // or up to 5 % longer, the others gain half as much)
     const int rc = launch_how(LaunchHow{true, 1, true}, "multi_dp_kernel", multi_dp_kernel, blocks, kMostDpWarps * 32, 0, s, ws, W, dist, 2u);
     if (rc != SR_OK) return rc;
     if (ev) SR_CUDA_TRY(cudaEventRecord(ev[3], s));
